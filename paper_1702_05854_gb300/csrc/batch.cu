@@ -97,25 +97,7 @@ __global__ void __launch_bounds__(256, 4) k_sample_batch(BatchParams B) {
         const uint4 x = node_draw(a, v, I.k0, I.k1);
         const bool live = x.x < rec.w;
         uint4 ra = make_uint4(0, 0, 0, 0), rb = make_uint4(0, 0, 0, 0);
-        if (live) {
-          if (rec.z) {
-            const uint32_t e = rec.x + x.x / rec.z;
-            ra = __ldg(&I.erec[2 * (size_t)e]);
-            rb = __ldg(&I.erec[2 * (size_t)e + 1]);
-          } else {
-            const size_t gp = 2 * ((size_t)rec.x + guide_bucket(x.x, rec.y, rec.w));
-            ra = __ldg(&I.grec[gp]);
-            rb = __ldg(&I.grec[gp + 1]);
-            uint32_t e = rec.x + rb.z;
-            if (x.x >= rb.y) {
-              do {
-                ++e;
-                rb = __ldg(&I.erec[2 * (size_t)e + 1]);
-              } while (x.x >= rb.y);
-              ra = __ldg(&I.erec[2 * (size_t)e]);
-            }
-          }
-        }
+        if (live) record_step(I.erec, I.grec, rec, x.x, ra, rb);
         const bool suspect = (sw >> (v & 31)) & 1u;
         if (suspect && (!I.p32 || source_coin(x.y, __ldg(&I.p32[v])))) {
           outcome = 1;

@@ -102,25 +102,7 @@ __global__ void __launch_bounds__(256, 6) k_sample(const __grid_constant__ Sampl
         const bool live = x.x < rec.w;
         uint4 ra = make_uint4(0, 0, 0, 0), rb = make_uint4(0, 0, 0, 0);
         uint32_t e = 0;
-        if (live) {
-          if (rec.z) {  // equal weights: j = r / w
-            e = rec.x + x.x / rec.z;
-            ra = __ldg(&P.erec[2 * (size_t)e]);
-            rb = __ldg(&P.erec[2 * (size_t)e + 1]);
-          } else {  // the bucket's candidate record, then step through the walk records
-            const size_t gp = 2 * ((size_t)rec.x + guide_bucket(x.x, rec.y, rec.w));
-            ra = __ldg(&P.grec[gp]);
-            rb = __ldg(&P.grec[gp + 1]);
-            e = rec.x + rb.z;
-            if (x.x >= rb.y) {
-              do {
-                ++e;
-                rb = __ldg(&P.erec[2 * (size_t)e + 1]);
-              } while (x.x >= rb.y);
-              ra = __ldg(&P.erec[2 * (size_t)e]);
-            }
-          }
-        }
+        if (live) e = record_step(P.erec, P.grec, rec, x.x, ra, rb);
         const bool suspect = (sw >> (v & 31)) & 1u;
         if (suspect && (!HAS_P || source_coin(x.y, __ldg(&P.p32[v])))) {
           outcome = 1;
