@@ -31,6 +31,7 @@ struct BatchInst {
   uint32_t n_attempts;  // window size
   uint32_t n_chunks;
   uint32_t chunk0;      // first global chunk of the window
+  uint32_t eq;          // the graph's walk-record layout
   uint32_t cap;         // hit records per chunk (a few standard deviations above the expected hits)
   uint64_t rec0;        // first record of the window
 };
@@ -96,8 +97,12 @@ __global__ void __launch_bounds__(256, 4) k_sample_batch(BatchParams B) {
         const uint32_t sw = __ldg(&I.s_bits[v >> 5]);
         const uint4 x = node_draw(a, v, I.k0, I.k1);
         const bool live = x.x < rec.w;
-        uint4 ra = make_uint4(0, 0, 0, 0), rb = make_uint4(0, 0, 0, 0);
-        if (live) record_step(I.erec, I.grec, rec, x.x, ra, rb);
+        uint4 next = make_uint4(0, 0, 0, 0);
+        uint32_t u = 0;
+        if (live) {
+          if (I.eq) record_step<true>(I.erec, I.grec, rec, x.x, u, next);
+          else record_step<false>(I.erec, I.grec, rec, x.x, u, next);
+        }
         const bool suspect = (sw >> (v & 31)) & 1u;
         if (suspect && (!I.p32 || source_coin(x.y, __ldg(&I.p32[v])))) {
           outcome = 1;
@@ -106,13 +111,12 @@ __global__ void __launch_bounds__(256, 4) k_sample_batch(BatchParams B) {
           if (!live) {
             outcome = 0;
           } else {
-            const uint32_t u = ra.x;
             if (ck.seen(u)) {
               outcome = 0;
             } else {
               ck.keep(u, len);
               v = u;
-              rec = make_uint4(ra.y, ra.z, ra.w, rb.x);
+              rec = next;
               if (++len > I.step_cap) {
                 atomicOr(B.status, BST_STEP_CAP);
                 outcome = 0;
@@ -243,6 +247,7 @@ hsaw_status batch_sample(const Graph* const* gs, const QueryDev* const* qds, Str
       BatchInst b{};
       b.node = g.node;
       b.erec = g.erec;
+      b.eq = g.eq ? 1u : 0u;
       b.grec = g.grec;
       b.s_bits = qd.s_bits;
       b.p32 = qd.p32;

@@ -151,7 +151,8 @@ __global__ void k_copy_edges(const int32_t* __restrict__ src, const uint32_t* __
 }
 
 // One warp per node: running in-weight sums (exact, 64-bit carry), the in-sum check
-// (<= 2^32 - 1), equal-weight detection and the node record.
+// (<= 2^32 - 1), equal-weight detection and the node record.  err[1] counts the nodes with
+// in-weight whose in-weights differ.
 __global__ void k_thresholds(const uint32_t* __restrict__ row_start, int64_t n, uint2* __restrict__ edge,
                              uint4* __restrict__ node, uint32_t* __restrict__ err) {
   const int lane = threadIdx.x & 31;
@@ -183,31 +184,35 @@ __global__ void k_thresholds(const uint32_t* __restrict__ row_start, int64_t n, 
     if (lane == 0) {
       uint32_t insum = (uint32_t)(carry > 0xFFFFFFFFull ? 0xFFFFFFFFull : carry);
       node[v] = make_uint4(b, deg, (uniform && deg) ? w0 : 0u, insum);
+      if (!uniform && insum) atomicAdd(err + 1, 1u);
     }
   }
 }
 
-// 32-byte walk records (see Graph::erec).
+// Walk records (see Graph::erec).
+template <bool EQ>
 __global__ void k_walk_records(const uint2* __restrict__ edge, const uint4* __restrict__ node, int64_t m,
                                uint4* __restrict__ erec) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
     const uint2 ed = edge[e];
     const uint4 nu = node[ed.x];
-    erec[2 * e] = make_uint4(ed.x, nu.x, nu.y, nu.z);
-    erec[2 * e + 1] = make_uint4(nu.w, ed.y, 0u, 0u);
+    if (EQ) {
+      erec[e] = make_uint4(ed.x, nu.x, nu.y, nu.z);
+    } else {
+      erec[2 * e] = make_uint4(ed.x, nu.x, nu.y, nu.z);
+      erec[2 * e + 1] = make_uint4(nu.w, ed.y, 0u, 0u);
+    }
   }
 }
 
 // Guide tables of the nodes with unequal in-weights (see Graph::guide); one warp per node.
 __global__ void k_guide(const uint4* __restrict__ node, const uint2* __restrict__ edge, int64_t n,
-                        uint32_t* __restrict__ guide, uint32_t* __restrict__ n_unequal) {
+                        uint32_t* __restrict__ guide) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  uint32_t cnt = 0;
   for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
     const uint4 nd = node[v];
     if (nd.y == 0 || nd.z != 0 || nd.w == 0) continue;  // no in-edge, equal weights, or zero in-sum
-    cnt += lane == 0 ? 1u : 0u;
     for (uint32_t b = lane; b < nd.y; b += 32) {
       const uint32_t lb = (uint32_t)(((uint64_t)b * nd.w + nd.y - 1) / nd.y);  // ceil(b * insum / deg)
       uint32_t lo = 0, hi = nd.y;
@@ -218,7 +223,6 @@ __global__ void k_guide(const uint4* __restrict__ node, const uint2* __restrict_
       guide[nd.x + b] = lo;
     }
   }
-  if (cnt) atomicAdd(n_unequal, cnt);
 }
 
 // Bucket records of the nodes with unequal in-weights (see Graph::grec); one warp per node.
@@ -242,10 +246,13 @@ __global__ void k_guide_records(const uint4* __restrict__ node, const uint32_t* 
 }
 
 // ------------------------------------------------------------------ host
-static hsaw_status check_err(uint32_t* d_err, cudaStream_t s) {
-  uint32_t h = 0;
-  HSAW_CK(cudaMemcpyAsync(&h, d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+// d_err: error bits, then the count of unequal nodes (k_thresholds) into *unequal.
+static hsaw_status check_err(uint32_t* d_err, cudaStream_t s, uint32_t* unequal = nullptr) {
+  uint32_t word[2] = {0, 0};
+  HSAW_CK(cudaMemcpyAsync(word, d_err, sizeof(word), cudaMemcpyDeviceToHost, s));
   HSAW_CK(cudaStreamSynchronize(s));
+  const uint32_t h = word[0];
+  if (unequal) *unequal = word[1];
   if (h & ERR_RANGE) return fail(HSAW_E_RANGE, "graph: a node index is outside [0, n)");
   if (h & ERR_ROWPTR) return fail(HSAW_E_INVALID, "graph: in_row_ptr is not a valid CSR offset array");
   if (h & ERR_WEIGHT) return fail(HSAW_E_WEIGHT_SUM, "graph: a node's in-weight sum exceeds 2^32 - 1");
@@ -303,7 +310,6 @@ static hsaw_status alloc_graph(Graph& g, int64_t n, int64_t m, bool with_index) 
   cudaGetDevice(&g.device);
   HSAW_CK(cudaMalloc((void**)&g.node, (size_t)n * sizeof(uint4)));
   HSAW_CK(cudaMalloc((void**)&g.edge, (size_t)(m ? m : 1) * sizeof(uint2)));
-  HSAW_CK(cudaMalloc((void**)&g.erec, (size_t)(m ? m : 1) * 2 * sizeof(uint4)));
   if (with_index) HSAW_CK(cudaMalloc((void**)&g.input_index, (size_t)(m ? m : 1) * sizeof(int64_t)));
   return HSAW_OK;
 }
@@ -348,39 +354,38 @@ static hsaw_status finish_graph(Graph& g, uint32_t* row_start, uint32_t* d_err, 
   count_launch();
   k_thresholds<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(row_start, n, g.edge, g.node, d_err);
   HSAW_CK(cudaGetLastError());
-  HSAW_TRY(check_err(d_err, s));
-  if (g.m) {
-    count_launch();
-    k_walk_records<<<grid_for(g.m, 256, 1u << 16), 256, 0, s>>>(g.edge, g.node, g.m, g.erec);
+  uint32_t unequal = 0;
+  HSAW_TRY(check_err(d_err, s, &unequal));
+  if (!g.m) return HSAW_OK;
+  g.eq = unequal == 0;
+  HSAW_CK(cudaMalloc((void**)&g.erec, (size_t)g.m * (g.eq ? 1 : 2) * sizeof(uint4)));
+  count_launch();
+  if (g.eq) {
+    k_walk_records<true><<<grid_for(g.m, 256, 1u << 16), 256, 0, s>>>(g.edge, g.node, g.m, g.erec);
     HSAW_CK(cudaGetLastError());
-    // guide tables and their bucket records, kept only when some node has unequal
-    // in-weights (the guide itself is a temporary)
-    uint32_t* guide = nullptr;
-    HSAW_TRY(dmalloc((void**)&guide, (size_t)g.m * sizeof(uint32_t), s));
-    HSAW_CK(cudaMemsetAsync(d_err, 0, sizeof(uint32_t), s));
-    count_launch();
-    k_guide<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(g.node, g.edge, n, guide, d_err);
-    uint32_t unequal = 0;
-    hsaw_status st = HSAW_OK;
-    if (cudaGetLastError() != cudaSuccess ||
-        cudaMemcpyAsync(&unequal, d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-      st = fail(HSAW_E_DEVICE, "graph: guide tables failed");
-    if (st == HSAW_OK && unequal) {
-      if (cudaMalloc((void**)&g.grec, (size_t)g.m * 2 * sizeof(uint4)) != cudaSuccess) {
-        cudaGetLastError();
-        g.grec = nullptr;
-        st = fail(HSAW_E_NOMEM, "graph: guide records do not fit in device memory");
-      } else {
-        count_launch();
-        k_guide_records<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(g.node, guide, n, g.erec, g.grec);
-        if (cudaGetLastError() != cudaSuccess) st = fail(HSAW_E_DEVICE, "graph: guide records failed");
-      }
-    }
-    dfree(guide, s);
-    HSAW_TRY(st);
+    return HSAW_OK;
   }
-  return HSAW_OK;
+  k_walk_records<false><<<grid_for(g.m, 256, 1u << 16), 256, 0, s>>>(g.edge, g.node, g.m, g.erec);
+  HSAW_CK(cudaGetLastError());
+  // guide tables (a temporary) and their bucket records
+  if (cudaMalloc((void**)&g.grec, (size_t)g.m * 2 * sizeof(uint4)) != cudaSuccess) {
+    cudaGetLastError();
+    g.grec = nullptr;
+    return fail(HSAW_E_NOMEM, "graph: guide records do not fit in device memory");
+  }
+  uint32_t* guide = nullptr;
+  HSAW_TRY(dmalloc((void**)&guide, (size_t)g.m * sizeof(uint32_t), s));
+  hsaw_status st = HSAW_OK;
+  count_launch();
+  k_guide<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(g.node, g.edge, n, guide);
+  if (cudaGetLastError() != cudaSuccess) st = fail(HSAW_E_DEVICE, "graph: guide tables failed");
+  if (st == HSAW_OK) {
+    count_launch();
+    k_guide_records<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(g.node, guide, n, g.erec, g.grec);
+    if (cudaGetLastError() != cudaSuccess) st = fail(HSAW_E_DEVICE, "graph: guide records failed");
+  }
+  dfree(guide, s);
+  return st;
 }
 
 static hsaw_status from_edges(int64_t n, int64_t m, const int32_t* src, const int32_t* dst, const uint32_t* w,
@@ -406,8 +411,8 @@ static hsaw_status from_edges(int64_t n, int64_t m, const int32_t* src, const in
   HSAW_TRY(stage(dst, (size_t)m, dev, s, &d_dst, &o2));
   if (o2) T.keep(d_dst);
   uint32_t* d_err = nullptr;
-  HSAW_TRY(T.get(&d_err, 1));
-  HSAW_CK(cudaMemsetAsync(d_err, 0, sizeof(uint32_t), s));
+  HSAW_TRY(T.get(&d_err, 2));
+  HSAW_CK(cudaMemsetAsync(d_err, 0, 2 * sizeof(uint32_t), s));
   if (m) {
     count_launch();
     k_validate_nodes<<<grid_for(m, 256, 8192), 256, 0, s>>>(d_dst, m, n, d_err);
@@ -475,9 +480,9 @@ static hsaw_status from_csr(int64_t n, int64_t m, const int64_t* rp, const int32
   HSAW_TRY(stage(w, (size_t)m, dev, s, &d_w, &o3));
   if (o3) T.keep(d_w);
   uint32_t *d_err, *row_start;
-  HSAW_TRY(T.get(&d_err, 1));
+  HSAW_TRY(T.get(&d_err, 2));
   HSAW_TRY(T.get(&row_start, n + 1));
-  HSAW_CK(cudaMemsetAsync(d_err, 0, sizeof(uint32_t), s));
+  HSAW_CK(cudaMemsetAsync(d_err, 0, 2 * sizeof(uint32_t), s));
   count_launch();
   k_csr_rows<<<grid_for(n + 1, 256, 8192), 256, 0, s>>>(d_rp, n, m, row_start, d_err);
   HSAW_CK(cudaGetLastError());

@@ -175,7 +175,7 @@ __global__ void k_bits_emit(const uint32_t* __restrict__ bits, const uint32_t* _
 
 // Length of each pooled hit: nodes walked up to and including its first real source.  A
 // walk that meets no source first (impossible for an attempt the index lists) sets bit 2.
-template <bool HAS_P>
+template <bool HAS_P, bool EQ>
 __global__ void k_hit_len(const uint4* __restrict__ node, const uint4* __restrict__ erec, const uint4* __restrict__ grec,
                           uint32_t n, uint32_t k0, uint32_t k1, const uint32_t* __restrict__ s_bits,
                           const uint32_t* __restrict__ p32, const uint64_t* __restrict__ aid, uint32_t count,
@@ -191,10 +191,7 @@ __global__ void k_hit_len(const uint4* __restrict__ node, const uint4* __restric
         atomicOr(status, 2u);
         break;
       }
-      uint4 ra, rb;
-      record_step(erec, grec, rec, x.x, ra, rb);
-      v = ra.x;
-      rec = make_uint4(ra.y, ra.z, ra.w, rb.x);
+      record_step<EQ>(erec, grec, rec, x.x, v, rec);
       ++l;
     }
     len[h] = l;
@@ -331,14 +328,10 @@ hsaw_status pool_hits(const Graph& g, const QueryDev& qd, Stream& st, uint64_t a
   HSAW_CK(cudaGetLastError());
   const unsigned hgrid = grid_for(h, 128, 1u << 16);
   count_launch();
-  if (qd.p32)
-    k_hit_len<true><<<hgrid, 128, 0, s>>>(g.node, g.erec, g.grec, (uint32_t)g.n, k0, k1, qd.s_bits, qd.p32,
-                                          st.aid.p + st.count, h, pool_step_cap(g), st.len.p + st.count,
-                                          st.ctrs.p + 3);
-  else
-    k_hit_len<false><<<hgrid, 128, 0, s>>>(g.node, g.erec, g.grec, (uint32_t)g.n, k0, k1, qd.s_bits, nullptr,
-                                           st.aid.p + st.count, h, pool_step_cap(g), st.len.p + st.count,
-                                           st.ctrs.p + 3);
+  const auto hit_len = qd.p32 ? (g.eq ? k_hit_len<true, true> : k_hit_len<true, false>)
+                              : (g.eq ? k_hit_len<false, true> : k_hit_len<false, false>);
+  hit_len<<<hgrid, 128, 0, s>>>(g.node, g.erec, g.grec, (uint32_t)g.n, k0, k1, qd.s_bits, qd.p32, st.aid.p + st.count, h,
+                                pool_step_cap(g), st.len.p + st.count, st.ctrs.p + 3);
   HSAW_CK(cudaGetLastError());
   uint32_t bad = 0;
   HSAW_CK(cudaMemcpyAsync(&bad, st.ctrs.p + 3, 4, cudaMemcpyDeviceToHost, s));

@@ -38,7 +38,7 @@ struct SampleParams {
   uint32_t k0, k1;
   uint64_t a0;           // first attempt of this launch
   uint32_t n_attempts;   // attempts in this launch
-  uint32_t chunk;        // attempts per chunk
+  uint32_t chunk_shift;  // chunks of 2^chunk_shift attempts
   uint32_t n_chunks;
   uint32_t cap;          // hit records per chunk
   uint32_t step_cap;
@@ -49,89 +49,123 @@ struct SampleParams {
   PhiloxKeys keys;       // round keys of (k0, k1)
 };
 
-template <bool HAS_P, bool HAS_REM>
-__global__ void __launch_bounds__(256, 6) k_sample(const __grid_constant__ SampleParams P) {
+// A warp draws the starts of its attempts 32 at a time, with every lane, into a buffer in
+// shared memory, and its lanes take their next attempt from there: the start draw and the
+// node record's latency are paid once per 32 attempts instead of in nearly every iteration
+// for the few lanes whose walk just ended.  A start at a node without in-weight that is no
+// suspect ends there, without a draw, and never takes a lane (half the nodes of an R-MAT
+// graph).  The next chunk is claimed one chunk ahead, so no warp waits for the counter.
+// Measured with the 16-byte records: 16 K-node Chung-Lu graph (L2-resident, bound by the ALU
+// and issue) 8.48 -> 6.50 ms per 200 K-hit solve; R-MAT 20 with unequal weights 281 -> 239 ms
+// per 1 M hits.  One loop that drew starts and live edges in the same Philox block instead
+// cost 10-23% more than refilling each lane by itself (fewer lanes active per instruction).
+constexpr int SAMPLE_WARPS = 8;
+constexpr int START_SLOTS = 64;  // at most 31 left when 32 more are drawn
+
+template <bool HAS_P, bool HAS_REM, bool EQ>
+__global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_constant__ SampleParams P) {
+  __shared__ uint4 start_rec[SAMPLE_WARPS][START_SLOTS];  // node record of the start
+  __shared__ uint2 start_at[SAMPLE_WARPS][START_SLOTS];   // attempt (within the launch), start node
   const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   uint32_t cur = 0, cur_end = 0;  // warp's attempt cursor within the launch
+  uint32_t ahead = 0;             // lane 0: the next chunk
+  if (lane == 0) ahead = atomicAdd(P.chunk_ctr, 1u);
+  uint32_t ready = 0;  // starts in the buffer
   bool more = true;
   bool active = false;
   uint32_t off = 0, v = 0, len = 0;
   uint4 rec = make_uint4(0, 0, 0, 0);  // node record of v: first in-edge, in-degree, equal weight, in-sum
   Ckpt ck;
   ck.reset(0);
-  unsigned long long my_steps = 0;
+  uint32_t my_steps = 0;
   for (;;) {
-    unsigned need = __ballot_sync(FULL, !active);
-    while (need) {
-      if (cur >= cur_end) {
-        if (!more) break;
-        uint32_t c = 0;
-        if (lane == 0) c = atomicAdd(P.chunk_ctr, 1u);
-        c = __shfl_sync(FULL, c, 0);
-        if (c >= P.n_chunks) { more = false; break; }
-        cur = c * P.chunk;
-        cur_end = min(cur + P.chunk, P.n_attempts);
-      }
-      const uint32_t avail = cur_end - cur;
-      const uint32_t rank = __popc(need & lt);
-      if (!active && rank < avail) {
-        off = cur + rank;
-        {
-          const uint64_t a = P.a0 + off;
-          v = __umulhi(philox4x32_10_rk(make_uint4((uint32_t)a, (uint32_t)(a >> 32), 0u, 1u), P.keys).x, P.n);
+    const unsigned need = __ballot_sync(FULL, !active);
+    if (need) {
+      const uint32_t want = __popc(need);
+      while (ready < want) {
+        if (cur >= cur_end) {
+          if (!more) break;
+          const uint32_t c = __shfl_sync(FULL, ahead, 0);
+          more = c < P.n_chunks;
+          if (!more) break;
+          cur = c << P.chunk_shift;
+          cur_end = min(cur + (1u << P.chunk_shift), P.n_attempts);
+          if (lane == 0) ahead = atomicAdd(P.chunk_ctr, 1u);
         }
-        rec = __ldg(&P.node[v]);
+        const uint32_t i = cur + lane;
+        bool walk = false;
+        uint32_t sv = 0;
+        uint4 srec = make_uint4(0, 0, 0, 0);
+        if (i < cur_end) {
+          const uint64_t a = P.a0 + i;
+          sv = __umulhi(philox4x32_10_rk(make_uint4((uint32_t)a, (uint32_t)(a >> 32), 0u, 1u), P.keys).x, P.n);
+          srec = __ldg(&P.node[sv]);
+          walk = ((__ldg(&P.s_bits[sv >> 5]) >> (sv & 31)) & 1u) || srec.w != 0;
+          if (HAS_REM && P.node_removed && P.node_removed[sv]) walk = false;
+        }
+        const unsigned got = __ballot_sync(FULL, walk);
+        if (walk) {
+          const uint32_t slot = ready + __popc(got & lt);
+          start_at[w][slot] = make_uint2(i, sv);
+          start_rec[w][slot] = srec;
+        }
+        ready += __popc(got);
+        cur = min(cur + 32u, cur_end);
+      }
+      __syncwarp();
+      const uint32_t take = min(want, ready);
+      if (take == 0 && need == FULL) break;
+      const uint32_t rank = __popc(need & lt);
+      if (!active && rank < take) {
+        const uint32_t slot = ready - 1 - rank;
+        const uint2 at = start_at[w][slot];
+        rec = start_rec[w][slot];
+        off = at.x;
+        v = at.y;
         ck.reset(v);
         len = 1;
         active = true;
       }
-      cur += min((uint32_t)__popc(need), avail);
-      need = __ballot_sync(FULL, !active);
+      ready -= take;
+      __syncwarp();  // slots are read before they are filled again
     }
-    if (!__any_sync(FULL, active)) break;
     if (active) {
       // one live-edge draw at node v (Alg. 1 lines 5-13); the tail's record comes with it
       const uint64_t a = P.a0 + off;
+      const uint32_t sw = __ldg(&P.s_bits[v >> 5]);
+      const uint4 x = philox4x32_10_rk(make_uint4((uint32_t)a, (uint32_t)(a >> 32), v, 0u), P.keys);
+      const bool live = x.x < rec.w;
+      uint4 next = make_uint4(0, 0, 0, 0);
+      uint32_t e = 0, u = 0;
+      if (live) e = record_step<EQ>(P.erec, P.grec, rec, x.x, u, next);
+      const bool suspect = (sw >> (v & 31)) & 1u;
       int outcome = -1;  // -1 continue, 0 miss, 1 hit
-      if (HAS_REM && len == 1 && P.node_removed && P.node_removed[v]) outcome = 0;
-      if (outcome < 0) {
-        const uint32_t sw = __ldg(&P.s_bits[v >> 5]);
-        const uint4 x = philox4x32_10_rk(make_uint4((uint32_t)a, (uint32_t)(a >> 32), v, 0u), P.keys);
-        const bool live = x.x < rec.w;
-        uint4 ra = make_uint4(0, 0, 0, 0), rb = make_uint4(0, 0, 0, 0);
-        uint32_t e = 0;
-        if (live) e = record_step(P.erec, P.grec, rec, x.x, ra, rb);
-        const bool suspect = (sw >> (v & 31)) & 1u;
-        if (suspect && (!HAS_P || source_coin(x.y, __ldg(&P.p32[v])))) {
-          outcome = 1;
+      if (suspect && (!HAS_P || source_coin(x.y, __ldg(&P.p32[v])))) {
+        outcome = 1;
+      } else {
+        ++my_steps;
+        if (!live) {
+          outcome = 0;  // no live in-edge
+        } else if (HAS_REM && ((P.edge_removed && P.edge_removed[e]) || (P.node_removed && P.node_removed[u]))) {
+          outcome = 0;
+        } else if (ck.seen(u)) {
+          outcome = 0;  // the walk closed a cycle
         } else {
-          ++my_steps;
-          if (!live) {
-            outcome = 0;  // no live in-edge
-          } else {
-            const uint32_t u = ra.x;
-            if (HAS_REM && ((P.edge_removed && P.edge_removed[e]) || (P.node_removed && P.node_removed[u]))) {
-              outcome = 0;
-            } else if (ck.seen(u)) {
-              outcome = 0;  // the walk closed a cycle
-            } else {
-              ck.keep(u, len);
-              v = u;
-              rec = make_uint4(ra.y, ra.z, ra.w, rb.x);
-              if (++len > P.step_cap) {
-                atomicOr(P.chunk_ctr + 1, ST_STEP_CAP);
-                outcome = 0;
-              }
-            }
+          ck.keep(u, len);
+          v = u;
+          rec = next;
+          if (++len > P.step_cap) {
+            atomicOr(P.chunk_ctr + 1, ST_STEP_CAP);
+            outcome = 0;
           }
         }
       }
       if (outcome >= 0) {
         active = false;
         if (outcome == 1) {
-          const uint32_t ck_i = off / P.chunk;
+          const uint32_t ck_i = off >> P.chunk_shift;
           const uint32_t slot = atomicAdd(&P.chunk_hits[ck_i], 1u);
           if (slot < P.cap) P.recs[(size_t)ck_i * P.cap + slot] = make_uint2(off, len);
           else atomicOr(P.chunk_ctr + 1, ST_OVERFLOW);
@@ -140,9 +174,10 @@ __global__ void __launch_bounds__(256, 6) k_sample(const __grid_constant__ Sampl
     }
   }
   // steps of this warp
+  unsigned long long warp_steps = my_steps;
 #pragma unroll
-  for (int o = 16; o; o >>= 1) my_steps += __shfl_down_sync(FULL, my_steps, o);
-  if (lane == 0 && my_steps) atomicAdd(P.steps, my_steps);
+  for (int o = 16; o; o >>= 1) warp_steps += __shfl_down_sync(FULL, warp_steps, o);
+  if (lane == 0 && warp_steps) atomicAdd(P.steps, warp_steps);
 }
 
 // Order each chunk's hits by attempt id and write them at the chunk's scanned offset.
@@ -183,6 +218,7 @@ __global__ void k_offsets(const uint64_t* __restrict__ excl, int64_t n, int64_t 
 }
 
 // Re-derive hit walks from their attempt ids (path encoding) into the flat buffers.
+template <bool EQ>
 __global__ void k_rewalk(const uint4* __restrict__ node, const uint4* __restrict__ erec, const uint4* __restrict__ grec,
                          uint32_t n, uint32_t k0, uint32_t k1, const uint64_t* __restrict__ aid,
                          const uint32_t* __restrict__ len, const int64_t* __restrict__ node_off, int64_t h0, int64_t h1,
@@ -197,12 +233,8 @@ __global__ void k_rewalk(const uint4* __restrict__ node, const uint4* __restrict
     for (uint32_t i = 1; i < l; ++i) {
       const uint4 x = node_draw(a, v, k0, k1);
       if (x.x >= rec.w) break;  // a hit's walk has a live in-edge at each of its first l - 1 nodes
-      uint4 ra, rb;
-      const uint32_t e = record_step(erec, grec, rec, x.x, ra, rb);
-      nodes[nb + i] = (int32_t)ra.x;
-      edges[eb + i - 1] = (int32_t)e;
-      v = ra.x;
-      rec = make_uint4(ra.y, ra.z, ra.w, rb.x);
+      edges[eb + i - 1] = (int32_t)record_step<EQ>(erec, grec, rec, x.x, v, rec);
+      nodes[nb + i] = (int32_t)v;
     }
   }
 }
@@ -337,7 +369,7 @@ static SampleParams make_params(const Graph& g, const QueryDev& qd) {
 static int sample_blocks_per_sm() {
   static const int cached = [] {
     int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sample<false, false>, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sample<false, false, true>, 256, 0);
     return b > 0 ? b : 1;
   }();
   return cached;
@@ -399,12 +431,19 @@ static void sample_tune_record(const Graph& g, int trial, double draws, float ms
             t.rate[1] / 1e6);
 }
 
-static void launch_sample(const SampleParams& P, unsigned grid, cudaStream_t s) {
+template <bool EQ>
+static void launch_sample_as(const SampleParams& P, unsigned grid, cudaStream_t s) {
   const bool hp = P.p32 != nullptr, hr = (P.edge_removed || P.node_removed);
-  if (hp && hr) { count_launch(); k_sample<true, true><<<grid, 256, 0, s>>>(P); }
-  else if (hp) { count_launch(); k_sample<true, false><<<grid, 256, 0, s>>>(P); }
-  else if (hr) { count_launch(); k_sample<false, true><<<grid, 256, 0, s>>>(P); }
-  else { count_launch(); k_sample<false, false><<<grid, 256, 0, s>>>(P); }
+  count_launch();
+  if (hp && hr) k_sample<true, true, EQ><<<grid, 256, 0, s>>>(P);
+  else if (hp) k_sample<true, false, EQ><<<grid, 256, 0, s>>>(P);
+  else if (hr) k_sample<false, true, EQ><<<grid, 256, 0, s>>>(P);
+  else k_sample<false, false, EQ><<<grid, 256, 0, s>>>(P);
+}
+
+static void launch_sample(const Graph& g, const SampleParams& P, unsigned grid, cudaStream_t s) {
+  if (g.eq) launch_sample_as<true>(P, grid, s);
+  else launch_sample_as<false>(P, grid, s);
 }
 
 // One sampler launch over attempts [st.next_attempt, + batch): hits are recorded per chunk
@@ -412,7 +451,7 @@ static void launch_sample(const SampleParams& P, unsigned grid, cudaStream_t s) 
 static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st, uint64_t batch, uint32_t* new_hits,
                                  cudaStream_t s) {
   SampleParams P = make_params(g, qd);
-  const uint32_t CHUNK = 256;
+  const uint32_t SHIFT = 8, CHUNK = 1u << SHIFT;
   const uint32_t n_chunks = (uint32_t)((batch + CHUNK - 1) / CHUNK);
   // records per chunk: a few standard deviations above the expected hits, else all
   double exp_hits = std::max(st.hit_rate, 0.0) * CHUNK;
@@ -429,7 +468,7 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
     HSAW_CK(cudaMemsetAsync(d_steps, 0, 8, s));
     P.a0 = st.next_attempt;
     P.n_attempts = (uint32_t)batch;
-    P.chunk = CHUNK;
+    P.chunk_shift = SHIFT;
     P.n_chunks = n_chunks;
     P.cap = cap;
     P.chunk_ctr = st.ctrs.p;
@@ -446,7 +485,7 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
     }
     if (trial >= 0) cudaEventRecord(tev[0], s);
     void* prof = profile_begin(s);
-    launch_sample(P, grid, s);
+    launch_sample(g, P, grid, s);
     profile_end(prof, s, batch);
     if (trial >= 0) cudaEventRecord(tev[1], s);
     HSAW_CK(cudaGetLastError());
@@ -550,11 +589,11 @@ hsaw_status stream_take_hits(const Graph& g, const QueryDev& qd, Stream& st, uin
   const int64_t tot = st.total_nodes + (int64_t)added;
   HSAW_TRY(st.nodes.ensure((size_t)tot, s, true));
   HSAW_TRY(st.edges.ensure((size_t)tot, s, true));
+  const unsigned grid = grid_for(new_hits, 128, 1u << 16);
+  const auto rewalk = g.eq ? k_rewalk<true> : k_rewalk<false>;
   count_launch();
-  k_rewalk<<<grid_for(new_hits, 128, 1u << 16), 128, 0, s>>>(g.node, g.erec, g.grec, (uint32_t)g.n, k0, k1, st.aid.p,
-                                                               st.len.p,
-                                                               st.node_off.p, st.count, st.count + new_hits,
-                                                               st.nodes.p, st.edges.p);
+  rewalk<<<grid, 128, 0, s>>>(g.node, g.erec, g.grec, (uint32_t)g.n, k0, k1, st.aid.p, st.len.p, st.node_off.p, st.count,
+                              st.count + new_hits, st.nodes.p, st.edges.p);
   HSAW_CK(cudaGetLastError());
   st.total_nodes = tot;
   st.count += new_hits;
@@ -593,7 +632,8 @@ hsaw_status classify_attempts(const Graph& g, const QueryDev& qd, uint64_t first
 // addresses are looked up once per device with cudaGetSymbolAddress.
 namespace hsaw {
 
-constexpr uint32_t STATIC_CHUNK = 256;
+constexpr uint32_t STATIC_SHIFT = 8;
+constexpr uint32_t STATIC_CHUNK = 1u << STATIC_SHIFT;
 constexpr uint32_t STATIC_CHUNKS = HSAW_STATIC_MAX_ATTEMPTS / STATIC_CHUNK;
 
 static __device__ __align__(256) uint32_t g_static_ctrs[8];                 // work counter, status, total
@@ -695,7 +735,7 @@ extern "C" hsaw_status hsaw_sample_hits_static(hsaw_graph g, const uint32_t* sus
   const uint32_t n_chunks = (uint32_t)((n_attempts + STATIC_CHUNK - 1) / STATIC_CHUNK);
   P.a0 = first_attempt;
   P.n_attempts = (uint32_t)n_attempts;
-  P.chunk = STATIC_CHUNK;
+  P.chunk_shift = STATIC_SHIFT;
   P.n_chunks = n_chunks;
   P.cap = STATIC_CHUNK;  // room for every attempt of a chunk to hit: no overflow
   P.chunk_ctr = sc->ctrs;
@@ -708,8 +748,7 @@ extern "C" hsaw_status hsaw_sample_hits_static(hsaw_graph g, const uint32_t* sus
   HSAW_CK(cudaMemsetAsync(sc->chunk_hits, 0, (size_t)n_chunks * sizeof(uint32_t), s));
   const unsigned grid = (unsigned)std::max(1, std::min<int>(sm_count() * sample_blocks_per_sm(),
                                                              (int)((n_chunks + 7) / 8)));
-  count_launch();
-  k_sample<false, false><<<grid, 256, 0, s>>>(P);
+  launch_sample(G, P, grid, s);
   HSAW_CK(cudaGetLastError());
   count_launch();
   k_static_scan<<<1, 1024, 0, s>>>(sc->chunk_hits, n_chunks, STATIC_CHUNK, sc->chunk_off, sc->ctrs + 2);
