@@ -245,6 +245,21 @@ __device__ __forceinline__ void load_record(const uint4* __restrict__ p, uint4& 
       : "l"(p));
 }
 
+// floor(r / w), w >= 1, from a float estimate that is never above it: the conversions, the
+// factor and the approximate quotient (2 ulp) are off by less than 2^-20 together, which the
+// factor takes off, so the estimate is the quotient or, below 2^19, at most one less.  About
+// half the instructions of the integer division.
+__device__ __forceinline__ uint32_t quotient(uint32_t r, uint32_t w) {
+  uint32_t q = __float2uint_rz(__fdividef(__uint2float_rn(r) * (1.0f - 0x1p-20f), __uint2float_rn(w)));
+  uint32_t rem = r - q * w;
+  if (rem >= w) {
+    ++q;
+    rem -= w;
+    if (rem >= w) q = r / w;
+  }
+  return q;
+}
+
 // The live in-edge e of a node with record rec = {first in-edge, in-degree, equal weight or
 // 0, in-sum} for a draw r < rec.w, read through the walk records (the same choice as
 // pick_in_edge: j = r / w at equal weights, otherwise the first j with r < thr[j], found
@@ -253,7 +268,7 @@ template <bool EQ>
 __device__ __forceinline__ uint32_t record_step(const uint4* __restrict__ erec, const uint4* __restrict__ grec,
                                                 uint4 rec, uint32_t r, uint32_t& u, uint4& next) {
   if (EQ) {
-    const uint32_t e = rec.x + r / rec.z;
+    const uint32_t e = rec.x + quotient(r, rec.z);
     const uint4 x = __ldg(&erec[e]);
     u = x.x;
     next = make_uint4(x.y, x.z, x.w, x.z * x.w);
@@ -262,7 +277,7 @@ __device__ __forceinline__ uint32_t record_step(const uint4* __restrict__ erec, 
   uint32_t e;
   uint4 ra, rb;
   if (rec.z) {
-    e = rec.x + r / rec.z;
+    e = rec.x + quotient(r, rec.z);
     load_record(erec + 2 * (size_t)e, ra, rb);
   } else {
     load_record(grec + 2 * ((size_t)rec.x + guide_bucket(r, rec.y, rec.w)), ra, rb);
