@@ -54,6 +54,15 @@ static hsaw_status upload_mask(const uint8_t* mask, size_t len, bool on_device, 
   return HSAW_OK;
 }
 
+// The bits of an optional removal mask of len bytes.
+static hsaw_status upload_removed(const uint8_t* mask, size_t len, bool on_device, cudaStream_t s, uint32_t** bits) {
+  uint8_t* bytes = nullptr;
+  hsaw_status st = upload_mask(mask, len, on_device, s, &bytes);
+  if (st == HSAW_OK && bytes) st = pack_mask(bytes, len, bits, s);
+  dfree(bytes, s);
+  return st;
+}
+
 static hsaw_status validate_common(const Graph& g, const hsaw_query* q, int64_t* n_cand) {
   if (q->mode != HSAW_EDGE && q->mode != HSAW_NODE) return fail(HSAW_E_INVALID, "query: unknown mode");
   const int64_t M = q->mode == HSAW_EDGE ? g.m : g.n;
@@ -252,8 +261,8 @@ hsaw_status hsaw_sample(hsaw_graph g, const hsaw_query* q, uint64_t first_attemp
   cudaGetDevice(&w->device);
   hsaw_status st = query_upload(g->g, q, w->qd, s);
   const bool dev = removed_flags & HSAW_INPUT_DEVICE;
-  if (st == HSAW_OK) st = upload_mask(edge_removed, (size_t)g->g.m, dev, s, &w->qd.edge_removed);
-  if (st == HSAW_OK) st = upload_mask(node_removed, (size_t)g->g.n, dev, s, &w->qd.node_removed);
+  if (st == HSAW_OK) st = upload_removed(edge_removed, (size_t)g->g.m, dev, s, &w->qd.edge_removed);
+  if (st == HSAW_OK) st = upload_removed(node_removed, (size_t)g->g.n, dev, s, &w->qd.node_removed);
   w->qd.owns_removed = true;
   if (st == HSAW_OK) st = stream_init(w->st, first_attempt, q->max_attempts, s);
   if (st == HSAW_OK) st = stream_extend(g->g, w->qd, w->st, n_hits, s);
@@ -271,8 +280,9 @@ hsaw_status hsaw_sample(hsaw_graph g, const hsaw_query* q, uint64_t first_attemp
   return HSAW_OK;
 }
 
-__global__ void k_mark_removed(const int64_t* __restrict__ ids, int32_t cnt, uint8_t* __restrict__ mask) {
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) mask[ids[i]] = 1;
+__global__ void k_mark_removed(const int64_t* __restrict__ ids, int32_t cnt, uint32_t* __restrict__ bits) {
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x)
+    atomicOr(&bits[ids[i] >> 5], 1u << (ids[i] & 31));
 }
 
 hsaw_status hsaw_estimate_spread(hsaw_graph g, const hsaw_query* q, const int64_t* removed, int32_t n_removed,
@@ -288,12 +298,13 @@ hsaw_status hsaw_estimate_spread(hsaw_graph g, const hsaw_query* q, const int64_
   SolveScratch W(s);
   HSAW_TRY(query_upload(G, q, W.qd, s));
   if (n_removed > 0) {
-    uint8_t* mask = nullptr;
+    uint32_t* mask = nullptr;
     int64_t* d_ids = nullptr;
-    HSAW_TRY(dmalloc((void**)&mask, (size_t)M, s));
+    const size_t bytes = ((size_t)M + 31) / 32 * 4;
+    HSAW_TRY(dmalloc((void**)&mask, bytes, s));
     (edges ? W.qd.edge_removed : W.qd.node_removed) = mask;
     W.qd.owns_removed = true;
-    HSAW_CK(cudaMemsetAsync(mask, 0, (size_t)M, s));
+    HSAW_CK(cudaMemsetAsync(mask, 0, bytes, s));
     HSAW_TRY(dmalloc((void**)&d_ids, (size_t)n_removed * 8, s));
     HSAW_CK(cudaMemcpyAsync(d_ids, removed, (size_t)n_removed * 8, cudaMemcpyHostToDevice, s));
     count_launch();

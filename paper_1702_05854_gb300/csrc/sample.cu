@@ -32,8 +32,8 @@ struct SampleParams {
   const uint4* __restrict__ grec;
   const uint32_t* __restrict__ s_bits;
   const uint32_t* __restrict__ p32;
-  const uint8_t* __restrict__ edge_removed;
-  const uint8_t* __restrict__ node_removed;
+  const uint32_t* __restrict__ edge_removed;
+  const uint32_t* __restrict__ node_removed;
   uint32_t n;
   uint32_t k0, k1;
   uint64_t a0;           // first attempt of this launch
@@ -48,6 +48,10 @@ struct SampleParams {
   unsigned long long* steps;
   PhiloxKeys keys;       // round keys of (k0, k1)
 };
+
+__device__ __forceinline__ bool bit_at(const uint32_t* __restrict__ bits, uint32_t x) {
+  return (__ldg(&bits[x >> 5]) >> (x & 31)) & 1u;
+}
 
 // A warp draws the starts of its attempts 32 at a time, with every lane, into a buffer in
 // shared memory, and its lanes take their next attempt from there: the start draw and the
@@ -102,8 +106,8 @@ __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_co
           const uint64_t a = P.a0 + i;
           sv = __umulhi(philox4x32_10_rk(make_uint4((uint32_t)a, (uint32_t)(a >> 32), 0u, 1u), P.keys).x, P.n);
           srec = __ldg(&P.node[sv]);
-          walk = ((__ldg(&P.s_bits[sv >> 5]) >> (sv & 31)) & 1u) || srec.w != 0;
-          if (HAS_REM && P.node_removed && P.node_removed[sv]) walk = false;
+          walk = bit_at(P.s_bits, sv) || srec.w != 0;
+          if (HAS_REM && P.node_removed && bit_at(P.node_removed, sv)) walk = false;
         }
         const unsigned got = __ballot_sync(FULL, walk);
         if (walk) {
@@ -140,6 +144,8 @@ __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_co
       uint4 next = make_uint4(0, 0, 0, 0);
       uint32_t e = 0, u = 0;
       if (live) e = record_step<EQ>(P.erec, P.grec, rec, x.x, u, next);
+      bool gone = false;  // the removal bit is read beside the walk record
+      if (HAS_REM && live && P.edge_removed) gone = bit_at(P.edge_removed, e);
       const bool suspect = (sw >> (v & 31)) & 1u;
       int outcome = -1;  // -1 continue, 0 miss, 1 hit
       if (suspect && (!HAS_P || source_coin(x.y, __ldg(&P.p32[v])))) {
@@ -148,7 +154,7 @@ __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_co
         ++my_steps;
         if (!live) {
           outcome = 0;  // no live in-edge
-        } else if (HAS_REM && ((P.edge_removed && P.edge_removed[e]) || (P.node_removed && P.node_removed[u]))) {
+        } else if (HAS_REM && (gone || (P.node_removed && bit_at(P.node_removed, u)))) {
           outcome = 0;
         } else if (ck.seen(u)) {
           outcome = 0;  // the walk closed a cycle
@@ -249,7 +255,7 @@ __global__ void k_classify(SampleParams P, uint64_t first, int64_t count, int8_t
     Ckpt ck;
     ck.reset(v);
     int out = -1;
-    if (HAS_REM && P.node_removed && P.node_removed[v]) out = 3;
+    if (HAS_REM && P.node_removed && bit_at(P.node_removed, v)) out = 3;
     while (out < 0) {
       const bool suspect = (__ldg(&P.s_bits[v >> 5]) >> (v & 31)) & 1u;
       const uint4 x = node_draw(a, v, P.k0, P.k1);
@@ -258,7 +264,10 @@ __global__ void k_classify(SampleParams P, uint64_t first, int64_t count, int8_t
       if (x.x >= nd.w) { out = 0; break; }
       const uint32_t e = nd.x + pick_in_edge(P.edge, nd, x.x);
       const uint32_t u = __ldg(&P.edge[e].x);
-      if (HAS_REM && ((P.edge_removed && P.edge_removed[e]) || (P.node_removed && P.node_removed[u]))) { out = 3; break; }
+      if (HAS_REM && ((P.edge_removed && bit_at(P.edge_removed, e)) || (P.node_removed && bit_at(P.node_removed, u)))) {
+        out = 3;
+        break;
+      }
       if (ck.seen(u)) { out = 2; break; }
       ck.keep(u, len);
       v = u;
@@ -315,6 +324,36 @@ hsaw_status query_upload(const Graph& g, const hsaw_query* q, QueryDev& qd, cuda
   dfree(d_p, s);
   if (le != cudaSuccess) return fail(HSAW_E_DEVICE, "query: suspect bits launch failed");
   qd.seed = q->seed;
+  return HSAW_OK;
+}
+
+// Removal masks are kept as bits: the walk reads one per draw at random, and m bytes would
+// push walk records out of L2 (R-MAT 22 eSI residual estimate of 100 K hits, 1,000 edges
+// removed: 67 MB of bytes against 8.4 MB of bits).
+__global__ void k_pack_mask(const uint8_t* __restrict__ bytes, size_t len, uint32_t* __restrict__ bits) {
+  const size_t words = (len + 31) / 32;
+  for (size_t w = blockIdx.x * (size_t)blockDim.x + threadIdx.x; w < words; w += (size_t)gridDim.x * blockDim.x) {
+    uint32_t b = 0;
+    if (w * 32 + 32 <= len) {  // bytes starts on a 16-byte boundary (an allocation of its own)
+      const uint4* p = reinterpret_cast<const uint4*>(bytes + w * 32);
+      const uint4 q[2] = {p[0], p[1]};
+      const uint32_t* x = reinterpret_cast<const uint32_t*>(q);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) b |= ((x[i] >> (8 * j)) & 0xFFu) ? 1u << (4 * i + j) : 0u;
+    } else {
+      for (size_t i = w * 32; i < len; ++i) b |= bytes[i] ? 1u << (i & 31) : 0u;
+    }
+    bits[w] = b;
+  }
+}
+
+hsaw_status pack_mask(const uint8_t* bytes, size_t len, uint32_t** bits, cudaStream_t s) {
+  HSAW_TRY(dmalloc((void**)bits, (len + 31) / 32 * 4, s));
+  count_launch();
+  k_pack_mask<<<grid_for((len + 31) / 32, 256, 8192), 256, 0, s>>>(bytes, len, *bits);
+  HSAW_CK(cudaGetLastError());
   return HSAW_OK;
 }
 

@@ -11,14 +11,16 @@ struct QueryDev {
   uint32_t* p32 = nullptr;        // n words or NULL (p == 1)
   int32_t* s_list = nullptr;      // n_src node ids of V_I
   int32_t n_src = 0;
-  uint8_t* edge_removed = nullptr;  // m bytes or NULL
-  uint8_t* node_removed = nullptr;  // n bytes or NULL
+  uint32_t* edge_removed = nullptr;  // m bits or NULL
+  uint32_t* node_removed = nullptr;  // n bits or NULL
   uint64_t seed = 0;
   bool owns_removed = false;
 };
 
 hsaw_status query_upload(const Graph& g, const hsaw_query* q, QueryDev& qd, cudaStream_t s);
 void query_release(QueryDev& qd, cudaStream_t s);
+// Bit x of *bits = (bytes[x] != 0), x < len; bytes is a device array.
+hsaw_status pack_mask(const uint8_t* bytes, size_t len, uint32_t** bits, cudaStream_t s);
 
 // The ordered HSAW stream R_1, R_2, ... of Alg. 3: hit j has attempt id aid[j], l_j =
 // len[j] nodes nodes[node_off[j] .. node_off[j+1]) and l_j - 1 edges starting at
