@@ -1129,7 +1129,11 @@ hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t 
   int32_t rounds = 0;
   hsaw_status st = HSAW_OK;
   bool done = false;
-  if (U > 0 && cv.walks > 0) {
+  // by gain levels, unless the environment asks for a version that takes one pick at a time
+  const bool one_by_one = getenv("HSAW_GREEDY") || getenv("HSAW_GREEDY_HEAVY") || getenv("HSAW_GREEDY_OWNED_MAX");
+  if (U > 0 && cv.walks > 0 && !one_by_one)
+    st = level_greedy(cv, cand_dev, k, ids.p, outs.p + k, &rounds, &done, s);
+  if (st == HSAW_OK && !done && U > 0 && cv.walks > 0) {
     HSAW_TRY(cv.cnt_work.ensure(U, s));
     HSAW_TRY(cv.covered.ensure((size_t)cv.walks, s));
     HSAW_TRY(cv.inv_ent.ensure((size_t)cv.entries, s));

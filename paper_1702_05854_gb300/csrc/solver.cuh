@@ -82,6 +82,10 @@ hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t
 // Greedy (Alg. 4 / 7) on a built Cover; cand (device, M bytes) may be NULL.
 hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t k, int64_t* ids_host,
                          uint32_t* gains_host, cudaStream_t s);
+// The same picks one gain level at a time (levels.cu), for cover_greedy: the first *rounds <= k
+// ids and gains (device, k of each); *done = false when no cluster can run it.
+hsaw_status level_greedy(Cover& cv, const uint8_t* cand, int32_t k, int64_t* ids, uint32_t* gains, int32_t* rounds,
+                         bool* done, cudaStream_t s);
 // #walks in [first, first + count) that contain an element of T (T host, k ids).
 hsaw_status cover_count(const Stream& st, hsaw_mode mode, int64_t first, int64_t count, const int64_t* T, int32_t k,
                         uint64_t* cov, cudaStream_t s);

@@ -67,3 +67,63 @@ def test_removal_mask_words(m, kind):
     walks = hs.hsaw_sample(g, hs.Query(sources=sources, seed=5), 0, 500, edge_removed=er, node_removed=nr)
     ost = oracle.Stream(oracle.Query(og, sources, edge_removed=er, node_removed=nr, seed=5)).extend(500)
     assert_same_stream(walks, ost, 500)
+
+
+@pytest.fixture(scope="module")
+def streams():
+    """20,000 walks on the 16 K-node Chung-Lu graph from few suspects (180 K walk elements: ranges of them run on one
+    CTA, at most 2^17 elements, or on the largest cluster) and from many (short walks, thousands of picks that gain)."""
+    d = synth.workload_c1()
+    g, og = hs.hsaw_graph_from_edges(d["n"], d["src"], d["dst"], d["w"]), oracle.Graph(d["n"], d["src"], d["dst"], d["w"])
+    got = {}
+    for name, sources in (("few", d["sources"]), ("many", synth.sources(d["n"], 9000, 5))):
+        got[name] = (hs.hsaw_sample(g, hs.Query(sources=sources, seed=21), 0, 20_000),
+                     oracle.Stream(oracle.Query(og, sources, seed=21)).extend(20_000))
+    return d, g, got
+
+
+@pytest.mark.parametrize("mode", [hs.HSAW_EDGE, hs.HSAW_NODE])
+@pytest.mark.parametrize("who,first,count,k,share", [
+    ("few", 0, 1, 3, 1.0),            # one walk, then zero-gain picks
+    ("few", 5, 33, 40, 1.0),          # every gain small
+    ("few", 0, 700, 1, 1.0),          # fewer elements kept per phase than there are
+    ("few", 100, 3000, 32, 0.5),      # candidate mask
+    ("few", 0, 20_000, 33, 1.0),      # the largest cluster
+    ("few", 0, 20_000, 1000, 0.05),   # few candidates: gains end before the picks do
+    ("many", 0, 20_000, 100, 1.0),    # many ties, several phases
+    ("many", 0, 20_000, 4096, 1.0),   # as many picks as one block orders
+    ("many", 0, 20_000, 7000, 1.0),   # more, levels down to 1, zero-gain picks in the edge mode
+    ("many", 3, 2000, 16_000, 0.9),   # gains of 1 and 2, then zero-gain picks
+])
+def test_greedy_by_levels(streams, mode, who, first, count, k, share):
+    """Greedy by gain levels: ids, gains and their order."""
+    d, g, got = streams
+    walks, ost = got[who]
+    M = d["m"] if mode == hs.HSAW_EDGE else d["n"]
+    mask = None if share == 1.0 else (np.random.default_rng(k).random(M) < share).astype(np.uint8)
+    if mask is not None:
+        k = min(k, int(mask.sum()))
+    ids, gains = hs.hsaw_greedy(walks, g, mode, first, count, k, candidate_mask=mask)
+    oids, ogains = ost.greedy(mode, first, count, M, k, cand_mask=mask, kept_gains=True)
+    assert np.array_equal(gains, ogains)
+    assert np.array_equal(ids, oids)
+
+
+def test_greedy_level_conflicts():
+    """Ties whose walks chain into each other: a level then takes several rounds.  A path 0 -> 1 -> ... -> n - 1 with
+    the suspect at 0 gives nested walks; a second copy with its ids interleaved gives equal gains."""
+    n = 40
+    even, odd = np.arange(0, 2 * n, 2, dtype=np.int32), np.arange(2 * n - 1, 0, -2, dtype=np.int32)
+    src = np.concatenate([even[:-1], odd[:-1]])
+    dst = np.concatenate([even[1:], odd[1:]])
+    w = np.full(src.size, int(ONE * 0.9), np.uint32)
+    sources = np.array([int(even[0]), int(odd[0])], np.int32)
+    g, og = hs.hsaw_graph_from_edges(2 * n, src, dst, w), oracle.Graph(2 * n, src, dst, w)
+    for seed in range(6):
+        walks = hs.hsaw_sample(g, hs.Query(sources=sources, seed=seed), 0, 400)
+        ost = oracle.Stream(oracle.Query(og, sources, seed=seed)).extend(400)
+        for mode, M in ((hs.HSAW_EDGE, src.size), (hs.HSAW_NODE, 2 * n)):
+            for first, count in ((0, 400), (3, 50), (100, 7)):
+                ids, gains = hs.hsaw_greedy(walks, g, mode, first, count, 30)
+                oids, ogains = ost.greedy(mode, first, count, M, 30)
+                assert np.array_equal(gains, ogains) and np.array_equal(ids, oids)
