@@ -157,7 +157,9 @@ __global__ void __launch_bounds__(256) k_rs_hist(const uint32_t* __restrict__ ke
 // One stable scatter pass.  The tile is first ordered by digit in shared memory (ranks
 // follow input order: warp sub-tiles in order, batches in order, lanes in order), then
 // written out in that order, so each digit's items leave as one contiguous run (about 16
-// items per digit and tile) instead of one scattered word per item.
+// items per digit and tile) instead of one scattered word per item.  All loads are issued
+// before the ranking, and an item's rank within its warp comes from the same match that
+// counts it.
 __global__ void __launch_bounds__(256) k_rs_scatter(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals,
                                                     size_t n, int shift, const uint32_t* __restrict__ offsets,
                                                     uint32_t tiles, uint32_t* __restrict__ keys_out,
@@ -171,18 +173,26 @@ __global__ void __launch_bounds__(256) k_rs_scatter(const uint32_t* __restrict__
   __syncthreads();
   const size_t tile0 = (size_t)blockIdx.x * RS_TILE;
   const size_t sub = tile0 + (size_t)w * RS_SUB;
-  uint32_t k[RS_BATCH], v[RS_BATCH];
+  const unsigned lt = (1u << lane) - 1u;
+  uint32_t k[RS_BATCH], v[RS_BATCH], rank[RS_BATCH];
 #pragma unroll
   for (int b = 0; b < RS_BATCH; ++b) {
-    size_t idx = sub + (size_t)b * 32 + lane;
-    bool ok = idx < n;
-    k[b] = ok ? keys[idx] : 0u;
-    v[b] = ok ? vals[idx] : 0u;
-    unsigned act = __ballot_sync(0xffffffffu, ok);
+    const size_t idx = sub + (size_t)b * 32 + lane;
+    k[b] = idx < n ? keys[idx] : 0u;
+    v[b] = idx < n ? vals[idx] : 0u;
+  }
+#pragma unroll
+  for (int b = 0; b < RS_BATCH; ++b) {
+    const bool ok = sub + (size_t)b * 32 + lane < n;
+    const unsigned act = __ballot_sync(0xffffffffu, ok);
+    rank[b] = 0;
     if (ok) {
-      uint32_t d = (k[b] >> shift) & 255u;
-      unsigned same = __match_any_sync(act, d);
-      if (lane == __ffs(same) - 1) wc[w][d] += __popc(same);
+      const uint32_t d = (k[b] >> shift) & 255u;
+      const unsigned same = __match_any_sync(act, d);
+      const uint32_t before = wc[w][d];
+      __syncwarp(act);
+      rank[b] = before + __popc(same & lt);
+      if (lane == __ffs(same) - 1) wc[w][d] = before + __popc(same);
     }
     __syncwarp();
   }
@@ -201,23 +211,13 @@ __global__ void __launch_bounds__(256) k_rs_scatter(const uint32_t* __restrict__
     }
   }
   __syncthreads();
-  const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
   for (int b = 0; b < RS_BATCH; ++b) {
-    size_t idx = sub + (size_t)b * 32 + lane;
-    bool ok = idx < n;
-    unsigned act = __ballot_sync(0xffffffffu, ok);
-    uint32_t d = (k[b] >> shift) & 255u;
-    unsigned same = ok ? __match_any_sync(act, d) : 0u;
-    uint32_t base = ok ? wc[w][d] : 0u;
-    __syncwarp();
-    if (ok) {
-      uint32_t pos = base + __popc(same & lt);
+    if (sub + (size_t)b * 32 + lane < n) {
+      const uint32_t pos = wc[w][(k[b] >> shift) & 255u] + rank[b];
       ks[pos] = k[b];
       vs[pos] = v[b];
-      if (lane == __ffs(same) - 1) wc[w][d] = base + __popc(same);
     }
-    __syncwarp();
   }
   __syncthreads();
   const uint32_t items = (uint32_t)min((size_t)RS_TILE, n - tile0);

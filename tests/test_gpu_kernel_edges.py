@@ -52,6 +52,18 @@ def test_equal_weight_pick(d, share):
     assert_same_stream(walks, oracle.Stream(oracle.Query(og, sources, seed=11)).extend(300), 300)
 
 
+@pytest.mark.parametrize("m", [1, 2, 31, 33, 511, 513, 4095, 4096, 4097, 8193, 70_000])
+def test_ingest_sort_tiles(m):
+    """Stable order by destination around the radix sort's batches and tiles, in graphs of few and many nodes."""
+    rng = np.random.default_rng(m)
+    for n in (1, 3, 257, 100_000):
+        src, dst = rng.integers(0, n, m).astype(np.int32), rng.integers(0, n, m).astype(np.int32)
+        w = synth.wc_weights(n, dst)
+        g, og = hs.hsaw_graph_from_edges(n, src, dst, w), oracle.Graph(n, src, dst, w)
+        for x, y in zip(g.export(), og.arrays()):
+            assert np.array_equal(x, y)
+
+
 @pytest.mark.parametrize("m", [1, 7, 31, 32, 33, 63, 64, 65, 200])
 @pytest.mark.parametrize("kind", ["edge", "node", "both"])
 def test_removal_mask_words(m, kind):
@@ -95,8 +107,8 @@ def streams():
     ("many", 0, 20_000, 7000, 1.0),   # more, levels down to 1, zero-gain picks in the edge mode
     ("many", 3, 2000, 16_000, 0.9),   # gains of 1 and 2, then zero-gain picks
 ])
-def test_greedy_by_levels(streams, mode, who, first, count, k, share):
-    """Greedy by gain levels: ids, gains and their order."""
+def test_greedy_by_peaks(streams, mode, who, first, count, k, share):
+    """Greedy by peaks: ids, gains and their order."""
     d, g, got = streams
     walks, ost = got[who]
     M = d["m"] if mode == hs.HSAW_EDGE else d["n"]
@@ -109,8 +121,8 @@ def test_greedy_by_levels(streams, mode, who, first, count, k, share):
     assert np.array_equal(ids, oids)
 
 
-def test_greedy_level_conflicts():
-    """Ties whose walks chain into each other: a level then takes several rounds.  A path 0 -> 1 -> ... -> n - 1 with
+def test_greedy_conflict_chains():
+    """Ties whose walks chain into each other: picks then take several rounds.  A path 0 -> 1 -> ... -> n - 1 with
     the suspect at 0 gives nested walks; a second copy with its ids interleaved gives equal gains."""
     n = 40
     even, odd = np.arange(0, 2 * n, 2, dtype=np.int32), np.arange(2 * n - 1, 0, -2, dtype=np.int32)
