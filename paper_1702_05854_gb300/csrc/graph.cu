@@ -150,42 +150,108 @@ __global__ void k_copy_edges(const int32_t* __restrict__ src, const uint32_t* __
   }
 }
 
-// One warp per node: running in-weight sums (exact, 64-bit carry), the in-sum check
-// (<= 2^32 - 1), equal-weight detection and the node record.  err[1] counts the nodes with
-// in-weight whose in-weights differ.
+// Running in-weight sums (exact, 64-bit carry), the in-sum check (<= 2^32 - 1), equal-weight
+// detection and the node record: one warp per node, and one block per hub (a node of more
+// than HUB_DEGREE in-edges), which the warp pass only lists.  A warp takes a list 32 edges at
+// a time with a scan each, so the longest list alone set the pass's time (R-MAT 22: 3.1 ms,
+// R-MAT 20: 1.3 ms).  err[1] counts the nodes with in-weight whose in-weights differ.
+constexpr uint32_t HUB_DEGREE = 1024;
+
+// Hubs of the graph: count, then node ids (at most m / HUB_DEGREE of them).
+struct Hubs {
+  uint32_t* count;
+  uint32_t* node;
+};
+
+__device__ __forceinline__ void write_node(uint4* __restrict__ node, int64_t v, uint32_t first, uint32_t deg,
+                                           bool uniform, uint32_t w0, uint64_t sum, uint32_t* __restrict__ err) {
+  const uint32_t insum = (uint32_t)(sum > 0xFFFFFFFFull ? 0xFFFFFFFFull : sum);
+  node[v] = make_uint4(first, deg, (uniform && deg) ? w0 : 0u, insum);
+  if (sum > 0xFFFFFFFFull) atomicOr(err, ERR_WEIGHT);
+  if (!uniform && insum) atomicAdd(err + 1, 1u);
+}
+
 __global__ void k_thresholds(const uint32_t* __restrict__ row_start, int64_t n, uint2* __restrict__ edge,
-                             uint4* __restrict__ node, uint32_t* __restrict__ err) {
+                             uint4* __restrict__ node, Hubs hubs, uint32_t* __restrict__ err) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
     const uint32_t b = row_start[v], e = row_start[v + 1];
     const uint32_t deg = e - b;
+    if (deg > HUB_DEGREE) {
+      if (lane == 0) hubs.node[atomicAdd(hubs.count, 1u)] = (uint32_t)v;
+      continue;
+    }
     uint64_t carry = 0;
-    uint32_t w0 = deg ? edge[b].y : 0u;
+    uint32_t w0 = 0;
     bool uniform = true;
     for (uint32_t base = b; base < e; base += 32) {
-      uint32_t q = base + lane;
-      uint64_t w = q < e ? edge[q].y : 0u;
-      if (q < e && (uint32_t)w != w0) uniform = false;
+      const uint32_t q = base + lane;
+      const uint32_t w = q < e ? edge[q].y : 0u;
+      if (base == b) w0 = __shfl_sync(0xffffffffu, w, 0);
+      if (q < e && w != w0) uniform = false;
       uint64_t x = w;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         uint64_t y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
       }
-      uint64_t run = carry + x;
-      if (q < e) {
-        if (run > 0xFFFFFFFFull) atomicOr(err, ERR_WEIGHT);
-        edge[q].y = (uint32_t)(run > 0xFFFFFFFFull ? 0xFFFFFFFFull : run);
-      }
+      const uint64_t run = carry + x;
+      if (q < e) edge[q].y = (uint32_t)(run > 0xFFFFFFFFull ? 0xFFFFFFFFull : run);
       carry += __shfl_sync(0xffffffffu, x, 31);
     }
     uniform = __all_sync(0xffffffffu, uniform);
-    if (lane == 0) {
-      uint32_t insum = (uint32_t)(carry > 0xFFFFFFFFull ? 0xFFFFFFFFull : carry);
-      node[v] = make_uint4(b, deg, (uniform && deg) ? w0 : 0u, insum);
-      if (!uniform && insum) atomicAdd(err + 1, 1u);
+    if (lane == 0) write_node(node, v, b, deg, uniform, w0, carry, err);
+  }
+}
+
+__global__ void __launch_bounds__(1024) k_hub_thresholds(const uint32_t* __restrict__ row_start,
+                                                         uint2* __restrict__ edge, uint4* __restrict__ node, Hubs hubs,
+                                                         uint32_t* __restrict__ err) {
+  constexpr uint32_t ITEMS = 4;
+  __shared__ uint64_t sums[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t count = *hubs.count;
+  for (uint32_t h = blockIdx.x; h < count; h += gridDim.x) {
+    const uint32_t v = hubs.node[h];
+    const uint32_t b = row_start[v], e = row_start[v + 1];
+    const uint32_t w0 = edge[b].y;
+    __syncthreads();  // every thread has read edge[b] before it is written
+    uint64_t carry = 0;
+    bool uniform = true;
+    for (uint32_t base = b; base < e; base += ITEMS * 1024) {
+      const uint32_t q = base + threadIdx.x * ITEMS;
+      uint64_t run[ITEMS], sum = 0;
+#pragma unroll
+      for (uint32_t i = 0; i < ITEMS; ++i) {
+        const uint32_t x = q + i < e ? edge[q + i].y : 0u;
+        if (q + i < e && x != w0) uniform = false;
+        run[i] = sum += x;
+      }
+      uint64_t inc = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      if (lane == 31) sums[w] = inc;
+      __syncthreads();
+      uint64_t mine = sums[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(0xffffffffu, mine, o);
+        if (lane >= o) mine += y;
+      }
+      const uint64_t before = w ? __shfl_sync(0xffffffffu, mine, w - 1) : 0ull;
+      const uint64_t at = carry + before + inc - sum;
+      carry += __shfl_sync(0xffffffffu, mine, 31);
+#pragma unroll
+      for (uint32_t i = 0; i < ITEMS; ++i)
+        if (q + i < e) edge[q + i].y = (uint32_t)(at + run[i] > 0xFFFFFFFFull ? 0xFFFFFFFFull : at + run[i]);
+      __syncthreads();  // sums is written again by the next tile
     }
+    uniform = __syncthreads_and(uniform);
+    if (threadIdx.x == 0) write_node(node, v, b, e - b, uniform, w0, carry, err);
   }
 }
 
@@ -205,43 +271,46 @@ __global__ void k_walk_records(const uint2* __restrict__ edge, const uint4* __re
   }
 }
 
-// Guide tables of the nodes with unequal in-weights (see Graph::guide); one warp per node.
+// Bucket record b of a node with unequal in-weights (see Graph::grec): the walk record of the
+// live in-edge of the bucket's smallest draw.
+__device__ __forceinline__ void guide_record(uint4 nd, uint32_t b, const uint2* __restrict__ edge,
+                                             const uint4* __restrict__ erec, uint4* __restrict__ grec) {
+  const uint32_t lb = (uint32_t)(((uint64_t)b * nd.w + nd.y - 1) / nd.y);  // ceil(b * insum / deg)
+  uint32_t lo = 0, hi = nd.y;
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (lb < edge[nd.x + mid].y) hi = mid; else lo = mid + 1;
+  }
+  const size_t p = 2 * ((size_t)nd.x + b), e = 2 * ((size_t)nd.x + lo);
+  grec[p] = erec[e];
+  uint4 second = erec[e + 1];
+  second.z = lo;
+  grec[p + 1] = second;
+}
+
+// One warp per node, and a block per slice of a hub's buckets (one warp on the longest list
+// took the whole pass: 4.7 ms on R-MAT 20).
 __global__ void k_guide(const uint4* __restrict__ node, const uint2* __restrict__ edge, int64_t n,
-                        uint32_t* __restrict__ guide) {
+                        const uint4* __restrict__ erec, uint4* __restrict__ grec) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
     const uint4 nd = node[v];
-    if (nd.y == 0 || nd.z != 0 || nd.w == 0) continue;  // no in-edge, equal weights, or zero in-sum
-    for (uint32_t b = lane; b < nd.y; b += 32) {
-      const uint32_t lb = (uint32_t)(((uint64_t)b * nd.w + nd.y - 1) / nd.y);  // ceil(b * insum / deg)
-      uint32_t lo = 0, hi = nd.y;
-      while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (lb < edge[nd.x + mid].y) hi = mid; else lo = mid + 1;
-      }
-      guide[nd.x + b] = lo;
-    }
+    if (nd.z != 0 || nd.w == 0 || nd.y > HUB_DEGREE) continue;  // equal weights, no in-weight, or a hub
+    for (uint32_t b = lane; b < nd.y; b += 32) guide_record(nd, b, edge, erec, grec);
   }
 }
 
-// Bucket records of the nodes with unequal in-weights (see Graph::grec); one warp per node.
-__global__ void k_guide_records(const uint4* __restrict__ node, const uint32_t* __restrict__ guide, int64_t n,
-                                const uint4* __restrict__ erec, uint4* __restrict__ grec) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
-    const uint4 nd = node[v];
-    if (nd.y == 0 || nd.z != 0 || nd.w == 0) continue;
-    for (uint32_t b = lane; b < nd.y; b += 32) {
-      const size_t p = (size_t)nd.x + b;
-      const uint32_t j0 = guide[p];
-      const size_t e0 = (size_t)nd.x + j0;
-      grec[2 * p] = erec[2 * e0];
-      uint4 hi = erec[2 * e0 + 1];
-      hi.z = j0;
-      grec[2 * p + 1] = hi;
-    }
+__global__ void __launch_bounds__(256) k_hub_guide(const uint4* __restrict__ node, const uint2* __restrict__ edge,
+                                                   Hubs hubs, const uint4* __restrict__ erec,
+                                                   uint4* __restrict__ grec) {
+  constexpr uint32_t SLICES = 16;
+  const uint64_t items = (uint64_t)*hubs.count * SLICES;
+  for (uint64_t i = blockIdx.x; i < items; i += gridDim.x) {
+    const uint4 nd = node[hubs.node[i / SLICES]];
+    if (nd.z != 0 || nd.w == 0) continue;
+    for (uint32_t b = (uint32_t)(i % SLICES) * blockDim.x + threadIdx.x; b < nd.y; b += SLICES * blockDim.x)
+      guide_record(nd, b, edge, erec, grec);
   }
 }
 
@@ -349,11 +418,21 @@ struct Temps {
   }
 };
 
-static hsaw_status finish_graph(Graph& g, uint32_t* row_start, uint32_t* d_err, cudaStream_t s) {
+static hsaw_status finish_graph(Graph& g, uint32_t* row_start, uint32_t* d_err, Temps& T, cudaStream_t s) {
   const int64_t n = g.n;
+  Hubs hubs;
+  HSAW_TRY(T.get(&hubs.count, 1 + (size_t)(g.m / HUB_DEGREE)));
+  hubs.node = hubs.count + 1;
+  HSAW_CK(cudaMemsetAsync(hubs.count, 0, sizeof(uint32_t), s));
   count_launch();
-  k_thresholds<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(row_start, n, g.edge, g.node, d_err);
+  k_thresholds<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(row_start, n, g.edge, g.node, hubs, d_err);
   HSAW_CK(cudaGetLastError());
+  if (g.m > HUB_DEGREE) {
+    count_launch();
+    k_hub_thresholds<<<grid_for((size_t)(g.m / HUB_DEGREE), 1, 2 * sm_count()), 1024, 0, s>>>(row_start, g.edge, g.node,
+                                                                                             hubs, d_err);
+    HSAW_CK(cudaGetLastError());
+  }
   uint32_t unequal = 0;
   HSAW_TRY(check_err(d_err, s, &unequal));
   if (!g.m) return HSAW_OK;
@@ -367,25 +446,20 @@ static hsaw_status finish_graph(Graph& g, uint32_t* row_start, uint32_t* d_err, 
   }
   k_walk_records<false><<<grid_for(g.m, 256, 1u << 16), 256, 0, s>>>(g.edge, g.node, g.m, g.erec);
   HSAW_CK(cudaGetLastError());
-  // guide tables (a temporary) and their bucket records
   if (cudaMalloc((void**)&g.grec, (size_t)g.m * 2 * sizeof(uint4)) != cudaSuccess) {
     cudaGetLastError();
     g.grec = nullptr;
     return fail(HSAW_E_NOMEM, "graph: guide records do not fit in device memory");
   }
-  uint32_t* guide = nullptr;
-  HSAW_TRY(dmalloc((void**)&guide, (size_t)g.m * sizeof(uint32_t), s));
-  hsaw_status st = HSAW_OK;
   count_launch();
-  k_guide<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(g.node, g.edge, n, guide);
-  if (cudaGetLastError() != cudaSuccess) st = fail(HSAW_E_DEVICE, "graph: guide tables failed");
-  if (st == HSAW_OK) {
+  k_guide<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(g.node, g.edge, n, g.erec, g.grec);
+  HSAW_CK(cudaGetLastError());
+  if (g.m > HUB_DEGREE) {
     count_launch();
-    k_guide_records<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(g.node, guide, n, g.erec, g.grec);
-    if (cudaGetLastError() != cudaSuccess) st = fail(HSAW_E_DEVICE, "graph: guide records failed");
+    k_hub_guide<<<8 * sm_count(), 256, 0, s>>>(g.node, g.edge, hubs, g.erec, g.grec);
+    HSAW_CK(cudaGetLastError());
   }
-  dfree(guide, s);
-  return st;
+  return HSAW_OK;
 }
 
 static hsaw_status from_edges(int64_t n, int64_t m, const int32_t* src, const int32_t* dst, const uint32_t* w,
@@ -460,7 +534,7 @@ static hsaw_status from_edges(int64_t n, int64_t m, const int32_t* src, const in
     k_gather_edges<<<grid_for(m, 256, 8192), 256, 0, s>>>(sv, d_src, d_w, m, g.edge, g.input_index);
     HSAW_CK(cudaGetLastError());
   }
-  return finish_graph(g, row_start, d_err, s);
+  return finish_graph(g, row_start, d_err, T, s);
 }
 
 static hsaw_status from_csr(int64_t n, int64_t m, const int64_t* rp, const int32_t* src, const uint32_t* w,
@@ -494,7 +568,7 @@ static hsaw_status from_csr(int64_t n, int64_t m, const int64_t* rp, const int32
     HSAW_CK(cudaGetLastError());
     HSAW_TRY(check_err(d_err, s));
   }
-  return finish_graph(g, row_start, d_err, s);
+  return finish_graph(g, row_start, d_err, T, s);
 }
 
 // node record -> host CSR export

@@ -64,6 +64,43 @@ def test_ingest_sort_tiles(m):
             assert np.array_equal(x, y)
 
 
+@pytest.mark.parametrize("deg", [31, 32, 33, 1023, 1024, 1025, 4096, 4097, 8192, 50_001])
+@pytest.mark.parametrize("kind", ["equal", "unequal", "zeros"])
+def test_hub_lists(deg, kind):
+    """Running sums, node records and guide records around the hub threshold and its tiles."""
+    rng = np.random.default_rng(deg)
+    n, src, dst, w = hub_graph(deg, int(ONE * 0.8) // deg)
+    if kind != "equal":  # the hub's in-weights differ; with "zeros" half of them are 0
+        x = rng.random(deg) + 0.01
+        if kind == "zeros":
+            x[rng.random(deg) < 0.5] = 0.0
+            x[0] = 0.5
+        w[:deg] = np.floor(x / x.sum() * 0.8 * ONE).astype(np.uint32)
+    order = rng.permutation(src.size)
+    src, dst, w = src[order], dst[order], w[order]
+    g, og = hs.hsaw_graph_from_edges(n, src, dst, w), oracle.Graph(n, src, dst, w)
+    for x, y in zip(g.export(), og.arrays()):
+        assert np.array_equal(x, y)
+    rp, s, _, _, _ = og.arrays()
+    gc = hs.hsaw_graph_from_csr(n, rp, s, w[og.arrays()[4]])
+    sources = np.arange(1, deg + 1, 5, dtype=np.int32)
+    ost = oracle.Stream(oracle.Query(og, sources, seed=9)).extend(300)
+    for graph in (g, gc):
+        assert_same_stream(hs.hsaw_sample(graph, hs.Query(sources=sources, seed=9), 0, 300), ost, 300)
+
+
+@pytest.mark.parametrize("deg", [1024, 1025, 9000])
+def test_hub_overweight(deg):
+    """An in-sum of 2^32 is refused, 2^32 - 1 accepted, above and below the hub threshold."""
+    n, src, dst, w = hub_graph(deg, ONE // deg)
+    w[0] += np.uint32(ONE - (ONE // deg) * deg)
+    hs.hsaw_graph_from_edges(n, src, dst, w).close()
+    w[deg // 2] += np.uint32(1)
+    with pytest.raises(hs.HsawError) as e:
+        hs.hsaw_graph_from_edges(n, src, dst, w)
+    assert e.value.status == -2
+
+
 @pytest.mark.parametrize("m", [1, 7, 31, 32, 33, 63, 64, 65, 200])
 @pytest.mark.parametrize("kind", ["edge", "node", "both"])
 def test_removal_mask_words(m, kind):
