@@ -27,7 +27,7 @@ void Cover::release(cudaStream_t s) {
   keys.release(s); vals.release(s); keys2.release(s); vals2.release(s); run_flag.release(s);
   uid.release(s); cnt.release(s); inv_off.release(s); inv_walk.release(s); entry_uidx.release(s);
   walk_eoff.release(s); cnt_work.release(s); covered.release(s); dirty.release(s); partial.release(s);
-  inv_ent.release(s); g_idx.release(s); g_list.release(s); g_cnt.release(s); g_entry.release(s); g_rng.release(s);
+  inv_ent.release(s); peak_list.release(s); g_idx.release(s); g_list.release(s); g_cnt.release(s); g_entry.release(s); g_rng.release(s);
 }
 
 // entry offsets of walks [first, first + count) relative to the first walk's first entry
@@ -1129,10 +1129,10 @@ hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t 
   int32_t rounds = 0;
   hsaw_status st = HSAW_OK;
   bool done = false;
-  // by gain levels, unless the environment asks for a version that takes one pick at a time
+  // by peaks, unless the environment asks for a version that takes one pick at a time
   const bool one_by_one = getenv("HSAW_GREEDY") || getenv("HSAW_GREEDY_HEAVY") || getenv("HSAW_GREEDY_OWNED_MAX");
   if (U > 0 && cv.walks > 0 && !one_by_one)
-    st = level_greedy(cv, cand_dev, k, ids.p, outs.p + k, &rounds, &done, s);
+    st = peak_greedy(cv, cand_dev, k, ids.p, outs.p + k, &rounds, &done, s);
   if (st == HSAW_OK && !done && U > 0 && cv.walks > 0) {
     HSAW_TRY(cv.cnt_work.ensure(U, s));
     HSAW_TRY(cv.covered.ensure((size_t)cv.walks, s));

@@ -71,7 +71,8 @@ struct Cover {
   DBuf<uint32_t> cnt_work;                  // greedy's running counts
   DBuf<uint32_t> covered;  // greedy: per walk, 0 or 1 + the pick that covered it
   DBuf<uint8_t> dirty;     // greedy (grid version): group dirty flags
-  DBuf<uint4> inv_ent;           // cluster greedy: inverted-index entries with their walk's entry range
+  DBuf<uint4> inv_ent;           // cluster greedy: inverted-index entries with their walk's entry range; peaks: pairs
+  DBuf<uint4> peak_list;         // greedy by peaks: the phase's elements
   DBuf<uint32_t> g_idx, g_list, g_cnt, g_entry;  // greedy on the heavy elements: index map, list, counts, entries
   DBuf<uint2> g_rng;             // greedy: each element's entries of inv_ent
   DBuf<unsigned long long> partial;
@@ -82,9 +83,9 @@ hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t
 // Greedy (Alg. 4 / 7) on a built Cover; cand (device, M bytes) may be NULL.
 hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t k, int64_t* ids_host,
                          uint32_t* gains_host, cudaStream_t s);
-// The same picks one gain level at a time (levels.cu), for cover_greedy: the first *rounds <= k
+// The same picks by peaks, many at a time (peaks.cu), for cover_greedy: the first *rounds <= k
 // ids and gains (device, k of each); *done = false when no cluster can run it.
-hsaw_status level_greedy(Cover& cv, const uint8_t* cand, int32_t k, int64_t* ids, uint32_t* gains, int32_t* rounds,
+hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, int64_t* ids, uint32_t* gains, int32_t* rounds,
                          bool* done, cudaStream_t s);
 // #walks in [first, first + count) that contain an element of T (T host, k ids).
 hsaw_status cover_count(const Stream& st, hsaw_mode mode, int64_t first, int64_t count, const int64_t* T, int32_t k,
