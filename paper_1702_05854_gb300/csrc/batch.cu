@@ -21,9 +21,7 @@ constexpr uint32_t BCHUNK = 256;                       // attempts per chunk
 constexpr uint64_t BATCH_ROUND_ATTEMPTS = 1ull << 32;  // attempts of all instances in one launch
 
 struct BatchInst {
-  const uint4* node;
-  const uint4* erec;
-  const uint4* grec;
+  WalkTables T;
   const uint32_t* s_bits;
   const uint32_t* p32;  // NULL: p == 1
   uint64_t a0;          // first attempt of this instance's window
@@ -31,7 +29,7 @@ struct BatchInst {
   uint32_t n_attempts;  // window size
   uint32_t n_chunks;
   uint32_t chunk0;      // first global chunk of the window
-  uint32_t eq;          // the graph's walk-record layout
+  Layout layout;        // REC16 or REC32
   uint32_t cap;         // hit records per chunk (a few standard deviations above the expected hits)
   uint64_t rec0;        // first record of the window
 };
@@ -82,7 +80,7 @@ __global__ void __launch_bounds__(256, 4) k_sample_batch(BatchParams B) {
         if (!active && rank < avail) {
           off = cur + rank;
           v = start_node(I.a0 + off, I.n, I.k0, I.k1);
-          rec = __ldg(&I.node[v]);
+          rec = __ldg(&I.T.node[v]);
           ck.reset(v);
           len = 1;
           active = true;
@@ -100,8 +98,8 @@ __global__ void __launch_bounds__(256, 4) k_sample_batch(BatchParams B) {
         uint4 next = make_uint4(0, 0, 0, 0);
         uint32_t u = 0;
         if (live) {
-          if (I.eq) record_step<true>(I.erec, I.grec, rec, x.x, u, next);
-          else record_step<false>(I.erec, I.grec, rec, x.x, u, next);
+          if (I.layout == REC16) record_step<REC16>(I.T, v, rec, x.x, u, next);
+          else record_step<REC32>(I.T, v, rec, x.x, u, next);
         }
         const bool suspect = (sw >> (v & 31)) & 1u;
         if (suspect && (!I.p32 || source_coin(x.y, __ldg(&I.p32[v])))) {
@@ -245,10 +243,8 @@ hsaw_status batch_sample(const Graph* const* gs, const QueryDev* const* qds, Str
       const Graph& g = *gs[i];
       const QueryDev& qd = *qds[i];
       BatchInst b{};
-      b.node = g.node;
-      b.erec = g.erec;
-      b.eq = g.eq ? 1u : 0u;
-      b.grec = g.grec;
+      b.T = g.tables();
+      b.layout = g.layout;
       b.s_bits = qd.s_bits;
       b.p32 = qd.p32;
       b.a0 = st.next_attempt;

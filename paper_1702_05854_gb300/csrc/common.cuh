@@ -62,22 +62,34 @@ struct DBuf {  // grow-only device buffer
 // (0 if the in-weights differ), in-sum}; edge[e] = {tail node u of (u, v), running sum of
 // v's in-weights through e}.  In-edge j of v is live for a draw r iff
 // thr[j-1] <= r < thr[j]; none is live when r >= in-sum.
-// Walk records give the tail node of an edge and everything the next draw at that node
-// needs in one read, so a walk makes one dependent DRAM access per live-edge draw at
-// equal-weight nodes (the tail's record is replicated per in-edge).  Two layouts:
-//   eq (every node with in-weight has equal in-weights, as weighted cascade gives): erec[e] =
-//     {u, node[u].x, node[u].y, node[u].z} of edge e = (u, v), 16 bytes; the in-sum is
-//     in-degree times weight.  Half the bytes put twice the records into L2: dependent random
-//     reads measured 83 G/s on a 0.27 GB table against 55 G/s on 0.54 GB, 41 on 2.1 GB.
-//   otherwise erec[2e], erec[2e+1] = {u, node[u].x, node[u].y, node[u].z}, {node[u].w, thr[e],
-//     0, 0}, 32 bytes, sector aligned.
-// Guide tables (only when some node has unequal in-weights): for node v and bucket
-// b = floor(r * deg / in-sum) in [0, deg), the guide entry is the live in-edge index j0 of
-// the smallest draw of the bucket, ceil(b * in-sum / deg); the answer for any r of the
-// bucket is at or after it (Chen & Asau's guide table), usually within a step or two.
-// grec[2p], grec[2p+1] (p = first(v) + b) hold the walk record of in-edge j0 with j0 in
-// the second half's third word, so a draw reads its candidate record directly (one
-// dependent access, like equal weights) and steps through erec only past it.
+// What a walk reads at each draw depends on where the graph's tables lie (Layout):
+//   REC16, REC32: walk records, larger than L2 or well inside it.  A record gives the tail
+//     node of an edge and everything the next draw at that node needs in one read, so a walk
+//     makes one dependent access per live-edge draw at equal-weight nodes (the tail's node
+//     record is replicated per in-edge).  REC16, where every node with in-weight has equal
+//     in-weights (as weighted cascade gives): erec[e] = {u, node[u].x, node[u].y, node[u].z}
+//     of edge e = (u, v); the in-sum is in-degree times weight.  REC32: erec[2e], erec[2e+1] =
+//     {u, node[u].x, node[u].y, node[u].z}, {node[u].w, thr[e], 0, 0}, sector aligned, and for
+//     nodes with unequal weights grec[2p], grec[2p+1] (p = first(v) + b), the walk record of
+//     the live in-edge j0 of the smallest draw of bucket b = floor(r * deg / in-sum), with j0
+//     in the second half's third word: the answer for any r of the bucket is at or after it
+//     (Chen & Asau's guide table), usually within a step or two through erec.
+//   TAIL4, EDGE8: two or three small reads that L2 holds instead of one that it does not.
+//     TAIL4 (equal weights): tail[e] = u, then node[u].  EDGE8: the first in-edge to look at
+//     from guide[] (one entry per four in-edges of a node, from guide_base), edges from there
+//     four at a time (a sector), then node[u].
+// Dependent random reads measured 290 G/s on tables that L2 holds, 83 G/s on 0.27 GB, 55 on
+// 0.54 GB, 41 on 2.1 GB and 38 beyond 8 GB.
+enum Layout { REC16 = 0, REC32 = 1, TAIL4 = 2, EDGE8 = 3 };
+struct WalkTables {
+  const uint4* __restrict__ node;
+  const uint2* __restrict__ edge;
+  const uint4* __restrict__ erec;
+  const uint4* __restrict__ grec;
+  const uint32_t* __restrict__ tail;
+  const uint32_t* __restrict__ guide;
+};
+
 // Walk pool (query-independent traces, kept as an inverted index): for walk seed `seed`,
 // trace a (a < attempts) is attempt a's walk ignoring sources - its nodes until no live
 // in-edge or a detected cycle.  A query's HSAW of attempt a is the trace's prefix up to its
@@ -102,9 +114,12 @@ struct Graph {
   WalkPool pool;
   uint4* node = nullptr;
   uint2* edge = nullptr;
-  uint4* erec = nullptr;
-  uint4* grec = nullptr;
-  bool eq = false;  // 16-byte walk records, no guide records
+  Layout layout = REC32;
+  uint4* erec = nullptr;      // REC16, REC32
+  uint4* grec = nullptr;      // REC32
+  uint32_t* tail = nullptr;   // TAIL4
+  uint32_t* guide = nullptr;  // EDGE8
+  WalkTables tables() const { return {node, edge, erec, grec, tail, guide}; }
   int64_t* input_index = nullptr;  // CSR position -> input edge index (NULL = identity)
   int device = 0;
 };
@@ -238,9 +253,11 @@ void phase_end(void* token, cudaStream_t s, int phase);
 // One 32-byte walk record in ONE 256-bit load (p is 32-byte aligned: records start at a
 // cudaMalloc base).  As two 16-byte loads every record costs two L1 and two L2 requests for
 // the same sector: dependent random reads measured 29-32 G/s that way on tables of 2-34 GB
-// and 205 G/s in L2, against 38-41 and 290 G/s as one load (6 blocks of 256 per SM).
+// and 205 G/s in L2, against 38-41 and 290 G/s as one load (6 blocks of 256 per SM).  volatile:
+// without it the compiler may take the read for free of effects and hoist it above the test
+// that makes its address valid.
 __device__ __forceinline__ void load_record(const uint4* __restrict__ p, uint4& a, uint4& b) {
-  asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+  asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
       : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
       : "l"(p));
 }
@@ -260,35 +277,73 @@ __device__ __forceinline__ uint32_t quotient(uint32_t r, uint32_t w) {
   return q;
 }
 
-// The live in-edge e of a node with record rec = {first in-edge, in-degree, equal weight or
-// 0, in-sum} for a draw r < rec.w, read through the walk records (the same choice as
-// pick_in_edge: j = r / w at equal weights, otherwise the first j with r < thr[j], found
-// from the guide bucket's candidate onward).  u receives e's tail, next the tail's record.
-template <bool EQ>
-__device__ __forceinline__ uint32_t record_step(const uint4* __restrict__ erec, const uint4* __restrict__ grec,
-                                                uint4 rec, uint32_t r, uint32_t& u, uint4& next) {
-  if (EQ) {
-    const uint32_t e = rec.x + quotient(r, rec.z);
-    const uint4 x = __ldg(&erec[e]);
+// EDGE8: node v's guide entries start here, one per four in-edges (rounded up), which bases of
+// consecutive nodes leave room for.
+__device__ __forceinline__ uint32_t guide_base(uint32_t first, uint32_t v) { return (first >> 2) + v; }
+// The guide entry of draw r < insum.  The float arithmetic is off by less than 2^-21 of the
+// bucket's number, so r >= b insum / buckets (1 - 2^-20): guide[] is built for that draw.
+__device__ __forceinline__ uint32_t guide_entry(uint32_t r, uint32_t deg, uint32_t insum) {
+  const uint32_t buckets = (deg + 3) >> 2;
+  const uint32_t b = __float2uint_rz(__uint2float_rz(r) *
+                                     __fdividef(__uint2float_rn(buckets), __uint2float_rn(insum)));
+  return min(b, buckets - 1);
+}
+
+// The live in-edge e of node v with record rec = {first in-edge, in-degree, equal weight or
+// 0, in-sum} for a draw r < rec.w, read through the graph's tables (the same choice as
+// pick_in_edge: j = r / w at equal weights, otherwise the first j with r < thr[j]).  u
+// receives e's tail, next the tail's record.
+template <Layout L>
+__device__ __forceinline__ uint32_t record_step(const WalkTables& T, uint32_t v, uint4 rec, uint32_t r, uint32_t& u,
+                                                uint4& next) {
+  uint32_t e;
+  if (L == REC16) {
+    e = rec.x + quotient(r, rec.z);
+    const uint4 x = __ldg(&T.erec[e]);
     u = x.x;
     next = make_uint4(x.y, x.z, x.w, x.z * x.w);
-    return e;
-  }
-  uint32_t e;
-  uint4 ra, rb;
-  if (rec.z) {
+  } else if (L == TAIL4) {
     e = rec.x + quotient(r, rec.z);
-    load_record(erec + 2 * (size_t)e, ra, rb);
-  } else {
-    load_record(grec + 2 * ((size_t)rec.x + guide_bucket(r, rec.y, rec.w)), ra, rb);
-    e = rec.x + rb.z;
-    while (r >= rb.y) {
-      ++e;
-      load_record(erec + 2 * (size_t)e, ra, rb);
+    u = __ldg(&T.tail[e]);
+    next = __ldg(&T.node[u]);
+  } else if (L == REC32) {
+    uint4 ra, rb;
+    if (rec.z) {
+      e = rec.x + quotient(r, rec.z);
+      load_record(T.erec + 2 * (size_t)e, ra, rb);
+    } else {
+      load_record(T.grec + 2 * ((size_t)rec.x + guide_bucket(r, rec.y, rec.w)), ra, rb);
+      e = rec.x + rb.z;
+      while (r >= rb.y) {
+        ++e;
+        load_record(T.erec + 2 * (size_t)e, ra, rb);
+      }
     }
+    u = ra.x;
+    next = make_uint4(ra.y, ra.z, ra.w, rb.x);
+  } else {
+    if (rec.z) {
+      e = rec.x + quotient(r, rec.z);
+      u = __ldg(&T.edge[e].x);
+    } else {
+      e = rec.x + __ldg(&T.guide[guide_base(rec.x, v) + guide_entry(r, rec.y, rec.w)]);
+      for (;;) {  // r < thr of the list's last edge, so the search ends inside the list
+        const uint32_t at = e & ~3u;
+        uint4 a, b;  // edges at .. at + 3, {tail, running sum} each
+        load_record(reinterpret_cast<const uint4*>(T.edge + at), a, b);
+        uint32_t past = (r < a.y ? 1u : 0u) | (r < a.w ? 2u : 0u) | (r < b.y ? 4u : 0u) | (r < b.w ? 8u : 0u);
+        past &= 0xFu << (e & 3u);
+        if (past) {
+          const uint32_t i = __ffs(past) - 1;
+          e = at + i;
+          u = i == 0 ? a.x : i == 1 ? a.z : i == 2 ? b.x : b.z;
+          break;
+        }
+        e = at + 4;
+      }
+    }
+    next = __ldg(&T.node[u]);
   }
-  u = ra.x;
-  next = make_uint4(ra.y, ra.z, ra.w, rb.x);
   return e;
 }
 

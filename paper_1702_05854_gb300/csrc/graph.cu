@@ -288,30 +288,57 @@ __device__ __forceinline__ void guide_record(uint4 nd, uint32_t b, const uint2* 
   grec[p + 1] = second;
 }
 
+// EDGE8: guide entry b of a node with unequal in-weights, the live in-edge of the smallest draw
+// that may look it up (see guide_entry).
+__device__ __forceinline__ void guide_first(uint4 nd, uint32_t v, uint32_t b, const uint2* __restrict__ edge,
+                                            uint32_t* __restrict__ guide) {
+  const uint32_t buckets = (nd.y + 3) >> 2;
+  const uint32_t at = (uint32_t)((uint64_t)b * nd.w / buckets), off = (at >> 20) + 1;
+  const uint32_t lb = at > off ? at - off : 0u;
+  uint32_t lo = 0, hi = nd.y;
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (lb < edge[nd.x + mid].y) hi = mid; else lo = mid + 1;
+  }
+  guide[guide_base(nd.x, v) + b] = lo;
+}
+
 // One warp per node, and a block per slice of a hub's buckets (one warp on the longest list
-// took the whole pass: 4.7 ms on R-MAT 20).
+// took the whole pass: 4.7 ms on R-MAT 20).  grec: bucket records (REC32), else guide (EDGE8).
 __global__ void k_guide(const uint4* __restrict__ node, const uint2* __restrict__ edge, int64_t n,
-                        const uint4* __restrict__ erec, uint4* __restrict__ grec) {
+                        const uint4* __restrict__ erec, uint4* __restrict__ grec, uint32_t* __restrict__ guide) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
     const uint4 nd = node[v];
     if (nd.z != 0 || nd.w == 0 || nd.y > HUB_DEGREE) continue;  // equal weights, no in-weight, or a hub
-    for (uint32_t b = lane; b < nd.y; b += 32) guide_record(nd, b, edge, erec, grec);
+    if (grec)
+      for (uint32_t b = lane; b < nd.y; b += 32) guide_record(nd, b, edge, erec, grec);
+    else
+      for (uint32_t b = lane; b < (nd.y + 3) >> 2; b += 32) guide_first(nd, (uint32_t)v, b, edge, guide);
   }
 }
 
 __global__ void __launch_bounds__(256) k_hub_guide(const uint4* __restrict__ node, const uint2* __restrict__ edge,
                                                    Hubs hubs, const uint4* __restrict__ erec,
-                                                   uint4* __restrict__ grec) {
+                                                   uint4* __restrict__ grec, uint32_t* __restrict__ guide) {
   constexpr uint32_t SLICES = 16;
   const uint64_t items = (uint64_t)*hubs.count * SLICES;
   for (uint64_t i = blockIdx.x; i < items; i += gridDim.x) {
-    const uint4 nd = node[hubs.node[i / SLICES]];
+    const uint32_t v = hubs.node[i / SLICES];
+    const uint4 nd = node[v];
     if (nd.z != 0 || nd.w == 0) continue;
-    for (uint32_t b = (uint32_t)(i % SLICES) * blockDim.x + threadIdx.x; b < nd.y; b += SLICES * blockDim.x)
-      guide_record(nd, b, edge, erec, grec);
+    const uint32_t buckets = grec ? nd.y : (nd.y + 3) >> 2;
+    for (uint32_t b = (uint32_t)(i % SLICES) * blockDim.x + threadIdx.x; b < buckets; b += SLICES * blockDim.x) {
+      if (grec) guide_record(nd, b, edge, erec, grec);
+      else guide_first(nd, v, b, edge, guide);
+    }
   }
+}
+
+__global__ void k_tails(const uint2* __restrict__ edge, int64_t m, uint32_t* __restrict__ tail) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x)
+    tail[e] = edge[e].x;
 }
 
 // ------------------------------------------------------------------ host
@@ -366,8 +393,12 @@ static void destroy_graph(Graph& g) {
   if (g.input_index) cudaFree(g.input_index);
   if (g.erec) cudaFree(g.erec);
   if (g.grec) cudaFree(g.grec);
+  if (g.tail) cudaFree(g.tail);
+  if (g.guide) cudaFree(g.guide);
   g.erec = nullptr;
   g.grec = nullptr;
+  g.tail = nullptr;
+  g.guide = nullptr;
   g.node = nullptr;
   g.edge = nullptr;
   g.input_index = nullptr;
@@ -378,7 +409,7 @@ static hsaw_status alloc_graph(Graph& g, int64_t n, int64_t m, bool with_index) 
   g.m = m;
   cudaGetDevice(&g.device);
   HSAW_CK(cudaMalloc((void**)&g.node, (size_t)n * sizeof(uint4)));
-  HSAW_CK(cudaMalloc((void**)&g.edge, (size_t)(m ? m : 1) * sizeof(uint2)));
+  HSAW_CK(cudaMalloc((void**)&g.edge, (size_t)(m + 4) / 4 * 4 * sizeof(uint2)));
   if (with_index) HSAW_CK(cudaMalloc((void**)&g.input_index, (size_t)(m ? m : 1) * sizeof(int64_t)));
   return HSAW_OK;
 }
@@ -418,6 +449,22 @@ struct Temps {
   }
 };
 
+// Walk tables by size (see Layout): the small ones where the records do not fit L2 and the
+// small ones do, or nearly.  Sampler, G draws/s, records against small tables, R-MAT edge
+// factor 16 (L2 129 MB): equal weights, scale 18 to 23: 171/135, 111/122, 70/98, 51/63, 44/46,
+// 40/36; random weights, scale 16 to 22: 78/84, 73/85, 65/82, 54/73, 46/58, 40/40, 36/30.
+static Layout choose_layout(int64_t n, int64_t m, bool eq) {
+  static const double l2 = [] {
+    int dev = 0, bytes = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&bytes, cudaDevAttrL2CacheSize, dev);
+    return (double)bytes;
+  }();
+  const double N = (double)n, M = (double)m;
+  if (eq) return 16 * M > l2 && 4 * M + 16 * N <= 3.0 * l2 ? TAIL4 : REC16;
+  return 64 * M > 0.25 * l2 && 9 * M + 20 * N <= 2.6 * l2 ? EDGE8 : REC32;
+}
+
 static hsaw_status finish_graph(Graph& g, uint32_t* row_start, uint32_t* d_err, Temps& T, cudaStream_t s) {
   const int64_t n = g.n;
   Hubs hubs;
@@ -436,27 +483,38 @@ static hsaw_status finish_graph(Graph& g, uint32_t* row_start, uint32_t* d_err, 
   uint32_t unequal = 0;
   HSAW_TRY(check_err(d_err, s, &unequal));
   if (!g.m) return HSAW_OK;
-  g.eq = unequal == 0;
-  HSAW_CK(cudaMalloc((void**)&g.erec, (size_t)g.m * (g.eq ? 1 : 2) * sizeof(uint4)));
-  count_launch();
-  if (g.eq) {
-    k_walk_records<true><<<grid_for(g.m, 256, 1u << 16), 256, 0, s>>>(g.edge, g.node, g.m, g.erec);
+  g.layout = choose_layout(n, g.m, unequal == 0);
+  if (g.layout == TAIL4) {
+    HSAW_CK(cudaMalloc((void**)&g.tail, (size_t)g.m * sizeof(uint32_t)));
+    count_launch();
+    k_tails<<<grid_for(g.m, 256, 1u << 16), 256, 0, s>>>(g.edge, g.m, g.tail);
     HSAW_CK(cudaGetLastError());
     return HSAW_OK;
   }
-  k_walk_records<false><<<grid_for(g.m, 256, 1u << 16), 256, 0, s>>>(g.edge, g.node, g.m, g.erec);
-  HSAW_CK(cudaGetLastError());
-  if (cudaMalloc((void**)&g.grec, (size_t)g.m * 2 * sizeof(uint4)) != cudaSuccess) {
-    cudaGetLastError();
-    g.grec = nullptr;
-    return fail(HSAW_E_NOMEM, "graph: guide records do not fit in device memory");
+  if (g.layout == EDGE8) {
+    HSAW_CK(cudaMalloc((void**)&g.guide, ((size_t)g.m / 4 + (size_t)n + 1) * sizeof(uint32_t)));
+  } else {
+    HSAW_CK(cudaMalloc((void**)&g.erec, (size_t)g.m * (g.layout == REC16 ? 1 : 2) * sizeof(uint4)));
+    count_launch();
+    if (g.layout == REC16) {
+      k_walk_records<true><<<grid_for(g.m, 256, 1u << 16), 256, 0, s>>>(g.edge, g.node, g.m, g.erec);
+      HSAW_CK(cudaGetLastError());
+      return HSAW_OK;
+    }
+    k_walk_records<false><<<grid_for(g.m, 256, 1u << 16), 256, 0, s>>>(g.edge, g.node, g.m, g.erec);
+    HSAW_CK(cudaGetLastError());
+    if (cudaMalloc((void**)&g.grec, (size_t)g.m * 2 * sizeof(uint4)) != cudaSuccess) {
+      cudaGetLastError();
+      g.grec = nullptr;
+      return fail(HSAW_E_NOMEM, "graph: guide records do not fit in device memory");
+    }
   }
   count_launch();
-  k_guide<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(g.node, g.edge, n, g.erec, g.grec);
+  k_guide<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(g.node, g.edge, n, g.erec, g.grec, g.guide);
   HSAW_CK(cudaGetLastError());
   if (g.m > HUB_DEGREE) {
     count_launch();
-    k_hub_guide<<<8 * sm_count(), 256, 0, s>>>(g.node, g.edge, hubs, g.erec, g.grec);
+    k_hub_guide<<<8 * sm_count(), 256, 0, s>>>(g.node, g.edge, hubs, g.erec, g.grec, g.guide);
     HSAW_CK(cudaGetLastError());
   }
   return HSAW_OK;

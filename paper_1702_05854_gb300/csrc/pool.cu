@@ -28,19 +28,19 @@ constexpr uint32_t POOL_SHIFT = 22;
 
 // Calls f(v) for every node of attempt a's trace (the detected repeat that ends it is not
 // passed); false when the step guard trips.
-template <class F>
-__device__ __forceinline__ bool for_trace(const uint4* __restrict__ node, const uint2* __restrict__ edge, uint32_t n,
-                                          uint32_t k0, uint32_t k1, uint64_t a, uint32_t step_cap, uint32_t* len,
-                                          F&& f) {
+template <Layout L, class F>
+__device__ __forceinline__ bool for_trace(const WalkTables& T, uint32_t n, uint32_t k0, uint32_t k1, uint64_t a,
+                                          uint32_t step_cap, uint32_t* len, F&& f) {
   uint32_t v = start_node(a, n, k0, k1), l = 1;
   f(v);
   Ckpt ck;
   ck.reset(v);
+  uint4 rec = __ldg(&T.node[v]);
   for (;;) {
     const uint4 x = node_draw(a, v, k0, k1);
-    const uint4 nd = __ldg(&node[v]);
-    if (x.x >= nd.w) break;  // no live in-edge
-    const uint32_t u = __ldg(&edge[nd.x + pick_in_edge(edge, nd, x.x)].x);
+    if (x.x >= rec.w) break;  // no live in-edge
+    uint32_t u;
+    record_step<L>(T, v, rec, x.x, u, rec);
     if (ck.seen(u)) break;  // cycle: u repeats an earlier node
     ++l;
     f(u);
@@ -56,7 +56,8 @@ __device__ __forceinline__ bool for_trace(const uint4* __restrict__ node, const 
 }
 
 // Pass 1: cnt[b (n + 1) + v] += trace nodes of block b's attempts at v; btot[b] += their sum.
-__global__ void k_pool_count(const uint4* __restrict__ node, const uint2* __restrict__ edge, uint32_t n, uint32_t k0,
+template <Layout L>
+__global__ void k_pool_count(const WalkTables T, uint32_t n, uint32_t k0,
                              uint32_t k1, uint64_t attempts, uint32_t step_cap, uint32_t* __restrict__ cnt,
                              unsigned long long* __restrict__ btot, uint32_t* __restrict__ status) {
   const int lane = threadIdx.x & 31;
@@ -72,7 +73,7 @@ __global__ void k_pool_count(const uint4* __restrict__ node, const uint2* __rest
     }
     const uint64_t base = b * ((uint64_t)n + 1);
     uint32_t len = 0;
-    const bool ok = for_trace(node, edge, n, k0, k1, a, step_cap, &len, [&](uint32_t v) {
+    const bool ok = for_trace<L>(T, n, k0, k1, a, step_cap, &len, [&](uint32_t v) {
       const unsigned long long key = base + v;
       const unsigned grp = __match_any_sync(__activemask(), key);
       if (lane == __ffs(grp) - 1) atomicAdd(&cnt[key], (uint32_t)__popc(grp));
@@ -85,7 +86,8 @@ __global__ void k_pool_count(const uint4* __restrict__ node, const uint2* __rest
 
 // Pass 2: each trace node v of attempt a takes the next slot of its list (cursor starts
 // as the node offsets) and receives a's id within its block.
-__global__ void k_pool_fill(const uint4* __restrict__ node, const uint2* __restrict__ edge, uint32_t n, uint32_t k0,
+template <Layout L>
+__global__ void k_pool_fill(const WalkTables T, uint32_t n, uint32_t k0,
                             uint32_t k1, uint64_t attempts, uint32_t step_cap, uint32_t* __restrict__ cursor,
                             const uint64_t* __restrict__ boff, uint32_t* __restrict__ ent) {
   const int lane = threadIdx.x & 31;
@@ -96,7 +98,7 @@ __global__ void k_pool_fill(const uint4* __restrict__ node, const uint2* __restr
     uint32_t* out = ent + boff[b];
     const uint32_t local = (uint32_t)(a - (b << POOL_SHIFT));
     uint32_t len = 0;
-    for_trace(node, edge, n, k0, k1, a, step_cap, &len, [&](uint32_t v) {
+    for_trace<L>(T, n, k0, k1, a, step_cap, &len, [&](uint32_t v) {
       const unsigned long long key = base + v;
       const unsigned grp = __match_any_sync(__activemask(), key);
       const int leader = __ffs(grp) - 1;
@@ -175,15 +177,14 @@ __global__ void k_bits_emit(const uint32_t* __restrict__ bits, const uint32_t* _
 
 // Length of each pooled hit: nodes walked up to and including its first real source.  A
 // walk that meets no source first (impossible for an attempt the index lists) sets bit 2.
-template <bool HAS_P, bool EQ>
-__global__ void k_hit_len(const uint4* __restrict__ node, const uint4* __restrict__ erec, const uint4* __restrict__ grec,
-                          uint32_t n, uint32_t k0, uint32_t k1, const uint32_t* __restrict__ s_bits,
+template <bool HAS_P, Layout L>
+__global__ void k_hit_len(const WalkTables T, uint32_t n, uint32_t k0, uint32_t k1, const uint32_t* __restrict__ s_bits,
                           const uint32_t* __restrict__ p32, const uint64_t* __restrict__ aid, uint32_t count,
                           uint32_t step_cap, uint32_t* __restrict__ len, uint32_t* __restrict__ status) {
   for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < count; h += gridDim.x * blockDim.x) {
     const uint64_t a = aid[h];
     uint32_t v = start_node(a, n, k0, k1), l = 1;
-    uint4 rec = __ldg(&node[v]);
+    uint4 rec = __ldg(&T.node[v]);
     for (;;) {
       const uint4 x = node_draw(a, v, k0, k1);
       if (((__ldg(&s_bits[v >> 5]) >> (v & 31)) & 1u) && (!HAS_P || source_coin(x.y, __ldg(&p32[v])))) break;
@@ -191,7 +192,7 @@ __global__ void k_hit_len(const uint4* __restrict__ node, const uint4* __restric
         atomicOr(status, 2u);
         break;
       }
-      record_step<EQ>(erec, grec, rec, x.x, v, rec);
+      record_step<L>(T, v, rec, x.x, v, rec);
       ++l;
     }
     len[h] = l;
@@ -246,7 +247,11 @@ hsaw_status pool_build(Graph& g, uint64_t seed, uint64_t attempts, cudaStream_t 
     return finish(fail(HSAW_E_DEVICE, "walk pool: clearing the counts failed"));
   const unsigned grid = (unsigned)(sm_count() * 16);
   count_launch();
-  k_pool_count<<<grid, 128, 0, s>>>(g.node, g.edge, (uint32_t)g.n, k0, k1, attempts, cap, p.noff, btot, status);
+  const decltype(&k_pool_count<REC16>) count_by[] = {k_pool_count<REC16>, k_pool_count<REC32>, k_pool_count<TAIL4>,
+                                                     k_pool_count<EDGE8>};
+  const decltype(&k_pool_fill<REC16>) fill_by[] = {k_pool_fill<REC16>, k_pool_fill<REC32>, k_pool_fill<TAIL4>,
+                                                   k_pool_fill<EDGE8>};
+  count_by[g.layout]<<<grid, 128, 0, s>>>(g.tables(), (uint32_t)g.n, k0, k1, attempts, cap, p.noff, btot, status);
   std::vector<unsigned long long> tot(blocks);
   uint32_t hs = 0;
   if (cudaGetLastError() != cudaSuccess ||
@@ -276,7 +281,7 @@ hsaw_status pool_build(Graph& g, uint64_t seed, uint64_t attempts, cudaStream_t 
   if (cudaMemcpyAsync(cursor, p.noff, noff_n * 4, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
     return finish(fail(HSAW_E_DEVICE, "walk pool: cursor copy failed"));
   count_launch();
-  k_pool_fill<<<grid, 128, 0, s>>>(g.node, g.edge, (uint32_t)g.n, k0, k1, attempts, cap, cursor, p.boff, p.ent);
+  fill_by[g.layout]<<<grid, 128, 0, s>>>(g.tables(), (uint32_t)g.n, k0, k1, attempts, cap, cursor, p.boff, p.ent);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
     return finish(fail(HSAW_E_DEVICE, "walk pool: index fill failed"));
   st = finish(HSAW_OK);
@@ -328,9 +333,11 @@ hsaw_status pool_hits(const Graph& g, const QueryDev& qd, Stream& st, uint64_t a
   HSAW_CK(cudaGetLastError());
   const unsigned hgrid = grid_for(h, 128, 1u << 16);
   count_launch();
-  const auto hit_len = qd.p32 ? (g.eq ? k_hit_len<true, true> : k_hit_len<true, false>)
-                              : (g.eq ? k_hit_len<false, true> : k_hit_len<false, false>);
-  hit_len<<<hgrid, 128, 0, s>>>(g.node, g.erec, g.grec, (uint32_t)g.n, k0, k1, qd.s_bits, qd.p32, st.aid.p + st.count, h,
+  const decltype(&k_hit_len<true, REC16>) by_layout[2][4] = {
+      {k_hit_len<false, REC16>, k_hit_len<false, REC32>, k_hit_len<false, TAIL4>, k_hit_len<false, EDGE8>},
+      {k_hit_len<true, REC16>, k_hit_len<true, REC32>, k_hit_len<true, TAIL4>, k_hit_len<true, EDGE8>}};
+  const auto hit_len = by_layout[qd.p32 ? 1 : 0][g.layout];
+  hit_len<<<hgrid, 128, 0, s>>>(g.tables(), (uint32_t)g.n, k0, k1, qd.s_bits, qd.p32, st.aid.p + st.count, h,
                                 pool_step_cap(g), st.len.p + st.count, st.ctrs.p + 3);
   HSAW_CK(cudaGetLastError());
   uint32_t bad = 0;

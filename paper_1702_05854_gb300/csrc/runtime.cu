@@ -36,6 +36,7 @@ static bool batchable(const hsaw_graph g, const hsaw_query& q) {
   if (!g || q.sampling != HSAW_FIXED_N || q.n_hsaw < 1 || q.n_sources < 1 || !q.sources) return false;
   const Graph& G = g->g;
   if (G.pool.ent && G.pool.seed == q.seed) return false;
+  if (G.layout != REC16 && G.layout != REC32) return false;  // the joint sampler walks records
   const bool ok = validate_query(G, &q) == HSAW_OK;  // an invalid one fails on its own path
   if (!ok) set_error("");
   return ok;

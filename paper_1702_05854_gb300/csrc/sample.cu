@@ -26,10 +26,7 @@ namespace hsaw {
 enum : uint32_t { ST_OVERFLOW = 1u, ST_STEP_CAP = 2u };
 
 struct SampleParams {
-  const uint4* __restrict__ node;
-  const uint2* __restrict__ edge;
-  const uint4* __restrict__ erec;
-  const uint4* __restrict__ grec;
+  WalkTables T;
   const uint32_t* __restrict__ s_bits;
   const uint32_t* __restrict__ p32;
   const uint32_t* __restrict__ edge_removed;
@@ -66,7 +63,7 @@ __device__ __forceinline__ bool bit_at(const uint32_t* __restrict__ bits, uint32
 constexpr int SAMPLE_WARPS = 8;
 constexpr int START_SLOTS = 64;  // at most 31 left when 32 more are drawn
 
-template <bool HAS_P, bool HAS_REM, bool EQ>
+template <bool HAS_P, bool HAS_REM, Layout L>
 __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_constant__ SampleParams P) {
   __shared__ uint4 start_rec[SAMPLE_WARPS][START_SLOTS];  // node record of the start
   __shared__ uint2 start_at[SAMPLE_WARPS][START_SLOTS];   // attempt (within the launch), start node
@@ -105,7 +102,7 @@ __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_co
         if (i < cur_end) {
           const uint64_t a = P.a0 + i;
           sv = __umulhi(philox4x32_10_rk(make_uint4((uint32_t)a, (uint32_t)(a >> 32), 0u, 1u), P.keys).x, P.n);
-          srec = __ldg(&P.node[sv]);
+          srec = __ldg(&P.T.node[sv]);
           walk = bit_at(P.s_bits, sv) || srec.w != 0;
           if (HAS_REM && P.node_removed && bit_at(P.node_removed, sv)) walk = false;
         }
@@ -143,7 +140,7 @@ __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_co
       const bool live = x.x < rec.w;
       uint4 next = make_uint4(0, 0, 0, 0);
       uint32_t e = 0, u = 0;
-      if (live) e = record_step<EQ>(P.erec, P.grec, rec, x.x, u, next);
+      if (live) e = record_step<L>(P.T, v, rec, x.x, u, next);
       bool gone = false;  // the removal bit is read beside the walk record
       if (HAS_REM && live && P.edge_removed) gone = bit_at(P.edge_removed, e);
       const bool suspect = (sw >> (v & 31)) & 1u;
@@ -224,9 +221,8 @@ __global__ void k_offsets(const uint64_t* __restrict__ excl, int64_t n, int64_t 
 }
 
 // Re-derive hit walks from their attempt ids (path encoding) into the flat buffers.
-template <bool EQ>
-__global__ void k_rewalk(const uint4* __restrict__ node, const uint4* __restrict__ erec, const uint4* __restrict__ grec,
-                         uint32_t n, uint32_t k0, uint32_t k1, const uint64_t* __restrict__ aid,
+template <Layout L>
+__global__ void k_rewalk(const WalkTables T, uint32_t n, uint32_t k0, uint32_t k1, const uint64_t* __restrict__ aid,
                          const uint32_t* __restrict__ len, const int64_t* __restrict__ node_off, int64_t h0, int64_t h1,
                          int32_t* __restrict__ nodes, int32_t* __restrict__ edges) {
   for (int64_t h = h0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; h < h1; h += (int64_t)gridDim.x * blockDim.x) {
@@ -235,11 +231,11 @@ __global__ void k_rewalk(const uint4* __restrict__ node, const uint4* __restrict
     const int64_t nb = node_off[h], eb = nb - h;
     uint32_t v = start_node(a, n, k0, k1);
     nodes[nb] = (int32_t)v;
-    uint4 rec = l > 1 ? __ldg(&node[v]) : make_uint4(0, 0, 0, 0);
+    uint4 rec = l > 1 ? __ldg(&T.node[v]) : make_uint4(0, 0, 0, 0);
     for (uint32_t i = 1; i < l; ++i) {
       const uint4 x = node_draw(a, v, k0, k1);
       if (x.x >= rec.w) break;  // a hit's walk has a live in-edge at each of its first l - 1 nodes
-      edges[eb + i - 1] = (int32_t)record_step<EQ>(erec, grec, rec, x.x, v, rec);
+      edges[eb + i - 1] = (int32_t)record_step<L>(T, v, rec, x.x, v, rec);
       nodes[nb + i] = (int32_t)v;
     }
   }
@@ -260,10 +256,10 @@ __global__ void k_classify(SampleParams P, uint64_t first, int64_t count, int8_t
       const bool suspect = (__ldg(&P.s_bits[v >> 5]) >> (v & 31)) & 1u;
       const uint4 x = node_draw(a, v, P.k0, P.k1);
       if (suspect && (!HAS_P || source_coin(x.y, __ldg(&P.p32[v])))) { out = 1; break; }
-      const uint4 nd = __ldg(&P.node[v]);
+      const uint4 nd = __ldg(&P.T.node[v]);
       if (x.x >= nd.w) { out = 0; break; }
-      const uint32_t e = nd.x + pick_in_edge(P.edge, nd, x.x);
-      const uint32_t u = __ldg(&P.edge[e].x);
+      const uint32_t e = nd.x + pick_in_edge(P.T.edge, nd, x.x);
+      const uint32_t u = __ldg(&P.T.edge[e].x);
       if (HAS_REM && ((P.edge_removed && bit_at(P.edge_removed, e)) || (P.node_removed && bit_at(P.node_removed, u)))) {
         out = 3;
         break;
@@ -389,10 +385,7 @@ hsaw_status stream_init(Stream& st, uint64_t first_attempt, uint64_t max_attempt
 
 static SampleParams make_params(const Graph& g, const QueryDev& qd) {
   SampleParams P{};
-  P.node = g.node;
-  P.edge = g.edge;
-  P.erec = g.erec;
-  P.grec = g.grec;
+  P.T = g.tables();
   P.s_bits = qd.s_bits;
   P.p32 = qd.p32;
   P.edge_removed = qd.edge_removed;
@@ -408,7 +401,7 @@ static SampleParams make_params(const Graph& g, const QueryDev& qd) {
 static int sample_blocks_per_sm() {
   static const int cached = [] {
     int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sample<false, false, true>, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sample<false, false, REC16>, 256, 0);
     return b > 0 ? b : 1;
   }();
   return cached;
@@ -470,19 +463,23 @@ static void sample_tune_record(const Graph& g, int trial, double draws, float ms
             t.rate[1] / 1e6);
 }
 
-template <bool EQ>
+template <Layout L>
 static void launch_sample_as(const SampleParams& P, unsigned grid, cudaStream_t s) {
   const bool hp = P.p32 != nullptr, hr = (P.edge_removed || P.node_removed);
   count_launch();
-  if (hp && hr) k_sample<true, true, EQ><<<grid, 256, 0, s>>>(P);
-  else if (hp) k_sample<true, false, EQ><<<grid, 256, 0, s>>>(P);
-  else if (hr) k_sample<false, true, EQ><<<grid, 256, 0, s>>>(P);
-  else k_sample<false, false, EQ><<<grid, 256, 0, s>>>(P);
+  if (hp && hr) k_sample<true, true, L><<<grid, 256, 0, s>>>(P);
+  else if (hp) k_sample<true, false, L><<<grid, 256, 0, s>>>(P);
+  else if (hr) k_sample<false, true, L><<<grid, 256, 0, s>>>(P);
+  else k_sample<false, false, L><<<grid, 256, 0, s>>>(P);
 }
 
 static void launch_sample(const Graph& g, const SampleParams& P, unsigned grid, cudaStream_t s) {
-  if (g.eq) launch_sample_as<true>(P, grid, s);
-  else launch_sample_as<false>(P, grid, s);
+  switch (g.layout) {
+    case REC16: launch_sample_as<REC16>(P, grid, s); break;
+    case REC32: launch_sample_as<REC32>(P, grid, s); break;
+    case TAIL4: launch_sample_as<TAIL4>(P, grid, s); break;
+    case EDGE8: launch_sample_as<EDGE8>(P, grid, s); break;
+  }
 }
 
 // One sampler launch over attempts [st.next_attempt, + batch): hits are recorded per chunk
@@ -629,9 +626,10 @@ hsaw_status stream_take_hits(const Graph& g, const QueryDev& qd, Stream& st, uin
   HSAW_TRY(st.nodes.ensure((size_t)tot, s, true));
   HSAW_TRY(st.edges.ensure((size_t)tot, s, true));
   const unsigned grid = grid_for(new_hits, 128, 1u << 16);
-  const auto rewalk = g.eq ? k_rewalk<true> : k_rewalk<false>;
+  const decltype(&k_rewalk<REC16>) by_layout[] = {k_rewalk<REC16>, k_rewalk<REC32>, k_rewalk<TAIL4>, k_rewalk<EDGE8>};
+  const auto rewalk = by_layout[g.layout];
   count_launch();
-  rewalk<<<grid, 128, 0, s>>>(g.node, g.erec, g.grec, (uint32_t)g.n, k0, k1, st.aid.p, st.len.p, st.node_off.p, st.count,
+  rewalk<<<grid, 128, 0, s>>>(g.tables(), (uint32_t)g.n, k0, k1, st.aid.p, st.len.p, st.node_off.p, st.count,
                               st.count + new_hits, st.nodes.p, st.edges.p);
   HSAW_CK(cudaGetLastError());
   st.total_nodes = tot;
@@ -761,10 +759,7 @@ extern "C" hsaw_status hsaw_sample_hits_static(hsaw_graph g, const uint32_t* sus
   HSAW_TRY(static_scratch(&sc));
   cudaStream_t s = (cudaStream_t)stream;
   SampleParams P{};
-  P.node = G.node;
-  P.edge = G.edge;
-  P.erec = G.erec;
-  P.grec = G.grec;
+  P.T = G.tables();
   P.s_bits = suspect_bits;
   P.n = (uint32_t)G.n;
   P.k0 = (uint32_t)seed;

@@ -89,6 +89,42 @@ def test_hub_lists(deg, kind):
         assert_same_stream(hs.hsaw_sample(graph, hs.Query(sources=sources, seed=9), 0, 300), ost, 300)
 
 
+def test_small_tables_unequal():
+    """Graphs whose records would not fit L2 are walked through edges and a guide of one entry per four in-edges:
+    in-lists of every length around the guide's groups, the sector and the hub threshold, with weights from uniform to
+    one that takes nearly all."""
+    rng = np.random.default_rng(3)
+    parts, base = [], 0
+    for deg in [*range(1, 14), 31, 32, 33, 63, 64, 65, 1023, 1024, 1025, 1027, 4096, 4099, 50_001, 600_000]:
+        for skew in (0.0, 3.0):
+            _, src, dst, w = hub_graph(deg, 1)
+            x = (rng.random(deg) + 1e-3) ** (1.0 + skew)
+            if skew:
+                x[rng.integers(deg)] = 20.0 * deg
+            w[:deg] = np.floor(x / x.sum() * rng.uniform(0.6, 1.0) * ONE).astype(np.uint32)
+            parts.append((src + base, dst + base, w))
+            base += deg + 1
+    src, dst, w = (np.concatenate(p) for p in zip(*parts))
+    order = rng.permutation(src.size)
+    src, dst, w = src[order], dst[order], w[order]
+    g, og = hs.hsaw_graph_from_edges(base, src, dst, w), oracle.Graph(base, src, dst, w)
+    sources = np.arange(1, base, 11, dtype=np.int32)
+    for first in (0, (1 << 32) - 500):
+        ost = oracle.Stream(oracle.Query(og, sources, seed=2), first_aid=first).extend(4000)
+        assert_same_stream(hs.hsaw_sample(g, hs.Query(sources=sources, seed=2), first, 4000), ost, 4000)
+
+
+def test_small_tables_equal():
+    """Equal weights beyond L2 as records: tails and node records."""
+    n, m = 400_003, 9_500_001
+    src, dst = synth.chung_lu_graph(n, m, 2.1, 6)
+    w = synth.wc_weights(n, dst)
+    g, og = hs.hsaw_graph_from_edges(n, src, dst, w), oracle.Graph(n, src, dst, w)
+    sources, p = synth.sources(n, 20_000, 8), synth.probabilities(20_000, 9)
+    ost = oracle.Stream(oracle.Query(og, sources, p_fixed=p, seed=2)).extend(3000)
+    assert_same_stream(hs.hsaw_sample(g, hs.Query(sources=sources, p_fixed=p, seed=2), 0, 3000), ost, 3000)
+
+
 @pytest.mark.parametrize("deg", [1024, 1025, 9000])
 def test_hub_overweight(deg):
     """An in-sum of 2^32 is refused, 2^32 - 1 accepted, above and below the hub threshold."""
