@@ -108,13 +108,12 @@ static hsaw_status fixed_tail(const Graph& g, const hsaw_query* q, Stream& st, C
   const int64_t M = q->mode == HSAW_EDGE ? g.m : g.n;
   const int32_t k = q->k;
   void* ph = phase_begin(s);
-  HSAW_TRY(cover_build(st, q->mode, 0, q->n_hsaw, cv, s));
+  HSAW_TRY(cover_build(st, q->mode, 0, q->n_hsaw, cv, s, true));
   phase_end(ph, s, PH_COUNT);
   ph = phase_begin(s);
-  HSAW_TRY(cover_greedy(cv, cand, M, k, r->ids, r->gains, s));
-  phase_end(ph, s, PH_GREEDY);
   uint64_t last = 0;
-  HSAW_TRY(aid_at(st, q->n_hsaw - 1, &last, s));
+  HSAW_TRY(cover_greedy(cv, cand, M, k, r->ids, r->gains, s, st.aid.p + q->n_hsaw - 1, &last));
+  phase_end(ph, s, PH_GREEDY);
   uint64_t cov = 0;
   for (int32_t i = 0; i < k; ++i) cov += r->gains[i];
   const double n = (double)g.n;
@@ -194,7 +193,7 @@ static hsaw_status solve(const Graph& g, const hsaw_query* q, hsaw_result* r, cu
       HSAW_TRY(stream_extend(g, W.qd, W.st, 2 * half, s));
       phase_end(ph, s, PH_SAMPLE);
       ph = phase_begin(s);
-      HSAW_TRY(cover_build(W.st, q->mode, 0, half, W.cv, s));
+      HSAW_TRY(cover_build(W.st, q->mode, 0, half, W.cv, s, true));
       phase_end(ph, s, PH_COUNT);
       ph = phase_begin(s);
       HSAW_TRY(cover_greedy(W.cv, W.cand, M, k, ids.data(), gains.data(), s));
@@ -203,13 +202,13 @@ static hsaw_status solve(const Graph& g, const hsaw_query* q, hsaw_result* r, cu
       for (int32_t i = 0; i < k; ++i) cov += gains[i];
       uint64_t covp = 0;
       ph = phase_begin(s);
-      HSAW_TRY(cover_count(W.st, q->mode, half, half, ids.data(), k, &covp, s));
+      const int64_t at[2] = {half - 1, 2 * half - 1};
+      uint64_t aids[2] = {0, 0};
+      HSAW_TRY(cover_count(W.st, q->mode, half, half, ids.data(), k, &covp, s, at, aids));
       phase_end(ph, s, PH_COVERAGE);
       double et;
       const int ok = check_bound((double)cov, (double)covp, (double)half, t, q->eps, lam1, &et);
-      uint64_t a_half = 0, a_all = 0;
-      HSAW_TRY(aid_at(W.st, half - 1, &a_half, s));
-      HSAW_TRY(aid_at(W.st, 2 * half - 1, &a_all, s));
+      const uint64_t a_half = aids[0], a_all = aids[1];
       for (int32_t i = 0; i < k; ++i) {
         r->ids[i] = ids[i];
         r->gains[i] = gains[i];
@@ -419,7 +418,7 @@ hsaw_status hsaw_greedy(hsaw_walks w, hsaw_graph g, hsaw_mode mode, int64_t firs
   Cover cv;
   uint8_t* cand = nullptr;
   hsaw_status st = upload_mask(candidate_mask, (size_t)M, false, s, &cand);
-  if (st == HSAW_OK) st = cover_build(w->st, mode, first, count, cv, s);
+  if (st == HSAW_OK) st = cover_build(w->st, mode, first, count, cv, s, true);
   if (st == HSAW_OK) st = cover_greedy(cv, cand, M, k, ids, gains, s);
   cudaStreamSynchronize(s);
   cv.release(s);

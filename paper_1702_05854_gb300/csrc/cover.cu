@@ -176,13 +176,43 @@ static int forced_strategy() {
 static hsaw_status cover_build_sort(const int32_t* el, uint32_t E, int64_t M, int64_t count, Cover& cv,
                                     cudaStream_t s);
 
-hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t count, Cover& cv, cudaStream_t s) {
+hsaw_status walk_offsets(const Stream& st, bool edges, int64_t first, int64_t count, Cover& cv, cudaStream_t s) {
+  count_launch();
+  k_walk_eoff<<<grid_for((size_t)count + 1, 256, 8192), 256, 0, s>>>(st.node_off.p, first, count, edges ? 1 : 0,
+                                                                      cv.walk_eoff.p);
+  HSAW_CK(cudaGetLastError());
+  return HSAW_OK;
+}
+
+// The environment asks for a greedy that takes one pick at a time, or for a histogram strategy.
+static bool one_by_one() {
+  return getenv("HSAW_GREEDY") || getenv("HSAW_GREEDY_HEAVY") || getenv("HSAW_GREEDY_OWNED_MAX");
+}
+
+// Counts by element id cost three passes over the element range and one atomic and one count
+// read per walk element, against about nine passes over the elements' sort and index: they are
+// cheaper while the counts lie in L2 (16 M of them), and beyond it while the range is at most
+// 8 times the elements (10 M edges of 67 M: 1.7 ms by the sort, 1.2 by id, greedy included).
+static bool counts_by_id(int64_t M, int64_t elements) {
+  return M > 0 && M < (1ll << 31) && (M <= (1ll << 24) || M <= 8 * elements);
+}
+
+hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t count, Cover& cv, cudaStream_t s,
+                        bool for_greedy) {
   cv.walks = count;
   cv.entries = 0;
   cv.unique = 0;
+  cv.by_id = false;
   if (count <= 0) return HSAW_OK;
   if (first < 0 || first + count > st.count) return fail(HSAW_E_INVALID, "cover: walk range outside the stream");
   const bool em = (mode == HSAW_EDGE);
+  const int64_t in_stream = em ? st.total_nodes - st.count : st.total_nodes;  // walk elements of the whole stream
+  if (for_greedy && !one_by_one() && !getenv("HSAW_HIST") && peak_cluster() && in_stream < 0xFFFFFFFFll &&
+      count < 0xFFFFFFFFll &&
+      counts_by_id(st.elem_range[em ? 1 : 0], (int64_t)((double)in_stream / (double)st.count * (double)count))) {
+    cv.short_walks = in_stream < 16 * st.count;
+    return count_by_id(st, em, first, count, st.elem_range[em ? 1 : 0], cv, s);
+  }
   int64_t nb[2];
   HSAW_CK(cudaMemcpyAsync(&nb[0], st.node_off.p + first, 8, cudaMemcpyDeviceToHost, s));
   HSAW_CK(cudaMemcpyAsync(&nb[1], st.node_off.p + first + count, 8, cudaMemcpyDeviceToHost, s));
@@ -192,10 +222,7 @@ hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t
   const uint32_t E = (uint32_t)E64;
   cv.entries = E;
   HSAW_TRY(cv.walk_eoff.ensure((size_t)count + 1, s));
-  count_launch();
-  k_walk_eoff<<<grid_for((size_t)count + 1, 256, 8192), 256, 0, s>>>(st.node_off.p, first, count, em ? 1 : 0,
-                                                                      cv.walk_eoff.p);
-  HSAW_CK(cudaGetLastError());
+  HSAW_TRY(walk_offsets(st, em, first, count, cv, s));
   if (E == 0) return HSAW_OK;
   const int32_t* el = em ? st.edges.p + (nb[0] - first) : st.nodes.p + nb[0];
   const int64_t M = st.elem_range[em ? 1 : 0];
@@ -1117,23 +1144,26 @@ __global__ void k_exclude_picks(const uint32_t* __restrict__ out_u, int32_t r, u
 }
 
 hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t k, int64_t* ids_host,
-                         uint32_t* gains_host, cudaStream_t s) {
+                         uint32_t* gains_host, cudaStream_t s, const uint64_t* aid_dev, uint64_t* aid_host) {
   if (k < 1) return fail(HSAW_E_INVALID, "greedy: k < 1");
   const uint32_t U = (uint32_t)cv.unique;
-  DBuf<int64_t> ids;
-  DBuf<uint32_t> outs;  // out_u[k], out_gain[k]
-  HSAW_TRY(ids.ensure(k, s));
-  HSAW_TRY(outs.ensure((size_t)2 * k + 8, s));
-  uint32_t* ctl = outs.p + 2 * (size_t)k;
-  HSAW_CK(cudaMemsetAsync(ctl, 0, 8 * sizeof(uint32_t), s));
+  DBuf<uint32_t> block, outs;
+  HSAW_TRY(block.ensure(PickBlock::copied_words(k) + PickBlock::WORK, s));
+  const PickBlock B = PickBlock::at(block.p, k);
+  std::vector<uint32_t> host(PickBlock::copied_words(k));
+  bool copied = false;
+  if (aid_dev) HSAW_CK(cudaMemcpyAsync(B.last_aid, aid_dev, 8, cudaMemcpyDeviceToDevice, s));
   int32_t rounds = 0;
   hsaw_status st = HSAW_OK;
   bool done = false;
   // by peaks, unless the environment asks for a version that takes one pick at a time
-  const bool one_by_one = getenv("HSAW_GREEDY") || getenv("HSAW_GREEDY_HEAVY") || getenv("HSAW_GREEDY_OWNED_MAX");
-  if (U > 0 && cv.walks > 0 && !one_by_one)
-    st = peak_greedy(cv, cand_dev, k, ids.p, outs.p + k, &rounds, &done, s);
+  if ((U > 0 || cv.by_id) && cv.walks > 0 && !one_by_one())
+    st = peak_greedy(cv, cand_dev, k, B, host.data(), &rounds, &done, &copied, s);
+  uint32_t* ctl = nullptr;
   if (st == HSAW_OK && !done && U > 0 && cv.walks > 0) {
+    HSAW_TRY(outs.ensure((size_t)2 * k + 8, s));  // out_u[k], out_gain[k]
+    ctl = outs.p + 2 * (size_t)k;
+    HSAW_CK(cudaMemsetAsync(ctl, 0, 8 * sizeof(uint32_t), s));
     HSAW_TRY(cv.cnt_work.ensure(U, s));
     HSAW_TRY(cv.covered.ensure((size_t)cv.walks, s));
     HSAW_TRY(cv.inv_ent.ensure((size_t)cv.entries, s));
@@ -1206,7 +1236,7 @@ hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t 
           }
           if (st == HSAW_OK && rounds > 0) {
             count_launch();
-            k_pick_ids<<<grid_for(rounds, 256, 1024), 256, 0, s>>>(outs.p, cv.uid.p, rounds, ids.p);
+            k_pick_ids<<<grid_for(rounds, 256, 1024), 256, 0, s>>>(outs.p, cv.uid.p, rounds, B.ids);
             if (cudaGetLastError() != cudaSuccess) st = fail(HSAW_E_DEVICE, "greedy: id launch failed");
           }
         }
@@ -1226,7 +1256,7 @@ hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t 
       st = cluster_greedy(cv, V, k, 1u, outs.p, outs.p + k, ctl, &rounds, &done, s);
       if (st == HSAW_OK && done && rounds > 0) {
         count_launch();
-        k_pick_ids<<<grid_for(rounds, 256, 1024), 256, 0, s>>>(outs.p, cv.uid.p, rounds, ids.p);
+        k_pick_ids<<<grid_for(rounds, 256, 1024), 256, 0, s>>>(outs.p, cv.uid.p, rounds, B.ids);
         if (cudaGetLastError() != cudaSuccess) st = fail(HSAW_E_DEVICE, "greedy: id launch failed");
       }
     }
@@ -1269,83 +1299,137 @@ hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t 
     rounds = (int32_t)h[3];
     if (st == HSAW_OK && rounds > 0) {
       count_launch();
-      k_pick_ids<<<grid_for(rounds, 256, 1024), 256, 0, s>>>(outs.p, cv.uid.p, rounds, ids.p);
+      k_pick_ids<<<grid_for(rounds, 256, 1024), 256, 0, s>>>(outs.p, cv.uid.p, rounds, B.ids);
       if (cudaGetLastError() != cudaSuccess) st = fail(HSAW_E_DEVICE, "greedy: id launch failed");
     }
   }
+  if (st == HSAW_OK && outs.p && rounds > 0 &&
+      cudaMemcpyAsync(B.gains, outs.p + k, (size_t)rounds * 4, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+    st = fail(HSAW_E_DEVICE, "greedy: gain copy failed");
   if (st == HSAW_OK && rounds < k) {
+    copied = false;
     uint32_t* bits = nullptr;
     const size_t words = (size_t)(M + 31) / 32;
     st = dmalloc((void**)&bits, words * 4, s);
     if (st == HSAW_OK) {
       cudaMemsetAsync(bits, 0, words * 4, s);
-      if (rounds > 0) { count_launch(); k_mark_bits<<<grid_for(rounds, 256, 1024), 256, 0, s>>>(ids.p, rounds, bits); }
+      if (rounds > 0) { count_launch(); k_mark_bits<<<grid_for(rounds, 256, 1024), 256, 0, s>>>(B.ids, rounds, bits); }
       count_launch();
-      k_zero_fill<<<1, 1024, 0, s>>>(M, cand_dev, bits, rounds, k, ids.p, outs.p + k);
+      k_zero_fill<<<1, 1024, 0, s>>>(M, cand_dev, bits, rounds, k, B.ids, B.gains);
       if (cudaGetLastError() != cudaSuccess) st = fail(HSAW_E_DEVICE, "greedy: zero-fill launch failed");
       dfree(bits, s);
     }
   }
+  if (st == HSAW_OK && !copied &&
+      (cudaMemcpyAsync(host.data(), block.p, host.size() * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+       cudaStreamSynchronize(s) != cudaSuccess))
+    st = fail(HSAW_E_DEVICE, "greedy: result copy failed");
   if (st == HSAW_OK) {
-    if (ids_host) cudaMemcpyAsync(ids_host, ids.p, (size_t)k * 8, cudaMemcpyDeviceToHost, s);
-    if (gains_host) cudaMemcpyAsync(gains_host, outs.p + k, (size_t)k * 4, cudaMemcpyDeviceToHost, s);
-    if (cudaStreamSynchronize(s) != cudaSuccess) st = fail(HSAW_E_DEVICE, "greedy: result copy failed");
+    if (ids_host) std::memcpy(ids_host, host.data(), (size_t)k * 8);
+    if (gains_host) std::memcpy(gains_host, host.data() + (B.gains - block.p), (size_t)k * 4);
+    if (aid_host) std::memcpy(aid_host, host.data() + (reinterpret_cast<uint32_t*>(B.last_aid) - block.p), 8);
   }
-  ids.release(s);
+  block.release(s);
   outs.release(s);
   return st;
 }
 
 // ------------------------------------------------------------------ coverage on R'_t
-__global__ void k_cover_count(const int64_t* __restrict__ node_off, const int32_t* __restrict__ nodes,
-                              const int32_t* __restrict__ edges, int edge_mode, int64_t first, int64_t count,
-                              const uint32_t* __restrict__ T_sorted, int32_t k, unsigned long long* __restrict__ cov) {
-  unsigned long long c = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t j = first + i;
-    const int64_t b = node_off[j] - (edge_mode ? j : 0), e = node_off[j + 1] - (edge_mode ? j + 1 : 0);
-    const int32_t* el = edge_mode ? edges : nodes;
-    for (int64_t p = b; p < e; ++p) {
-      const uint32_t x = (uint32_t)el[p];
-      int32_t lo = 0, hi = k;
-      while (lo < hi) {
-        const int32_t mid = (lo + hi) >> 1;
-        if (T_sorted[mid] < x) lo = mid + 1; else hi = mid;
-      }
-      if (lo < k && T_sorted[lo] == x) { ++c; break; }
-    }
+// LANES lanes read a walk, 32-byte sectors at a time; a bit filter of T in shared memory turns
+// almost every other element away, and what passes is searched in T (sorted).  One thread per
+// walk, each element searched, was bound by its uncoalesced reads (150 K walks of 68 edges, k =
+// 1,000: 0.39 ms).
+constexpr uint32_t FILTER_BITS = 1u << 15;
+__device__ __forceinline__ uint32_t filter_bit(uint32_t x) { return (x * 0x9E3779B1u) >> 17; }
+
+template <int LANES>
+__global__ void __launch_bounds__(256) k_cover_count(const int64_t* __restrict__ node_off,
+                                                     const int32_t* __restrict__ el, int edge_mode, int64_t first,
+                                                     int64_t count, const uint32_t* __restrict__ T_sorted, int32_t k,
+                                                     const uint64_t* __restrict__ aid, int64_t at0, int64_t at1,
+                                                     unsigned long long* __restrict__ out) {
+  __shared__ uint32_t filter[FILTER_BITS / 32];
+  for (uint32_t i = threadIdx.x; i < FILTER_BITS / 32; i += blockDim.x) filter[i] = 0;
+  __syncthreads();
+  for (int32_t i = threadIdx.x; i < k; i += blockDim.x) {
+    const uint32_t b = filter_bit(T_sorted[i]);
+    atomicOr(&filter[b >> 5], 1u << (b & 31));
   }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(cov, c);
+  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && aid) {
+    out[1] = aid[at0];
+    out[2] = aid[at1];
+  }
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, group = lane / LANES;
+  const unsigned mine = LANES == 32 ? FULL : ((1u << (LANES & 31)) - 1u) << (group * LANES);
+  constexpr int PER = 32 / LANES;  // walks a warp at a time
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  uint32_t c = 0;
+  for (int64_t i0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * PER; i0 < count; i0 += warps * PER) {
+    const int64_t j = first + i0 + group;
+    int64_t p = 0, e = 0;
+    if (i0 + group < count) {
+      p = node_off[j] - (edge_mode ? j : 0) + lane % LANES;
+      e = node_off[j + 1] - (edge_mode ? j + 1 : 0);
+    }
+    bool hit = false;
+    while (__any_sync(FULL, !hit && p < e)) {
+      bool here = false;
+      if (!hit && p < e) {
+        const uint32_t x = (uint32_t)__ldg(&el[p]);
+        const uint32_t b = filter_bit(x);
+        if ((filter[b >> 5] >> (b & 31)) & 1u) {
+          int32_t lo = 0, hi = k;
+          while (lo < hi) {
+            const int32_t mid = (lo + hi) >> 1;
+            if (T_sorted[mid] < x) lo = mid + 1; else hi = mid;
+          }
+          here = lo < k && T_sorted[lo] == x;
+        }
+      }
+      if (__ballot_sync(FULL, here) & mine) hit = true;
+      p += LANES;
+    }
+    if (hit && lane % LANES == 0) ++c;
+  }
+  c = __reduce_add_sync(FULL, c);
+  if (lane == 0 && c) atomicAdd(out, (unsigned long long)c);
 }
 
 hsaw_status cover_count(const Stream& st, hsaw_mode mode, int64_t first, int64_t count, const int64_t* T, int32_t k,
-                        uint64_t* cov, cudaStream_t s) {
+                        uint64_t* cov, cudaStream_t s, const int64_t* at, uint64_t* aids) {
   *cov = 0;
   if (count <= 0 || k <= 0) return HSAW_OK;
   if (first < 0 || first + count > st.count) return fail(HSAW_E_INVALID, "coverage: walk range outside the stream");
   // T is a host array of k ids: sort it here (k is at most a few thousand) and search it on the device
   std::vector<uint32_t> sorted(T, T + k);
   std::sort(sorted.begin(), sorted.end());
-  uint32_t* buf = nullptr;
-  HSAW_TRY(dmalloc((void**)&buf, (size_t)k * 4 + 64, s));
-  unsigned long long* dcov = (unsigned long long*)(((uintptr_t)(buf + k) + 15) & ~(uintptr_t)7);
+  unsigned long long* out = nullptr;  // coverage, two attempt ids, then T
+  HSAW_TRY(dmalloc((void**)&out, 32 + (size_t)k * 4, s));
+  uint32_t* buf = reinterpret_cast<uint32_t*>(out + 4);
   hsaw_status stt = HSAW_OK;
-  unsigned long long h = 0;
+  unsigned long long h[3] = {0, 0, 0};
   if (cudaMemcpyAsync(buf, sorted.data(), (size_t)k * 4, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      cudaMemsetAsync(dcov, 0, 8, s) != cudaSuccess) {
+      cudaMemsetAsync(out, 0, 32, s) != cudaSuccess) {
     stt = fail(HSAW_E_DEVICE, "coverage: upload failed");
   } else {
+    const bool em = mode == HSAW_EDGE, small = st.total_nodes < 16 * st.count;
+    const auto kernel = small ? k_cover_count<8> : k_cover_count<32>;
     count_launch();
-    k_cover_count<<<grid_for(count, 256, 8192), 256, 0, s>>>(st.node_off.p, st.nodes.p, st.edges.p,
-                                                             mode == HSAW_EDGE ? 1 : 0, first, count, buf, k, dcov);
-    cudaMemcpyAsync(&h, dcov, 8, cudaMemcpyDeviceToHost, s);
+    kernel<<<grid_for((size_t)count * (small ? 8 : 32), 256, 8 * sm_count()), 256, 0, s>>>(
+        st.node_off.p, em ? st.edges.p : st.nodes.p, em ? 1 : 0, first, count, buf, k, aids ? st.aid.p : nullptr,
+        aids ? at[0] : 0, aids ? at[1] : 0, out);
+    cudaMemcpyAsync(h, out, sizeof(h), cudaMemcpyDeviceToHost, s);
     if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess)
       stt = fail(HSAW_E_DEVICE, "coverage kernel failed");
   }
-  *cov = h;
-  dfree(buf, s);
+  *cov = h[0];
+  if (aids) {
+    aids[0] = h[1];
+    aids[1] = h[2];
+  }
+  dfree(out, s);
   return stt;
 }
 

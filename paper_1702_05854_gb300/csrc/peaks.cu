@@ -24,6 +24,7 @@
 
 #include <algorithm>
 #include <cstdlib>
+#include <cstring>
 
 #include "solver.cuh"
 
@@ -33,13 +34,13 @@ namespace cg = cooperative_groups;
 
 namespace {
 
-constexpr uint32_t NOT_CANDIDATE = 0x80000000u;  // bit 31 of a running count
-constexpr uint32_t COUNT_BINS = 4096;            // counts from COUNT_BINS - 1 up share the last bin
-constexpr uint32_t SORT_MAX = 4096;              // picks ordered by one block
+constexpr uint32_t COUNT_BINS = 4096;  // counts from COUNT_BINS - 1 up share the last bin
+constexpr uint32_t SORT_MAX = 4096;    // picks ranked against each other from shared memory
 
 // ctl words of a run; the list's length (high half) and its pairs (low half) grow together in
 // one 64-bit word
-enum { PC_PICKS = 0, PC_FLOOR = 1, PC_GAIN = 2, PC_ROUNDS = 3, PC_STUCK = 4, PC_LIST = 6 /* 64 bits */, PC_WORDS = 16 };
+enum { PC_PICKS = 0, PC_FLOOR = 1, PC_GAIN = 2, PC_ROUNDS = 3, PC_STUCK = 4, PC_TOTAL = 5, PC_LIST = 6 /* 64 bits */,
+       PC_WORDS = 16 };
 
 // A walk of a listed element: {walk, element, index in the list, 1 for the element's first}.
 using Pair = uint4;
@@ -48,9 +49,12 @@ struct PeakParams {
   const Pair* pairs;
   uint32_t* failed;            // per listed element: the last round in which it was no peak
   uint2* seen;                 // and the last round that looked at it, with its count then
-  uint32_t* cnt;               // running counts | NOT_CANDIDATE
-  const uint32_t* walk_eoff;   // per walk: its entries of entry_uidx
-  const uint32_t* entry_uidx;
+  uint32_t* cnt;               // running counts
+  const uint32_t* walk_eoff;   // per walk: its entries, from the range's first
+  const uint32_t* entry;       // element of each entry; the range's first is entry[*from - from_sub] (from NULL: 0)
+  const int64_t* from;
+  int64_t from_sub;
+  uint32_t list_cap, pair_cap;
   uint32_t* stamp;             // per walk: 0, or the round that covered it
   unsigned long long* top[2];  // per walk, by the round's parity: the largest key signed on it
   uint32_t* out_u;
@@ -67,7 +71,8 @@ __device__ __forceinline__ unsigned long long peak_key(uint32_t count, uint32_t 
 
 // The counts of the entries [range.x, range.y) of the walks of the lanes in `mine` go down by
 // one, the whole warp on each.  Four walks' entries are in flight at a time.
-__device__ __forceinline__ void take_down(const PeakParams& P, unsigned mine, uint2 range, int lane) {
+__device__ __forceinline__ void take_down(const PeakParams& P, const uint32_t* __restrict__ entry, unsigned mine,
+                                          uint2 range, int lane) {
   while (mine) {
     uint32_t b[4], e[4], x[4];
 #pragma unroll
@@ -76,12 +81,12 @@ __device__ __forceinline__ void take_down(const PeakParams& P, unsigned mine, ui
       b[j] = __shfl_sync(0xffffffffu, range.x, src) + lane;
       e[j] = mine ? __shfl_sync(0xffffffffu, range.y, src) : 0u;
       mine &= mine - 1;
-      x[j] = b[j] < e[j] ? __ldg(&P.entry_uidx[b[j]]) : 0u;
+      x[j] = b[j] < e[j] ? __ldg(&entry[b[j]]) : 0u;
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       if (b[j] < e[j]) atomicSub(&P.cnt[x[j]], 1u);
-      for (uint32_t p = b[j] + 32; p < e[j]; p += 32) atomicSub(&P.cnt[__ldg(&P.entry_uidx[p])], 1u);
+      for (uint32_t p = b[j] + 32; p < e[j]; p += 32) atomicSub(&P.cnt[__ldg(&entry[p])], 1u);
     }
   }
 }
@@ -101,6 +106,8 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
   const uint32_t gtid = rank * blockDim.x + threadIdx.x, threads = C * blockDim.x;
   const uint32_t gwarp = gtid >> 5, warps = threads >> 5;
   const uint32_t n = __ldcg(&P.ctl[PC_LIST]);
+  if (n > P.pair_cap || __ldcg(&P.ctl[PC_LIST + 1]) > P.list_cap) return;  // the host makes room and comes back
+  const uint32_t* __restrict__ entry = P.entry + (P.from ? *P.from - P.from_sub : 0);
   const uint32_t stripe = (n + 31) / 32;
   const uint32_t floor_gain = __ldcg(&P.ctl[PC_FLOOR]);
   uint32_t picks = 0, g = 0, r = P.round0;
@@ -184,7 +191,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
           }
         }
       }
-      take_down(P, __ballot_sync(FULL, fresh), range, lane);
+      take_down(P, entry, __ballot_sync(FULL, fresh), range, lane);
     }
     cluster.sync();
   }
@@ -196,30 +203,43 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
   }
 }
 
-// Histogram of the running counts of the candidates (counts from 1 up).  first: the counts
-// are taken from cnt and the candidate mask first.  Most R-MAT walk elements occur once or
-// twice: those two bins are counted by ballot, not by atomics on one word.
-__global__ void __launch_bounds__(512) k_peak_hist(bool first, const int32_t* __restrict__ uid,
-                                                    const uint32_t* __restrict__ cnt, const uint8_t* __restrict__ cand,
-                                                    uint32_t U, uint32_t* __restrict__ work,
-                                                    uint32_t* __restrict__ hist) {
+// Counts of the elements of walks [first, first + count), by element id.
+__global__ void __launch_bounds__(256) k_count_elements(const int64_t* __restrict__ node_off, int64_t first,
+                                                        int64_t count, int edge_mode, const int32_t* __restrict__ el,
+                                                        uint32_t* __restrict__ cnt) {
+  const int64_t b = node_off[first] - (edge_mode ? first : 0);
+  const int64_t e = node_off[first + count] - (edge_mode ? first + count : 0);
+  for (int64_t p = b + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < e; p += (int64_t)gridDim.x * blockDim.x)
+    atomicAdd(&cnt[el[p]], 1u);
+}
+
+// Histogram of the counts of the candidates (counts from 1 up).  Most R-MAT walk elements occur
+// once or twice: those two bins are kept in registers, not counted by atomics on one word.
+// uid: element id of each count, NULL if counts are by id.
+__global__ void __launch_bounds__(512) k_peak_hist(const uint32_t* __restrict__ cnt, const int32_t* __restrict__ uid,
+                                                   const uint8_t* __restrict__ cand, uint32_t U,
+                                                   uint32_t* __restrict__ hist) {
   __shared__ uint32_t h[COUNT_BINS];
   for (uint32_t i = threadIdx.x; i < COUNT_BINS; i += blockDim.x) h[i] = 0;
   __syncthreads();
   uint32_t one = 0, two = 0;
-  for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < U; u += gridDim.x * blockDim.x) {
-    uint32_t v;
-    if (first) {
-      v = cnt[u] | ((cand && !cand[uid[u]]) ? NOT_CANDIDATE : 0u);
-      work[u] = v;
-    } else {
-      v = work[u];
-    }
-    if (v & NOT_CANDIDATE) continue;
+  auto add = [&](uint32_t u, uint32_t v) {
+    if (v == 0 || (cand && !cand[uid ? uid[u] : u])) return;
     if (v == 1) ++one;
     else if (v == 2) ++two;
-    else if (v) atomicAdd(&h[min(v, COUNT_BINS - 1)], 1u);
+    else atomicAdd(&h[min(v, COUNT_BINS - 1)], 1u);
+  };
+  const uint4* cnt4 = reinterpret_cast<const uint4*>(cnt);  // a buffer of its own: 16-byte aligned
+  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < U / 4; q += gridDim.x * blockDim.x) {
+    const uint4 v = cnt4[q];
+    if (v.x | v.y | v.z | v.w) {
+      add(4 * q, v.x);
+      add(4 * q + 1, v.y);
+      add(4 * q + 2, v.z);
+      add(4 * q + 3, v.w);
+    }
   }
+  if (blockIdx.x == 0 && threadIdx.x < U % 4) add(U / 4 * 4 + threadIdx.x, cnt[U / 4 * 4 + threadIdx.x]);
   one = __reduce_add_sync(0xffffffffu, one);
   two = __reduce_add_sync(0xffffffffu, two);
   if ((threadIdx.x & 31) == 0) {
@@ -232,14 +252,16 @@ __global__ void __launch_bounds__(512) k_peak_hist(bool first, const int32_t* __
 }
 
 // The phase's floor and the list of candidates that reach it, {element, its first entry of
-// inv_walk, its first pair}, in no order.  Every listed element may be picked and covered, and
+// inv_walk, its first pair, 0}, in no order.  Every listed element may be picked and covered, and
 // is read in each round, so the list holds half as many again as the k picks wanted (1,000
 // R-MAT edge picks came from the first 1,100-1,500) and a few, and more while it is short.
 __global__ void __launch_bounds__(512) k_peak_list(const uint32_t* __restrict__ hist, uint32_t k,
-                                                   const uint32_t* __restrict__ work,
-                                                   const uint32_t* __restrict__ inv_off, uint32_t U,
+                                                   const uint32_t* __restrict__ cnt, const int32_t* __restrict__ uid,
+                                                   const uint8_t* __restrict__ cand,
+                                                   const uint32_t* __restrict__ inv_off, uint32_t U, uint32_t list_cap,
                                                    uint4* __restrict__ list, uint32_t* __restrict__ failed,
-                                                   uint2* __restrict__ seen, uint32_t* __restrict__ ctl) {
+                                                   uint2* __restrict__ seen, uint32_t* __restrict__ index,
+                                                   uint32_t* __restrict__ ctl) {
   constexpr uint32_t PER = COUNT_BINS / 512;
   constexpr unsigned long long FEW_WALKS = 1ull << 15;
   __shared__ uint32_t n_warp[16], s_few, s_want;
@@ -296,37 +318,60 @@ __global__ void __launch_bounds__(512) k_peak_list(const uint32_t* __restrict__ 
   }
   __syncthreads();
   const uint32_t floor_gain = total ? min(s_few, s_want) : 1u;
-  if (blockIdx.x == 0 && threadIdx.x == 0) ctl[PC_FLOOR] = floor_gain;
-  for (uint32_t u0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; u0 < U; u0 += gridDim.x * blockDim.x) {
-    const uint32_t u = u0 + lane;
-    const uint32_t v = u < U ? work[u] : 0u;
-    const bool in = !(v & NOT_CANDIDATE) && v >= floor_gain;
-    const unsigned b = __ballot_sync(0xffffffffu, in);
-    if (!b) continue;
-    const uint32_t q0 = in ? inv_off[u] : 0u, len = in ? inv_off[u + 1] - q0 : 0u;
-    unsigned long long inc = len;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    ctl[PC_FLOOR] = floor_gain;
+    ctl[PC_TOTAL] = total;
+  }
+  // 128 counts a warp at a time: few reach the floor, so most are looked at once, four a lane
+  const uint4* cnt4 = reinterpret_cast<const uint4*>(cnt);
+  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+  for (uint32_t g0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; (uint64_t)g0 * 128 < U; g0 += warps) {
+    const uint32_t at4 = g0 * 32 + lane;  // the lane's four counts
+    uint4 q = make_uint4(0u, 0u, 0u, 0u);
+    if (at4 < U / 4) {
+      q = cnt4[at4];
+    } else if (at4 == U / 4) {
+      const uint32_t left = U % 4;
+      q.x = left > 0 ? cnt[4 * at4] : 0u;
+      q.y = left > 1 ? cnt[4 * at4 + 1] : 0u;
+      q.z = left > 2 ? cnt[4 * at4 + 2] : 0u;
     }
-    unsigned long long at = 0;
-    if (lane == 31) at = atomicAdd(reinterpret_cast<unsigned long long*>(&ctl[PC_LIST]),
-                                   ((unsigned long long)__popc(b) << 32) | inc);
-    at = __shfl_sync(0xffffffffu, at, 31);
-    if (in) {
+    if (!__any_sync(0xffffffffu, max(max(q.x, q.y), max(q.z, q.w)) >= floor_gain)) continue;
+#pragma unroll
+    for (int part = 0; part < 4; ++part) {
+      const uint32_t u = 4 * at4 + part;
+      const uint32_t v = part == 0 ? q.x : part == 1 ? q.y : part == 2 ? q.z : q.w;
+      const bool in = v >= floor_gain && (!cand || cand[uid ? uid[u] : u]);
+      const unsigned b = __ballot_sync(0xffffffffu, in);
+      if (!b) continue;
+      const uint32_t q0 = in && inv_off ? inv_off[u] : 0u, len = !in ? 0u : inv_off ? inv_off[u + 1] - q0 : v;
+      unsigned long long inc = len;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      unsigned long long at = 0;
+      if (lane == 31) at = atomicAdd(reinterpret_cast<unsigned long long*>(&ctl[PC_LIST]),
+                                     ((unsigned long long)__popc(b) << 32) | inc);
+      at = __shfl_sync(0xffffffffu, at, 31);
       const uint32_t i = (uint32_t)(at >> 32) + __popc(b & ((1u << lane) - 1u));
-      list[i] = make_uint4(u, q0, (uint32_t)at + (uint32_t)(inc - len), 0u);
-      failed[i] = 0u;
-      seen[i] = make_uint2(0u, 0u);
+      if (in && i < list_cap) {
+        list[i] = make_uint4(u, q0, (uint32_t)at + (uint32_t)(inc - len), 0u);
+        failed[i] = 0u;
+        seen[i] = make_uint2(0u, 0u);
+        if (index) index[u] = i;
+      }
     }
   }
 }
 
-// The list's (element, walk) pairs, element by element.
+// The list's (element, walk) pairs, element by element, from the inverted index.
 __global__ void __launch_bounds__(256) k_peak_pairs(const uint4* __restrict__ list, const uint32_t* __restrict__ inv_walk,
-                                                    const uint32_t* __restrict__ ctl, Pair* __restrict__ pairs) {
+                                                    const uint32_t* __restrict__ ctl, uint32_t list_cap,
+                                                    uint32_t pair_cap, Pair* __restrict__ pairs) {
   const uint32_t n = ctl[PC_LIST], elements = ctl[PC_LIST + 1];
+  if (n > pair_cap || elements > list_cap) return;
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
     uint32_t lo = 0, hi = elements;  // the last element whose first pair is at or before i
     while (hi - lo > 1) {
@@ -338,36 +383,55 @@ __global__ void __launch_bounds__(256) k_peak_pairs(const uint4* __restrict__ li
   }
 }
 
-// Picks in the greedy's order: gain down, element up (bitonic sort in one block); the first k
-// of them as ids and gains.  More than SORT_MAX picks are left to the radix sort.
-__global__ void __launch_bounds__(1024) k_peak_order(const uint32_t* __restrict__ out_u,
-                                                      const uint32_t* __restrict__ out_gain,
-                                                      const uint32_t* __restrict__ ctl,
-                                                      const int32_t* __restrict__ uid, uint32_t k,
-                                                      int64_t* __restrict__ ids, uint32_t* __restrict__ gains) {
+// The same pairs from the walks themselves, where counts are by element id and no inverted index
+// was made: LANES lanes read a walk that no pick covers yet, and each entry whose count reaches
+// the floor takes the next pair of its element.  Reads every entry once, with its count.
+template <int LANES>
+__global__ void __launch_bounds__(256) k_walk_pairs(const __grid_constant__ PeakParams P, uint32_t walks,
+                                                    const uint8_t* __restrict__ cand,
+                                                    const uint32_t* __restrict__ index, uint4* __restrict__ list,
+                                                    Pair* __restrict__ pairs) {
+  if (P.ctl[PC_LIST] > P.pair_cap || P.ctl[PC_LIST + 1] > P.list_cap) return;
+  const uint32_t floor_gain = P.ctl[PC_FLOOR];
+  const uint32_t* __restrict__ entry = P.entry + (*P.from - P.from_sub);
+  const uint32_t lane = threadIdx.x % LANES;
+  const uint32_t groups = gridDim.x * blockDim.x / LANES;
+  for (uint32_t j = (blockIdx.x * blockDim.x + threadIdx.x) / LANES; j < walks; j += groups) {
+    const uint32_t b = P.walk_eoff[j], e = P.walk_eoff[j + 1];
+    if (P.stamp[j] != 0u) continue;
+    for (uint32_t p = b + lane; p < e; p += LANES) {
+      const uint32_t x = __ldg(&entry[p]);
+      if (__ldg(&P.cnt[x]) < floor_gain || (cand && !cand[x])) continue;
+      const uint32_t i = index[x];
+      const uint32_t at = atomicAdd(&list[i].w, 1u);
+      pairs[list[i].z + at] = make_uint4(j, x, i, at == 0 ? 1u : 0u);
+    }
+  }
+}
+
+// Picks in the greedy's order: gain down, element up; the first k of them as ids and gains.  A
+// thread ranks one pick against all of them from shared memory.  More than SORT_MAX picks are
+// left to the radix sort.
+__global__ void __launch_bounds__(128) k_peak_order(const uint32_t* __restrict__ out_u,
+                                                    const uint32_t* __restrict__ out_gain,
+                                                    const uint32_t* __restrict__ ctl, const int32_t* __restrict__ uid,
+                                                    uint32_t k, int64_t* __restrict__ ids,
+                                                    uint32_t* __restrict__ gains) {
   __shared__ unsigned long long key[SORT_MAX];
   const uint32_t n = ctl[PC_PICKS];
-  if (n > SORT_MAX) return;
-  uint32_t size = 32;
-  while (size < n) size *= 2;
-  for (uint32_t i = threadIdx.x; i < size; i += blockDim.x)
-    key[i] = i < n ? ((unsigned long long)(~out_gain[i]) << 32) | out_u[i] : ~0ull;
-  for (uint32_t span = 2; span <= size; span *= 2)
-    for (uint32_t step = span / 2; step; step /= 2) {
-      __syncthreads();
-      for (uint32_t t = threadIdx.x; t < size / 2; t += blockDim.x) {
-        const uint32_t i = 2 * t - (t & (step - 1)), j = i + step;
-        const unsigned long long a = key[i], b = key[j];
-        if ((a > b) == ((i & span) == 0)) {
-          key[i] = b;
-          key[j] = a;
-        }
-      }
-    }
+  if (n > SORT_MAX || blockIdx.x * blockDim.x >= n) return;
+  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) key[i] = peak_key(out_gain[i], out_u[i]);
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < min(n, k); i += blockDim.x) {
-    ids[i] = uid[(uint32_t)key[i]];
-    gains[i] = ~(uint32_t)(key[i] >> 32);
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const unsigned long long mine = key[i];
+  uint32_t rank = 0;
+#pragma unroll 8
+  for (uint32_t j = 0; j < n; ++j) rank += key[j] > mine ? 1u : 0u;
+  if (rank < k) {
+    const uint32_t u = 0xFFFFFFFFu - (uint32_t)mine;
+    ids[rank] = uid ? uid[u] : (int64_t)u;
+    gains[rank] = (uint32_t)(mine >> 32);
   }
 }
 
@@ -379,13 +443,13 @@ __global__ void k_peak_emit(const uint32_t* __restrict__ u, const uint32_t* __re
                              const int32_t* __restrict__ uid, int64_t* __restrict__ ids,
                              uint32_t* __restrict__ gains) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    ids[i] = uid[u[i]];
+    ids[i] = uid ? uid[u[i]] : (int64_t)u[i];
     gains[i] = ~flipped_gain[i];
   }
 }
 
 // The largest cluster (16 CTAs, else 8) that k_greedy_peaks can run on; 0: none.
-static int peak_cluster() {
+int peak_cluster() {
   static const int cached = [] {
     const int want[2] = {16, 8};
     for (int c : want) {
@@ -413,31 +477,53 @@ static int peak_cluster() {
   return cached;
 }
 
-hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, int64_t* ids, uint32_t* gains, int32_t* rounds,
-                        bool* done, cudaStream_t s) {
-  *done = false;
-  const int largest = peak_cluster();
-  if (!largest) return HSAW_OK;
-  const uint32_t U = (uint32_t)cv.unique, W = (uint32_t)cv.walks;
-  const uint32_t most = std::min(U, W);  // a pick covers a walk of its own
+// Counts by element id and walk offsets of walks [first, first + count), with no read back: the
+// rest of the greedy takes sizes from the device.  M elements.
+hsaw_status count_by_id(const Stream& st, bool edges, int64_t first, int64_t count, int64_t M, Cover& cv,
+                        cudaStream_t s) {
+  HSAW_TRY(cv.walk_eoff.ensure((size_t)count + 1, s));
+  HSAW_TRY(cv.keys.ensure((size_t)M, s));
+  HSAW_CK(cudaMemsetAsync(cv.keys.p, 0, (size_t)M * 4, s));
+  const int32_t* el = edges ? st.edges.p : st.nodes.p;
+  count_launch();
+  k_count_elements<<<8 * sm_count(), 256, 0, s>>>(st.node_off.p, first, count, edges ? 1 : 0, el, cv.keys.p);
+  HSAW_CK(cudaGetLastError());
+  HSAW_TRY(walk_offsets(st, edges, first, count, cv, s));
+  cv.by_id = true;
+  cv.el = el;
+  cv.from = st.node_off.p + first;
+  cv.from_sub = edges ? first : 0;
+  cv.elements = M;
+  return HSAW_OK;
+}
+
+hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlock& out, uint32_t* host,
+                        int32_t* rounds, bool* done, bool* copied, cudaStream_t s) {
+  *done = *copied = false;
+  int64_t* const ids = out.ids;
+  uint32_t *const gains = out.gains, *const ctl = out.ctl, *const hist = out.work;
+  static_assert(PC_WORDS == PickBlock::CTL && COUNT_BINS == PickBlock::WORK, "layout of the picks' block");
   // always the largest cluster: greedy and coverage on streams of 150-1,000 walks take 0.26-0.29
   // ms on 1 to 16 CTAs alike, on 2,500 walks 0.57, 0.41 and 0.35 ms on 1, 4 and 16, and more
   // beyond
-  const uint32_t csize = (uint32_t)largest;
-  HSAW_TRY(cv.cnt_work.ensure(U, s));
-  HSAW_TRY(cv.peak_list.ensure(U, s));
-  HSAW_TRY(cv.inv_ent.ensure((size_t)cv.entries, s));  // pairs
-  HSAW_TRY(cv.g_list.ensure(U, s));
-  HSAW_TRY(cv.g_rng.ensure(U, s));
+  const int csize = peak_cluster();
+  if (!csize) return HSAW_OK;
+  const bool by_id = cv.by_id;
+  const uint32_t U = (uint32_t)(by_id ? cv.elements : cv.unique), W = (uint32_t)cv.walks;
+  const uint32_t most = std::min(U, W);  // a pick covers a walk of its own
+  // room for the list and its pairs; a phase that needs more says so and is run again
+  uint32_t list_cap = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(16ull * k, 1ull << 15), 1ull << 20);
+  uint32_t pair_cap = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(256ull * k, 1ull << 18), 1ull << 22);
+  uint32_t* const cnt = by_id ? cv.keys.p : cv.cnt.p;
+  const int32_t* const uid = by_id ? nullptr : cv.uid.p;
+  if (by_id) HSAW_TRY(cv.vals.ensure(U, s));  // list index of each listed element
   HSAW_TRY(cv.covered.ensure(W, s));
   HSAW_TRY(cv.partial.ensure(2 * (size_t)W, s));
-  HSAW_TRY(cv.g_cnt.ensure((size_t)4 * most + COUNT_BINS + PC_WORDS + 2, s));  // picks (and room to sort), bins, ctl
+  HSAW_TRY(cv.g_cnt.ensure((size_t)4 * most, s));  // picks, and room to sort them
   uint32_t* out_u = cv.g_cnt.p;
   uint32_t* out_gain = out_u + most;
-  uint32_t* hist = out_u + ((4 * (size_t)most + 1) & ~(size_t)1);  // ctl holds a 64-bit word
-  uint32_t* ctl = hist + COUNT_BINS;
   HSAW_CK(cudaMemsetAsync(cv.covered.p, 0, (size_t)W * 4, s));
-  HSAW_CK(cudaMemsetAsync(hist, 0, (COUNT_BINS + PC_WORDS) * 4, s));
+  HSAW_CK(cudaMemsetAsync(ctl, 0, (PC_WORDS + COUNT_BINS) * 4, s));
   const bool log = getenv("HSAW_LOG_LAUNCHES") != nullptr;  // measurement aid
   cudaEvent_t ev[2] = {nullptr, nullptr};
   if (log) {
@@ -445,31 +531,37 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, int64_t* ids,
     cudaEventCreate(&ev[1]);
     cudaEventRecord(ev[0], s);
   }
-  uint32_t h[PC_WORDS] = {0}, phases = 0;
+  uint32_t h[PC_WORDS] = {0}, phases = 0, unique = 0;
+  bool again = false;  // the phase did not fit its list or pairs
   do {
-    if (phases++) {  // every pick down to the floor is made: the candidates below it
-      HSAW_CK(cudaMemsetAsync(hist, 0, COUNT_BINS * 4, s));
-      HSAW_CK(cudaMemsetAsync(ctl + PC_LIST, 0, 2 * 4, s));
+    if (!again) {
+      if (phases++) HSAW_CK(cudaMemsetAsync(hist, 0, COUNT_BINS * 4, s));  // the candidates below the last floor
+      count_launch();
+      k_peak_hist<<<grid_for((U + 3) / 4, 512, 4 * sm_count()), 512, 0, s>>>(cnt, uid, cand, U, hist);
+      HSAW_CK(cudaGetLastError());
+      HSAW_CK(cudaMemsetAsync(cv.partial.p, 0, (size_t)W * 16, s));
     }
-    HSAW_CK(cudaMemsetAsync(cv.partial.p, 0, (size_t)W * 16, s));
+    if (again || phases > 1) HSAW_CK(cudaMemsetAsync(ctl + PC_LIST, 0, 2 * 4, s));
+    HSAW_TRY(cv.peak_list.ensure(list_cap, s));
+    HSAW_TRY(cv.g_list.ensure(list_cap, s));
+    HSAW_TRY(cv.g_rng.ensure(list_cap, s));
+    HSAW_TRY(cv.inv_ent.ensure(pair_cap, s));
     count_launch();
-    k_peak_hist<<<grid_for(U, 512, 4 * sm_count()), 512, 0, s>>>(phases == 1, cv.uid.p, cv.cnt.p, cand, U, cv.cnt_work.p,
-                                                                hist);
-    HSAW_CK(cudaGetLastError());
-    count_launch();
-    k_peak_list<<<grid_for(U, 512, 4 * sm_count()), 512, 0, s>>>(hist, (uint32_t)k, cv.cnt_work.p, cv.inv_off.p, U,
-                                                                cv.peak_list.p, cv.g_list.p, cv.g_rng.p, ctl);
-    HSAW_CK(cudaGetLastError());
-    count_launch();
-    k_peak_pairs<<<4 * sm_count(), 256, 0, s>>>(cv.peak_list.p, cv.inv_walk.p, ctl, cv.inv_ent.p);
+    k_peak_list<<<grid_for((U + 3) / 4, 512, 4 * sm_count()), 512, 0, s>>>(
+        hist, (uint32_t)k, cnt, uid, cand, by_id ? nullptr : cv.inv_off.p, U, list_cap, cv.peak_list.p, cv.g_list.p,
+        cv.g_rng.p, by_id ? cv.vals.p : nullptr, ctl);
     HSAW_CK(cudaGetLastError());
     PeakParams P;
     P.pairs = cv.inv_ent.p;
     P.failed = cv.g_list.p;
     P.seen = cv.g_rng.p;
-    P.cnt = cv.cnt_work.p;
+    P.cnt = cnt;
     P.walk_eoff = cv.walk_eoff.p;
-    P.entry_uidx = cv.entry_uidx.p;
+    P.entry = by_id ? reinterpret_cast<const uint32_t*>(cv.el) : cv.entry_uidx.p;
+    P.from = by_id ? cv.from : nullptr;
+    P.from_sub = cv.from_sub;
+    P.list_cap = list_cap;
+    P.pair_cap = pair_cap;
     P.stamp = cv.covered.p;
     P.top[0] = cv.partial.p;
     P.top[1] = cv.partial.p + W;
@@ -479,6 +571,16 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, int64_t* ids,
     P.k = (uint32_t)k;
     P.round0 = h[PC_ROUNDS];
     P.max_rounds = most;  // a round makes a pick
+    count_launch();
+    if (!by_id)
+      k_peak_pairs<<<4 * sm_count(), 256, 0, s>>>(cv.peak_list.p, cv.inv_walk.p, ctl, list_cap, pair_cap, cv.inv_ent.p);
+    else if (cv.short_walks)
+      k_walk_pairs<8><<<grid_for((size_t)W * 8, 256, 8 * sm_count()), 256, 0, s>>>(P, W, cand, cv.vals.p,
+                                                                                  cv.peak_list.p, cv.inv_ent.p);
+    else
+      k_walk_pairs<32><<<grid_for((size_t)W * 32, 256, 8 * sm_count()), 256, 0, s>>>(P, W, cand, cv.vals.p,
+                                                                                    cv.peak_list.p, cv.inv_ent.p);
+    HSAW_CK(cudaGetLastError());
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -493,12 +595,20 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, int64_t* ids,
     count_launch();
     HSAW_CK(cudaLaunchKernelEx(&cfg, k_greedy_peaks, P));
     count_launch();
-    k_peak_order<<<1, 1024, 0, s>>>(out_u, out_gain, ctl, cv.uid.p, (uint32_t)k, ids, gains);
+    k_peak_order<<<SORT_MAX / 128, 128, 0, s>>>(out_u, out_gain, ctl, uid, (uint32_t)k, ids, gains);
     HSAW_CK(cudaGetLastError());
-    HSAW_CK(cudaMemcpyAsync(h, ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
+    // picks and control words come back in one copy
+    HSAW_CK(cudaMemcpyAsync(host, out.ids, PickBlock::copied_words(k) * 4, cudaMemcpyDeviceToHost, s));
     HSAW_CK(cudaStreamSynchronize(s));
+    std::memcpy(h, host + (out.ctl - reinterpret_cast<uint32_t*>(out.ids)), sizeof(h));
     if (h[PC_STUCK]) return fail(HSAW_E_DEVICE, "greedy: a round made no pick");
-  } while (h[PC_PICKS] < (uint32_t)k && h[PC_FLOOR] > 1);
+    if (phases == 1) unique = h[PC_TOTAL];
+    again = h[PC_LIST] > pair_cap || h[PC_LIST + 1] > list_cap;
+    if (again) {
+      pair_cap = std::max(pair_cap, h[PC_LIST]);
+      list_cap = std::max(list_cap, h[PC_LIST + 1]);
+    }
+  } while (again || (h[PC_PICKS] < (uint32_t)k && h[PC_FLOOR] > 1));
   const uint32_t made = h[PC_PICKS], kept = std::min<uint32_t>(made, (uint32_t)k);
   if (made > SORT_MAX) {  // by element, then (stable) by gain downwards
     uint32_t *k1 = out_u, *v1 = out_gain, *k2 = out_u + 2 * (size_t)most, *v2 = k2 + most;
@@ -516,19 +626,22 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, int64_t* ids,
   if (log) {
     // a greedy on one cluster with counts in global memory, like k_greedy_cluster, whose record
     // this is
+    uint32_t entries = 0;
+    cudaMemcpyAsync(&entries, cv.walk_eoff.p + W, 4, cudaMemcpyDeviceToHost, s);
     cudaEventRecord(ev[1], s);
     cudaEventSynchronize(ev[1]);
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ev[0], ev[1]);
     fprintf(stderr,
-            "hsaw: k_greedy_cluster walks=%lld entries=%lld unique=%u cluster=%u gshift=0 k=%d picks=%u spread=0 "
-            "rounds=%u phases=%u pairs=%u made=%u ms=%.3f\n",
-            (long long)cv.walks, (long long)cv.entries, U, csize, k, kept, h[PC_ROUNDS], phases, h[PC_LIST], made, ms);
+            "hsaw: k_greedy_cluster walks=%lld entries=%u unique=%u cluster=%d gshift=0 k=%d picks=%u spread=0 "
+            "rounds=%u phases=%u pairs=%u made=%u by_id=%d ms=%.3f\n",
+            (long long)cv.walks, entries, unique, csize, k, kept, h[PC_ROUNDS], phases, h[PC_LIST], made, by_id ? 1 : 0, ms);
     cudaEventDestroy(ev[0]);
     cudaEventDestroy(ev[1]);
   }
   *rounds = (int32_t)kept;
   *done = true;
+  *copied = made <= SORT_MAX;
   return HSAW_OK;
 }
 

@@ -76,20 +76,52 @@ struct Cover {
   DBuf<uint32_t> g_idx, g_list, g_cnt, g_entry;  // greedy on the heavy elements: index map, list, counts, entries
   DBuf<uint2> g_rng;             // greedy: each element's entries of inv_ent
   DBuf<unsigned long long> partial;
+  // counts by element id (for_greedy): keys holds the counts of `elements` ids, the entries of
+  // the walks are el[*from - from_sub ...], and entries, unique, uid and the inverted index are
+  // not made
+  bool by_id = false;
+  bool short_walks = false;  // mean walk below 16 elements, about
+  const int32_t* el = nullptr;
+  const int64_t* from = nullptr;
+  int64_t from_sub = 0, elements = 0;
   void release(cudaStream_t s);
 };
 
-hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t count, Cover& cv, cudaStream_t s);
-// Greedy (Alg. 4 / 7) on a built Cover; cand (device, M bytes) may be NULL.
+// for_greedy: only cover_greedy follows, so counts by element id do where they are the cheaper.
+hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t count, Cover& cv, cudaStream_t s,
+                        bool for_greedy = false);
+// Entry offsets of walks [first, first + count) from the range's first, in cv.walk_eoff.
+hsaw_status walk_offsets(const Stream& st, bool edges, int64_t first, int64_t count, Cover& cv, cudaStream_t s);
+hsaw_status count_by_id(const Stream& st, bool edges, int64_t first, int64_t count, int64_t M, Cover& cv,
+                        cudaStream_t s);
+int peak_cluster();  // CTAs of the cluster that the greedy by peaks runs on; 0: it cannot
+// Greedy (Alg. 4 / 7) on a built Cover; cand (device, M bytes) may be NULL.  *aid_host (may be
+// NULL) receives *aid_dev with the picks.
 hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t k, int64_t* ids_host,
-                         uint32_t* gains_host, cudaStream_t s);
+                         uint32_t* gains_host, cudaStream_t s, const uint64_t* aid_dev = nullptr,
+                         uint64_t* aid_host = nullptr);
 // The same picks by peaks, many at a time (peaks.cu), for cover_greedy: the first *rounds <= k
 // ids and gains (device, k of each); *done = false when no cluster can run it.
-hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, int64_t* ids, uint32_t* gains, int32_t* rounds,
-                         bool* done, cudaStream_t s);
-// #walks in [first, first + count) that contain an element of T (T host, k ids).
+struct PickBlock {  // one device buffer, so that one copy brings a greedy's results back
+  static constexpr int CTL = 16, WORK = 4096;
+  int64_t* ids;       // k
+  uint32_t* gains;    // k
+  uint64_t* last_aid; // an attempt id for the caller
+  uint32_t* ctl;      // CTL words
+  uint32_t* work;     // WORK words, not copied
+  static size_t copied_words(int32_t k) { return ((size_t)3 * k + 1) / 2 * 2 + 2 + CTL; }
+  static PickBlock at(uint32_t* p, int32_t k) {
+    uint32_t* e = p + ((size_t)3 * k + 1) / 2 * 2;
+    return {reinterpret_cast<int64_t*>(p), p + 2 * (size_t)k, reinterpret_cast<uint64_t*>(e), e + 2, e + 2 + CTL};
+  }
+};
+// host: room for PickBlock::copied_words(k) words; *copied: the picks are there already.
+hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlock& out, uint32_t* host,
+                        int32_t* rounds, bool* done, bool* copied, cudaStream_t s);
+// #walks in [first, first + count) that contain an element of T (T host, k ids).  aids (may be
+// NULL) receives the attempt ids of walks at[0] and at[1] with it.
 hsaw_status cover_count(const Stream& st, hsaw_mode mode, int64_t first, int64_t count, const int64_t* T, int32_t k,
-                        uint64_t* cov, cudaStream_t s);
+                        uint64_t* cov, cudaStream_t s, const int64_t* at = nullptr, uint64_t* aids = nullptr);
 
 // Walk pool (pool.cu).
 void pool_release(WalkPool& p);
