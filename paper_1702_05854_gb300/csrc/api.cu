@@ -162,6 +162,7 @@ static hsaw_status solve(const Graph& g, const hsaw_query* q, hsaw_result* r, cu
   HSAW_TRY(query_upload(g, q, W.qd, s));
   HSAW_TRY(upload_mask(q->candidate_mask, (size_t)M, false, s, &W.cand));
   HSAW_TRY(stream_init(W.st, 0, q->max_attempts, s));
+  W.st.least_window = 65536.0;
   r->n_selected = k;
   r->rounds_t = 0;
   r->cov_Rprime = r->hits_Rprime = r->attempts_Rprime = 0;
@@ -312,6 +313,8 @@ hsaw_status hsaw_estimate_spread(hsaw_graph g, const hsaw_query* q, const int64_
     dfree(d_ids, s);
   }
   HSAW_TRY(stream_init(W.st, 0, q->max_attempts, s));
+  W.st.least_window = 65536.0;
+  W.st.ids_only = true;
   HSAW_TRY(stream_extend(G, W.qd, W.st, q->n_hsaw, s));
   uint64_t last = 0;
   HSAW_TRY(aid_at(W.st, q->n_hsaw - 1, &last, s));

@@ -409,26 +409,30 @@ __global__ void __launch_bounds__(256) k_walk_pairs(const __grid_constant__ Peak
   }
 }
 
-// Picks in the greedy's order: gain down, element up; the first k of them as ids and gains.  A
-// thread ranks one pick against all of them from shared memory.  More than SORT_MAX picks are
+// Picks in the greedy's order: gain down, element up; the first k of them as ids and gains.
+// Eight lanes rank a pick against all of them from shared memory.  More than SORT_MAX picks are
 // left to the radix sort.
-__global__ void __launch_bounds__(128) k_peak_order(const uint32_t* __restrict__ out_u,
-                                                    const uint32_t* __restrict__ out_gain,
-                                                    const uint32_t* __restrict__ ctl, const int32_t* __restrict__ uid,
-                                                    uint32_t k, int64_t* __restrict__ ids,
-                                                    uint32_t* __restrict__ gains) {
+constexpr int RANK_LANES = 8, RANK_THREADS = 128;
+__global__ void __launch_bounds__(RANK_THREADS) k_peak_order(const uint32_t* __restrict__ out_u,
+                                                             const uint32_t* __restrict__ out_gain,
+                                                             const uint32_t* __restrict__ ctl,
+                                                             const int32_t* __restrict__ uid, uint32_t k,
+                                                             int64_t* __restrict__ ids,
+                                                             uint32_t* __restrict__ gains) {
+  constexpr uint32_t PICKS = RANK_THREADS / RANK_LANES;
   __shared__ unsigned long long key[SORT_MAX];
   const uint32_t n = ctl[PC_PICKS];
-  if (n > SORT_MAX || blockIdx.x * blockDim.x >= n) return;
+  if (n > SORT_MAX || blockIdx.x * PICKS >= n) return;
   for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) key[i] = peak_key(out_gain[i], out_u[i]);
   __syncthreads();
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const unsigned long long mine = key[i];
+  const uint32_t i = blockIdx.x * PICKS + threadIdx.x / RANK_LANES;
+  const unsigned long long mine = i < n ? key[i] : 0ull;
   uint32_t rank = 0;
-#pragma unroll 8
-  for (uint32_t j = 0; j < n; ++j) rank += key[j] > mine ? 1u : 0u;
-  if (rank < k) {
+#pragma unroll 4
+  for (uint32_t j = threadIdx.x % RANK_LANES; j < n; j += RANK_LANES) rank += key[j] > mine ? 1u : 0u;
+#pragma unroll
+  for (int o = RANK_LANES / 2; o; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+  if (i < n && threadIdx.x % RANK_LANES == 0 && rank < k) {
     const uint32_t u = 0xFFFFFFFFu - (uint32_t)mine;
     ids[rank] = uid ? uid[u] : (int64_t)u;
     gains[rank] = (uint32_t)(mine >> 32);
@@ -595,7 +599,7 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     count_launch();
     HSAW_CK(cudaLaunchKernelEx(&cfg, k_greedy_peaks, P));
     count_launch();
-    k_peak_order<<<SORT_MAX / 128, 128, 0, s>>>(out_u, out_gain, ctl, uid, (uint32_t)k, ids, gains);
+    k_peak_order<<<SORT_MAX * RANK_LANES / RANK_THREADS, RANK_THREADS, 0, s>>>(out_u, out_gain, ctl, uid, (uint32_t)k, ids, gains);
     HSAW_CK(cudaGetLastError());
     // picks and control words come back in one copy
     HSAW_CK(cudaMemcpyAsync(host, out.ids, PickBlock::copied_words(k) * 4, cudaMemcpyDeviceToHost, s));

@@ -180,7 +180,9 @@ __global__ void k_bits_emit(const uint32_t* __restrict__ bits, const uint32_t* _
 template <bool HAS_P, Layout L>
 __global__ void k_hit_len(const WalkTables T, uint32_t n, uint32_t k0, uint32_t k1, const uint32_t* __restrict__ s_bits,
                           const uint32_t* __restrict__ p32, const uint64_t* __restrict__ aid, uint32_t count,
-                          uint32_t step_cap, uint32_t* __restrict__ len, uint32_t* __restrict__ status) {
+                          uint32_t step_cap, uint32_t* __restrict__ len, uint32_t* __restrict__ status,
+                          unsigned long long* __restrict__ nodes) {
+  uint32_t sum = 0;
   for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < count; h += gridDim.x * blockDim.x) {
     const uint64_t a = aid[h];
     uint32_t v = start_node(a, n, k0, k1), l = 1;
@@ -196,7 +198,12 @@ __global__ void k_hit_len(const WalkTables T, uint32_t n, uint32_t k0, uint32_t 
       ++l;
     }
     len[h] = l;
+    sum += l;
   }
+  unsigned long long warp_sum = sum;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) warp_sum += __shfl_down_sync(0xffffffffu, warp_sum, o);
+  if ((threadIdx.x & 31) == 0 && warp_sum) atomicAdd(nodes, warp_sum);
 }
 
 void pool_release(WalkPool& p) {
@@ -290,9 +297,10 @@ hsaw_status pool_build(Graph& g, uint64_t seed, uint64_t attempts, cudaStream_t 
 }
 
 hsaw_status pool_hits(const Graph& g, const QueryDev& qd, Stream& st, uint64_t a0, uint64_t a1, uint32_t* new_hits,
-                      cudaStream_t s) {
+                      int64_t* new_nodes, cudaStream_t s) {
   const WalkPool& pl = g.pool;
   *new_hits = 0;
+  *new_nodes = 0;
   if (a1 <= a0) return HSAW_OK;
   const uint32_t k0 = (uint32_t)qd.seed, k1 = (uint32_t)(qd.seed >> 32);
   const uint64_t b0 = a0 >> pl.shift, b1 = (a1 - 1) >> pl.shift;
@@ -338,13 +346,15 @@ hsaw_status pool_hits(const Graph& g, const QueryDev& qd, Stream& st, uint64_t a
       {k_hit_len<true, REC16>, k_hit_len<true, REC32>, k_hit_len<true, TAIL4>, k_hit_len<true, EDGE8>}};
   const auto hit_len = by_layout[qd.p32 ? 1 : 0][g.layout];
   hit_len<<<hgrid, 128, 0, s>>>(g.tables(), (uint32_t)g.n, k0, k1, qd.s_bits, qd.p32, st.aid.p + st.count, h,
-                                pool_step_cap(g), st.len.p + st.count, st.ctrs.p + 3);
+                                pool_step_cap(g), st.len.p + st.count, st.ctrs.p + 3,
+                                reinterpret_cast<unsigned long long*>(st.ctrs.p + 4));
   HSAW_CK(cudaGetLastError());
-  uint32_t bad = 0;
-  HSAW_CK(cudaMemcpyAsync(&bad, st.ctrs.p + 3, 4, cudaMemcpyDeviceToHost, s));
+  uint32_t back[3] = {0, 0, 0};  // status, then the nodes (64 bits)
+  HSAW_CK(cudaMemcpyAsync(back, st.ctrs.p + 3, sizeof(back), cudaMemcpyDeviceToHost, s));
   HSAW_CK(cudaStreamSynchronize(s));
-  if (bad) return fail(HSAW_E_DEVICE, "walk pool: a listed attempt did not reach a source");
+  if (back[0]) return fail(HSAW_E_DEVICE, "walk pool: a listed attempt did not reach a source");
   *new_hits = h;
+  *new_nodes = (int64_t)(((uint64_t)back[2] << 32) | back[1]);
   return HSAW_OK;
 }
 

@@ -119,7 +119,7 @@ static hsaw_status run_batch(const hsaw_graph* gs, const hsaw_query* qs, hsaw_re
       if (i >= count) break;
       if (is_joint[i]) {
         const int32_t j = pos_of[i];
-        if (st[i] == HSAW_OK) st[i] = stream_take_hits(gs[i]->g, qds[j], sts[j], (uint32_t)staged[j], s);
+        if (st[i] == HSAW_OK) st[i] = stream_take_hits(gs[i]->g, qds[j], sts[j], (uint32_t)staged[j], -1, s);
         if (st[i] == HSAW_OK) st[i] = solve_fixed_from_stream(gs[i]->g, &qs[i], sts[j], &rs[i], s);
       } else if (!gs[i]) {
         st[i] = fail(HSAW_E_INVALID, "batch: NULL graph");

@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <cstring>
 #include <mutex>
 #include <unordered_map>
 #include <vector>
@@ -24,6 +25,11 @@
 namespace hsaw {
 
 enum : uint32_t { ST_OVERFLOW = 1u, ST_STEP_CAP = 2u };
+
+// Control words of a sampler launch, before its chunks' hit counts (cleared together, read back
+// in one copy): work counter, status bits, hits, live-edge draws and the hits' nodes (64 bits
+// each).
+enum SampleCtl { SC_NEXT = 0, SC_STATUS = 1, SC_HITS = 2, SC_STEPS = 4, SC_NODES = 6, SC_WORDS = 8 };
 
 struct SampleParams {
   WalkTables T;
@@ -39,10 +45,9 @@ struct SampleParams {
   uint32_t n_chunks;
   uint32_t cap;          // hit records per chunk
   uint32_t step_cap;
-  uint32_t* chunk_ctr;   // [0] work counter, [1] status bits
+  uint32_t* ctl;         // SampleCtl words
   uint32_t* chunk_hits;  // n_chunks
   uint2* recs;           // n_chunks * cap
-  unsigned long long* steps;
   PhiloxKeys keys;       // round keys of (k0, k1)
 };
 
@@ -72,7 +77,7 @@ __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_co
   const unsigned lt = (1u << lane) - 1u;
   uint32_t cur = 0, cur_end = 0;  // warp's attempt cursor within the launch
   uint32_t ahead = 0;             // lane 0: the next chunk
-  if (lane == 0) ahead = atomicAdd(P.chunk_ctr, 1u);
+  if (lane == 0) ahead = atomicAdd(P.ctl + SC_NEXT, 1u);
   uint32_t ready = 0;  // starts in the buffer
   bool more = true;
   bool active = false;
@@ -80,7 +85,7 @@ __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_co
   uint4 rec = make_uint4(0, 0, 0, 0);  // node record of v: first in-edge, in-degree, equal weight, in-sum
   Ckpt ck;
   ck.reset(0);
-  uint32_t my_steps = 0;
+  uint32_t my_steps = 0, my_nodes = 0;
   for (;;) {
     const unsigned need = __ballot_sync(FULL, !active);
     if (need) {
@@ -93,7 +98,7 @@ __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_co
           if (!more) break;
           cur = c << P.chunk_shift;
           cur_end = min(cur + (1u << P.chunk_shift), P.n_attempts);
-          if (lane == 0) ahead = atomicAdd(P.chunk_ctr, 1u);
+          if (lane == 0) ahead = atomicAdd(P.ctl + SC_NEXT, 1u);
         }
         const uint32_t i = cur + lane;
         bool walk = false;
@@ -160,7 +165,7 @@ __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_co
           v = u;
           rec = next;
           if (++len > P.step_cap) {
-            atomicOr(P.chunk_ctr + 1, ST_STEP_CAP);
+            atomicOr(P.ctl + SC_STATUS, ST_STEP_CAP);
             outcome = 0;
           }
         }
@@ -168,33 +173,39 @@ __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_co
       if (outcome >= 0) {
         active = false;
         if (outcome == 1) {
+          my_nodes += len;
           const uint32_t ck_i = off >> P.chunk_shift;
           const uint32_t slot = atomicAdd(&P.chunk_hits[ck_i], 1u);
           if (slot < P.cap) P.recs[(size_t)ck_i * P.cap + slot] = make_uint2(off, len);
-          else atomicOr(P.chunk_ctr + 1, ST_OVERFLOW);
+          else atomicOr(P.ctl + SC_STATUS, ST_OVERFLOW);
         }
       }
     }
   }
-  // steps of this warp
-  unsigned long long warp_steps = my_steps;
+  // draws and hit nodes of this warp
+  unsigned long long warp_steps = my_steps, warp_nodes = my_nodes;
 #pragma unroll
-  for (int o = 16; o; o >>= 1) warp_steps += __shfl_down_sync(FULL, warp_steps, o);
-  if (lane == 0 && warp_steps) atomicAdd(P.steps, warp_steps);
+  for (int o = 16; o; o >>= 1) {
+    warp_steps += __shfl_down_sync(FULL, warp_steps, o);
+    warp_nodes += __shfl_down_sync(FULL, warp_nodes, o);
+  }
+  if (lane == 0 && warp_steps) atomicAdd(reinterpret_cast<unsigned long long*>(P.ctl + SC_STEPS), warp_steps);
+  if (lane == 0 && warp_nodes) atomicAdd(reinterpret_cast<unsigned long long*>(P.ctl + SC_NODES), warp_nodes);
 }
 
-// Order each chunk's hits by attempt id and write them at the chunk's scanned offset.
-// One warp per chunk; rank = number of the chunk's records with a smaller offset.
-__global__ void k_compact(const uint32_t* __restrict__ chunk_hits, const uint32_t* __restrict__ chunk_off,
+// Order each chunk's hits by attempt id and write them at the chunk's scanned offset (*total:
+// the hits of all chunks).  One warp per chunk; rank = number of the chunk's records with a
+// smaller offset.
+__global__ void k_compact(const uint32_t* __restrict__ chunk_off, const uint32_t* __restrict__ total,
                           const uint2* __restrict__ recs, uint32_t cap, uint32_t n_chunks, uint64_t a0,
                           uint64_t* __restrict__ out_aid, uint32_t* __restrict__ out_len) {
   const int lane = threadIdx.x & 31;
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
   for (uint32_t ck = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; ck < n_chunks; ck += warps) {
-    const uint32_t c = min(chunk_hits[ck], cap);
+    const uint32_t base = chunk_off[ck];
+    const uint32_t c = (ck + 1 < n_chunks ? chunk_off[ck + 1] : *total) - base;
     if (c == 0) continue;
     const uint2* r = recs + (size_t)ck * cap;
-    const uint32_t base = chunk_off[ck];
     for (uint32_t i = lane; i < c; i += 32) {
       const uint2 me = r[i];
       uint32_t rank = 0;
@@ -205,19 +216,73 @@ __global__ void k_compact(const uint32_t* __restrict__ chunk_hits, const uint32_
   }
 }
 
-__global__ void k_clamp(const uint32_t* __restrict__ in, uint32_t* __restrict__ out, uint32_t n, uint32_t cap) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) out[i] = min(in[i], cap);
+// node_off[i] = base + len[0] + ... + len[i - 1], i <= n: sums of 4,096-walk tiles, their scan,
+// then the tiles' own scans.
+constexpr int OFF_THREADS = 512, OFF_TILE = 4096;
+__device__ __forceinline__ uint64_t block_scan_u64(uint64_t v, uint64_t* sums, uint64_t* total) {  // exclusive
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  uint64_t inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) sums[w] = inc;
+  __syncthreads();
+  uint64_t before = 0, all = 0;
+  for (int i = 0; i < OFF_THREADS / 32; ++i) {
+    const uint64_t x = sums[i];
+    if (i < w) before += x;
+    all += x;
+  }
+  *total = all;
+  return before + inc - v;
 }
 
-__global__ void k_len_to_u64(const uint32_t* __restrict__ len, int64_t n, uint64_t* __restrict__ out) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = len[i];
+__global__ void __launch_bounds__(OFF_THREADS) k_len_tiles(const uint32_t* __restrict__ len, int64_t n,
+                                                           uint64_t* __restrict__ tile_sum) {
+  __shared__ uint64_t sums[OFF_THREADS / 32];
+  uint64_t v = 0, total;
+  const int64_t base = (int64_t)blockIdx.x * OFF_TILE;
+  for (int i = threadIdx.x; i < OFF_TILE; i += OFF_THREADS)
+    if (base + i < n) v += len[base + i];
+  block_scan_u64(v, sums, &total);
+  if (threadIdx.x == 0) tile_sum[blockIdx.x] = total;
 }
 
-__global__ void k_offsets(const uint64_t* __restrict__ excl, int64_t n, int64_t base, int64_t* __restrict__ node_off,
-                          const uint64_t* __restrict__ total) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= n; i += (int64_t)gridDim.x * blockDim.x)
-    node_off[i] = base + (int64_t)(i < n ? excl[i] : *total);
+__global__ void __launch_bounds__(OFF_THREADS) k_len_offsets(const uint32_t* __restrict__ len, int64_t n,
+                                                             const uint64_t* __restrict__ tile_off, int64_t base,
+                                                             int64_t* __restrict__ node_off) {
+  constexpr int PER = OFF_TILE / OFF_THREADS;
+  __shared__ uint64_t sums[OFF_THREADS / 32];
+  const int64_t i0 = (int64_t)blockIdx.x * OFF_TILE + threadIdx.x * PER;
+  uint32_t l[PER];
+  uint64_t v = 0, total;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) v += l[i] = i0 + i < n ? len[i0 + i] : 0u;
+  uint64_t run = block_scan_u64(v, sums, &total) + base + (tile_off ? tile_off[blockIdx.x] : 0ull);
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    if (i0 + i <= n) node_off[i0 + i] = (int64_t)run;
+    run += l[i];
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == OFF_THREADS - 1 && i0 + PER == n) node_off[n] = (int64_t)run;
+}
+
+static hsaw_status len_offsets(const uint32_t* len, int64_t n, int64_t base, int64_t* node_off, DBuf<uint64_t>& tmp,
+                               cudaStream_t s) {
+  const int64_t tiles = (n + OFF_TILE - 1) / OFF_TILE;
+  if (tiles > 1) {
+    HSAW_TRY(tmp.ensure((size_t)tiles, s));
+    count_launch();
+    k_len_tiles<<<(unsigned)tiles, OFF_THREADS, 0, s>>>(len, n, tmp.p);
+    HSAW_CK(cudaGetLastError());
+    HSAW_TRY(exclusive_scan_u64(tmp.p, (size_t)tiles, nullptr, s));
+  }
+  count_launch();
+  k_len_offsets<<<(unsigned)tiles, OFF_THREADS, 0, s>>>(len, n, tiles > 1 ? tmp.p : nullptr, base, node_off);
+  HSAW_CK(cudaGetLastError());
+  return HSAW_OK;
 }
 
 // Re-derive hit walks from their attempt ids (path encoding) into the flat buffers.
@@ -267,7 +332,7 @@ __global__ void k_classify(SampleParams P, uint64_t first, int64_t count, int8_t
       if (ck.seen(u)) { out = 2; break; }
       ck.keep(u, len);
       v = u;
-      if (++len > P.step_cap) { atomicOr(P.chunk_ctr + 1, ST_STEP_CAP); out = 0; break; }
+      if (++len > P.step_cap) { atomicOr(P.ctl + SC_STATUS, ST_STEP_CAP); out = 0; break; }
     }
     outcome[i] = (int8_t)out;
     length[i] = (int32_t)len;
@@ -320,6 +385,9 @@ hsaw_status query_upload(const Graph& g, const hsaw_query* q, QueryDev& qd, cuda
   dfree(d_p, s);
   if (le != cudaSuccess) return fail(HSAW_E_DEVICE, "query: suspect bits launch failed");
   qd.seed = q->seed;
+  double real = 0.0;  // expected number of real sources
+  for (int32_t i = 0; i < q->n_sources; ++i) real += q->p_fixed ? (double)q->p_fixed[i] / 4294967296.0 : 1.0;
+  qd.start_rate = real / (double)g.n;
   return HSAW_OK;
 }
 
@@ -482,35 +550,41 @@ static void launch_sample(const Graph& g, const SampleParams& P, unsigned grid, 
   }
 }
 
+// Attempts per chunk: 256, or fewer (32 at least) where that leaves resident warps without one.
+// A lane then walks one attempt or few, so a short launch ends with its longest walk instead of
+// the longest sum of eight: 4,096 attempts on a 16 K-node graph, 105 -> 60 us.
+static uint32_t chunk_shift_for(uint64_t attempts) {
+  const uint64_t warps = (uint64_t)sm_count() * sample_blocks_per_sm() * SAMPLE_WARPS;
+  uint32_t shift = 8;
+  while (shift > 5 && (attempts >> shift) < warps) --shift;
+  return shift;
+}
+
 // One sampler launch over attempts [st.next_attempt, + batch): hits are recorded per chunk
-// and compacted in attempt order into aid/len at st.count; *new_hits receives their number.
+// and compacted in attempt order into aid/len at st.count; *new_hits receives their number,
+// *new_nodes their nodes.
 static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st, uint64_t batch, uint32_t* new_hits,
-                                 cudaStream_t s) {
+                                 int64_t* new_nodes, cudaStream_t s) {
   SampleParams P = make_params(g, qd);
-  const uint32_t SHIFT = 8, CHUNK = 1u << SHIFT;
-  const uint32_t n_chunks = (uint32_t)((batch + CHUNK - 1) / CHUNK);
+  const uint32_t shift = chunk_shift_for(batch), chunk = 1u << shift;
+  const uint32_t n_chunks = (uint32_t)((batch + chunk - 1) >> shift);
   // records per chunk: a few standard deviations above the expected hits, else all
-  double exp_hits = std::max(st.hit_rate, 0.0) * CHUNK;
-  uint32_t cap = (uint32_t)std::min<double>(CHUNK, std::ceil(exp_hits + 6.0 * std::sqrt(exp_hits + 1.0) + 8.0));
-  if (st.hit_rate == 0.0) cap = CHUNK;
+  const double exp_hits = std::max(st.hit_rate, 0.0) * chunk;
+  uint32_t cap = (uint32_t)std::min<double>(chunk, std::ceil(exp_hits + 6.0 * std::sqrt(exp_hits + 1.0) + 8.0));
+  if (st.hit_rate == 0.0) cap = chunk;
   for (;;) {
-    HSAW_TRY(st.tmp64.ensure(1, s));
-    HSAW_TRY(st.chunk_hits.ensure(n_chunks, s));
-    HSAW_TRY(st.chunk_off.ensure(n_chunks, s));
+    HSAW_TRY(st.chunk_hits.ensure((size_t)SC_WORDS + n_chunks, s));
     HSAW_TRY(st.recs.ensure((size_t)n_chunks * cap, s));
-    HSAW_CK(cudaMemsetAsync(st.chunk_hits.p, 0, (size_t)n_chunks * 4, s));
-    HSAW_CK(cudaMemsetAsync(st.ctrs.p, 0, 8 * 4, s));
-    unsigned long long* d_steps = reinterpret_cast<unsigned long long*>(st.tmp64.p);
-    HSAW_CK(cudaMemsetAsync(d_steps, 0, 8, s));
+    uint32_t* const ctl = st.chunk_hits.p;
+    HSAW_CK(cudaMemsetAsync(ctl, 0, ((size_t)SC_WORDS + n_chunks) * 4, s));
     P.a0 = st.next_attempt;
     P.n_attempts = (uint32_t)batch;
-    P.chunk_shift = SHIFT;
+    P.chunk_shift = shift;
     P.n_chunks = n_chunks;
     P.cap = cap;
-    P.chunk_ctr = st.ctrs.p;
-    P.chunk_hits = st.chunk_hits.p;
+    P.ctl = ctl;
+    P.chunk_hits = ctl + SC_WORDS;
     P.recs = st.recs.p;
-    P.steps = d_steps;
     int trial = -1;
     const int bps = sample_blocks_for(g, batch, &trial);
     const unsigned grid = (unsigned)std::max(1, std::min<int>(sm_count() * bps, (int)((n_chunks + 7) / 8)));
@@ -525,24 +599,24 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
     profile_end(prof, s, batch);
     if (trial >= 0) cudaEventRecord(tev[1], s);
     HSAW_CK(cudaGetLastError());
-    count_launch();
-    k_clamp<<<grid_for(n_chunks, 256, 4096), 256, 0, s>>>(st.chunk_hits.p, st.chunk_off.p, n_chunks, cap);
-    HSAW_CK(cudaGetLastError());
-    HSAW_TRY(exclusive_scan_u32(st.chunk_off.p, n_chunks, st.ctrs.p + 2, s));
-    uint32_t h[4];
-    unsigned long long hs = 0;
-    HSAW_CK(cudaMemcpyAsync(h, st.ctrs.p, 16, cudaMemcpyDeviceToHost, s));
-    HSAW_CK(cudaMemcpyAsync(&hs, d_steps, 8, cudaMemcpyDeviceToHost, s));
+    // the counts' offsets in place (a chunk with more hits than records makes the launch run
+    // again, whatever they say)
+    HSAW_TRY(exclusive_scan_u32(P.chunk_hits, n_chunks, ctl + SC_HITS, s));
+    uint32_t h[SC_WORDS];
+    HSAW_CK(cudaMemcpyAsync(h, ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
     HSAW_CK(cudaStreamSynchronize(s));
+    unsigned long long hs = 0, hn = 0;
+    std::memcpy(&hs, h + SC_STEPS, 8);
+    std::memcpy(&hn, h + SC_NODES, 8);
     if (trial >= 0) {
       float ms = 0.f;
       if (cudaEventElapsedTime(&ms, tev[0], tev[1]) == cudaSuccess) sample_tune_record(g, trial, (double)hs, ms);
       cudaEventDestroy(tev[0]);
       cudaEventDestroy(tev[1]);
     }
-    if (h[1] & ST_STEP_CAP) return fail(HSAW_E_STEP_CAP, "sampling: a walk exceeded its step guard");
-    if ((h[1] & ST_OVERFLOW) && cap < CHUNK) {
-      cap = CHUNK;  // rare: rerun this launch with room for every attempt to hit
+    if (h[SC_STATUS] & ST_STEP_CAP) return fail(HSAW_E_STEP_CAP, "sampling: a walk exceeded its step guard");
+    if ((h[SC_STATUS] & ST_OVERFLOW) && cap < chunk) {
+      cap = chunk;  // rare: rerun this launch with room for every attempt to hit
       continue;
     }
     st.steps += hs;
@@ -550,14 +624,15 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
     if (getenv("HSAW_LOG_LAUNCHES"))  // measurement aid: attempts and live-edge draws of each sampler launch
       fprintf(stderr, "hsaw: k_sample launch attempts=%llu draws=%llu blocks_per_sm=%d\n", (unsigned long long)batch,
               hs, bps);
-    *new_hits = h[2];
-    if (h[2]) {
-      HSAW_TRY(st.aid.ensure((size_t)st.count + h[2], s, true));
-      HSAW_TRY(st.len.ensure((size_t)st.count + h[2], s, true));
+    *new_hits = h[SC_HITS];
+    *new_nodes = (int64_t)hn;
+    if (*new_hits) {
+      HSAW_TRY(st.aid.ensure((size_t)st.count + *new_hits, s, true));
+      HSAW_TRY(st.len.ensure((size_t)st.count + *new_hits, s, true));
       count_launch();
-      k_compact<<<grid_for((size_t)n_chunks * 32, 256, 8192), 256, 0, s>>>(
-          st.chunk_hits.p, st.chunk_off.p, st.recs.p, cap, n_chunks, st.next_attempt, st.aid.p + st.count,
-          st.len.p + st.count);
+      k_compact<<<grid_for((size_t)n_chunks * 32, 256, 8192), 256, 0, s>>>(P.chunk_hits, ctl + SC_HITS, st.recs.p, cap,
+                                                                         n_chunks, st.next_attempt, st.aid.p + st.count,
+                                                                         st.len.p + st.count);
       HSAW_CK(cudaGetLastError());
     }
     return HSAW_OK;
@@ -575,54 +650,60 @@ hsaw_status stream_extend(const Graph& g, const QueryDev& qd, Stream& st, int64_
     if (cancel_requested()) return fail(HSAW_E_CANCELLED, "sampling: query cancelled");
     const uint64_t used = st.next_attempt - st.first_attempt;
     if (used >= st.max_attempts) return fail(HSAW_E_TIMEOUT, "sampling: attempt budget exhausted before enough hits");
-    // window size from the hit rate so far (2^20 .. 2^28 attempts; doubling while no hit),
+    // window size from the hit rate so far (2^20 .. 2^28 attempts; doubling while no hit; down
+    // to 2^16 where the walks of a window past the last hit asked for are of no use to the
+    // caller, the first then by the rate that start nodes alone give),
     // with a margin of 4 standard deviations of the rate estimate (st.count hits seen) and
     // of the window's own hit count (need): attempts past the last hit a solve uses are
     // wasted, and a window that falls short only costs one more launch
     const double need = (double)(want - st.count);
     st.hit_rate = used ? (double)st.count / (double)used : 0.0;
     const double margin = std::min(1.25, 1.0 + 4.0 / std::sqrt(std::max(1.0, (double)st.count)) + 4.0 / std::sqrt(need));
-    double target = st.hit_rate > 0 ? need / st.hit_rate * margin + 4096.0 : std::max(1048576.0, 2.0 * (double)used);
-    target = std::max(target, 1048576.0);
+    const double least = st.least_window;
+    double target = st.hit_rate > 0 ? need / st.hit_rate * margin + 4096.0
+                    : used          ? std::max(1048576.0, 2.0 * (double)used)
+                                    : std::min(1048576.0, need / std::max(qd.start_rate, 1e-12));
+    target = std::max(target, least);
     target = std::min(target, 268435456.0);
     uint64_t batch = (uint64_t)target;
     batch = std::min<uint64_t>(batch, st.max_attempts - used);
     uint32_t new_hits = 0;
+    int64_t new_nodes = 0;
     if (pool_ok && st.next_attempt < g.pool.attempts) {
       // whole blocks of the index where the pool and the budget allow
       const uint64_t B = 1ull << g.pool.shift;
       uint64_t a1 = std::min<uint64_t>(g.pool.attempts, (st.next_attempt + batch + B - 1) / B * B);
       a1 = std::min<uint64_t>(a1, st.next_attempt + (st.max_attempts - used));
       batch = a1 - st.next_attempt;
-      HSAW_TRY(pool_hits(g, qd, st, st.next_attempt, a1, &new_hits, s));
+      HSAW_TRY(pool_hits(g, qd, st, st.next_attempt, a1, &new_hits, &new_nodes, s));
     } else {
       batch = (batch + CHUNK - 1) / CHUNK * CHUNK;
-      HSAW_TRY(sample_window(g, qd, st, batch, &new_hits, s));
+      HSAW_TRY(sample_window(g, qd, st, batch, &new_hits, &new_nodes, s));
     }
-    HSAW_TRY(stream_take_hits(g, qd, st, new_hits, s));
+    HSAW_TRY(stream_take_hits(g, qd, st, new_hits, new_nodes, s));
     st.next_attempt += batch;
   }
   return HSAW_OK;
 }
 
-hsaw_status stream_take_hits(const Graph& g, const QueryDev& qd, Stream& st, uint32_t new_hits, cudaStream_t s) {
+hsaw_status stream_take_hits(const Graph& g, const QueryDev& qd, Stream& st, uint32_t new_hits, int64_t new_nodes,
+                             cudaStream_t s) {
   if (!new_hits) return HSAW_OK;
+  if (st.ids_only) {
+    st.count += new_hits;
+    return HSAW_OK;
+  }
   const uint32_t k0 = (uint32_t)qd.seed, k1 = (uint32_t)(qd.seed >> 32);
   // walk offsets, then the hits' nodes and edges re-drawn from their attempt ids
   HSAW_TRY(st.node_off.ensure((size_t)st.count + new_hits + 1, s, true));
-  HSAW_TRY(st.tmp64.ensure((size_t)new_hits + 1, s));
-  count_launch();
-  k_len_to_u64<<<grid_for(new_hits, 256, 4096), 256, 0, s>>>(st.len.p + st.count, new_hits, st.tmp64.p);
-  HSAW_CK(cudaGetLastError());
-  HSAW_TRY(exclusive_scan_u64(st.tmp64.p, new_hits, st.tmp64.p + new_hits, s));
-  count_launch();
-  k_offsets<<<grid_for((size_t)new_hits + 1, 256, 4096), 256, 0, s>>>(
-      st.tmp64.p, new_hits, st.total_nodes, st.node_off.p + st.count, st.tmp64.p + new_hits);
-  HSAW_CK(cudaGetLastError());
-  uint64_t added = 0;
-  HSAW_CK(cudaMemcpyAsync(&added, st.tmp64.p + new_hits, 8, cudaMemcpyDeviceToHost, s));
-  HSAW_CK(cudaStreamSynchronize(s));
-  const int64_t tot = st.total_nodes + (int64_t)added;
+  HSAW_TRY(len_offsets(st.len.p + st.count, new_hits, st.total_nodes, st.node_off.p + st.count, st.tmp64, s));
+  if (new_nodes < 0) {
+    int64_t end = 0;
+    HSAW_CK(cudaMemcpyAsync(&end, st.node_off.p + st.count + new_hits, 8, cudaMemcpyDeviceToHost, s));
+    HSAW_CK(cudaStreamSynchronize(s));
+    new_nodes = end - st.total_nodes;
+  }
+  const int64_t tot = st.total_nodes + new_nodes;
   HSAW_TRY(st.nodes.ensure((size_t)tot, s, true));
   HSAW_TRY(st.edges.ensure((size_t)tot, s, true));
   const unsigned grid = grid_for(new_hits, 128, 1u << 16);
@@ -643,7 +724,7 @@ hsaw_status classify_attempts(const Graph& g, const QueryDev& qd, uint64_t first
   uint32_t* d_ctr = nullptr;
   HSAW_TRY(dmalloc((void**)&d_ctr, 16, s));
   HSAW_CK(cudaMemsetAsync(d_ctr, 0, 16, s));
-  P.chunk_ctr = d_ctr;
+  P.ctl = d_ctr;
   const unsigned grid = grid_for(count, 128, 1u << 16);
   const bool hp = P.p32 != nullptr, hr = (P.edge_removed || P.node_removed);
   if (hp && hr) { count_launch(); k_classify<true, true><<<grid, 128, 0, s>>>(P, first, count, outcome, length); }
@@ -669,21 +750,13 @@ hsaw_status classify_attempts(const Graph& g, const QueryDev& qd, uint64_t first
 // addresses are looked up once per device with cudaGetSymbolAddress.
 namespace hsaw {
 
-constexpr uint32_t STATIC_SHIFT = 8;
-constexpr uint32_t STATIC_CHUNK = 1u << STATIC_SHIFT;
-constexpr uint32_t STATIC_CHUNKS = HSAW_STATIC_MAX_ATTEMPTS / STATIC_CHUNK;
+constexpr uint32_t STATIC_CHUNKS = HSAW_STATIC_MAX_ATTEMPTS / 32;  // chunks of at least 32 attempts
 
-static __device__ __align__(256) uint32_t g_static_ctrs[8];                 // work counter, status, total
-static __device__ __align__(256) unsigned long long g_static_steps[1];
-static __device__ __align__(256) uint32_t g_static_chunk_hits[STATIC_CHUNKS];
-static __device__ __align__(256) uint32_t g_static_chunk_off[STATIC_CHUNKS];
-static __device__ __align__(256) uint2 g_static_recs[STATIC_CHUNKS * STATIC_CHUNK];
+static __device__ __align__(256) uint32_t g_static_ctl[SC_WORDS + STATIC_CHUNKS];  // control words, chunk hits
+static __device__ __align__(256) uint2 g_static_recs[HSAW_STATIC_MAX_ATTEMPTS];
 
 struct StaticScratch {
-  uint32_t* ctrs = nullptr;
-  unsigned long long* steps = nullptr;
-  uint32_t* chunk_hits = nullptr;
-  uint32_t* chunk_off = nullptr;
+  uint32_t* ctl = nullptr;
   uint2* recs = nullptr;
   bool ready = false;
 };
@@ -698,10 +771,7 @@ static hsaw_status static_scratch(StaticScratch** out) {
   std::lock_guard<std::mutex> lk(g_static_mu);
   StaticScratch& s = g_static_dev[dev];
   if (!s.ready) {
-    HSAW_CK(cudaGetSymbolAddress((void**)&s.ctrs, g_static_ctrs));
-    HSAW_CK(cudaGetSymbolAddress((void**)&s.steps, g_static_steps));
-    HSAW_CK(cudaGetSymbolAddress((void**)&s.chunk_hits, g_static_chunk_hits));
-    HSAW_CK(cudaGetSymbolAddress((void**)&s.chunk_off, g_static_chunk_off));
+    HSAW_CK(cudaGetSymbolAddress((void**)&s.ctl, g_static_ctl));
     HSAW_CK(cudaGetSymbolAddress((void**)&s.recs, g_static_recs));
     s.ready = true;
   }
@@ -709,34 +779,66 @@ static hsaw_status static_scratch(StaticScratch** out) {
   return HSAW_OK;
 }
 
-// Single-block exclusive scan of at most STATIC_CHUNKS counts (clamped to cap); writes the
-// total to *total.  One block of 1024 threads, no temporary memory.
-__global__ void __launch_bounds__(1024) k_static_scan(const uint32_t* __restrict__ in, uint32_t n, uint32_t cap,
-                                                      uint32_t* __restrict__ out, uint32_t* __restrict__ total) {
-  __shared__ uint32_t warp_sum[32];
-  __shared__ uint32_t carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
+// The hits of all chunks in attempt order, as k_compact, with no scan before it: a block owns
+// STATIC_BLOCK chunks and sums the counts of those before them itself (at most 32 KB, from L2).
+// Writes nothing when there are more than out_cap hits; the total goes to ctl.
+constexpr uint32_t STATIC_BLOCK = 128;
+__global__ void __launch_bounds__(256) k_static_finish(const uint32_t* __restrict__ chunk_hits, uint32_t n_chunks,
+                                                       const uint2* __restrict__ recs, uint32_t chunk_shift,
+                                                       uint64_t a0, int64_t out_cap, uint32_t* __restrict__ ctl,
+                                                       uint64_t* __restrict__ out_aid,
+                                                       uint32_t* __restrict__ out_len) {
+  __shared__ uint32_t before_w[8], total_w[8], own[STATIC_BLOCK], off[STATIC_BLOCK];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (uint32_t base = 0; base < n; base += blockDim.x) {
-    const uint32_t i = base + threadIdx.x;
-    const uint32_t v = i < n ? min(in[i], cap) : 0u;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_sum[w] = x;
-    __syncthreads();
-    uint32_t before = carry;
-    for (int k = 0; k < w; ++k) before += warp_sum[k];
-    if (i < n) out[i] = before + x - v;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry = before + x;
-    __syncthreads();
+  const uint32_t c0 = blockIdx.x * STATIC_BLOCK;
+  uint32_t before = 0, total = 0;
+  for (uint32_t i = threadIdx.x; i < n_chunks; i += blockDim.x) {
+    const uint32_t c = chunk_hits[i];
+    total += c;
+    if (i < c0) before += c;
+    if (i >= c0 && i < c0 + STATIC_BLOCK) own[i - c0] = c;
   }
-  if (threadIdx.x == 0) *total = carry;
+  before = __reduce_add_sync(0xffffffffu, before);
+  total = __reduce_add_sync(0xffffffffu, total);
+  if (lane == 0) {
+    before_w[w] = before;
+    total_w[w] = total;
+  }
+  __syncthreads();
+  before = total = 0;
+  for (int i = 0; i < 8; ++i) {
+    before += before_w[i];
+    total += total_w[i];
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctl[SC_HITS] = total;
+  if ((int64_t)total > out_cap || (ctl[SC_STATUS] & ST_STEP_CAP)) return;
+  const uint32_t mine = min(STATIC_BLOCK, n_chunks - c0);
+  if (w == 0) {  // offsets of the block's chunks
+    uint32_t run = before;
+    for (uint32_t i0 = 0; i0 < mine; i0 += 32) {
+      const uint32_t v = i0 + lane < mine ? own[i0 + lane] : 0u;
+      uint32_t x = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      if (i0 + lane < mine) off[i0 + lane] = run + x - v;
+      run += __shfl_sync(0xffffffffu, x, 31);
+    }
+  }
+  __syncthreads();
+  for (uint32_t ck = w; ck < mine; ck += 8) {
+    const uint32_t c = own[ck];
+    const uint2* r = recs + ((size_t)(c0 + ck) << chunk_shift);
+    for (uint32_t i = lane; i < c; i += 32) {
+      const uint2 me = r[i];
+      uint32_t rank = 0;
+      for (uint32_t j = 0; j < c; ++j) rank += (r[j].x < me.x) ? 1u : 0u;
+      out_aid[off[ck] + rank] = a0 + me.x;
+      out_len[off[ck] + rank] = me.y;
+    }
+  }
 }
 
 }  // namespace hsaw
@@ -766,39 +868,32 @@ extern "C" hsaw_status hsaw_sample_hits_static(hsaw_graph g, const uint32_t* sus
   P.k1 = (uint32_t)(seed >> 32);
   P.keys = philox_round_keys(P.k0, P.k1);
   P.step_cap = (uint32_t)std::min<uint64_t>(4ull * (uint64_t)G.n + 64ull, 0xFFFFFFF0ull);
-  const uint32_t n_chunks = (uint32_t)((n_attempts + STATIC_CHUNK - 1) / STATIC_CHUNK);
+  const uint32_t shift = chunk_shift_for((uint64_t)n_attempts);
+  const uint32_t n_chunks = (uint32_t)((n_attempts + (1 << shift) - 1) >> shift);
   P.a0 = first_attempt;
   P.n_attempts = (uint32_t)n_attempts;
-  P.chunk_shift = STATIC_SHIFT;
+  P.chunk_shift = shift;
   P.n_chunks = n_chunks;
-  P.cap = STATIC_CHUNK;  // room for every attempt of a chunk to hit: no overflow
-  P.chunk_ctr = sc->ctrs;
-  P.chunk_hits = sc->chunk_hits;
+  P.cap = 1u << shift;  // room for every attempt of a chunk to hit: no overflow
+  P.ctl = sc->ctl;
+  P.chunk_hits = sc->ctl + SC_WORDS;
   P.recs = sc->recs;
-  P.steps = sc->steps;
   // the shared scratch keeps the previous call's contents: clear what must start at zero
-  HSAW_CK(cudaMemsetAsync(sc->ctrs, 0, sizeof(g_static_ctrs), s));
-  HSAW_CK(cudaMemsetAsync(sc->steps, 0, sizeof(g_static_steps), s));
-  HSAW_CK(cudaMemsetAsync(sc->chunk_hits, 0, (size_t)n_chunks * sizeof(uint32_t), s));
+  HSAW_CK(cudaMemsetAsync(sc->ctl, 0, ((size_t)SC_WORDS + n_chunks) * sizeof(uint32_t), s));
   const unsigned grid = (unsigned)std::max(1, std::min<int>(sm_count() * sample_blocks_per_sm(),
                                                              (int)((n_chunks + 7) / 8)));
   launch_sample(G, P, grid, s);
   HSAW_CK(cudaGetLastError());
   count_launch();
-  k_static_scan<<<1, 1024, 0, s>>>(sc->chunk_hits, n_chunks, STATIC_CHUNK, sc->chunk_off, sc->ctrs + 2);
+  k_static_finish<<<(n_chunks + STATIC_BLOCK - 1) / STATIC_BLOCK, 256, 0, s>>>(P.chunk_hits, n_chunks, sc->recs, shift,
+                                                                             first_attempt, out_cap, sc->ctl, aid_out,
+                                                                             len_out);
   HSAW_CK(cudaGetLastError());
-  uint32_t h[4] = {0, 0, 0, 0};
-  HSAW_CK(cudaMemcpyAsync(h, sc->ctrs, sizeof(h), cudaMemcpyDeviceToHost, s));
+  uint32_t h[SC_WORDS] = {0};
+  HSAW_CK(cudaMemcpyAsync(h, sc->ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
   HSAW_CK(cudaStreamSynchronize(s));
-  if (h[1] & ST_STEP_CAP) return fail(HSAW_E_STEP_CAP, "static sampler: a walk exceeded its step guard");
-  *n_hits = h[2];
-  if ((int64_t)h[2] > out_cap) return fail(HSAW_E_INVALID, "static sampler: more hits than out_cap");
-  if (h[2]) {
-    count_launch();
-    k_compact<<<grid_for((size_t)n_chunks * 32, 256, 8192), 256, 0, s>>>(
-        sc->chunk_hits, sc->chunk_off, sc->recs, STATIC_CHUNK, n_chunks, first_attempt, aid_out, len_out);
-    HSAW_CK(cudaGetLastError());
-  }
-  HSAW_CK(cudaStreamSynchronize(s));
+  if (h[SC_STATUS] & ST_STEP_CAP) return fail(HSAW_E_STEP_CAP, "static sampler: a walk exceeded its step guard");
+  *n_hits = h[SC_HITS];
+  if ((int64_t)h[SC_HITS] > out_cap) return fail(HSAW_E_INVALID, "static sampler: more hits than out_cap");
   return HSAW_OK;
 }

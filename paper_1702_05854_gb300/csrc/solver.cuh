@@ -15,6 +15,7 @@ struct QueryDev {
   uint32_t* node_removed = nullptr;  // n bits or NULL
   uint64_t seed = 0;
   bool owns_removed = false;
+  double start_rate = 0.0;  // chance that a start node is a real source
 };
 
 hsaw_status query_upload(const Graph& g, const hsaw_query* q, QueryDev& qd, cudaStream_t s);
@@ -44,6 +45,8 @@ struct Stream {
   DBuf<uint32_t> pbits;  // walk pool: one bit per attempt of a window
   DBuf<uint64_t> pcnt;   // walk pool: entries per (source, block), then their prefix
   double hit_rate = 0.0;  // running estimate for launch sizing
+  double least_window = 1048576.0;  // attempts per sampler launch; a caller's handle holds all hits of its windows
+  bool ids_only = false;  // only attempt ids and lengths are wanted, no walks
   int64_t elem_range[2] = {0, 0};  // [node mode, edge mode]: element ids lie in [0, n) / [0, m)
   void release(cudaStream_t s);
 };
@@ -53,7 +56,9 @@ hsaw_status stream_init(Stream& st, uint64_t first_attempt, uint64_t max_attempt
 hsaw_status stream_extend(const Graph& g, const QueryDev& qd, Stream& st, int64_t want, cudaStream_t s);
 // Adopt new_hits hits whose attempt ids and lengths are already at aid/len[st.count ..]:
 // their walk offsets, nodes and edges (re-drawn from the attempt ids), and the count.
-hsaw_status stream_take_hits(const Graph& g, const QueryDev& qd, Stream& st, uint32_t new_hits, cudaStream_t s);
+// new_nodes: their nodes, or -1 if not known.
+hsaw_status stream_take_hits(const Graph& g, const QueryDev& qd, Stream& st, uint32_t new_hits, int64_t new_nodes,
+                             cudaStream_t s);
 hsaw_status classify_attempts(const Graph& g, const QueryDev& qd, uint64_t first, int64_t count, int8_t* outcome,
                               int32_t* length, cudaStream_t s);
 
@@ -127,9 +132,9 @@ hsaw_status cover_count(const Stream& st, hsaw_mode mode, int64_t first, int64_t
 void pool_release(WalkPool& p);
 hsaw_status pool_build(Graph& g, uint64_t seed, uint64_t attempts, cudaStream_t s);
 // Append to st (aid, len at st.count) the hits among attempts [a0, a1) (a1 <= pool.attempts),
-// in attempt order; *new_hits receives their number.
+// in attempt order; *new_hits receives their number, *new_nodes their nodes.
 hsaw_status pool_hits(const Graph& g, const QueryDev& qd, Stream& st, uint64_t a0, uint64_t a1, uint32_t* new_hits,
-                      cudaStream_t s);
+                      int64_t* new_nodes, cudaStream_t s);
 
 // Cancellation of the calling thread's current solve (set by the server's workers):
 // checked between sampler launches and between stopping-rule rounds.

@@ -212,3 +212,22 @@ def test_greedy_conflict_chains():
                 ids, gains = hs.hsaw_greedy(walks, g, mode, first, count, 30)
                 oids, ogains = ost.greedy(mode, first, count, M, 30)
                 assert np.array_equal(gains, ogains) and np.array_equal(ids, oids)
+
+
+@pytest.mark.parametrize("count", [1, 31, 32, 33, 127, 4095, 4097, 116_735, 116_737, 233_471, 233_473, 1 << 18])
+def test_static_chunks(count):
+    """The allocation-free sampler's chunks of 32 to 256 attempts, and its blocks of 128 chunks."""
+    d = synth.workload_c1()
+    g = hs.hsaw_graph_from_edges(d["n"], d["src"], d["dst"], d["w"])
+    og = oracle.Graph(d["n"], d["src"], d["dst"], d["w"])
+    bits = np.zeros((d["n"] + 31) // 32, np.uint32)
+    np.bitwise_or.at(bits, d["sources"] >> 5, np.uint32(1) << (d["sources"] & 31).astype(np.uint32))
+    aid = torch.full((count,), -1, dtype=torch.int64, device="cuda")
+    length = torch.full((count,), -1, dtype=torch.int32, device="cuda")
+    first = 12_345
+    n = hs.hsaw_sample_hits_static(g, torch.from_numpy(bits.view(np.int32)).cuda(), 4, first, count, aid, length)
+    out, ln = oracle.Query(og, d["sources"], seed=4).classify(first, count)
+    hit = np.nonzero(out == 1)[0]
+    assert n == hit.size
+    assert np.array_equal(aid[:n].cpu().numpy(), first + hit) and np.array_equal(length[:n].cpu().numpy(), ln[hit])
+    assert bool((aid[n:] == -1).all()) and bool((length[n:] == -1).all())
