@@ -215,8 +215,10 @@ struct Ckpt {
   __device__ __forceinline__ void keep(uint32_t u, uint32_t pos) {
     if (pos < next) return;
     c7 = c6; c6 = c5; c5 = c4; c4 = c3; c3 = c2; c2 = c1; c1 = c0; c0 = u;
-    next = next + max(1u, next >> 2);
+    next = after(next);
   }
+  // the position kept after `pos`: 1, 2, ..., 8, 10, 12, 15, ...
+  static __device__ __forceinline__ uint32_t after(uint32_t pos) { return pos + max(1u, pos >> 2); }
 };
 
 // ------------------------------------------------------------------ primitives (primitives.cu)

@@ -181,12 +181,14 @@ template <bool HAS_P, Layout L>
 __global__ void k_hit_len(const WalkTables T, uint32_t n, uint32_t k0, uint32_t k1, const uint32_t* __restrict__ s_bits,
                           const uint32_t* __restrict__ p32, const uint64_t* __restrict__ aid, uint32_t count,
                           uint32_t step_cap, uint32_t* __restrict__ len, uint32_t* __restrict__ status,
-                          unsigned long long* __restrict__ nodes) {
+                          unsigned long long* __restrict__ nodes, uint4* __restrict__ kept) {
   uint32_t sum = 0;
   for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < count; h += gridDim.x * blockDim.x) {
     const uint64_t a = aid[h];
     uint32_t v = start_node(a, n, k0, k1), l = 1;
     uint4 rec = __ldg(&T.node[v]);
+    Ckpt ck;  // only for its checkpoints: a listed attempt reaches its source before any repeat
+    ck.reset(v);
     for (;;) {
       const uint4 x = node_draw(a, v, k0, k1);
       if (((__ldg(&s_bits[v >> 5]) >> (v & 31)) & 1u) && (!HAS_P || source_coin(x.y, __ldg(&p32[v])))) break;
@@ -195,9 +197,12 @@ __global__ void k_hit_len(const WalkTables T, uint32_t n, uint32_t k0, uint32_t 
         break;
       }
       record_step<L>(T, v, rec, x.x, v, rec);
+      ck.keep(v, l);
       ++l;
     }
     len[h] = l;
+    kept[2 * (size_t)h] = make_uint4(ck.c0, ck.c1, ck.c2, ck.c3);
+    kept[2 * (size_t)h + 1] = make_uint4(ck.c4, ck.c5, ck.c6, ck.c7);
     sum += l;
   }
   unsigned long long warp_sum = sum;
@@ -336,6 +341,8 @@ hsaw_status pool_hits(const Graph& g, const QueryDev& qd, Stream& st, uint64_t a
   if (!h) return HSAW_OK;
   HSAW_TRY(st.aid.ensure((size_t)st.count + h, s, true));
   HSAW_TRY(st.len.ensure((size_t)st.count + h, s, true));
+  HSAW_TRY(st.kept.ensure(2 * (size_t)h, s));
+  st.kept_hits = h;
   count_launch();
   k_bits_emit<<<grid_for(words, 256, 8192), 256, 0, s>>>(st.pbits.p, st.chunk_off.p, words, a0, st.aid.p + st.count);
   HSAW_CK(cudaGetLastError());
@@ -347,7 +354,7 @@ hsaw_status pool_hits(const Graph& g, const QueryDev& qd, Stream& st, uint64_t a
   const auto hit_len = by_layout[qd.p32 ? 1 : 0][g.layout];
   hit_len<<<hgrid, 128, 0, s>>>(g.tables(), (uint32_t)g.n, k0, k1, qd.s_bits, qd.p32, st.aid.p + st.count, h,
                                 pool_step_cap(g), st.len.p + st.count, st.ctrs.p + 3,
-                                reinterpret_cast<unsigned long long*>(st.ctrs.p + 4));
+                                reinterpret_cast<unsigned long long*>(st.ctrs.p + 4), st.kept.p);
   HSAW_CK(cudaGetLastError());
   uint32_t back[3] = {0, 0, 0};  // status, then the nodes (64 bits)
   HSAW_CK(cudaMemcpyAsync(back, st.ctrs.p + 3, sizeof(back), cudaMemcpyDeviceToHost, s));

@@ -48,6 +48,7 @@ struct SampleParams {
   uint32_t* ctl;         // SampleCtl words
   uint32_t* chunk_hits;  // n_chunks
   uint2* recs;           // n_chunks * cap
+  uint4* kept;           // 2 per record, or NULL: the checkpoints of the hit's walk, newest first
   PhiloxKeys keys;       // round keys of (k0, k1)
 };
 
@@ -176,8 +177,14 @@ __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_co
           my_nodes += len;
           const uint32_t ck_i = off >> P.chunk_shift;
           const uint32_t slot = atomicAdd(&P.chunk_hits[ck_i], 1u);
-          if (slot < P.cap) P.recs[(size_t)ck_i * P.cap + slot] = make_uint2(off, len);
-          else atomicOr(P.ctl + SC_STATUS, ST_OVERFLOW);
+          if (slot < P.cap) {
+            const size_t at = (size_t)ck_i * P.cap + slot;
+            P.recs[at] = make_uint2(off, len);
+            if (P.kept) {
+              P.kept[2 * at] = make_uint4(ck.c0, ck.c1, ck.c2, ck.c3);
+              P.kept[2 * at + 1] = make_uint4(ck.c4, ck.c5, ck.c6, ck.c7);
+            }
+          } else atomicOr(P.ctl + SC_STATUS, ST_OVERFLOW);
         }
       }
     }
@@ -198,7 +205,8 @@ __global__ void __launch_bounds__(SAMPLE_WARPS * 32, 6) k_sample(const __grid_co
 // smaller offset.
 __global__ void k_compact(const uint32_t* __restrict__ chunk_off, const uint32_t* __restrict__ total,
                           const uint2* __restrict__ recs, uint32_t cap, uint32_t n_chunks, uint64_t a0,
-                          uint64_t* __restrict__ out_aid, uint32_t* __restrict__ out_len) {
+                          const uint4* __restrict__ kept, uint64_t* __restrict__ out_aid,
+                          uint32_t* __restrict__ out_len, uint4* __restrict__ out_kept) {
   const int lane = threadIdx.x & 31;
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
   for (uint32_t ck = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; ck < n_chunks; ck += warps) {
@@ -212,6 +220,10 @@ __global__ void k_compact(const uint32_t* __restrict__ chunk_off, const uint32_t
       for (uint32_t j = 0; j < c; ++j) rank += (r[j].x < me.x) ? 1u : 0u;
       out_aid[base + rank] = a0 + me.x;
       out_len[base + rank] = me.y;
+      if (kept) {
+        out_kept[2 * (size_t)(base + rank)] = kept[2 * ((size_t)ck * cap + i)];
+        out_kept[2 * (size_t)(base + rank) + 1] = kept[2 * ((size_t)ck * cap + i) + 1];
+      }
     }
   }
 }
@@ -302,6 +314,52 @@ __global__ void k_rewalk(const WalkTables T, uint32_t n, uint32_t k0, uint32_t k
       if (x.x >= rec.w) break;  // a hit's walk has a live in-edge at each of its first l - 1 nodes
       edges[eb + i - 1] = (int32_t)record_step<L>(T, v, rec, x.x, v, rec);
       nodes[nb + i] = (int32_t)v;
+    }
+  }
+}
+
+// The same by segments: the walk's last eight checkpoints (kept, newest first) are known, so its
+// parts between them are walked side by side, each a fifth of the walk at most.  A launch takes
+// as long as its longest chain of dependent reads: the longest hit of a window is 5-10 times
+// the mean.
+constexpr int SEGMENTS = 9;
+template <Layout L>
+__global__ void k_rewalk_segments(const WalkTables T, uint32_t n, uint32_t k0, uint32_t k1,
+                                  const uint64_t* __restrict__ aid, const uint32_t* __restrict__ len,
+                                  const int64_t* __restrict__ node_off, const uint32_t* __restrict__ kept, int64_t h0,
+                                  int64_t h1, int32_t* __restrict__ nodes, int32_t* __restrict__ edges) {
+  const int64_t total = (h1 - h0) * SEGMENTS;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t h = h0 + i / SEGMENTS;
+    const uint32_t seg = (uint32_t)(i % SEGMENTS);  // from the checkpoint that is seg-th from the end; 8: from the start
+    const uint32_t l = len[h];
+    // the positions kept before l, newest first: how many, and those this segment lies between
+    uint32_t count = 0;
+    for (uint32_t p = 1; p < l; p = Ckpt::after(p)) ++count;
+    const uint32_t have = min(count, 8u);
+    if (seg < 8 && seg >= have) continue;
+    const uint32_t from_rank = seg < 8 ? count - seg : 0u;              // rank 0: the start, at position 0
+    const uint32_t to_rank = seg < 8 ? from_rank + 1 : count - have + 1;  // rank count + 1: the end
+    uint32_t from = 0, to = l - 1, p = 1;
+    for (uint32_t rank = 1; rank <= count; ++rank, p = Ckpt::after(p)) {
+      if (rank == from_rank) from = p;
+      if (rank == to_rank) to = p;
+    }
+    const uint64_t a = aid[h];
+    const int64_t nb = node_off[h], eb = nb - h;
+    uint32_t v;
+    if (seg < 8) {
+      v = kept[8 * (h - h0) + seg];
+    } else {
+      v = start_node(a, n, k0, k1);
+      nodes[nb] = (int32_t)v;
+    }
+    uint4 rec = to > from ? __ldg(&T.node[v]) : make_uint4(0, 0, 0, 0);
+    for (uint32_t q = from; q < to; ++q) {
+      const uint4 x = node_draw(a, v, k0, k1);
+      if (x.x >= rec.w) break;  // a hit's walk has a live in-edge at each of its first l - 1 nodes
+      edges[eb + q] = (int32_t)record_step<L>(T, v, rec, x.x, v, rec);
+      nodes[nb + q + 1] = (int32_t)v;
     }
   }
 }
@@ -434,7 +492,7 @@ void query_release(QueryDev& qd, cudaStream_t s) {
 
 void Stream::release(cudaStream_t s) {
   aid.release(s); len.release(s); node_off.release(s); nodes.release(s); edges.release(s);
-  chunk_hits.release(s); chunk_off.release(s); ctrs.release(s); recs.release(s); tmp64.release(s);
+  chunk_hits.release(s); chunk_off.release(s); chunk_kept.release(s); kept.release(s); ctrs.release(s); recs.release(s); tmp64.release(s);
   pbits.release(s); pcnt.release(s);
 }
 
@@ -575,6 +633,7 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
   for (;;) {
     HSAW_TRY(st.chunk_hits.ensure((size_t)SC_WORDS + n_chunks, s));
     HSAW_TRY(st.recs.ensure((size_t)n_chunks * cap, s));
+    HSAW_TRY(st.chunk_kept.ensure(st.ids_only ? 0 : 2 * (size_t)n_chunks * cap, s));
     uint32_t* const ctl = st.chunk_hits.p;
     HSAW_CK(cudaMemsetAsync(ctl, 0, ((size_t)SC_WORDS + n_chunks) * 4, s));
     P.a0 = st.next_attempt;
@@ -585,6 +644,7 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
     P.ctl = ctl;
     P.chunk_hits = ctl + SC_WORDS;
     P.recs = st.recs.p;
+    P.kept = st.ids_only ? nullptr : st.chunk_kept.p;
     int trial = -1;
     const int bps = sample_blocks_for(g, batch, &trial);
     const unsigned grid = (unsigned)std::max(1, std::min<int>(sm_count() * bps, (int)((n_chunks + 7) / 8)));
@@ -629,10 +689,12 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
     if (*new_hits) {
       HSAW_TRY(st.aid.ensure((size_t)st.count + *new_hits, s, true));
       HSAW_TRY(st.len.ensure((size_t)st.count + *new_hits, s, true));
+      HSAW_TRY(st.kept.ensure(st.ids_only ? 0 : 2 * (size_t)*new_hits, s));
+      st.kept_hits = st.ids_only ? 0 : *new_hits;
       count_launch();
-      k_compact<<<grid_for((size_t)n_chunks * 32, 256, 8192), 256, 0, s>>>(P.chunk_hits, ctl + SC_HITS, st.recs.p, cap,
-                                                                         n_chunks, st.next_attempt, st.aid.p + st.count,
-                                                                         st.len.p + st.count);
+      k_compact<<<grid_for((size_t)n_chunks * 32, 256, 8192), 256, 0, s>>>(
+          P.chunk_hits, ctl + SC_HITS, st.recs.p, cap, n_chunks, st.next_attempt, P.kept, st.aid.p + st.count,
+          st.len.p + st.count, st.kept.p);
       HSAW_CK(cudaGetLastError());
     }
     return HSAW_OK;
@@ -706,12 +768,22 @@ hsaw_status stream_take_hits(const Graph& g, const QueryDev& qd, Stream& st, uin
   const int64_t tot = st.total_nodes + new_nodes;
   HSAW_TRY(st.nodes.ensure((size_t)tot, s, true));
   HSAW_TRY(st.edges.ensure((size_t)tot, s, true));
-  const unsigned grid = grid_for(new_hits, 128, 1u << 16);
-  const decltype(&k_rewalk<REC16>) by_layout[] = {k_rewalk<REC16>, k_rewalk<REC32>, k_rewalk<TAIL4>, k_rewalk<EDGE8>};
-  const auto rewalk = by_layout[g.layout];
+  // by segments where walks are long enough for their start-up (a node record each) to pay
+  const bool segments = st.kept_hits == new_hits && new_nodes >= 16 * (int64_t)new_hits;
+  st.kept_hits = 0;
   count_launch();
-  rewalk<<<grid, 128, 0, s>>>(g.tables(), (uint32_t)g.n, k0, k1, st.aid.p, st.len.p, st.node_off.p, st.count,
-                              st.count + new_hits, st.nodes.p, st.edges.p);
+  if (segments) {
+    const decltype(&k_rewalk_segments<REC16>) by_layout[] = {k_rewalk_segments<REC16>, k_rewalk_segments<REC32>,
+                                                             k_rewalk_segments<TAIL4>, k_rewalk_segments<EDGE8>};
+    by_layout[g.layout]<<<grid_for((size_t)new_hits * SEGMENTS, 128, 1u << 16), 128, 0, s>>>(
+        g.tables(), (uint32_t)g.n, k0, k1, st.aid.p, st.len.p, st.node_off.p, reinterpret_cast<uint32_t*>(st.kept.p),
+        st.count, st.count + new_hits, st.nodes.p, st.edges.p);
+  } else {
+    const decltype(&k_rewalk<REC16>) by_layout[] = {k_rewalk<REC16>, k_rewalk<REC32>, k_rewalk<TAIL4>, k_rewalk<EDGE8>};
+    by_layout[g.layout]<<<grid_for(new_hits, 128, 1u << 16), 128, 0, s>>>(
+        g.tables(), (uint32_t)g.n, k0, k1, st.aid.p, st.len.p, st.node_off.p, st.count, st.count + new_hits, st.nodes.p,
+        st.edges.p);
+  }
   HSAW_CK(cudaGetLastError());
   st.total_nodes = tot;
   st.count += new_hits;

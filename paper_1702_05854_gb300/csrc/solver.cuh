@@ -41,6 +41,9 @@ struct Stream {
   // per-launch workspace
   DBuf<uint32_t> chunk_hits, chunk_off, ctrs;
   DBuf<uint2> recs;
+  DBuf<uint4> chunk_kept;  // checkpoints of the records' walks, two per record
+  DBuf<uint4> kept;        // and of the hits just found, in order
+  uint32_t kept_hits = 0;  // hits that kept holds
   DBuf<uint64_t> tmp64;
   DBuf<uint32_t> pbits;  // walk pool: one bit per attempt of a window
   DBuf<uint64_t> pcnt;   // walk pool: entries per (source, block), then their prefix

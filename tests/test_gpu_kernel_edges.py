@@ -231,3 +231,18 @@ def test_static_chunks(count):
     assert n == hit.size
     assert np.array_equal(aid[:n].cpu().numpy(), first + hit) and np.array_equal(length[:n].cpu().numpy(), ln[hit])
     assert bool((aid[n:] == -1).all()) and bool((length[n:] == -1).all())
+
+
+@pytest.mark.parametrize("n,keep", [(40, 1.0), (700, 1.0), (3000, 1.0), (3000, 0.999)])
+def test_rewalk_segments(n, keep):
+    """Walks of every length up to n: on a path to the only suspect a hit started at node j has j + 1 nodes, so the
+    checkpoints, none to far more than the eight kept, cut it in every way.  From the sampler and from a walk pool."""
+    src, dst = np.arange(n - 1, dtype=np.int32), np.arange(1, n, dtype=np.int32)
+    w = np.full(n - 1, int(ONE * keep), np.uint32)
+    g, og = hs.hsaw_graph_from_edges(n, src, dst, w), oracle.Graph(n, src, dst, w)
+    sources = np.array([0], np.int32)
+    ost = oracle.Stream(oracle.Query(og, sources, seed=6)).extend(1500)
+    for pool in (False, True):
+        if pool:
+            g.build_walk_pool(seed=6, attempts=1 << 14)
+        assert_same_stream(hs.hsaw_sample(g, hs.Query(sources=sources, seed=6), 0, 1500), ost, 1500)
