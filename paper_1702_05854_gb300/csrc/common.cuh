@@ -229,6 +229,12 @@ hsaw_status exclusive_scan_u64(uint64_t* d, size_t n, uint64_t* total, cudaStrea
 // result ends in (keys, vals) or (keys_alt, vals_alt); *in_alt tells which.
 hsaw_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, uint32_t* vals_alt, size_t n,
                              int bits, cudaStream_t s, bool* in_alt);
+// The edge list (src, dst, w) sorted by dst, stable: edge = {src, w} and index = input position in
+// sorted order; *sorted_dst is keys or keys_alt.  A node at or above `nodes` (2 at least) sets bit
+// 0 of *err.  keys, keys_alt, vals, vals_alt, pay: room for m each; m >= 1.
+hsaw_status radix_sort_edges(const int32_t* src, const int32_t* dst, const uint32_t* w, size_t m, uint32_t nodes,
+                             uint32_t* keys, uint32_t* keys_alt, uint32_t* vals, uint32_t* vals_alt, uint2* pay,
+                             uint2* edge, int64_t* index, uint32_t** sorted_dst, uint32_t* err, cudaStream_t s);
 int bit_width(uint64_t x);  // bits needed for values in [0, x]
 
 // ------------------------------------------------------------------ launch helpers

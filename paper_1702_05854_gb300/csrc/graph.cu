@@ -545,6 +545,24 @@ static hsaw_status from_edges(int64_t n, int64_t m, const int32_t* src, const in
   uint32_t* d_err = nullptr;
   HSAW_TRY(T.get(&d_err, 2));
   HSAW_CK(cudaMemsetAsync(d_err, 0, 2 * sizeof(uint32_t), s));
+  uint32_t *keys, *vals, *keys2, *vals2, *row_start;
+  HSAW_TRY(T.get(&row_start, n + 1));
+  if (!overlap && m > 0 && n > 1) {  // the whole list is here: tails and weights ride along
+    HSAW_TRY(alloc_graph(g, n, m, true));
+    uint2* pay = nullptr;
+    uint32_t* sorted = nullptr;
+    HSAW_TRY(T.get(&keys, m));
+    HSAW_TRY(T.get(&vals, m));
+    HSAW_TRY(T.get(&keys2, m));
+    HSAW_TRY(T.get(&vals2, m));
+    HSAW_TRY(T.get(&pay, m));
+    HSAW_TRY(radix_sort_edges(d_src, d_dst, d_w, (size_t)m, (uint32_t)n, keys, keys2, vals, vals2, pay, g.edge,
+                              g.input_index, &sorted, d_err, s));
+    count_launch();
+    k_row_from_sorted<<<grid_for(n + 1, 256, 8192), 256, 0, s>>>(sorted, m, n, row_start);
+    HSAW_CK(cudaGetLastError());
+    return finish_graph(g, row_start, d_err, T, s);
+  }
   if (m) {
     count_launch();
     k_validate_nodes<<<grid_for(m, 256, 8192), 256, 0, s>>>(d_dst, m, n, d_err);
@@ -555,12 +573,10 @@ static hsaw_status from_edges(int64_t n, int64_t m, const int32_t* src, const in
     HSAW_CK(cudaGetLastError());
     HSAW_TRY(check_err(d_err, s));
   }
-  uint32_t *keys, *vals, *keys2, *vals2, *row_start;
   HSAW_TRY(T.get(&keys, m));
   HSAW_TRY(T.get(&vals, m));
   HSAW_TRY(T.get(&keys2, m));
   HSAW_TRY(T.get(&vals2, m));
-  HSAW_TRY(T.get(&row_start, n + 1));
   if (m) {
     count_launch();
     k_iota_dst<<<grid_for(m, 256, 8192), 256, 0, s>>>(d_dst, m, keys, vals);
