@@ -714,7 +714,8 @@ hsaw_status stream_extend(const Graph& g, const QueryDev& qd, Stream& st, int64_
     if (used >= st.max_attempts) return fail(HSAW_E_TIMEOUT, "sampling: attempt budget exhausted before enough hits");
     // window size from the hit rate so far (2^20 .. 2^28 attempts; doubling while no hit; down
     // to 2^16 where the walks of a window past the last hit asked for are of no use to the
-    // caller, the first then by the rate that start nodes alone give),
+    // caller, the first then by 16 times the rate that start nodes alone give: most walks see
+    // more nodes than that, and one that falls short costs a launch),
     // with a margin of 4 standard deviations of the rate estimate (st.count hits seen) and
     // of the window's own hit count (need): attempts past the last hit a solve uses are
     // wasted, and a window that falls short only costs one more launch
@@ -724,7 +725,7 @@ hsaw_status stream_extend(const Graph& g, const QueryDev& qd, Stream& st, int64_
     const double least = st.least_window;
     double target = st.hit_rate > 0 ? need / st.hit_rate * margin + 4096.0
                     : used          ? std::max(1048576.0, 2.0 * (double)used)
-                                    : std::min(1048576.0, need / std::max(qd.start_rate, 1e-12));
+                                    : std::min(1048576.0, need / 16.0 / std::max(qd.start_rate, 1e-12));
     target = std::max(target, least);
     target = std::min(target, 268435456.0);
     uint64_t batch = (uint64_t)target;
