@@ -77,12 +77,13 @@ static hsaw_status validate_common(const Graph& g, const hsaw_query* q, int64_t*
 }
 
 struct SolveScratch {
+  Slab slab;  // outlives the buffers below
   QueryDev qd;
   Stream st;
   Cover cv;
   uint8_t* cand = nullptr;
   cudaStream_t s;
-  explicit SolveScratch(cudaStream_t st_) : s(st_) {}
+  explicit SolveScratch(cudaStream_t st_) : slab(st_), s(st_) {}
   ~SolveScratch() {
     cudaStreamSynchronize(s);
     query_release(qd, s);
@@ -418,6 +419,7 @@ hsaw_status hsaw_greedy(hsaw_walks w, hsaw_graph g, hsaw_mode mode, int64_t firs
   }
   if (k < 1 || k > c) return fail(HSAW_E_INVALID, "greedy: need 1 <= k <= |C|");
   cudaStream_t s = (cudaStream_t)stream;
+  Slab slab(s);
   Cover cv;
   uint8_t* cand = nullptr;
   hsaw_status st = upload_mask(candidate_mask, (size_t)M, false, s, &cand);

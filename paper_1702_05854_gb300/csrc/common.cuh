@@ -34,6 +34,27 @@ hsaw_status cuda_fail(cudaError_t e, const char* what, const char* file, int lin
 hsaw_status dmalloc(void** p, size_t bytes, cudaStream_t s);
 void dfree(void* p, cudaStream_t s);
 
+// One allocation that a call's small buffers are cut from: while it lives, dmalloc on its thread
+// and stream takes what fits from it and dfree leaves that alone.  A small solve makes about 30
+// allocations and as many frees, each a microsecond or two and a lock that solves on other
+// threads want too.  Buffers cut from it must be gone before it is.
+class Slab {
+ public:
+  explicit Slab(cudaStream_t s);
+  ~Slab();
+  Slab(const Slab&) = delete;
+  Slab& operator=(const Slab&) = delete;
+  void* cut(size_t bytes, cudaStream_t s);
+  bool holds(const void* p) const { return p >= base_ && p < base_ + cap_; }
+
+ private:
+  static constexpr size_t BYTES = 32ull << 20;
+  cudaStream_t s_;
+  char* base_ = nullptr;
+  size_t cap_ = 0, used_ = 0;
+  Slab* outer_;
+};
+
 template <typename T>
 struct DBuf {  // grow-only device buffer
   T* p = nullptr;

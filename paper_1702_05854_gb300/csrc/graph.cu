@@ -44,6 +44,34 @@ static std::vector<std::unique_ptr<ScratchAllocator>> g_alloc_all;  // every one
 static std::atomic<const ScratchAllocator*> g_alloc{nullptr};
 static std::atomic<long long> g_held{0};                   // scratch blocks handed out, not yet released
 
+static thread_local Slab* t_slab = nullptr;
+
+Slab::Slab(cudaStream_t s) : s_(s), outer_(t_slab) {
+  void* p = nullptr;
+  t_slab = nullptr;  // its own block comes from the allocator
+  if (dmalloc(&p, BYTES, s) == HSAW_OK) {
+    base_ = static_cast<char*>(p);
+    cap_ = BYTES;
+  } else {
+    set_error("");  // small buffers are then allocated one by one
+  }
+  t_slab = this;
+}
+
+Slab::~Slab() {
+  t_slab = nullptr;
+  dfree(base_, s_);
+  t_slab = outer_;
+}
+
+void* Slab::cut(size_t bytes, cudaStream_t s) {
+  bytes = (bytes + 255) & ~(size_t)255;
+  if (s != s_ || bytes > cap_ - used_) return nullptr;
+  void* p = base_ + used_;
+  used_ += bytes;
+  return p;
+}
+
 hsaw_status dmalloc(void** p, size_t bytes, cudaStream_t s) {
   if (g_fail_countdown.load(std::memory_order_relaxed) > 0 && g_fail_countdown.fetch_sub(1) == 1) {
     *p = nullptr;
@@ -51,6 +79,7 @@ hsaw_status dmalloc(void** p, size_t bytes, cudaStream_t s) {
     return HSAW_E_NOMEM;
   }
   if (bytes == 0) bytes = 16;
+  if (t_slab && (*p = t_slab->cut(bytes, s))) return HSAW_OK;
   if (const ScratchAllocator* a = g_alloc.load(std::memory_order_acquire)) {
     *p = a->alloc(bytes, (void*)s, a->ctx);
     if (!*p) {
@@ -84,7 +113,7 @@ hsaw_status dmalloc(void** p, size_t bytes, cudaStream_t s) {
   return HSAW_OK;
 }
 void dfree(void* p, cudaStream_t s) {
-  if (!p) return;
+  if (!p || (t_slab && t_slab->holds(p))) return;
   if (const ScratchAllocator* a = g_alloc.load(std::memory_order_acquire))
     a->release(p, (void*)s, a->ctx);
   else
