@@ -145,9 +145,6 @@ struct Graph {
   int device = 0;
 };
 
-// Sampler occupancy autotuner state of a graph (sample.cu): forget it when the graph goes.
-void sample_tune_forget(const Graph& g);
-
 // ------------------------------------------------------------------ Philox4x32-10
 // Salmon, Moraes, Dror, Shaw, SC'11: 10 rounds of two 32x32->64 multiplies with the
 // published multipliers, key bumped by the published Weyl constants between rounds.

@@ -17,7 +17,6 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
-#include <unordered_map>
 #include <vector>
 
 #include "solver.cuh"
@@ -533,60 +532,16 @@ static int sample_blocks_per_sm() {
   return cached;
 }
 
-// Sampler occupancy autotuner.  A walk makes one dependent record read per draw; with the
-// records in DRAM the random-read rate of this GPU peaks at 1-2 blocks of 256 per SM and
-// falls a little as more requests queue, while graphs whose records sit in L2 are bound by
-// issue and want every warp.  So each graph's first two sampler launches of at least 2^23
-// attempts run with 6 and 3 blocks per SM (draws per ms by CUDA events on the launching
-// stream), and its later launches use 3 if it was faster by more than 3%, else 6.  (Trials
-// at 4 and 2 blocks per SM gained nothing on the billion-edge graph and cost up to 47% of a
-// launch on L2-resident ones.)  The grid does not change any result: hits are ordered by
-// attempt id.  HSAW_SAMPLE_BLOCKS=b in the environment forces b blocks per SM (measurement).
-namespace {
-constexpr int kTuneN = 2;
-constexpr int kTuneCands[kTuneN] = {6, 3};
-struct SampleTune {
-  int next_trial = 0, done = 0, best = 0;
-  float rate[kTuneN] = {0.f, 0.f};
-};
-std::mutex g_stune_mu;
-std::unordered_map<const void*, SampleTune> g_stune;  // keyed by the graph's node array
-}  // namespace
-
-void sample_tune_forget(const Graph& g) {
-  std::lock_guard<std::mutex> lk(g_stune_mu);
-  g_stune.erase(g.node);
-}
-
-// Blocks per SM for the next launch over `batch` attempts; *trial >= 0 when it is a timed trial.
-static int sample_blocks_for(const Graph& g, uint64_t batch, int* trial) {
-  *trial = -1;
+// Blocks per SM: all that fit, 6.  G draws/s with 4 and 6 blocks, R-MAT: equal weights at scale
+// 17 to 23: 173/185, 153/173, 111/112, 101/100, 67/65, 49/48, 39/40; random weights at 16 to 22:
+// 71/84, 71/83, 47/59, 37/40, 34/37.  (With two loads a record, 3 blocks were the faster on
+// graphs far beyond L2; one load does not need that.)  HSAW_SAMPLE_BLOCKS=b in the environment
+// asks for b (measurement).
+static int sample_blocks() {
   const int full = sample_blocks_per_sm();
-  if (const char* f = getenv("HSAW_SAMPLE_BLOCKS")) {
-    const int b = atoi(f);
-    return std::max(1, std::min(full, b > 0 ? b : full));
-  }
-  std::lock_guard<std::mutex> lk(g_stune_mu);
-  SampleTune& t = g_stune[g.node];
-  if (t.best) return std::min(full, t.best);
-  if (batch < (1ull << 23) || t.next_trial >= kTuneN) return full;
-  *trial = t.next_trial++;
-  return std::min(full, kTuneCands[*trial]);
-}
-
-static void sample_tune_record(const Graph& g, int trial, double draws, float ms) {
-  if (trial < 0 || !(ms > 0.f)) return;
-  std::lock_guard<std::mutex> lk(g_stune_mu);
-  SampleTune& t = g_stune[g.node];
-  t.rate[trial] = (float)(draws / ms);
-  if (++t.done < kTuneN) return;
-  int best = 0;
-  for (int i = 1; i < kTuneN; ++i)
-    if (t.rate[i] > t.rate[best] * 1.03f) best = i;
-  t.best = kTuneCands[best];
-  if (getenv("HSAW_LOG_LAUNCHES"))
-    fprintf(stderr, "hsaw: k_sample tuned blocks_per_sm=%d (G draws/s: 6 %.1f, 3 %.1f)\n", t.best, t.rate[0] / 1e6,
-            t.rate[1] / 1e6);
+  const char* f = getenv("HSAW_SAMPLE_BLOCKS");
+  const int b = f ? atoi(f) : 0;
+  return b > 0 ? std::min(full, b) : full;
 }
 
 template <Layout L>
@@ -645,19 +600,11 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
     P.chunk_hits = ctl + SC_WORDS;
     P.recs = st.recs.p;
     P.kept = st.ids_only ? nullptr : st.chunk_kept.p;
-    int trial = -1;
-    const int bps = sample_blocks_for(g, batch, &trial);
+    const int bps = sample_blocks();
     const unsigned grid = (unsigned)std::max(1, std::min<int>(sm_count() * bps, (int)((n_chunks + 7) / 8)));
-    cudaEvent_t tev[2] = {nullptr, nullptr};
-    if (trial >= 0 && (cudaEventCreate(&tev[0]) != cudaSuccess || cudaEventCreate(&tev[1]) != cudaSuccess)) {
-      cudaGetLastError();
-      trial = -1;
-    }
-    if (trial >= 0) cudaEventRecord(tev[0], s);
     void* prof = profile_begin(s);
     launch_sample(g, P, grid, s);
     profile_end(prof, s, batch);
-    if (trial >= 0) cudaEventRecord(tev[1], s);
     HSAW_CK(cudaGetLastError());
     // the counts' offsets in place (a chunk with more hits than records makes the launch run
     // again, whatever they say)
@@ -668,12 +615,6 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
     unsigned long long hs = 0, hn = 0;
     std::memcpy(&hs, h + SC_STEPS, 8);
     std::memcpy(&hn, h + SC_NODES, 8);
-    if (trial >= 0) {
-      float ms = 0.f;
-      if (cudaEventElapsedTime(&ms, tev[0], tev[1]) == cudaSuccess) sample_tune_record(g, trial, (double)hs, ms);
-      cudaEventDestroy(tev[0]);
-      cudaEventDestroy(tev[1]);
-    }
     if (h[SC_STATUS] & ST_STEP_CAP) return fail(HSAW_E_STEP_CAP, "sampling: a walk exceeded its step guard");
     if ((h[SC_STATUS] & ST_OVERFLOW) && cap < chunk) {
       cap = chunk;  // rare: rerun this launch with room for every attempt to hit
