@@ -16,8 +16,8 @@
 //
 // The greedy with one pick per barrier (cover.cu) is bound by latency, 3.4-8 us a pick.  Per
 // greedy against it: k = 1000 edges, 150 K R-MAT 22 walks, 5.1 -> 0.25 ms; k = 300 edges,
-// 7 K-222 K R-MAT 18 walks, 1.1-2.0 -> 0.11-0.18 ms; k = 100 nodes of 8 K with random coins,
-// 5.3 K walks, 0.59 -> 0.35 ms (33 rounds).  Taking one gain level a round instead (the picks of
+// 7 K-222 K R-MAT 18 walks, 1.1-2.0 -> 0.10-0.14 ms; k = 100 nodes of 8 K with random coins,
+// 5.3 K walks, 0.59 -> 0.30 ms (33 rounds).  Taking one gain level a round instead (the picks of
 // a level are an independent set) needed 9-104 rounds there and measured 0.15-1.1 ms.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
+#include <utility>
 
 #include "solver.cuh"
 
@@ -40,7 +41,7 @@ constexpr uint32_t SORT_MAX = 4096;    // picks ranked against each other from s
 // ctl words of a run; the list's length (high half) and its pairs (low half) grow together in
 // one 64-bit word
 enum { PC_PICKS = 0, PC_FLOOR = 1, PC_GAIN = 2, PC_ROUNDS = 3, PC_STUCK = 4, PC_TOTAL = 5, PC_LIST = 6 /* 64 bits */,
-       PC_WORDS = 16 };
+       PC_OWNED = 8 /* counts were not taken down */, PC_WORDS = 16 };
 
 // A walk of a listed element: {walk, element, index in the list, 1 for the element's first}.
 using Pair = uint4;
@@ -91,11 +92,62 @@ __device__ __forceinline__ void take_down(const PeakParams& P, const uint32_t* _
   }
 }
 
+// A CTA's own part of the list: whole elements, their pairs in registers, their counts in shared
+// memory.
+constexpr int OWN_PAIRS = 16;            // pairs a thread
+constexpr uint32_t OWN_ELEMENTS = 3072;  // elements a CTA (16 bits each in registers)
+
+struct OwnPart {
+  uint32_t count[OWN_ELEMENTS];   // uncovered walks of the element
+  uint32_t id[OWN_ELEMENTS];
+  uint32_t failed[OWN_ELEMENTS];  // the last round in which it was no peak
+  uint32_t first[2];              // the CTA's first pair, and the next CTA's
+  uint32_t none[16];              // per CTA: 1 if its part has no room
+};
+
+// This CTA's part, [first[0], first[1]): an even share of the pairs, moved up to where an element
+// begins.  True if each CTA of the cluster has room for its own.
+__device__ __forceinline__ bool own_part(const PeakParams& P, uint32_t n, OwnPart& O, cg::cluster_group& cluster) {
+  constexpr uint32_t NONE = 0xffffffffu;
+  const uint32_t rank = cluster.block_rank(), C = cluster.num_blocks();
+  const uint32_t from[2] = {(uint32_t)((uint64_t)n * rank / C), (uint32_t)((uint64_t)n * (rank + 1) / C)};
+  cg::cluster_group::arrival_token started = cluster.barrier_arrive();
+  if (threadIdx.x < 2) O.first[threadIdx.x] = NONE;
+  __syncthreads();
+  for (uint32_t j = 0; j < OWN_PAIRS; ++j) {  // an element longer than that has no room in a CTA
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const uint32_t i = from[q] + j * blockDim.x + threadIdx.x;
+      if (i >= n) atomicMin(&O.first[q], n);
+      else if (__ldg(&P.pairs[i].w)) atomicMin(&O.first[q], i);
+    }
+    __syncthreads();
+    const bool found = O.first[0] != NONE && O.first[1] != NONE;
+    __syncthreads();
+    if (found) break;
+  }
+  const uint32_t b = O.first[0], e = O.first[1];
+  bool room = b != NONE && e != NONE && e - b <= OWN_PAIRS * blockDim.x;
+  if (room && e > b) room = __ldg(&P.pairs[e - 1].z) - __ldg(&P.pairs[b].z) < OWN_ELEMENTS;
+  cluster.barrier_wait(std::move(started));  // the peers run: their shared memory can be written
+  if (threadIdx.x < C) *cluster.map_shared_rank(&O.none[rank], threadIdx.x) = room ? 0u : 1u;
+  cluster.sync();
+  return !__any_sync(0xffffffffu, (threadIdx.x & 31) < C && O.none[threadIdx.x & 31]);
+}
+
 }  // namespace
 
-// One cluster, a thread per (element, walk) pair of the list; counts, stamps and
-// keys in global memory (L2).  Bound by latency: three barriers a round, two or three
-// dependent L2 reads before each.
+// One cluster, a thread per (element, walk) pair of the list; stamps and keys in global memory
+// (L2).  Bound by latency: the barriers of a round and the dependent L2 reads before each.
+//
+// Where whole elements of the list fit the CTAs (OwnPart: 2^18 pairs on 16 CTAs, less what the
+// division at elements costs), an element's walks are looked at by one CTA alone: its count is
+// that of its pairs whose walk has no stamp, so no pick takes counts down walk entry by walk
+// entry (k_take_down does that for all of a phase's walks if another phase follows), and whether
+// it is a peak is settled within the CTA, which leaves two cluster barriers a round of three.
+// Against counts in global memory: the greedy of 5.3 K node walks and k = 100 (33 rounds) 360 -> 295 us,
+// of 7-222 K edge walks and k = 300 110-220 -> 95-139 us.
+// Longer lists, or an element in more walks than a CTA has room for, keep counts in global memory.
 __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant__ PeakParams P) {
   __shared__ uint32_t s_red[32];
   __shared__ uint32_t slot[2][16];  // by round parity, per CTA: its largest count
@@ -110,6 +162,38 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
   const uint32_t* __restrict__ entry = P.entry + (P.from ? *P.from - P.from_sub : 0);
   const uint32_t stripe = (n + 31) / 32;
   const uint32_t floor_gain = __ldcg(&P.ctl[PC_FLOOR]);
+  __shared__ OwnPart O;
+  const bool owned = own_part(P, n, O, cluster);
+  uint32_t walk[OWN_PAIRS], el2[OWN_PAIRS / 2] = {}, alive = 0;  // this thread's pairs; elements in 16 bits
+  auto el = [&](int j) { return el2[j / 2] >> 16 * (j & 1) & 0xFFFFu; };
+  const uint32_t own_first = owned ? O.first[0] : 0u, own_n = owned ? O.first[1] - own_first : 0u;
+  const uint32_t el_first = own_n ? __ldg(&P.pairs[own_first].z) : 0u;
+  const uint32_t own_elements = own_n ? __ldg(&P.pairs[own_first + own_n - 1].z) - el_first + 1 : 0u;
+  if (owned) {
+    for (uint32_t e = threadIdx.x; e < own_elements; e += blockDim.x) O.count[e] = O.failed[e] = 0u;
+#pragma unroll
+    for (int j = 0; j < OWN_PAIRS; ++j) {
+      const uint32_t i = j * blockDim.x + threadIdx.x;
+      walk[j] = 0u;
+      if (i < own_n) {
+        const Pair x = __ldg(&P.pairs[own_first + i]);
+        walk[j] = x.x;
+        const uint32_t e = x.z - el_first;
+        el2[j / 2] |= e << 16 * (j & 1);
+        alive |= 1u << j;
+        if (x.w) O.id[e] = x.y;
+      }
+    }
+    __syncthreads();
+    // walks that earlier phases cover are no longer counted
+#pragma unroll
+    for (int j = 0; j < OWN_PAIRS; ++j) {
+      if (!(alive >> j & 1u)) continue;
+      if (__ldcg(&P.stamp[walk[j]])) alive &= ~(1u << j);
+      else atomicAdd(&O.count[el(j)], 1u);
+    }
+    __syncthreads();
+  }
   uint32_t picks = 0, g = 0, r = P.round0;
   bool stuck = false;
   for (;;) {
@@ -119,8 +203,29 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
     // count
     unsigned long long* const top = P.top[r & 1];
     uint32_t m = 0;
+    if (owned) {
+      if (r > P.round0 + 1) {  // the last round's walks leave the counts
+        uint32_t gone = 0;
+#pragma unroll
+        for (int j = 0; j < OWN_PAIRS; ++j)
+          if (alive >> j & 1u) gone |= (__ldcg(&P.stamp[walk[j]]) ? 1u : 0u) << j;
+#pragma unroll
+        for (int j = 0; j < OWN_PAIRS; ++j)
+          if (gone >> j & 1u) atomicSub(&O.count[el(j)], 1u);
+        alive &= ~gone;
+        __syncthreads();
+      }
+#pragma unroll
+      for (int j = 0; j < OWN_PAIRS; ++j) {
+        if (!(alive >> j & 1u)) continue;
+        const uint32_t c = O.count[el(j)];
+        if (c < floor_gain) continue;
+        m = max(m, c);
+        atomicMax(&top[walk[j]], peak_key(c, O.id[el(j)]));
+      }
+    }
 #pragma unroll 4
-    for (uint32_t i = gtid; i < n; i += threads) {
+    for (uint32_t i = owned ? n : gtid; i < n; i += threads) {
       const Pair x = __ldg(&P.pairs[i]);
       const uint32_t c = __ldcg(&P.cnt[x.y]), st = __ldcg(&P.stamp[x.x]);
       if (c >= floor_gain) {
@@ -156,6 +261,35 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
     // other parity's words are cleared for the next round on the way: a walk that no element
     // at or above the floor reaches any more is not looked at again.
     unsigned long long* const other = P.top[(r + 1) & 1];
+    if (owned) {
+      unsigned long long t[4];
+#pragma unroll
+      for (int j0 = 0; j0 < OWN_PAIRS; j0 += 4) {
+#pragma unroll
+        for (int j = j0; j < j0 + 4; ++j) t[j - j0] = alive >> j & 1u ? __ldcg(&top[walk[j]]) : 0ull;
+#pragma unroll
+        for (int j = j0; j < j0 + 4; ++j) {
+          const uint32_t c = alive >> j & 1u ? O.count[el(j)] : 0u;
+          if (c < floor_gain) continue;
+          if (t[j - j0] != peak_key(c, O.id[el(j)])) O.failed[el(j)] = r;
+          other[walk[j]] = 0ull;
+        }
+      }
+      __syncthreads();
+      // 3. peaks are picks, their walks are stamped
+      for (uint32_t e = threadIdx.x; e < own_elements; e += blockDim.x) {
+        const uint32_t c = O.count[e];
+        if (c < floor_gain || O.failed[e] == r) continue;
+        const uint32_t pos = atomicAdd(&P.ctl[PC_PICKS], 1u);
+        P.out_u[pos] = O.id[e];
+        P.out_gain[pos] = c;
+      }
+#pragma unroll
+      for (int j = 0; j < OWN_PAIRS; ++j)
+        if ((alive >> j & 1u) && O.count[el(j)] >= floor_gain && O.failed[el(j)] != r) P.stamp[walk[j]] = r;
+      cluster.sync();
+      continue;
+    }
 #pragma unroll 4
     for (uint32_t i = gtid; i < n; i += threads) {
       const Pair x = __ldg(&P.pairs[i]);
@@ -200,6 +334,21 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
     P.ctl[PC_GAIN] = g;
     P.ctl[PC_ROUNDS] = r;
     P.ctl[PC_STUCK] = stuck ? 1u : 0u;
+    P.ctl[PC_OWNED] = owned ? 1u : 0u;
+  }
+}
+
+// Counts without the walks stamped after round `round0`: a warp looks at 32 stamps and reads those
+// walks' entries one walk at a time.
+__global__ void __launch_bounds__(256) k_take_down(const __grid_constant__ PeakParams P, uint32_t walks, uint32_t round0) {
+  const uint32_t* __restrict__ entry = P.entry + (P.from ? *P.from - P.from_sub : 0);
+  const int lane = threadIdx.x & 31;
+  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+  for (uint32_t j0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; (uint64_t)j0 * 32 < walks; j0 += warps) {
+    const uint32_t j = j0 * 32 + lane;
+    const bool mine = j < walks && P.stamp[j] > round0;
+    const uint2 range = mine ? make_uint2(__ldg(&P.walk_eoff[j]), __ldg(&P.walk_eoff[j + 1])) : make_uint2(0u, 0u);
+    take_down(P, entry, __ballot_sync(0xffffffffu, mine), range, lane);
   }
 }
 
@@ -536,10 +685,18 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     cudaEventRecord(ev[0], s);
   }
   uint32_t h[PC_WORDS] = {0}, phases = 0, unique = 0;
+  PeakParams P = {};
   bool again = false;  // the phase did not fit its list or pairs
   do {
     if (!again) {
-      if (phases++) HSAW_CK(cudaMemsetAsync(hist, 0, COUNT_BINS * 4, s));  // the candidates below the last floor
+      if (phases++) {  // the candidates below the last floor
+        HSAW_CK(cudaMemsetAsync(hist, 0, COUNT_BINS * 4, s));
+        if (h[PC_OWNED]) {
+          count_launch();
+          k_take_down<<<grid_for(W, 256, 8 * sm_count()), 256, 0, s>>>(P, W, P.round0);
+          HSAW_CK(cudaGetLastError());
+        }
+      }
       count_launch();
       k_peak_hist<<<grid_for((U + 3) / 4, 512, 4 * sm_count()), 512, 0, s>>>(cnt, uid, cand, U, hist);
       HSAW_CK(cudaGetLastError());
@@ -555,7 +712,6 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
         hist, (uint32_t)k, cnt, uid, cand, by_id ? nullptr : cv.inv_off.p, U, list_cap, cv.peak_list.p, cv.g_list.p,
         cv.g_rng.p, by_id ? cv.vals.p : nullptr, ctl);
     HSAW_CK(cudaGetLastError());
-    PeakParams P;
     P.pairs = cv.inv_ent.p;
     P.failed = cv.g_list.p;
     P.seen = cv.g_rng.p;
@@ -638,8 +794,9 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     cudaEventElapsedTime(&ms, ev[0], ev[1]);
     fprintf(stderr,
             "hsaw: k_greedy_cluster walks=%lld entries=%u unique=%u cluster=%d gshift=0 k=%d picks=%u spread=0 "
-            "rounds=%u phases=%u pairs=%u made=%u by_id=%d ms=%.3f\n",
-            (long long)cv.walks, entries, unique, csize, k, kept, h[PC_ROUNDS], phases, h[PC_LIST], made, by_id ? 1 : 0, ms);
+            "rounds=%u phases=%u pairs=%u made=%u by_id=%d owned=%u ms=%.3f\n",
+            (long long)cv.walks, entries, unique, csize, k, kept, h[PC_ROUNDS], phases, h[PC_LIST], made, by_id ? 1 : 0,
+            h[PC_OWNED], ms);
     cudaEventDestroy(ev[0]);
     cudaEventDestroy(ev[1]);
   }

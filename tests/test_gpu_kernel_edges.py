@@ -214,6 +214,24 @@ def test_greedy_conflict_chains():
                 assert np.array_equal(gains, ogains) and np.array_equal(ids, oids)
 
 
+@pytest.mark.parametrize("count", [16_000, 16_384, 16_385, 20_000, 60_000])
+def test_greedy_elements_of_many_walks(count):
+    """Elements in about as many walks as a thread block keeps to itself (16,384 pairs), or more."""
+    n = 30
+    src, dst = np.arange(n - 1, dtype=np.int32), np.arange(1, n, dtype=np.int32)
+    src, dst = np.concatenate([src, [n + 1]]).astype(np.int32), np.concatenate([dst, [n - 1]]).astype(np.int32)
+    w = np.full(src.size, ONE // 2 - 1, np.uint32)
+    sources = np.array([0, n - 3, n + 1], np.int32)
+    g, og = hs.hsaw_graph_from_edges(n + 2, src, dst, w), oracle.Graph(n + 2, src, dst, w)
+    walks = hs.hsaw_sample(g, hs.Query(sources=sources, seed=3), 0, count)
+    ost = oracle.Stream(oracle.Query(og, sources, seed=3)).extend(count)
+    for mode, M in ((hs.HSAW_EDGE, src.size), (hs.HSAW_NODE, n + 2)):
+        for k in (1, 3, 25):
+            ids, gains = hs.hsaw_greedy(walks, g, mode, 0, count, k)
+            oids, ogains = ost.greedy(mode, 0, count, M, k)
+            assert np.array_equal(gains, ogains) and np.array_equal(ids, oids)
+
+
 @pytest.mark.parametrize("count", [1, 31, 32, 33, 127, 4095, 4097, 116_735, 116_737, 233_471, 233_473, 1 << 18])
 def test_static_chunks(count):
     """The allocation-free sampler's chunks of 32 to 256 attempts, and its blocks of 128 chunks."""
