@@ -180,10 +180,9 @@ __global__ void k_copy_edges(const int32_t* __restrict__ src, const uint32_t* __
 }
 
 // Running in-weight sums (exact, 64-bit carry), the in-sum check (<= 2^32 - 1), equal-weight
-// detection and the node record: one warp per node, and one block per hub (a node of more
-// than HUB_DEGREE in-edges), which the warp pass only lists.  A warp takes a list 32 edges at
-// a time with a scan each, so the longest list alone set the pass's time (R-MAT 22: 3.1 ms,
-// R-MAT 20: 1.3 ms).  err[1] counts the nodes with in-weight whose in-weights differ.
+// detection and the node record: a warp per 32 nodes, and a block per hub (a node of more
+// than HUB_DEGREE in-edges), which the warp pass only lists.  In the warp pass the longest list
+// alone set the pass's time (R-MAT 22: 3.1 ms, R-MAT 20: 1.3 ms).  err[1] counts the nodes with in-weight whose in-weights differ.
 constexpr uint32_t HUB_DEGREE = 1024;
 
 // Hubs of the graph: count, then node ids (at most m / HUB_DEGREE of them).
@@ -192,70 +191,141 @@ struct Hubs {
   uint32_t* node;
 };
 
+__device__ __forceinline__ uint32_t clamp32(uint64_t x) { return x > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)x; }
+
 __device__ __forceinline__ void write_node(uint4* __restrict__ node, int64_t v, uint32_t first, uint32_t deg,
                                            bool uniform, uint32_t w0, uint64_t sum, uint32_t* __restrict__ err) {
-  const uint32_t insum = (uint32_t)(sum > 0xFFFFFFFFull ? 0xFFFFFFFFull : sum);
-  node[v] = make_uint4(first, deg, (uniform && deg) ? w0 : 0u, insum);
+  node[v] = make_uint4(first, deg, (uniform && deg) ? w0 : 0u, clamp32(sum));
   if (sum > 0xFFFFFFFFull) atomicOr(err, ERR_WEIGHT);
-  if (!uniform && insum) atomicAdd(err + 1, 1u);
 }
 
-__global__ void k_thresholds(const uint32_t* __restrict__ row_start, int64_t n, uint2* __restrict__ edge,
-                             uint4* __restrict__ node, Hubs hubs, uint32_t* __restrict__ err) {
+// A warp takes 32 nodes, a lane each for lists of up to SHORT_LIST edges; longer lists are taken
+// 32 edges at a time by the whole warp, the next 32 (of the same node or the next) being read
+// meanwhile.  Where 32 in-weights are equal their sums are multiples, without a scan.  Bound by
+// instructions before (a warp a node, a 64-bit scan for every 32 edges):
+// R-MAT 22, equal weights, 656 -> 324 us; R-MAT 20, random weights, 292 -> 232 us.
+__global__ void __launch_bounds__(256) k_thresholds(const uint32_t* __restrict__ row_start, int64_t n,
+                                                    uint2* __restrict__ edge, uint4* __restrict__ node, Hubs hubs,
+                                                    uint32_t* __restrict__ err) {
+  constexpr uint32_t SHORT_LIST = 8;
+  const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t v = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
-    const uint32_t b = row_start[v], e = row_start[v + 1];
-    const uint32_t deg = e - b;
-    if (deg > HUB_DEGREE) {
-      if (lane == 0) hubs.node[atomicAdd(hubs.count, 1u)] = (uint32_t)v;
-      continue;
-    }
-    uint64_t carry = 0;
+  for (int64_t v0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 32; v0 < n; v0 += warps * 32) {
+    const int64_t v = v0 + lane;
+    const uint32_t b = v < n ? row_start[v] : 0u, e = v < n ? row_start[v + 1] : 0u, deg = e - b;
+    const bool hub = deg > HUB_DEGREE;
+    if (hub) hubs.node[atomicAdd(hubs.count, 1u)] = (uint32_t)v;
+    uint64_t sum = 0;
     uint32_t w0 = 0;
     bool uniform = true;
-    for (uint32_t base = b; base < e; base += 32) {
-      const uint32_t q = base + lane;
-      const uint32_t w = q < e ? edge[q].y : 0u;
-      if (base == b) w0 = __shfl_sync(0xffffffffu, w, 0);
-      if (q < e && w != w0) uniform = false;
-      uint64_t x = w;
+    if (deg && deg <= SHORT_LIST) {
+      uint32_t w[SHORT_LIST];
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        uint64_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
+      for (uint32_t i = 0; i < SHORT_LIST; ++i) w[i] = i < deg ? edge[b + i].y : 0u;
+      w0 = w[0];
+#pragma unroll
+      for (uint32_t i = 0; i < SHORT_LIST; ++i) {
+        if (i >= deg) break;
+        sum += w[i];
+        uniform &= w[i] == w0;
+        edge[b + i].y = clamp32(sum);
       }
-      const uint64_t run = carry + x;
-      if (q < e) edge[q].y = (uint32_t)(run > 0xFFFFFFFFull ? 0xFFFFFFFFull : run);
-      carry += __shfl_sync(0xffffffffu, x, 31);
     }
-    uniform = __all_sync(0xffffffffu, uniform);
-    if (lane == 0) write_node(node, v, b, deg, uniform, w0, carry, err);
+    unsigned left = __ballot_sync(FULL, deg > SHORT_LIST && !hub);
+    int cur = left ? __ffs(left) - 1 : -1;
+    uint32_t first = __shfl_sync(FULL, b, cur & 31), end = __shfl_sync(FULL, e, cur & 31), base = first;
+    uint32_t w = cur >= 0 && base + lane < end ? edge[base + lane].y : 0u;
+    uint64_t carry = 0;
+    uint32_t start_w = 0;
+    bool same = true;  // all of the node's in-weights so far
+    while (cur >= 0) {
+      int next = cur;
+      uint32_t next_first = first, next_end = end, next_base = base + 32;
+      if (next_base >= end) {
+        left &= left - 1;
+        next = left ? __ffs(left) - 1 : -1;
+        next_first = next_base = __shfl_sync(FULL, b, next & 31);
+        next_end = __shfl_sync(FULL, e, next & 31);
+      }
+      const uint32_t next_w = next >= 0 && next_base + lane < next_end ? edge[next_base + lane].y : 0u;
+      if (base == first) {
+        carry = 0;
+        same = true;
+        start_w = __shfl_sync(FULL, w, 0);
+      }
+      const bool in = base + lane < end;
+      uint64_t x, all;
+      if (__all_sync(FULL, !in || w == start_w)) {
+        x = (uint64_t)start_w * (lane + 1);
+        all = (uint64_t)start_w * min(32u, end - base);
+      } else {
+        same = false;
+        x = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint64_t y = __shfl_up_sync(FULL, x, o);
+          if (lane >= o) x += y;
+        }
+        all = __shfl_sync(FULL, x, 31);
+      }
+      if (in) edge[base + lane].y = clamp32(carry + x);
+      carry += all;
+      if (next != cur && lane == cur) {
+        sum = carry;
+        w0 = start_w;
+        uniform = same;
+      }
+      cur = next;
+      first = next_first;
+      end = next_end;
+      base = next_base;
+      w = next_w;
+    }
+    if (v < n && !hub) write_node(node, v, b, deg, uniform, w0, sum, err);
+    const unsigned unequal = __ballot_sync(FULL, !uniform && clamp32(sum));
+    if (lane == 0 && unequal) atomicAdd(err + 1, (uint32_t)__popc(unequal));
   }
 }
 
-__global__ void __launch_bounds__(1024) k_hub_thresholds(const uint32_t* __restrict__ row_start,
+// A block a hub, a tile of 2 K edges at a time, the next tile's in-weights being read while this
+// one's sums are made: many hubs have a tile or two, so four small blocks an SM, not one of 1,024
+// threads (R-MAT 22 358 -> 240 us, R-MAT 20 93 -> 70 us; 301 and 72 us with tiles of 8 K).
+constexpr int HUB_WARPS = 8;
+__global__ void __launch_bounds__(HUB_WARPS * 32, 4) k_hub_thresholds(const uint32_t* __restrict__ row_start,
                                                          uint2* __restrict__ edge, uint4* __restrict__ node, Hubs hubs,
                                                          uint32_t* __restrict__ err) {
-  constexpr uint32_t ITEMS = 4;
-  __shared__ uint64_t sums[32];
+  constexpr uint32_t ITEMS = 8, TILE = ITEMS * HUB_WARPS * 32;
+  __shared__ uint64_t sums[2][HUB_WARPS];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t count = *hubs.count;
   for (uint32_t h = blockIdx.x; h < count; h += gridDim.x) {
     const uint32_t v = hubs.node[h];
     const uint32_t b = row_start[v], e = row_start[v + 1];
     const uint32_t w0 = edge[b].y;
+    uint32_t x[ITEMS];
+#pragma unroll
+    for (uint32_t i = 0; i < ITEMS; ++i) {
+      const uint32_t q = b + threadIdx.x * ITEMS + i;
+      x[i] = q < e ? edge[q].y : 0u;
+    }
     __syncthreads();  // every thread has read edge[b] before it is written
     uint64_t carry = 0;
     bool uniform = true;
-    for (uint32_t base = b; base < e; base += ITEMS * 1024) {
+    uint32_t turn = 0;
+    for (uint32_t base = b; base < e; base += TILE, turn ^= 1) {
       const uint32_t q = base + threadIdx.x * ITEMS;
-      uint64_t run[ITEMS], sum = 0;
+      uint32_t next[ITEMS];
+      uint64_t sum = 0;
 #pragma unroll
       for (uint32_t i = 0; i < ITEMS; ++i) {
-        const uint32_t x = q + i < e ? edge[q + i].y : 0u;
-        if (q + i < e && x != w0) uniform = false;
-        run[i] = sum += x;
+        const uint64_t p = (uint64_t)q + TILE + i;
+        next[i] = p < e ? edge[p].y : 0u;
+      }
+#pragma unroll
+      for (uint32_t i = 0; i < ITEMS; ++i) {
+        if (q + i < e && x[i] != w0) uniform = false;
+        sum += x[i];
       }
       uint64_t inc = sum;
 #pragma unroll
@@ -263,24 +333,29 @@ __global__ void __launch_bounds__(1024) k_hub_thresholds(const uint32_t* __restr
         const uint64_t y = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += y;
       }
-      if (lane == 31) sums[w] = inc;
-      __syncthreads();
-      uint64_t mine = sums[lane];
+      if (lane == 31) sums[turn][w] = inc;
+      __syncthreads();  // the other turn's sums are read before this, and written after the next
+      uint64_t mine = lane < HUB_WARPS ? sums[turn][lane] : 0ull;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
+      for (int o = 1; o < HUB_WARPS; o <<= 1) {
         const uint64_t y = __shfl_up_sync(0xffffffffu, mine, o);
         if (lane >= o) mine += y;
       }
-      const uint64_t before = w ? __shfl_sync(0xffffffffu, mine, w - 1) : 0ull;
-      const uint64_t at = carry + before + inc - sum;
-      carry += __shfl_sync(0xffffffffu, mine, 31);
+      const uint64_t before = __shfl_sync(0xffffffffu, mine, (w + 31) & 31);
+      uint64_t at = carry + (w ? before : 0ull) + inc - sum;
+      carry += __shfl_sync(0xffffffffu, mine, HUB_WARPS - 1);
 #pragma unroll
-      for (uint32_t i = 0; i < ITEMS; ++i)
-        if (q + i < e) edge[q + i].y = (uint32_t)(at + run[i] > 0xFFFFFFFFull ? 0xFFFFFFFFull : at + run[i]);
-      __syncthreads();  // sums is written again by the next tile
+      for (uint32_t i = 0; i < ITEMS; ++i) {
+        at += x[i];
+        if (q + i < e) edge[q + i].y = clamp32(at);
+        x[i] = next[i];
+      }
     }
     uniform = __syncthreads_and(uniform);
-    if (threadIdx.x == 0) write_node(node, v, b, e - b, uniform, w0, carry, err);
+    if (threadIdx.x == 0) {
+      write_node(node, v, b, e - b, uniform, w0, carry, err);
+      if (!uniform && clamp32(carry)) atomicAdd(err + 1, 1u);
+    }
   }
 }
 
@@ -501,12 +576,12 @@ static hsaw_status finish_graph(Graph& g, uint32_t* row_start, uint32_t* d_err, 
   hubs.node = hubs.count + 1;
   HSAW_CK(cudaMemsetAsync(hubs.count, 0, sizeof(uint32_t), s));
   count_launch();
-  k_thresholds<<<grid_for((size_t)n * 32, 256, 1u << 20), 256, 0, s>>>(row_start, n, g.edge, g.node, hubs, d_err);
+  k_thresholds<<<grid_for((size_t)n, 256, 1u << 20), 256, 0, s>>>(row_start, n, g.edge, g.node, hubs, d_err);
   HSAW_CK(cudaGetLastError());
   if (g.m > HUB_DEGREE) {
     count_launch();
-    k_hub_thresholds<<<grid_for((size_t)(g.m / HUB_DEGREE), 1, 2 * sm_count()), 1024, 0, s>>>(row_start, g.edge, g.node,
-                                                                                             hubs, d_err);
+    k_hub_thresholds<<<grid_for((size_t)(g.m / HUB_DEGREE), 1, 4 * sm_count()), HUB_WARPS * 32, 0, s>>>(
+        row_start, g.edge, g.node, hubs, d_err);
     HSAW_CK(cudaGetLastError());
   }
   uint32_t unequal = 0;

@@ -89,6 +89,37 @@ def test_hub_lists(deg, kind):
         assert_same_stream(hs.hsaw_sample(graph, hs.Query(sources=sources, seed=9), 0, 300), ost, 300)
 
 
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 1000])
+def test_running_sums_of_neighbours(n):
+    """In-lists of every kind side by side in one warp's 32 nodes: none, up to 8 edges, up to and beyond 32 at a time,
+    and hubs around their tiles of 2,048; equal weights, equal but one, weights of 0, and all different."""
+    rng = np.random.default_rng(n)
+    degs = [0, 1, 2, 7, 8, 9, 31, 32, 33, 63, 64, 65, 96, 1023, 1024, 1025]
+    big = iter([2047, 2048, 2049, 4096, 4097, 8193])
+    dst, w = [], []
+    for v in range(n):
+        deg = next(big, 0) if v % 13 == 12 else int(rng.choice(degs))
+        x = np.full(deg, 1.0)
+        kind = rng.integers(4)
+        if kind == 1 and deg:
+            x[rng.integers(deg)] = 2.0
+        elif kind == 2:
+            x[rng.random(deg) < 0.5] = 0.0
+        elif kind == 3:
+            x = rng.random(deg)
+        dst.append(np.full(deg, v, np.int32))
+        w.append(np.floor(x / max(1.0, x.sum()) * ONE * (1.0 - 2.0 ** -20)).astype(np.uint32))
+    dst, w = np.concatenate(dst), np.concatenate(w)
+    order = rng.permutation(dst.size)
+    dst, w = dst[order], w[order]
+    src = rng.integers(0, n, dst.size).astype(np.int32)
+    og = oracle.Graph(n, src, dst, w)
+    rp, s, _, _, index = og.arrays()
+    for g in (hs.hsaw_graph_from_edges(n, src, dst, w), hs.hsaw_graph_from_csr(n, rp, s, w[index])):
+        for x, y in zip(g.export()[:4], og.arrays()[:4]):
+            assert np.array_equal(x, y)
+
+
 def test_small_tables_unequal():
     """Graphs whose records would not fit L2 are walked through edges and a guide of one entry per four in-edges:
     in-lists of every length around the guide's groups, the sector and the hub threshold, with weights from uniform to
