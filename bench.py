@@ -39,8 +39,8 @@ BYTES_PER_STEP = 96  # three random 32-byte sectors per live-edge draw: node rec
 # DRAM bytes (read + write) per live-edge draw of the sampler kernel from an ncu capture,
 # keyed by (hash of the kernel's source, workload).  A workload without a capture of the
 # current kernel reports traffic = null.
-NCU_TRAFFIC = {("783e77c95bea", "rmat22-wc-eSI"): 122.9,   # profiles/k_sample_rmat22_dram.md
-               ("783e77c95bea", "rmat26-wc-eSI"): 122.9}   # the scale-22 figure, scaled by draws
+NCU_TRAFFIC = {("3ac37996ed07", "rmat23-wc-eSI"): 124.5,   # profiles/k_sample_rmat23_dram.md
+               ("3ac37996ed07", "rmat26-wc-eSI"): 124.5}   # the scale-23 figure, scaled by draws
 
 
 def sampler_hash():
@@ -48,7 +48,7 @@ def sampler_hash():
     edge pick, checkpoints in common.cuh)."""
     csrc = os.path.join(ROOT, "paper_1702_05854_gb300", "csrc")
     src = open(os.path.join(csrc, "sample.cu")).read()
-    i = src.index("template <bool HAS_P, bool HAS_REM>\n__global__ void __launch_bounds__(256, 6) k_sample")
+    i = src.index("constexpr int SAMPLE_WARPS")
     j = src.index("\n}\n", i)
     common = open(os.path.join(csrc, "common.cuh")).read()
     a = common.index("// ------------------------------------------------------------------ Philox4x32-10")
