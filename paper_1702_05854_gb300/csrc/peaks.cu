@@ -17,7 +17,7 @@
 // The greedy with one pick per barrier (cover.cu) is bound by latency, 3.4-8 us a pick.  Per
 // greedy against it: k = 1000 edges, 150 K R-MAT 22 walks, 5.1 -> 0.25 ms; k = 300 edges,
 // 7 K-222 K R-MAT 18 walks, 1.1-2.0 -> 0.10-0.14 ms; k = 100 nodes of 8 K with random coins,
-// 5.3 K walks, 0.59 -> 0.30 ms (33 rounds).  Taking one gain level a round instead (the picks of
+// 5.3 K walks, 0.59 -> 0.27 ms (33 rounds).  Taking one gain level a round instead (the picks of
 // a level are an independent set) needed 9-104 rounds there and measured 0.15-1.1 ms.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -145,8 +145,8 @@ __device__ __forceinline__ bool own_part(const PeakParams& P, uint32_t n, OwnPar
 // that of its pairs whose walk has no stamp, so no pick takes counts down walk entry by walk
 // entry (k_take_down does that for all of a phase's walks if another phase follows), and whether
 // it is a peak is settled within the CTA, which leaves two cluster barriers a round of three.
-// Against counts in global memory: the greedy of 5.3 K node walks and k = 100 (33 rounds) 360 -> 295 us,
-// of 7-222 K edge walks and k = 300 110-220 -> 95-139 us.
+// Against counts in global memory, 1,024 threads a CTA: the greedy of 5.3 K node walks and k = 100 (33 rounds)
+// 360 -> 298 us, of 7-222 K edge walks and k = 300 110-220 -> 94-137 us.
 // Longer lists, or an element in more walks than a CTA has room for, keep counts in global memory.
 __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant__ PeakParams P) {
   __shared__ uint32_t s_red[32];
@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
   const uint32_t stripe = (n + 31) / 32;
   const uint32_t floor_gain = __ldcg(&P.ctl[PC_FLOOR]);
   __shared__ OwnPart O;
+  if (threadIdx.x < 32) s_red[threadIdx.x] = 0u;  // a block may have fewer than 32 warps
   const bool owned = own_part(P, n, O, cluster);
   uint32_t walk[OWN_PAIRS], el2[OWN_PAIRS / 2] = {}, alive = 0;  // this thread's pairs; elements in 16 bits
   auto el = [&](int j) { return el2[j / 2] >> 16 * (j & 1) & 0xFFFFu; };
@@ -748,7 +749,11 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(csize);
-    cfg.blockDim = dim3(1024);
+    // Fewer warps meet at a barrier sooner, and have half the loads in flight and half the room
+    // for whole elements: 512 threads against 1,024 on 5.3 K walks 266 against 298 us (stopping
+    // rule query 677 against 730 us), 7-28 K walks of a pool 91-102 against 94-106, 55-222 K walks
+    // 107-143 against 103-137; 32 instances of 20 K walks at once 7.47 against 7.08 ms.
+    cfg.blockDim = dim3(W <= (1u << 14) ? 512 : 1024);
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = 1;
