@@ -24,10 +24,14 @@ namespace hsaw {
 enum : uint32_t { GS_BARRIER_TIMEOUT = 1u };
 
 void Cover::release(cudaStream_t s) {
+  release_index(s);
   keys.release(s); vals.release(s); keys2.release(s); vals2.release(s); run_flag.release(s);
-  uid.release(s); cnt.release(s); inv_off.release(s); inv_walk.release(s); entry_uidx.release(s);
   walk_eoff.release(s); cnt_work.release(s); covered.release(s); dirty.release(s); partial.release(s);
   inv_ent.release(s); peak_list.release(s); g_idx.release(s); g_list.release(s); g_cnt.release(s); g_entry.release(s); g_rng.release(s);
+}
+
+void Cover::release_index(cudaStream_t s) {
+  uid.release(s); cnt.release(s); inv_off.release(s); inv_walk.release(s); entry_uidx.release(s);
 }
 
 // entry offsets of walks [first, first + count) relative to the first walk's first entry
@@ -211,6 +215,7 @@ hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t
       count < 0xFFFFFFFFll &&
       counts_by_id(st.elem_range[em ? 1 : 0], (int64_t)((double)in_stream / (double)st.count * (double)count))) {
     cv.short_walks = in_stream < 16 * st.count;
+    cv.release_index(s);  // a stopping rule's earlier rounds may have counted by sorting
     return count_by_id(st, em, first, count, st.elem_range[em ? 1 : 0], cv, s);
   }
   int64_t nb[2];

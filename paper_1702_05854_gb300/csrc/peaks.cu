@@ -785,7 +785,7 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     HSAW_CK(cudaGetLastError());
     HSAW_TRY(radix_sort_pairs(key, val, key2, val2, made, 32, s, &alt));
     count_launch();
-    k_peak_emit<<<grid_for(kept, 256, 1024), 256, 0, s>>>(alt ? val2 : val, alt ? key2 : key, kept, cv.uid.p, ids, gains);
+    k_peak_emit<<<grid_for(kept, 256, 1024), 256, 0, s>>>(alt ? val2 : val, alt ? key2 : key, kept, uid, ids, gains);
     HSAW_CK(cudaGetLastError());
   }
   if (log) {

@@ -92,6 +92,7 @@ struct Cover {
   const int32_t* el = nullptr;
   const int64_t* from = nullptr;
   int64_t from_sub = 0, elements = 0;
+  void release_index(cudaStream_t s);  // uid, cnt and the inverted index, which counts by id do not make
   void release(cudaStream_t s);
 };
 

@@ -295,3 +295,25 @@ def test_rewalk_segments(n, keep):
         if pool:
             g.build_walk_pool(seed=6, attempts=1 << 14)
         assert_same_stream(hs.hsaw_sample(g, hs.Query(sources=sources, seed=6), 0, 1500), ost, 1500)
+
+
+def test_stopping_rule_counts_by_sort_then_by_id():
+    """A stopping rule on more than 2^24 edges with 5,000 picks: its early rounds sort the walk elements, its last has
+    an eighth as many of them as there are edges and counts by id, and more picks are made than one block orders."""
+    n, k, eps = 1 << 20, 5000, 0.45
+    src, dst = synth.rmat_graph(20, 17)
+    w, sources = synth.wc_weights(n, dst), synth.sources(n, 1000)
+    M = src.size
+    g = hs.hsaw_graph_from_edges(n, src, dst, w)
+    ids, gains, r = hs.hsaw_solve(g, hs.Query(sources=sources, mode=hs.HSAW_EDGE, k=k, sampling=hs.HSAW_STOP_RULE,
+                                              eps=eps, seed=synth.SEED_WALKS))
+    og = oracle.Graph(n, src, dst, w)
+    half = r["hits"] // 2
+    ost = oracle.Stream(oracle.Query(og, sources, seed=synth.SEED_WALKS)).extend_threads(2 * half, threads=8)
+    off = ost.export().node_off
+    elements, before = (int(off[h] - off[0]) - h for h in (half, half // 2))
+    assert M > 1 << 24 and M <= 8 * elements and M > 8 * before  # the two rounds count in different ways
+    oids, ogains = ost.greedy(oracle.MODE_EDGE, 0, half, M, k, kept_gains=True)
+    assert ogains[-1] > 0
+    assert np.array_equal(gains, ogains) and np.array_equal(ids, oids)
+    assert r["cov_Rprime"] == ost.coverage(oracle.MODE_EDGE, half, half, M, oids)
