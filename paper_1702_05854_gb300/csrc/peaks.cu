@@ -685,7 +685,7 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     cudaEventCreate(&ev[1]);
     cudaEventRecord(ev[0], s);
   }
-  uint32_t h[PC_WORDS] = {0}, phases = 0, unique = 0;
+  uint32_t h[PC_WORDS] = {0}, phases = 0, owned_phases = 0, unique = 0;
   PeakParams P = {};
   bool again = false;  // the phase did not fit its list or pairs
   do {
@@ -772,6 +772,8 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     if (again) {
       pair_cap = std::max(pair_cap, h[PC_LIST]);
       list_cap = std::max(list_cap, h[PC_LIST + 1]);
+    } else {
+      owned_phases += h[PC_OWNED];
     }
   } while (again || (h[PC_PICKS] < (uint32_t)k && h[PC_FLOOR] > 1));
   const uint32_t made = h[PC_PICKS], kept = std::min<uint32_t>(made, (uint32_t)k);
@@ -789,8 +791,7 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     HSAW_CK(cudaGetLastError());
   }
   if (log) {
-    // a greedy on one cluster with counts in global memory, like k_greedy_cluster, whose record
-    // this is
+    // the kernel and what is its own, then the fields that the one-pick greedies' records have too
     uint32_t entries = 0;
     cudaMemcpyAsync(&entries, cv.walk_eoff.p + W, 4, cudaMemcpyDeviceToHost, s);
     cudaEventRecord(ev[1], s);
@@ -798,10 +799,10 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     float ms = 0.f;
     cudaEventElapsedTime(&ms, ev[0], ev[1]);
     fprintf(stderr,
-            "hsaw: k_greedy_cluster walks=%lld entries=%u unique=%u cluster=%d gshift=0 k=%d picks=%u spread=0 "
-            "rounds=%u phases=%u pairs=%u made=%u by_id=%d owned=%u ms=%.3f\n",
-            (long long)cv.walks, entries, unique, csize, k, kept, h[PC_ROUNDS], phases, h[PC_LIST], made, by_id ? 1 : 0,
-            h[PC_OWNED], ms);
+            "hsaw: k_greedy_peaks rounds=%u phases=%u owned=%u pairs=%u made=%u by_id=%d ms=%.3f, as k_greedy_cluster "
+            "walks=%lld entries=%u unique=%u cluster=%d gshift=0 k=%d picks=%u spread=0\n",
+            h[PC_ROUNDS], phases, owned_phases, h[PC_LIST], made, by_id ? 1 : 0, ms, (long long)cv.walks, entries, unique,
+            csize, k, kept);
     cudaEventDestroy(ev[0]);
     cudaEventDestroy(ev[1]);
   }

@@ -2,6 +2,8 @@
 
 Everything compared is a whole number, so equality is exact.
 """
+import re
+
 import numpy as np
 import pytest
 
@@ -317,3 +319,27 @@ def test_stopping_rule_counts_by_sort_then_by_id():
     assert ogains[-1] > 0
     assert np.array_equal(gains, ogains) and np.array_equal(ids, oids)
     assert r["cov_Rprime"] == ost.coverage(oracle.MODE_EDGE, half, half, M, oids)
+
+
+def greedy_records(err):
+    """The launch records of the greedy by peaks, as dicts."""
+    return [dict((k, float(v)) for k, v in re.findall(r"(\w+)=([\d.]+)", line))
+            for line in err.splitlines() if line.startswith("hsaw: k_greedy_peaks ")]
+
+
+@pytest.mark.parametrize("count", [300, 20_000])
+def test_greedy_record_names_its_kernel(streams, capfd, monkeypatch, count):
+    """The launch record says which greedy ran: the one by peaks unless the environment asks for another."""
+    d, g, got = streams
+    monkeypatch.setenv("HSAW_LOG_LAUNCHES", "1")
+    for force in (None, "cluster", "grid"):
+        monkeypatch.setenv("HSAW_GREEDY", force) if force else monkeypatch.delenv("HSAW_GREEDY", raising=False)
+        capfd.readouterr()
+        hs.hsaw_greedy(got["many"][0], g, hs.HSAW_EDGE, 0, count, 20)
+        err = capfd.readouterr().err
+        runs = greedy_records(err)
+        assert len(runs) == (0 if force else 1)
+        if runs:
+            assert runs[0]["walks"] == count and runs[0]["picks"] == 20 and runs[0]["owned"] <= runs[0]["phases"]
+        else:
+            assert ("hsaw: k_greedy_cluster " in err) == (force == "cluster")
