@@ -109,7 +109,7 @@ static hsaw_status fixed_tail(const Graph& g, const hsaw_query* q, Stream& st, C
   const int64_t M = q->mode == HSAW_EDGE ? g.m : g.n;
   const int32_t k = q->k;
   void* ph = phase_begin(s);
-  HSAW_TRY(cover_build(st, q->mode, 0, q->n_hsaw, cv, s, true));
+  HSAW_TRY(cover_build(st, q->mode, 0, q->n_hsaw, cv, s, k, !cand));
   phase_end(ph, s, PH_COUNT);
   ph = phase_begin(s);
   uint64_t last = 0;
@@ -195,7 +195,7 @@ static hsaw_status solve(const Graph& g, const hsaw_query* q, hsaw_result* r, cu
       HSAW_TRY(stream_extend(g, W.qd, W.st, 2 * half, s));
       phase_end(ph, s, PH_SAMPLE);
       ph = phase_begin(s);
-      HSAW_TRY(cover_build(W.st, q->mode, 0, half, W.cv, s, true));
+      HSAW_TRY(cover_build(W.st, q->mode, 0, half, W.cv, s, k, !W.cand));
       phase_end(ph, s, PH_COUNT);
       ph = phase_begin(s);
       HSAW_TRY(cover_greedy(W.cv, W.cand, M, k, ids.data(), gains.data(), s));
@@ -423,7 +423,7 @@ hsaw_status hsaw_greedy(hsaw_walks w, hsaw_graph g, hsaw_mode mode, int64_t firs
   Cover cv;
   uint8_t* cand = nullptr;
   hsaw_status st = upload_mask(candidate_mask, (size_t)M, false, s, &cand);
-  if (st == HSAW_OK) st = cover_build(w->st, mode, first, count, cv, s, true);
+  if (st == HSAW_OK) st = cover_build(w->st, mode, first, count, cv, s, k, !cand);
   if (st == HSAW_OK) st = cover_greedy(cv, cand, M, k, ids, gains, s);
   cudaStreamSynchronize(s);
   cv.release(s);

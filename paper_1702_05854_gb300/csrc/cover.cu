@@ -188,7 +188,7 @@ hsaw_status walk_offsets(const Stream& st, bool edges, int64_t first, int64_t co
   return HSAW_OK;
 }
 
-// The environment asks for a greedy that takes one pick at a time, or for a histogram strategy.
+// The environment asks for a greedy that takes one pick at a time.
 static bool one_by_one() {
   return getenv("HSAW_GREEDY") || getenv("HSAW_GREEDY_HEAVY") || getenv("HSAW_GREEDY_OWNED_MAX");
 }
@@ -201,22 +201,37 @@ static bool counts_by_id(int64_t M, int64_t elements) {
   return M > 0 && M < (1ll << 31) && (M <= (1ll << 24) || M <= 8 * elements);
 }
 
+// Streams whose listed elements would be in too many walks for the greedy by peaks (half of peak_pairs,
+// and more than its CTAs hold) even if all elements were in equally many: it would leave them, so it is
+// not begun.  Greedy of 60 K nested walks on 30 nodes, k = 1: 0.85 ms by peaks, 0.26 one pick at a time.
+static bool crowded(int64_t M, int64_t elements, int64_t walks, int32_t k) {
+  const double listed = (double)std::min<uint64_t>((uint64_t)M, peak_list_goal((uint64_t)k));
+  const double pairs = listed * (double)elements / (double)M;
+  return pairs > (double)peak_room(walks) && 2.0 * pairs > (double)peak_pairs(walks, elements, k);
+}
+
 hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t count, Cover& cv, cudaStream_t s,
-                        bool for_greedy) {
+                        int32_t k, bool all) {
   cv.walks = count;
   cv.entries = 0;
   cv.unique = 0;
   cv.by_id = false;
+  cv.crowded = false;
   if (count <= 0) return HSAW_OK;
   if (first < 0 || first + count > st.count) return fail(HSAW_E_INVALID, "cover: walk range outside the stream");
   const bool em = (mode == HSAW_EDGE);
   const int64_t in_stream = em ? st.total_nodes - st.count : st.total_nodes;  // walk elements of the whole stream
-  if (for_greedy && !one_by_one() && !getenv("HSAW_HIST") && peak_cluster() && in_stream < 0xFFFFFFFFll &&
-      count < 0xFFFFFFFFll &&
-      counts_by_id(st.elem_range[em ? 1 : 0], (int64_t)((double)in_stream / (double)st.count * (double)count))) {
+  const int64_t M = st.elem_range[em ? 1 : 0];
+  cv.about = (int64_t)((double)in_stream / (double)st.count * (double)count);
+  cv.crowded = k > 0 && all && M > 0 && crowded(M, cv.about, count, k);
+  if (k > 0 && !cv.crowded && !one_by_one() && !getenv("HSAW_HIST") && peak_cluster() && in_stream < 0xFFFFFFFFll &&
+      count < 0xFFFFFFFFll && counts_by_id(M, cv.about)) {
     cv.short_walks = in_stream < 16 * st.count;
+    cv.stream = &st;
+    cv.mode = mode;
+    cv.first = first;
     cv.release_index(s);  // a stopping rule's earlier rounds may have counted by sorting
-    return count_by_id(st, em, first, count, st.elem_range[em ? 1 : 0], cv, s);
+    return count_by_id(st, em, first, count, M, cv, s);
   }
   int64_t nb[2];
   HSAW_CK(cudaMemcpyAsync(&nb[0], st.node_off.p + first, 8, cudaMemcpyDeviceToHost, s));
@@ -230,7 +245,6 @@ hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t
   HSAW_TRY(walk_offsets(st, em, first, count, cv, s));
   if (E == 0) return HSAW_OK;
   const int32_t* el = em ? st.edges.p + (nb[0] - first) : st.nodes.p + nb[0];
-  const int64_t M = st.elem_range[em ? 1 : 0];
   const bool dense_ok = M > 0 && M <= (1ll << 28) && M <= 64ll * (int64_t)E + (1 << 20);
   int strat = forced_strategy();
   if (strat == HIST_DENSE && !dense_ok) strat = HIST_SORT;
@@ -1151,7 +1165,6 @@ __global__ void k_exclude_picks(const uint32_t* __restrict__ out_u, int32_t r, u
 hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t k, int64_t* ids_host,
                          uint32_t* gains_host, cudaStream_t s, const uint64_t* aid_dev, uint64_t* aid_host) {
   if (k < 1) return fail(HSAW_E_INVALID, "greedy: k < 1");
-  const uint32_t U = (uint32_t)cv.unique;
   DBuf<uint32_t> block, outs;
   HSAW_TRY(block.ensure(PickBlock::copied_words(k) + PickBlock::WORK, s));
   const PickBlock B = PickBlock::at(block.p, k);
@@ -1161,9 +1174,12 @@ hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t 
   int32_t rounds = 0;
   hsaw_status st = HSAW_OK;
   bool done = false;
-  // by peaks, unless the environment asks for a version that takes one pick at a time
-  if ((U > 0 || cv.by_id) && cv.walks > 0 && !one_by_one())
+  // by peaks, unless that is the slower or the environment asks for a version that takes one pick
+  // at a time
+  if ((cv.unique > 0 || cv.by_id) && cv.walks > 0 && !cv.crowded && !one_by_one())
     st = peak_greedy(cv, cand_dev, k, B, host.data(), &rounds, &done, &copied, s);
+  if (st == HSAW_OK && !done && cv.by_id) st = cover_build(*cv.stream, cv.mode, cv.first, cv.walks, cv, s);
+  const uint32_t U = (uint32_t)cv.unique;
   uint32_t* ctl = nullptr;
   if (st == HSAW_OK && !done && U > 0 && cv.walks > 0) {
     HSAW_TRY(outs.ensure((size_t)2 * k + 8, s));  // out_u[k], out_gain[k]

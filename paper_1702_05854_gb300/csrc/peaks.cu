@@ -41,7 +41,8 @@ constexpr uint32_t SORT_MAX = 4096;    // picks ranked against each other from s
 // ctl words of a run; the list's length (high half) and its pairs (low half) grow together in
 // one 64-bit word
 enum { PC_PICKS = 0, PC_FLOOR = 1, PC_GAIN = 2, PC_ROUNDS = 3, PC_STUCK = 4, PC_TOTAL = 5, PC_LIST = 6 /* 64 bits */,
-       PC_OWNED = 8 /* counts were not taken down */, PC_WORDS = 16 };
+       PC_OWNED = 8 /* counts were not taken down */, PC_LEFT = 9 /* it takes too long this way */,
+       PC_KEEP = 10 /* pairs that may lie outside the CTAs */, PC_WORDS = 16 };
 
 // A walk of a listed element: {walk, element, index in the list, 1 for the element's first}.
 using Pair = uint4;
@@ -64,6 +65,7 @@ struct PeakParams {
   uint32_t k;
   uint32_t round0;             // rounds of earlier phases
   uint32_t max_rounds;
+  uint32_t room;               // pairs that the CTAs hold
 };
 
 __device__ __forceinline__ unsigned long long peak_key(uint32_t count, uint32_t u) {
@@ -147,7 +149,10 @@ __device__ __forceinline__ bool own_part(const PeakParams& P, uint32_t n, OwnPar
 // it is a peak is settled within the CTA, which leaves two cluster barriers a round of three.
 // Against counts in global memory, 1,024 threads a CTA: the greedy of 5.3 K node walks and k = 100 (33 rounds)
 // 360 -> 298 us, of 7-222 K edge walks and k = 300 110-220 -> 94-137 us.
-// Longer lists, or an element in more walks than a CTA has room for, keep counts in global memory.
+// Longer lists, or an element in more walks than a CTA has room for, keep counts in global memory:
+// about 0.15-0.25 ns a pair and round, against 5 us a pick and an index of the walks (65 us a million
+// elements) for the greedy that takes one pick at a time.  Which is the faster then depends on the
+// rounds, which nothing tells beforehand: peak_pairs draws the line.
 __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant__ PeakParams P) {
   __shared__ uint32_t s_red[32];
   __shared__ uint32_t slot[2][16];  // by round parity, per CTA: its largest count
@@ -158,7 +163,9 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
   const uint32_t gtid = rank * blockDim.x + threadIdx.x, threads = C * blockDim.x;
   const uint32_t gwarp = gtid >> 5, warps = threads >> 5;
   const uint32_t n = __ldcg(&P.ctl[PC_LIST]);
-  if (n > P.pair_cap || __ldcg(&P.ctl[PC_LIST + 1]) > P.list_cap) return;  // the host makes room and comes back
+  const uint32_t keep = __ldcg(&P.ctl[PC_KEEP]);
+  // the host makes room and comes back, or leaves it
+  if (n > min(P.pair_cap, max(keep, P.room)) || __ldcg(&P.ctl[PC_LIST + 1]) > P.list_cap) return;
   const uint32_t* __restrict__ entry = P.entry + (P.from ? *P.from - P.from_sub : 0);
   const uint32_t stripe = (n + 31) / 32;
   const uint32_t floor_gain = __ldcg(&P.ctl[PC_FLOOR]);
@@ -196,10 +203,16 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
     __syncthreads();
   }
   uint32_t picks = 0, g = 0, r = P.round0;
-  bool stuck = false;
+  bool stuck = false, left = false;
+  const uint32_t picks0 = __ldcg(&P.ctl[PC_PICKS]);
   for (;;) {
     ++r;
     picks = __ldcg(&P.ctl[PC_PICKS]);
+    if (!owned &&
+        (n > keep || (uint64_t)n * (r - P.round0) > 16ull * keep + (picks - picks0) * PEAK_PICK)) {
+      left = true;  // the same decision in every CTA
+      break;
+    }
     // 1. elements at or above the floor sign their keys on their uncovered walks; the largest
     // count
     unsigned long long* const top = P.top[r & 1];
@@ -336,6 +349,7 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
     P.ctl[PC_ROUNDS] = r;
     P.ctl[PC_STUCK] = stuck ? 1u : 0u;
     P.ctl[PC_OWNED] = owned ? 1u : 0u;
+    P.ctl[PC_LEFT] = left ? 1u : 0u;
   }
 }
 
@@ -405,7 +419,8 @@ __global__ void __launch_bounds__(512) k_peak_hist(const uint32_t* __restrict__ 
 // inv_walk, its first pair, 0}, in no order.  Every listed element may be picked and covered, and
 // is read in each round, so the list holds half as many again as the k picks wanted (1,000
 // R-MAT edge picks came from the first 1,100-1,500) and a few, and more while it is short.
-__global__ void __launch_bounds__(512) k_peak_list(const uint32_t* __restrict__ hist, uint32_t k,
+__global__ void __launch_bounds__(512) k_peak_list(const uint32_t* __restrict__ hist, uint32_t k, uint32_t keep,
+                                                   uint32_t sparse, uint64_t elements,
                                                    const uint32_t* __restrict__ cnt, const int32_t* __restrict__ uid,
                                                    const uint8_t* __restrict__ cand,
                                                    const uint32_t* __restrict__ inv_off, uint32_t U, uint32_t list_cap,
@@ -454,7 +469,7 @@ __global__ void __launch_bounds__(512) k_peak_list(const uint32_t* __restrict__ 
       walks_above += w_warp[i];
     }
   }
-  const uint32_t want = (uint32_t)min((unsigned long long)total, (unsigned long long)k + k / 2 + 64);
+  const uint32_t want = (uint32_t)min((uint64_t)total, peak_list_goal(k));
   const unsigned long long few = max(16ull * k, 1024ull);
 #pragma unroll
   for (uint32_t i = 0; i < PER; ++i) {
@@ -471,6 +486,7 @@ __global__ void __launch_bounds__(512) k_peak_list(const uint32_t* __restrict__ 
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ctl[PC_FLOOR] = floor_gain;
     ctl[PC_TOTAL] = total;
+    ctl[PC_KEEP] = keep + (elements < (uint64_t)total * PEAK_SPARSE ? sparse : 0u);
   }
   // 128 counts a warp at a time: few reach the floor, so most are looked at once, four a lane
   const uint4* cnt4 = reinterpret_cast<const uint4*>(cnt);
@@ -541,7 +557,7 @@ __global__ void __launch_bounds__(256) k_walk_pairs(const __grid_constant__ Peak
                                                     const uint8_t* __restrict__ cand,
                                                     const uint32_t* __restrict__ index, uint4* __restrict__ list,
                                                     Pair* __restrict__ pairs) {
-  if (P.ctl[PC_LIST] > P.pair_cap || P.ctl[PC_LIST + 1] > P.list_cap) return;
+  if (P.ctl[PC_LIST] > min(P.pair_cap, max(P.ctl[PC_KEEP], P.room)) || P.ctl[PC_LIST + 1] > P.list_cap) return;
   const uint32_t floor_gain = P.ctl[PC_FLOOR];
   const uint32_t* __restrict__ entry = P.entry + (*P.from - P.from_sub);
   const uint32_t lane = threadIdx.x % LANES;
@@ -631,6 +647,13 @@ int peak_cluster() {
   return cached;
 }
 
+// Threads of a CTA.  Fewer warps meet at a barrier sooner, and have half the loads in flight and half
+// the room for whole elements: 512 threads against 1,024 on 5.3 K walks 266 against 298 us (stopping
+// rule query 677 against 730 us), 7-28 K walks of a pool 91-102 against 94-106, 55-222 K walks
+// 107-143 against 103-137; 32 instances of 20 K walks at once 7.47 against 7.08 ms.
+static unsigned peak_threads(int64_t walks) { return walks <= (1 << 14) ? 512 : 1024; }
+uint64_t peak_room(int64_t walks) { return (uint64_t)peak_cluster() * peak_threads(walks) * OWN_PAIRS; }
+
 // Counts by element id and walk offsets of walks [first, first + count), with no read back: the
 // rest of the greedy takes sizes from the device.  M elements.
 hsaw_status count_by_id(const Stream& st, bool edges, int64_t first, int64_t count, int64_t M, Cover& cv,
@@ -687,7 +710,10 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
   }
   uint32_t h[PC_WORDS] = {0}, phases = 0, owned_phases = 0, unique = 0;
   PeakParams P = {};
+  const uint64_t about = by_id ? cv.about : cv.entries;
+  const uint32_t room = (uint32_t)peak_room(W), keep = (uint32_t)std::min<uint64_t>(peak_pairs(W, about, k), 0xF0000000u);
   bool again = false;  // the phase did not fit its list or pairs
+  bool left = false;   // to the greedy that takes one pick at a time
   do {
     if (!again) {
       if (phases++) {  // the candidates below the last floor
@@ -710,7 +736,7 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     HSAW_TRY(cv.inv_ent.ensure(pair_cap, s));
     count_launch();
     k_peak_list<<<grid_for((U + 3) / 4, 512, 4 * sm_count()), 512, 0, s>>>(
-        hist, (uint32_t)k, cnt, uid, cand, by_id ? nullptr : cv.inv_off.p, U, list_cap, cv.peak_list.p, cv.g_list.p,
+        hist, (uint32_t)k, keep, peak_sparse_pairs(k), about, cnt, uid, cand, by_id ? nullptr : cv.inv_off.p, U, list_cap, cv.peak_list.p, cv.g_list.p,
         cv.g_rng.p, by_id ? cv.vals.p : nullptr, ctl);
     HSAW_CK(cudaGetLastError());
     P.pairs = cv.inv_ent.p;
@@ -732,6 +758,7 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     P.k = (uint32_t)k;
     P.round0 = h[PC_ROUNDS];
     P.max_rounds = most;  // a round makes a pick
+    P.room = room;
     count_launch();
     if (!by_id)
       k_peak_pairs<<<4 * sm_count(), 256, 0, s>>>(cv.peak_list.p, cv.inv_walk.p, ctl, list_cap, pair_cap, cv.inv_ent.p);
@@ -749,11 +776,7 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(csize);
-    // Fewer warps meet at a barrier sooner, and have half the loads in flight and half the room
-    // for whole elements: 512 threads against 1,024 on 5.3 K walks 266 against 298 us (stopping
-    // rule query 677 against 730 us), 7-28 K walks of a pool 91-102 against 94-106, 55-222 K walks
-    // 107-143 against 103-137; 32 instances of 20 K walks at once 7.47 against 7.08 ms.
-    cfg.blockDim = dim3(W <= (1u << 14) ? 512 : 1024);
+    cfg.blockDim = dim3(peak_threads(W));
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = 1;
@@ -769,6 +792,8 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
     if (h[PC_STUCK]) return fail(HSAW_E_DEVICE, "greedy: a round made no pick");
     if (phases == 1) unique = h[PC_TOTAL];
     again = h[PC_LIST] > pair_cap || h[PC_LIST + 1] > list_cap;
+    left = h[PC_LIST] > std::max(h[PC_KEEP], room) || (!again && h[PC_LEFT]);
+    if (left) break;
     if (again) {
       pair_cap = std::max(pair_cap, h[PC_LIST]);
       list_cap = std::max(list_cap, h[PC_LIST + 1]);
@@ -776,6 +801,15 @@ hsaw_status peak_greedy(Cover& cv, const uint8_t* cand, int32_t k, const PickBlo
       owned_phases += h[PC_OWNED];
     }
   } while (again || (h[PC_PICKS] < (uint32_t)k && h[PC_FLOOR] > 1));
+  if (left) {
+    if (log) {
+      fprintf(stderr, "hsaw: k_greedy_peaks left rounds=%u phases=%u pairs=%u picks=%u walks=%lld\n", h[PC_ROUNDS], phases,
+              h[PC_LIST], h[PC_PICKS], (long long)cv.walks);
+      cudaEventDestroy(ev[0]);
+      cudaEventDestroy(ev[1]);
+    }
+    return HSAW_OK;
+  }
   const uint32_t made = h[PC_PICKS], kept = std::min<uint32_t>(made, (uint32_t)k);
   if (made > SORT_MAX) {  // by element, then (stable) by gain downwards
     uint32_t *k1 = out_u, *v1 = out_gain, *k2 = out_u + 2 * (size_t)most, *v2 = k2 + most;

@@ -1,6 +1,8 @@
 // Internal state of a query: device suspect set, the ordered HSAW stream and the
 // counting / greedy workspaces (not part of the ABI).
 #pragma once
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace hsaw {
@@ -92,25 +94,55 @@ struct Cover {
   const int32_t* el = nullptr;
   const int64_t* from = nullptr;
   int64_t from_sub = 0, elements = 0;
+  const struct Stream* stream = nullptr;  // where the walks lie, for an index made after all
+  hsaw_mode mode = HSAW_EDGE;
+  int64_t first = 0;
+  int64_t about = 0;      // walk elements of the range (counts by id: about)
+  bool crowded = false;   // by peaks would be the slower greedy (cover_build)
   void release_index(cudaStream_t s);  // uid, cnt and the inverted index, which counts by id do not make
   void release(cudaStream_t s);
 };
 
-// for_greedy: only cover_greedy follows, so counts by element id do where they are the cheaper.
+// k > 0: only cover_greedy of k picks follows (any element a candidate if all), so counts by element
+// id do where they are the cheaper.
 hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t count, Cover& cv, cudaStream_t s,
-                        bool for_greedy = false);
+                        int32_t k = 0, bool all = true);
 // Entry offsets of walks [first, first + count) from the range's first, in cv.walk_eoff.
 hsaw_status walk_offsets(const Stream& st, bool edges, int64_t first, int64_t count, Cover& cv, cudaStream_t s);
 hsaw_status count_by_id(const Stream& st, bool edges, int64_t first, int64_t count, int64_t M, Cover& cv,
                         cudaStream_t s);
 int peak_cluster();  // CTAs of the cluster that the greedy by peaks runs on; 0: it cannot
+uint64_t peak_room(int64_t walks);  // pairs that its CTAs hold
 // Greedy (Alg. 4 / 7) on a built Cover; cand (device, M bytes) may be NULL.  *aid_host (may be
 // NULL) receives *aid_dev with the picks.
 hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t k, int64_t* ids_host,
                          uint32_t* gains_host, cudaStream_t s, const uint64_t* aid_dev = nullptr,
                          uint64_t* aid_host = nullptr);
 // The same picks by peaks, many at a time (peaks.cu), for cover_greedy: the first *rounds <= k
-// ids and gains (device, k of each); *done = false when no cluster can run it.
+// ids and gains (device, k of each); *done = false when no cluster can run it, or it is left to the
+// greedy that takes one pick at a time.
+// The greedy by peaks keeps a phase whose elements do not fit its CTAs whole while their (element, walk)
+// pairs are at most this many, and its rounds have not looked at 16 times as many and PEAK_PICK a pick;
+// otherwise the greedy that takes one pick at a time has it.  Greedy by peaks against one pick at a
+// time, ms, where the lists are longer: 4 M node walks of R-MAT 18 (115 M elements), k = 100, 700
+// against 65; 1 M of R-MAT 13 (8.2 M), k = 1,000, 102 against 9.9; 1 M on a path of 30, k = 1, 0.85
+// against 0.26; though also 200 K edge walks of the 16 K Chung-Lu graph, k = 100, 1.3 against 4.5
+// (16 picks cover all: the list does not tell).  Within it: 4 M edge walks of R-MAT 18 (111 M
+// elements, 310 K pairs), k = 1,000, 3.9 against 15.7; 1 M of R-MAT 13 with random weights (1.6 M,
+// 443 K pairs), k = 1,000, 3.6 against 5.1; 100 K node walks of R-MAT 13 (224 K pairs), k = 10, 0.75
+// against 0.64.  Where the mean candidate is in fewer than 32 walks, few picks touch each other and
+// lists may be longer: 1 M node walks of a 1 M Chung-Lu graph with random weights (16 walks a candidate,
+// 1.1 M pairs), k = 100, 1.7 against 2.6.
+constexpr uint64_t PEAK_PICK = 1ull << 15;
+inline uint64_t peak_pairs(int64_t walks, int64_t elements, int32_t k) {
+  return peak_room(walks) / 8 * 7 + (uint64_t)elements / 20 + 200ull * k;
+}
+constexpr uint32_t PEAK_SPARSE = 32;  // elements / candidates below which a list may be longer,
+inline uint32_t peak_sparse_pairs(int32_t k) {  // by this many pairs: fewer where many picks mean many rounds
+  return (uint32_t)std::min<uint64_t>(10000ull * k, 1000000000ull / (1000 + (uint64_t)k));
+}
+// Elements that a phase lists, about: half as many again as the picks wanted, and a few.
+__host__ __device__ inline uint64_t peak_list_goal(uint64_t k) { return k + k / 2 + 64; }
 struct PickBlock {  // one device buffer, so that one copy brings a greedy's results back
   static constexpr int CTL = 16, WORK = 4096;
   int64_t* ids;       // k

@@ -343,3 +343,50 @@ def test_greedy_record_names_its_kernel(streams, capfd, monkeypatch, count):
             assert runs[0]["walks"] == count and runs[0]["picks"] == 20 and runs[0]["owned"] <= runs[0]["phases"]
         else:
             assert ("hsaw: k_greedy_cluster " in err) == (force == "cluster")
+
+
+def concentrated(name):
+    """(n, src, dst, w, sources, mode) of streams in which few elements are in many walks."""
+    if name.startswith("path"):  # nested walks
+        n = int(name[4:])
+        src, dst = np.arange(n - 1, dtype=np.int32), np.arange(1, n, dtype=np.int32)
+        return n, src, dst, np.full(n - 1, ONE, np.uint32), np.array([0], np.int32), hs.HSAW_NODE
+    if name == "chung-lu":
+        d = synth.workload_c1()
+        return d["n"], d["src"], d["dst"], d["w"], d["sources"], hs.HSAW_EDGE
+    src, dst = synth.rmat_graph(13, 5)
+    return 1 << 13, src, dst, synth.wc_weights(1 << 13, dst), synth.sources(1 << 13, 1000), hs.HSAW_NODE
+
+
+# Pairs of each list against those that the thread blocks hold and those with which the greedy by peaks goes on, from
+# the oracle's counts: 932 K (262 K, 276 K), 177 K (262 K, 253 K; an element in more walks than a block holds),
+# 131 K (131 K, 124 K; elements of up to 2,700 do not share out evenly), 376 K (262 K, 321 K), 344 K (262 K, 451 K;
+# 60 picks in 27 rounds).
+@pytest.mark.parametrize("name,count,k,route", [
+    ("path30", 60_000, 1, "not begun"),
+    ("chung-lu", 100_000, 10, "kept"),
+    ("path100", 2_700, 10, "left at once"),
+    ("rmat", 120_000, 300, "left at once"),
+    ("rmat", 80_000, 1000, "left later"),
+])
+def test_greedy_leaves_long_lists(capfd, monkeypatch, name, count, k, route):
+    """Lists of many walks go to the greedy that takes one pick at a time: before the first round, or when the rounds
+    take longer than their picks are worth.  The picks are the same either way."""
+    n, src, dst, w, sources, mode = concentrated(name)
+    M = src.size if mode == hs.HSAW_EDGE else n
+    g, og = hs.hsaw_graph_from_edges(n, src, dst, w), oracle.Graph(n, src, dst, w)
+    ost = oracle.Stream(oracle.Query(og, sources, seed=4)).extend_threads(count, threads=8)
+    walks = hs.hsaw_sample(g, hs.Query(sources=sources, seed=4), 0, count)
+    monkeypatch.setenv("HSAW_LOG_LAUNCHES", "1")
+    capfd.readouterr()
+    ids, gains = hs.hsaw_greedy(walks, g, mode, 0, count, k)
+    err = capfd.readouterr().err
+    peaks = [line for line in err.splitlines() if line.startswith("hsaw: k_greedy_peaks ")]
+    one_pick = "hsaw: k_greedy_cluster " in err or "hsaw: k_greedy_onchip " in err
+    assert len(peaks) == (0 if route == "not begun" else 1)
+    assert one_pick == (route != "kept") and any(" left " in line for line in peaks) == route.startswith("left")
+    if route.startswith("left"):
+        rounds = int(re.search(r"rounds=(\d+)", peaks[0])[1])
+        assert rounds <= 1 if route == "left at once" else rounds > 2
+    oids, ogains = ost.greedy(mode, 0, count, M, k, kept_gains=True)
+    assert np.array_equal(gains, ogains) and np.array_equal(ids, oids)
