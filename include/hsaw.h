@@ -187,9 +187,10 @@ HSAW_API hsaw_status hsaw_debug_fail_alloc_after(int64_t n);
  *   must outlive the server) and starts `workers` threads (<= 0: 8).  mem_budget (bytes,
  *   0 = 3/4 of the free device memory at creation) bounds the summed device-memory
  *   estimates of the queries on the GPU.  hsaw_server_submit copies the query's host
- *   arrays and returns a ticket; a query whose estimate alone exceeds the budget is
- *   refused with HSAW_E_REJECTED.  Queries start in submission order as soon as a worker
- *   is free and the budget has room, while earlier ones are still running.
+ *   arrays and returns a ticket; a query whose walks alone (by estimate) exceed the budget
+ *   is refused with HSAW_E_REJECTED.  Queries start in submission order as soon as a worker
+ *   is free and the budget has room, while earlier ones are still running; one whose whole
+ *   estimate exceeds the budget starts when no other runs.
  *   hsaw_server_poll waits up to timeout_ms (< 0: forever) for the ticket: HSAW_E_PENDING
  *   if still running (the ticket stays valid), else the query's own status, with r
  *   filled as by hsaw_solve and *latency_ms (may be NULL) = completion - submission;

@@ -269,6 +269,8 @@ hsaw_status hsaw_sample(hsaw_graph g, const hsaw_query* q, uint64_t first_attemp
   if (st == HSAW_OK) st = stream_extend(g->g, w->qd, w->st, n_hits, s);
   if (st == HSAW_OK) {
     if (cudaStreamSynchronize(s) != cudaSuccess) st = fail(HSAW_E_DEVICE, "sample: stream sync failed");
+    w->st.chunk_kept.release(s);  // of no use to the handle
+    w->st.kept.release(s);
   }
   if (st != HSAW_OK) {
     cudaStreamSynchronize(s);

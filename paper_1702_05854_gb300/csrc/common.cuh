@@ -46,9 +46,9 @@ class Slab {
   Slab& operator=(const Slab&) = delete;
   void* cut(size_t bytes, cudaStream_t s);
   bool holds(const void* p) const { return p >= base_ && p < base_ + cap_; }
+  static constexpr size_t BYTES = 32ull << 20;
 
  private:
-  static constexpr size_t BYTES = 32ull << 20;
   cudaStream_t s_;
   char* base_ = nullptr;
   size_t cap_ = 0, used_ = 0;

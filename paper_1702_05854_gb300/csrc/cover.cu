@@ -197,7 +197,7 @@ static bool one_by_one() {
 // read per walk element, against about nine passes over the elements' sort and index: they are
 // cheaper while the counts lie in L2 (16 M of them), and beyond it while the range is at most
 // 8 times the elements (10 M edges of 67 M: 1.7 ms by the sort, 1.2 by id, greedy included).
-static bool counts_by_id(int64_t M, int64_t elements) {
+bool counts_by_id(int64_t M, int64_t elements) {
   return M > 0 && M < (1ll << 31) && (M <= (1ll << 24) || M <= 8 * elements);
 }
 

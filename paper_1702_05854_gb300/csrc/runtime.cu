@@ -189,17 +189,22 @@ struct Server {
   std::vector<std::thread> workers;
 };
 
-// Device bytes a query is expected to hold: its walk stream (aid, len, offsets and
-// elements per walk) plus the counting workspace (about 32 B per walk entry) and the
-// suspect bitmap / masks.
-static size_t estimate_bytes(const Server& S, const Ticket& t) {
+// Device bytes that a query is expected to hold.  walks: its walk stream (aid, len, offsets and elements
+// per walk), the counting workspace (about 32 B per walk entry) and the suspect bitmap / masks.  all:
+// with it the scratch whose size does not follow from the walks: the slab, counts and list indexes by
+// element id, and the sampler's records and their checkpoints.
+struct Estimate {
+  size_t walks, all;
+};
+
+static Estimate estimate_bytes(const Server& S, const Ticket& t) {
   const Graph& g = S.graphs[t.graph]->g;
   const double len = S.len_avg[t.graph] > 0 ? S.len_avg[t.graph] : 16.0;
+  const int64_t M = t.q.mode == HSAW_EDGE ? g.m : g.n;
   double hits;
   if (t.q.sampling == HSAW_FIXED_N) {
     hits = (double)t.q.n_hsaw;
   } else {
-    const int64_t M = t.q.mode == HSAW_EDGE ? g.m : g.n;
     double c6[6];
     const double delta = t.q.delta > 0 ? t.q.delta : 1.0 / (double)g.n;
     stop_constants(M, t.q.k, (t.q.eps > 0 && t.q.eps < 1) ? t.q.eps : 0.1, delta, c6);
@@ -207,8 +212,17 @@ static size_t estimate_bytes(const Server& S, const Ticket& t) {
   }
   const double per_walk = 24.0 + 8.0 * len + 40.0 * len;
   const double masks = (double)g.n / 8.0 + (t.q.p_fixed ? 4.0 * (double)g.n : 0.0) +
-                       (t.q.candidate_mask ? (double)(t.q.mode == HSAW_EDGE ? g.m : g.n) : 0.0);
-  return (size_t)(hits * 1.1 * per_walk + masks + (64 << 20));
+                       (t.q.candidate_mask ? (double)M : 0.0);
+  const double walks = hits * 1.1 * per_walk + masks + (64 << 20);
+  double ids = 1024.0;
+  if (counts_by_id(M, (int64_t)std::min(hits * len, 1e18)))
+    while (ids < (double)M) ids *= 2.0;  // as buffers grow
+  // a walk of len nodes meets a suspect about len times as often as its start is one
+  const double rate = std::min(1.0, std::max(1e-9, len * (double)t.q.n_sources / (double)g.n));
+  const double attempts = std::min((double)MOST_ATTEMPTS, std::max(1048576.0, 1.25 * hits / rate));
+  const double records = attempts / 256.0 * hit_records(rate, 256);
+  const double window = records * 8.0 + std::min(records, (double)kept_records(hits * len)) * 32.0;
+  return {(size_t)walks, (size_t)(walks + (double)Slab::BYTES + 8.0 * ids + window)};
 }
 
 static void server_worker(Server* S) {
@@ -344,8 +358,9 @@ hsaw_status hsaw_server_submit(hsaw_server h, int32_t graph_idx, const hsaw_quer
   t->t_submit = std::chrono::steady_clock::now();
   {
     std::lock_guard<std::mutex> lk(S.mu);
-    t->estimate = estimate_bytes(S, *t);
-    if (t->estimate > S.budget) return fail(HSAW_E_REJECTED, "server: query's memory estimate exceeds the budget");
+    const Estimate e = estimate_bytes(S, *t);
+    t->estimate = e.all;  // more than the budget: it runs alone
+    if (e.walks > S.budget) return fail(HSAW_E_REJECTED, "server: query's memory estimate exceeds the budget");
     t->id = S.next_id++;
     S.tickets[t->id] = t;
     S.queue.push_back(t);

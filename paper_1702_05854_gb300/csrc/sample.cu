@@ -581,14 +581,15 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
   SampleParams P = make_params(g, qd);
   const uint32_t shift = chunk_shift_for(batch), chunk = 1u << shift;
   const uint32_t n_chunks = (uint32_t)((batch + chunk - 1) >> shift);
-  // records per chunk: a few standard deviations above the expected hits, else all
-  const double exp_hits = std::max(st.hit_rate, 0.0) * chunk;
-  uint32_t cap = (uint32_t)std::min<double>(chunk, std::ceil(exp_hits + 6.0 * std::sqrt(exp_hits + 1.0) + 8.0));
-  if (st.hit_rate == 0.0) cap = chunk;
+  // with no hit yet, the rate is below a few in the attempts so far
+  const uint64_t used = st.next_attempt - st.first_attempt;
+  uint32_t cap = hit_records(st.hit_rate > 0.0 ? st.hit_rate : used ? 1.0 / (double)used : 1.0, chunk);
   for (;;) {
     HSAW_TRY(st.chunk_hits.ensure((size_t)SC_WORDS + n_chunks, s));
     HSAW_TRY(st.recs.ensure((size_t)n_chunks * cap, s));
-    HSAW_TRY(st.chunk_kept.ensure(st.ids_only ? 0 : 2 * (size_t)n_chunks * cap, s));
+    const double elements = st.count ? st.hit_rate * (double)batch * (double)st.total_nodes / (double)st.count : 0.0;
+    const bool keep = !st.ids_only && (st.count || !used) && (uint64_t)n_chunks * cap <= kept_records(elements);
+    HSAW_TRY(st.chunk_kept.ensure(keep ? 2 * (size_t)n_chunks * cap : 0, s));
     uint32_t* const ctl = st.chunk_hits.p;
     HSAW_CK(cudaMemsetAsync(ctl, 0, ((size_t)SC_WORDS + n_chunks) * 4, s));
     P.a0 = st.next_attempt;
@@ -599,7 +600,7 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
     P.ctl = ctl;
     P.chunk_hits = ctl + SC_WORDS;
     P.recs = st.recs.p;
-    P.kept = st.ids_only ? nullptr : st.chunk_kept.p;
+    P.kept = keep ? st.chunk_kept.p : nullptr;
     const int bps = sample_blocks();
     const unsigned grid = (unsigned)std::max(1, std::min<int>(sm_count() * bps, (int)((n_chunks + 7) / 8)));
     void* prof = profile_begin(s);
@@ -630,8 +631,8 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
     if (*new_hits) {
       HSAW_TRY(st.aid.ensure((size_t)st.count + *new_hits, s, true));
       HSAW_TRY(st.len.ensure((size_t)st.count + *new_hits, s, true));
-      HSAW_TRY(st.kept.ensure(st.ids_only ? 0 : 2 * (size_t)*new_hits, s));
-      st.kept_hits = st.ids_only ? 0 : *new_hits;
+      HSAW_TRY(st.kept.ensure(keep ? 2 * (size_t)*new_hits : 0, s));
+      st.kept_hits = keep ? *new_hits : 0;
       count_launch();
       k_compact<<<grid_for((size_t)n_chunks * 32, 256, 8192), 256, 0, s>>>(
           P.chunk_hits, ctl + SC_HITS, st.recs.p, cap, n_chunks, st.next_attempt, P.kept, st.aid.p + st.count,
@@ -668,7 +669,7 @@ hsaw_status stream_extend(const Graph& g, const QueryDev& qd, Stream& st, int64_
                     : used          ? std::max(1048576.0, 2.0 * (double)used)
                                     : std::min(1048576.0, need / 16.0 / std::max(qd.start_rate, 1e-12));
     target = std::max(target, least);
-    target = std::min(target, 268435456.0);
+    target = std::min(target, (double)MOST_ATTEMPTS);
     uint64_t batch = (uint64_t)target;
     batch = std::min<uint64_t>(batch, st.max_attempts - used);
     uint32_t new_hits = 0;

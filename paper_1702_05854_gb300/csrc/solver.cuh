@@ -2,6 +2,7 @@
 // counting / greedy workspaces (not part of the ABI).
 #pragma once
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 
@@ -56,6 +57,18 @@ struct Stream {
   void release(cudaStream_t s);
 };
 
+// Hit records that a sampler launch has room for per chunk of attempts: a few standard deviations above
+// the hits expected at `rate` a attempt, at most all.  A launch that needs more runs again with all.
+inline uint32_t hit_records(double rate, uint32_t chunk) {
+  const double hits = std::max(rate, 0.0) * chunk;
+  return (uint32_t)std::min<double>(chunk, std::ceil(hits + 6.0 * std::sqrt(hits + 1.0) + 8.0));
+}
+// Checkpoints (32 bytes a record) are kept for launches of up to this many records: 134 MB, or half of what
+// the counts and the index of the walks expected will take (48 bytes an element); without them the walks
+// are drawn again from their starts.
+inline uint64_t kept_records(double elements) { return std::max(1ull << 22, (unsigned long long)(0.75 * elements)); }
+constexpr uint64_t MOST_ATTEMPTS = 1ull << 28;  // of a launch
+
 hsaw_status stream_init(Stream& st, uint64_t first_attempt, uint64_t max_attempts, cudaStream_t s);
 // Extend the stream until it holds at least want hits (Alg. 3 loop).
 hsaw_status stream_extend(const Graph& g, const QueryDev& qd, Stream& st, int64_t want, cudaStream_t s);
@@ -103,6 +116,8 @@ struct Cover {
   void release(cudaStream_t s);
 };
 
+// Whether the greedy's counts are by element id (M elements in all, `elements` in the walks).
+bool counts_by_id(int64_t M, int64_t elements);
 // k > 0: only cover_greedy of k picks follows (any element a candidate if all), so counts by element
 // id do where they are the cheaper.
 hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t count, Cover& cv, cudaStream_t s,

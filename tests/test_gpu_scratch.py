@@ -1,0 +1,118 @@
+"""Scratch device memory: what calls hold at most, and what is left when an allocation fails.
+
+Counted by an allocator of the tests' own (hsaw_set_allocator) over torch's caching allocator; failures are made on the
+host, by that allocator or by the library's own hook.
+"""
+import threading
+
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+hs = pytest.importorskip("paper_1702_05854_gb300")
+
+MB = 1 << 20
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.init()
+
+
+class Scratch:
+    """Installs an allocator that counts the bytes held and refuses what `refuse(nbytes, held)` says."""
+
+    def __init__(self, refuse=lambda nbytes, held: False):
+        self.live, self.held, self.peak, self.asked, self.refuse = {}, 0, 0, 0, refuse
+        self.lock = threading.Lock()
+
+    def alloc(self, nbytes, stream):
+        with self.lock:
+            self.asked += 1
+            if self.refuse(nbytes, self.held):
+                return 0
+            p = torch.cuda.caching_allocator_alloc(nbytes, stream=stream)
+            self.live[p] = nbytes
+            self.held += nbytes
+            self.peak = max(self.peak, self.held)
+            return p
+
+    def release(self, ptr, stream):
+        with self.lock:
+            self.held -= self.live.pop(ptr)
+            torch.cuda.caching_allocator_delete(ptr)
+
+    def __enter__(self):
+        hs.hsaw_set_allocator(self.alloc, self.release)
+        return self
+
+    def __exit__(self, *exc):
+        torch.cuda.synchronize()
+        hs.hsaw_set_allocator()
+
+
+def test_server_budget_bounds_scratch():
+    """Queries of few walks on 2^24 edges: the counts by edge id, the slab and the sampler's records, not the walks, are
+    what they hold; together they stay within the budget."""
+    d = synth.workload_rmat(20, "wc", 1000, 50, "edge")
+    g = hs.hsaw_graph_from_edges(d["n"], d["src"], d["dst"], d["w"])
+    queries = [hs.Query(sources=d["sources"], mode=hs.HSAW_EDGE, k=50, n_hsaw=2000, seed=s) for s in range(48)]
+    alone = [hs.hsaw_solve(g, q) for q in queries]
+    budget = 700 * MB
+    with Scratch() as a:
+        srv = hs.Server([g], mem_budget=budget, workers=8)
+        tickets = [srv.submit(0, q) for q in queries]
+        got = [srv.poll(t) for t in tickets]
+        srv.close()
+        assert 128 * MB < a.peak <= budget, a.peak / MB
+    for (ids, gains, r), (ids2, gains2, r2, *_) in zip(alone, got):
+        assert np.array_equal(ids, ids2) and np.array_equal(gains, gains2) and r["attempts"] == r2["attempts"]
+
+
+def test_server_takes_what_its_walks_fit():
+    """A query whose walks fit the budget is served, alone, though its scratch does not."""
+    d = synth.workload_rmat(20, "wc", 1000, 50, "edge")
+    g = hs.hsaw_graph_from_edges(d["n"], d["src"], d["dst"], d["w"])
+    srv = hs.Server([g], mem_budget=80 * MB, workers=2)
+    q = hs.Query(sources=d["sources"], mode=hs.HSAW_EDGE, k=50, n_hsaw=2000, seed=1)
+    ids, gains = hs.hsaw_solve(g, q)[:2]
+    for t in [srv.submit(0, q) for _ in range(4)]:
+        got = srv.poll(t)
+        assert np.array_equal(got[0], ids) and np.array_equal(got[1], gains)
+    srv.close()
+
+
+def test_scratch_while_no_attempt_hits():
+    """One suspect among 2^25 isolated nodes: launches grow to tens of millions of attempts before the first hit, and have
+    room for the few hits that can be expected, not for one an attempt (8 bytes each: 268 MB and more)."""
+    n = 1 << 25
+    one = np.zeros(1, np.int32)
+    g = hs.hsaw_graph_from_edges(n, one, one + 1, np.ones(1, np.uint32))
+    og = oracle.Graph(n, one, one + 1, np.ones(1, np.uint32))
+    sources = np.array([12_345_678], np.int32)
+    with Scratch() as a:
+        ids, gains, r = hs.hsaw_solve(g, hs.Query(sources=sources, mode=hs.HSAW_NODE, k=1, n_hsaw=2, seed=8))
+        assert a.peak < 192 * MB, a.peak / MB
+    st = oracle.Stream(oracle.Query(og, sources, seed=8)).extend_threads(2, threads=8)
+    aid = st.export().aid
+    assert r["attempts"] == aid[1] + 1 and r["attempts"] > 1 << 24 and ids[0] == sources[0] and gains[0] == 2
+
+
+def test_walks_handle_keeps_no_checkpoints():
+    """What a handle holds: its walks and the sampler's records of one launch of 2^20 attempts (8 bytes each)."""
+    d = synth.workload_c1()
+    g = hs.hsaw_graph_from_edges(d["n"], d["src"], d["dst"], d["w"])
+    with Scratch() as a:
+        w = hs.hsaw_sample(g, hs.Query(sources=d["sources"], seed=4), 0, 1000)
+        i = w.info()
+        walks = 20 * i["count"] + 8 + 8 * i["total_nodes"]  # ids, lengths, offsets; nodes and edges
+        assert a.held <= 2 * walks + (8 << 20) + 2 * MB, (a.held / MB, walks / MB)
+        w.close()
+        assert not a.live
