@@ -45,11 +45,11 @@ static std::atomic<const ScratchAllocator*> g_alloc{nullptr};
 static std::atomic<long long> g_held{0};                   // scratch blocks handed out, not yet released
 
 static thread_local Slab* t_slab = nullptr;
+static hsaw_status allocate(void** p, size_t bytes, cudaStream_t s);
 
 Slab::Slab(cudaStream_t s) : s_(s), outer_(t_slab) {
   void* p = nullptr;
-  t_slab = nullptr;  // its own block comes from the allocator
-  if (dmalloc(&p, BYTES, s) == HSAW_OK) {
+  if (allocate(&p, BYTES, s) == HSAW_OK) {
     base_ = static_cast<char*>(p);
     cap_ = BYTES;
   } else {
@@ -80,6 +80,11 @@ hsaw_status dmalloc(void** p, size_t bytes, cudaStream_t s) {
   }
   if (bytes == 0) bytes = 16;
   if (t_slab && (*p = t_slab->cut(bytes, s))) return HSAW_OK;
+  return allocate(p, bytes, s);
+}
+
+// From the allocator itself.
+static hsaw_status allocate(void** p, size_t bytes, cudaStream_t s) {
   if (const ScratchAllocator* a = g_alloc.load(std::memory_order_acquire)) {
     *p = a->alloc(bytes, (void*)s, a->ctx);
     if (!*p) {

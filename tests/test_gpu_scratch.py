@@ -116,3 +116,22 @@ def test_walks_handle_keeps_no_checkpoints():
         assert a.held <= 2 * walks + (8 << 20) + 2 * MB, (a.held / MB, walks / MB)
         w.close()
         assert not a.live
+
+
+def test_injected_failure_reaches_the_caller():
+    """The n-th allocation fails as if memory were out, and the call with it, the first too."""
+    d = synth.workload_c1()
+    g = hs.hsaw_graph_from_edges(d["n"], d["src"], d["dst"], d["w"])
+    q = hs.Query(sources=d["sources"], mode=hs.HSAW_EDGE, k=10, n_hsaw=1000, seed=4)
+    walks = hs.hsaw_sample(g, q, 0, 1000)
+    calls = [lambda: hs.hsaw_solve(g, q), lambda: hs.hsaw_estimate_spread(g, q, [3]),
+             lambda: hs.hsaw_greedy(walks, g, hs.HSAW_EDGE, 0, 1000, 10), lambda: hs.hsaw_sample(g, q, 0, 1000)]
+    try:
+        for call in calls:
+            for n in (1, 2, 3):
+                hs.hsaw_debug_fail_alloc_after(n)
+                with pytest.raises(hs.HsawError) as e:
+                    call()
+                assert e.value.status == -4
+    finally:
+        hs.hsaw_debug_fail_alloc_after(0)
