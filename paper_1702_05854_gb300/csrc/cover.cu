@@ -1165,7 +1165,15 @@ __global__ void k_exclude_picks(const uint32_t* __restrict__ out_u, int32_t r, u
 hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t k, int64_t* ids_host,
                          uint32_t* gains_host, cudaStream_t s, const uint64_t* aid_dev, uint64_t* aid_host) {
   if (k < 1) return fail(HSAW_E_INVALID, "greedy: k < 1");
-  DBuf<uint32_t> block, outs;
+  struct Held {  // given back on every way out
+    DBuf<uint32_t> block, outs;
+    cudaStream_t s;
+    ~Held() {
+      block.release(s);
+      outs.release(s);
+    }
+  } held{{}, {}, s};
+  DBuf<uint32_t>&block = held.block, &outs = held.outs;
   HSAW_TRY(block.ensure(PickBlock::copied_words(k) + PickBlock::WORK, s));
   const PickBlock B = PickBlock::at(block.p, k);
   std::vector<uint32_t> host(PickBlock::copied_words(k));
@@ -1350,8 +1358,6 @@ hsaw_status cover_greedy(Cover& cv, const uint8_t* cand_dev, int64_t M, int32_t 
     if (gains_host) std::memcpy(gains_host, host.data() + (B.gains - block.p), (size_t)k * 4);
     if (aid_host) std::memcpy(aid_host, host.data() + (reinterpret_cast<uint32_t*>(B.last_aid) - block.p), 8);
   }
-  block.release(s);
-  outs.release(s);
   return st;
 }
 

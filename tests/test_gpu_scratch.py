@@ -135,3 +135,50 @@ def test_injected_failure_reaches_the_caller():
                 assert e.value.status == -4
     finally:
         hs.hsaw_debug_fail_alloc_after(0)
+        walks.close()
+
+
+def test_nothing_is_held_after_a_failed_call():
+    """Allocations of a call refused from the n-th on, for every n, with and without room for the slab: the call ends
+    with HSAW_E_NOMEM and gives everything back."""
+    d = synth.workload_c1()
+    g = hs.hsaw_graph_from_edges(d["n"], d["src"], d["dst"], d["w"])
+    kw = dict(sources=d["sources"], mode=hs.HSAW_EDGE, seed=4)
+    fixed = hs.Query(k=10, n_hsaw=1000, **kw)
+    walks = hs.hsaw_sample(g, fixed, 0, 1000)
+    calls = [lambda: hs.hsaw_solve(g, fixed), lambda: hs.hsaw_solve(g, hs.Query(k=5, sampling=hs.HSAW_STOP_RULE, eps=0.4, **kw)),
+             lambda: hs.hsaw_greedy(walks, g, hs.HSAW_EDGE, 0, 1000, 10), lambda: hs.hsaw_histogram(walks, hs.HSAW_NODE, 0, 1000),
+             lambda: hs.hsaw_coverage(walks, hs.HSAW_EDGE, 0, 1000, [3, 5]), lambda: hs.hsaw_estimate_spread(g, fixed, [3]),
+             lambda: hs.hsaw_sample(g, fixed, 0, 1000, edge_removed=np.zeros(d["m"], np.uint8)).close(),
+             lambda: hs.hsaw_classify(g, fixed, 0, 1000),
+             lambda: hs.hsaw_solve_batch([g, g], [fixed, fixed], concurrency=1)]
+    walks.close()  # its blocks are of the allocator of before: made again below
+    for greedy in (None, "cluster", "grid"):
+        for slab in (True, False):
+            for i, call in enumerate(calls):
+                if (greedy and i > 2) or (not slab and i in (3, 4, 6, 7)):  # the latter have no slab
+                    continue
+                nth = 0
+                while True:
+                    nth += 1
+                    with pytest.MonkeyPatch.context() as mp, Scratch() as a:
+                        if greedy:
+                            mp.setenv("HSAW_GREEDY", greedy)
+                        walks = hs.hsaw_sample(g, fixed, 0, 1000)
+                        held, first = set(a.live), a.asked
+                        a.refuse = lambda b, h: (not slab and b >= 32 * MB) or a.asked - first >= nth
+                        done = False
+                        try:
+                            out = call()
+                            done = i != len(calls) - 1 or all(s == 0 for s, *_ in out)
+                            if i == len(calls) - 1 and not done:
+                                assert all(s in (0, -4) for s, *_ in out)
+                        except hs.HsawError as e:
+                            assert e.status == -4
+                        torch.cuda.synchronize()
+                        assert set(a.live) == held, (i, nth, len(a.live) - len(held))
+                        used = a.asked - first
+                        walks.close()
+                    if done and used < nth:
+                        break
+                    assert nth < 400, (greedy, slab, i, used)
