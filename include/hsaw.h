@@ -331,7 +331,8 @@ HSAW_API hsaw_status hsaw_probe_gather(uint64_t table_bytes, int32_t chains, uin
  * installs an allocator of its own, such as a framework's caching allocator:
  *   alloc(bytes, stream, ctx) returns device memory on the current device, aligned to at
  *     least 256 bytes, usable in stream order on `stream`, or NULL when it has none (the
- *     call in progress then fails with HSAW_E_NOMEM);
+ *     call in progress is then made once more with as little scratch as it can do with, and
+ *     fails with HSAW_E_NOMEM if that is refused too);
  *   release(ptr, stream, ctx) takes back a block alloc returned, in stream order on
  *     `stream`.
  * The library calls them from whichever threads run its calls (batch and server workers

@@ -142,14 +142,16 @@ hsaw_status solve_fixed_from_stream(const Graph& g, const hsaw_query* q, Stream&
   HSAW_TRY(validate_common(g, q, &n_cand));
   if (q->n_hsaw < 1 || st.count < q->n_hsaw) return fail(HSAW_E_INVALID, "solve: stream shorter than n_hsaw");
   const int64_t M = q->mode == HSAW_EDGE ? g.m : g.n;
-  Cover cv;
-  uint8_t* cand = nullptr;
-  hsaw_status rc = upload_mask(q->candidate_mask, (size_t)M, false, s, &cand);
-  if (rc == HSAW_OK) rc = fixed_tail(g, q, st, cv, cand, r, s);
-  cudaStreamSynchronize(s);
-  cv.release(s);
-  dfree(cand, s);
-  return rc;
+  return within_memory([&] {
+    Cover cv;
+    uint8_t* cand = nullptr;
+    hsaw_status rc = upload_mask(q->candidate_mask, (size_t)M, false, s, &cand);
+    if (rc == HSAW_OK) rc = fixed_tail(g, q, st, cv, cand, r, s);
+    cudaStreamSynchronize(s);
+    cv.release(s);
+    dfree(cand, s);
+    return rc;
+  });
 }
 
 static hsaw_status solve(const Graph& g, const hsaw_query* q, hsaw_result* r, cudaStream_t s) {
@@ -236,7 +238,7 @@ static hsaw_status solve(const Graph& g, const hsaw_query* q, hsaw_result* r, cu
 }
 
 hsaw_status solve_one(const Graph& g, const hsaw_query* q, hsaw_result* r, cudaStream_t s) {
-  return solve(g, q, r, s);
+  return within_memory([&] { return solve(g, q, r, s); });
 }
 
 }  // namespace hsaw
@@ -247,7 +249,7 @@ extern "C" {
 
 hsaw_status hsaw_solve(hsaw_graph g, const hsaw_query* q, hsaw_result* r, void* stream) {
   if (!g) return fail(HSAW_E_INVALID, "solve: NULL graph");
-  return solve(g->g, q, r, (cudaStream_t)stream);
+  return solve_one(g->g, q, r, (cudaStream_t)stream);
 }
 
 hsaw_status hsaw_sample(hsaw_graph g, const hsaw_query* q, uint64_t first_attempt, int64_t n_hits,
@@ -260,24 +262,29 @@ hsaw_status hsaw_sample(hsaw_graph g, const hsaw_query* q, uint64_t first_attemp
   auto* w = new (std::nothrow) hsaw_walks_s();
   if (!w) return fail(HSAW_E_NOMEM, "sample: host allocation");
   cudaGetDevice(&w->device);
-  hsaw_status st = query_upload(g->g, q, w->qd, s);
-  const bool dev = removed_flags & HSAW_INPUT_DEVICE;
-  if (st == HSAW_OK) st = upload_removed(edge_removed, (size_t)g->g.m, dev, s, &w->qd.edge_removed);
-  if (st == HSAW_OK) st = upload_removed(node_removed, (size_t)g->g.n, dev, s, &w->qd.node_removed);
-  w->qd.owns_removed = true;
-  if (st == HSAW_OK) st = stream_init(w->st, first_attempt, q->max_attempts, s);
-  if (st == HSAW_OK) st = stream_extend(g->g, w->qd, w->st, n_hits, s);
-  if (st == HSAW_OK) {
-    if (cudaStreamSynchronize(s) != cudaSuccess) st = fail(HSAW_E_DEVICE, "sample: stream sync failed");
-    w->st.chunk_kept.release(s);  // of no use to the handle
-    w->st.kept.release(s);
-  }
-  if (st != HSAW_OK) {
-    cudaStreamSynchronize(s);
-    query_release(w->qd, s);
-    w->st.release(s);
-    delete w;
+  const hsaw_status rc = within_memory([&] {
+    hsaw_status st = query_upload(g->g, q, w->qd, s);
+    const bool dev = removed_flags & HSAW_INPUT_DEVICE;
+    if (st == HSAW_OK) st = upload_removed(edge_removed, (size_t)g->g.m, dev, s, &w->qd.edge_removed);
+    if (st == HSAW_OK) st = upload_removed(node_removed, (size_t)g->g.n, dev, s, &w->qd.node_removed);
+    w->qd.owns_removed = true;
+    if (st == HSAW_OK) st = stream_init(w->st, first_attempt, q->max_attempts, s);
+    if (st == HSAW_OK) st = stream_extend(g->g, w->qd, w->st, n_hits, s);
+    if (st == HSAW_OK) {
+      if (cudaStreamSynchronize(s) != cudaSuccess) st = fail(HSAW_E_DEVICE, "sample: stream sync failed");
+      w->st.chunk_kept.release(s);  // of no use to the handle
+      w->st.kept.release(s);
+    }
+    if (st != HSAW_OK) {
+      cudaStreamSynchronize(s);
+      query_release(w->qd, s);
+      w->st.release(s);
+    }
     return st;
+  });
+  if (rc != HSAW_OK) {
+    delete w;
+    return rc;
   }
   *out = w;
   return HSAW_OK;
@@ -298,33 +305,35 @@ hsaw_status hsaw_estimate_spread(hsaw_graph g, const hsaw_query* q, const int64_
   for (int32_t i = 0; i < n_removed; ++i)
     if (removed[i] < 0 || removed[i] >= M) return fail(HSAW_E_RANGE, "estimate: removed id out of range");
   cudaStream_t s = (cudaStream_t)stream;
-  SolveScratch W(s);
-  HSAW_TRY(query_upload(G, q, W.qd, s));
-  if (n_removed > 0) {
-    uint32_t* mask = nullptr;
-    int64_t* d_ids = nullptr;
-    const size_t bytes = ((size_t)M + 31) / 32 * 4;
-    HSAW_TRY(dmalloc((void**)&mask, bytes, s));
-    (edges ? W.qd.edge_removed : W.qd.node_removed) = mask;
-    W.qd.owns_removed = true;
-    HSAW_CK(cudaMemsetAsync(mask, 0, bytes, s));
-    HSAW_TRY(dmalloc((void**)&d_ids, (size_t)n_removed * 8, s));
-    HSAW_CK(cudaMemcpyAsync(d_ids, removed, (size_t)n_removed * 8, cudaMemcpyHostToDevice, s));
-    count_launch();
-    k_mark_removed<<<grid_for(n_removed, 256, 1024), 256, 0, s>>>(d_ids, n_removed, mask);
-    HSAW_CK(cudaGetLastError());
-    dfree(d_ids, s);
-  }
-  HSAW_TRY(stream_init(W.st, 0, q->max_attempts, s));
-  W.st.least_window = 65536.0;
-  W.st.ids_only = true;
-  HSAW_TRY(stream_extend(G, W.qd, W.st, q->n_hsaw, s));
-  uint64_t last = 0;
-  HSAW_TRY(aid_at(W.st, q->n_hsaw - 1, &last, s));
-  const double A = (double)(last + 1), f = (double)q->n_hsaw / A, n = (double)G.n;
-  *spread = n * (double)q->n_hsaw / A;
-  if (std_err) *std_err = n * std::sqrt(f * (1.0 - f) / A);
-  return HSAW_OK;
+  return within_memory([&]() -> hsaw_status {
+    SolveScratch W(s);
+    HSAW_TRY(query_upload(G, q, W.qd, s));
+    if (n_removed > 0) {
+      uint32_t* mask = nullptr;
+      int64_t* d_ids = nullptr;
+      const size_t bytes = ((size_t)M + 31) / 32 * 4;
+      HSAW_TRY(dmalloc((void**)&mask, bytes, s));
+      (edges ? W.qd.edge_removed : W.qd.node_removed) = mask;
+      W.qd.owns_removed = true;
+      HSAW_CK(cudaMemsetAsync(mask, 0, bytes, s));
+      HSAW_TRY(dmalloc((void**)&d_ids, (size_t)n_removed * 8, s));
+      HSAW_CK(cudaMemcpyAsync(d_ids, removed, (size_t)n_removed * 8, cudaMemcpyHostToDevice, s));
+      count_launch();
+      k_mark_removed<<<grid_for(n_removed, 256, 1024), 256, 0, s>>>(d_ids, n_removed, mask);
+      HSAW_CK(cudaGetLastError());
+      dfree(d_ids, s);
+    }
+    HSAW_TRY(stream_init(W.st, 0, q->max_attempts, s));
+    W.st.least_window = 65536.0;
+    W.st.ids_only = true;
+    HSAW_TRY(stream_extend(G, W.qd, W.st, q->n_hsaw, s));
+    uint64_t last = 0;
+    HSAW_TRY(aid_at(W.st, q->n_hsaw - 1, &last, s));
+    const double A = (double)(last + 1), f = (double)q->n_hsaw / A, n = (double)G.n;
+    *spread = n * (double)q->n_hsaw / A;
+    if (std_err) *std_err = n * std::sqrt(f * (1.0 - f) / A);
+    return HSAW_OK;
+  });
 }
 
 hsaw_status hsaw_walks_info(hsaw_walks w, int64_t* count, int64_t* total_nodes, uint64_t* attempts, uint64_t* steps) {
@@ -421,16 +430,18 @@ hsaw_status hsaw_greedy(hsaw_walks w, hsaw_graph g, hsaw_mode mode, int64_t firs
   }
   if (k < 1 || k > c) return fail(HSAW_E_INVALID, "greedy: need 1 <= k <= |C|");
   cudaStream_t s = (cudaStream_t)stream;
-  Slab slab(s);
-  Cover cv;
-  uint8_t* cand = nullptr;
-  hsaw_status st = upload_mask(candidate_mask, (size_t)M, false, s, &cand);
-  if (st == HSAW_OK) st = cover_build(w->st, mode, first, count, cv, s, k, !cand);
-  if (st == HSAW_OK) st = cover_greedy(cv, cand, M, k, ids, gains, s);
-  cudaStreamSynchronize(s);
-  cv.release(s);
-  dfree(cand, s);
-  return st;
+  return within_memory([&] {
+    Slab slab(s);
+    Cover cv;
+    uint8_t* cand = nullptr;
+    hsaw_status st = upload_mask(candidate_mask, (size_t)M, false, s, &cand);
+    if (st == HSAW_OK) st = cover_build(w->st, mode, first, count, cv, s, k, !cand);
+    if (st == HSAW_OK) st = cover_greedy(cv, cand, M, k, ids, gains, s);
+    cudaStreamSynchronize(s);
+    cv.release(s);
+    dfree(cand, s);
+    return st;
+  });
 }
 
 hsaw_status hsaw_coverage(hsaw_walks w, hsaw_mode mode, int64_t first, int64_t count, const int64_t* T, int32_t k,

@@ -55,6 +55,22 @@ class Slab {
   Slab* outer_;
 };
 
+// A call that ran out of device memory is made once more without the scratch that only buys time: no
+// slab, no counts by element id, no greedy by peaks, no checkpoints of walks, no payload in the edge
+// sort.  lean() is true meanwhile, on the call's thread.  call: makes and releases all that it holds.
+bool lean();
+bool begin_lean(hsaw_status st);  // false: not for a failure that was injected, nor twice
+struct LeanEnd {
+  ~LeanEnd();
+};
+template <typename F>
+hsaw_status within_memory(F&& call) {
+  const hsaw_status st = call();
+  if (!begin_lean(st)) return st;
+  LeanEnd end;
+  return call();
+}
+
 template <typename T>
 struct DBuf {  // grow-only device buffer
   T* p = nullptr;

@@ -223,7 +223,7 @@ hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t
   const int64_t in_stream = em ? st.total_nodes - st.count : st.total_nodes;  // walk elements of the whole stream
   const int64_t M = st.elem_range[em ? 1 : 0];
   cv.about = (int64_t)((double)in_stream / (double)st.count * (double)count);
-  cv.crowded = k > 0 && all && M > 0 && crowded(M, cv.about, count, k);
+  cv.crowded = lean() || (k > 0 && all && M > 0 && crowded(M, cv.about, count, k));
   if (k > 0 && !cv.crowded && !one_by_one() && !getenv("HSAW_HIST") && peak_cluster() && in_stream < 0xFFFFFFFFll &&
       count < 0xFFFFFFFFll && counts_by_id(M, cv.about)) {
     cv.short_walks = in_stream < 16 * st.count;

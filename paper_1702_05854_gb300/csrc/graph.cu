@@ -21,10 +21,20 @@ hsaw_status fail(hsaw_status st, const std::string& msg) {
   t_err = msg;
   return st;
 }
+static thread_local bool t_lean = false, t_refused = false;  // the allocator had no memory
+bool lean() { return t_lean; }
+bool begin_lean(hsaw_status st) {
+  const bool again = st == HSAW_E_NOMEM && t_refused && !t_lean;
+  t_refused = false;
+  if (again) t_lean = true;
+  return again;
+}
+LeanEnd::~LeanEnd() { t_lean = false; }
 hsaw_status cuda_fail(cudaError_t e, const char* what, const char* file, int line) {
   char buf[512];
   snprintf(buf, sizeof(buf), "%s failed: %s (%s:%d)", what, cudaGetErrorString(e), file, line);
   t_err = buf;
+  if (e == cudaErrorMemoryAllocation) t_refused = true;
   return (e == cudaErrorMemoryAllocation) ? HSAW_E_NOMEM : HSAW_E_DEVICE;
 }
 
@@ -49,11 +59,12 @@ static hsaw_status allocate(void** p, size_t bytes, cudaStream_t s);
 
 Slab::Slab(cudaStream_t s) : s_(s), outer_(t_slab) {
   void* p = nullptr;
-  if (allocate(&p, BYTES, s) == HSAW_OK) {
+  if (!lean() && allocate(&p, BYTES, s) == HSAW_OK) {
     base_ = static_cast<char*>(p);
     cap_ = BYTES;
   } else {
     set_error("");  // small buffers are then allocated one by one
+    t_refused = false;
   }
   t_slab = this;
 }
@@ -75,6 +86,7 @@ void* Slab::cut(size_t bytes, cudaStream_t s) {
 hsaw_status dmalloc(void** p, size_t bytes, cudaStream_t s) {
   if (g_fail_countdown.load(std::memory_order_relaxed) > 0 && g_fail_countdown.fetch_sub(1) == 1) {
     *p = nullptr;
+    t_refused = false;
     t_err = "device allocation failed (injected by hsaw_debug_fail_alloc_after)";
     return HSAW_E_NOMEM;
   }
@@ -88,6 +100,7 @@ static hsaw_status allocate(void** p, size_t bytes, cudaStream_t s) {
   if (const ScratchAllocator* a = g_alloc.load(std::memory_order_acquire)) {
     *p = a->alloc(bytes, (void*)s, a->ctx);
     if (!*p) {
+      t_refused = true;
       char buf[128];
       snprintf(buf, sizeof(buf), "device allocation of %zu bytes failed (caller's allocator)", bytes);
       t_err = buf;
@@ -109,6 +122,7 @@ static hsaw_status allocate(void** p, size_t bytes, cudaStream_t s) {
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
+    t_refused = true;
     char buf[128];
     snprintf(buf, sizeof(buf), "device allocation of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
     t_err = buf;
@@ -615,6 +629,7 @@ static hsaw_status finish_graph(Graph& g, uint32_t* row_start, uint32_t* d_err, 
     if (cudaMalloc((void**)&g.grec, (size_t)g.m * 2 * sizeof(uint4)) != cudaSuccess) {
       cudaGetLastError();
       g.grec = nullptr;
+      t_refused = true;
       return fail(HSAW_E_NOMEM, "graph: guide records do not fit in device memory");
     }
   }
@@ -656,7 +671,7 @@ static hsaw_status from_edges(int64_t n, int64_t m, const int32_t* src, const in
   HSAW_CK(cudaMemsetAsync(d_err, 0, 2 * sizeof(uint32_t), s));
   uint32_t *keys, *vals, *keys2, *vals2, *row_start;
   HSAW_TRY(T.get(&row_start, n + 1));
-  if (!overlap && m > 0 && n > 1) {  // the whole list is here: tails and weights ride along
+  if (!overlap && m > 0 && n > 1 && !lean()) {  // the whole list is here: tails and weights ride along
     HSAW_TRY(alloc_graph(g, n, m, true));
     uint2* pay = nullptr;
     uint32_t* sorted = nullptr;
@@ -800,10 +815,15 @@ hsaw_status hsaw_graph_from_edges(int64_t n, int64_t m, const int32_t* src, cons
   *out = nullptr;
   auto* h = new (std::nothrow) hsaw_graph_s();
   if (!h) return fail(HSAW_E_NOMEM, "graph: host allocation");
-  hsaw_status st = from_edges(n, m, src, dst, w_fixed, flags, (cudaStream_t)stream, h->g);
+  const hsaw_status st = within_memory([&] {
+    const hsaw_status r = from_edges(n, m, src, dst, w_fixed, flags, (cudaStream_t)stream, h->g);
+    if (r != HSAW_OK) {
+      cudaStreamSynchronize((cudaStream_t)stream);
+      destroy_graph(h->g);
+    }
+    return r;
+  });
   if (st != HSAW_OK) {
-    cudaStreamSynchronize((cudaStream_t)stream);
-    destroy_graph(h->g);
     delete h;
     return st;
   }

@@ -588,7 +588,7 @@ static hsaw_status sample_window(const Graph& g, const QueryDev& qd, Stream& st,
     HSAW_TRY(st.chunk_hits.ensure((size_t)SC_WORDS + n_chunks, s));
     HSAW_TRY(st.recs.ensure((size_t)n_chunks * cap, s));
     const double elements = st.count ? st.hit_rate * (double)batch * (double)st.total_nodes / (double)st.count : 0.0;
-    const bool keep = !st.ids_only && (st.count || !used) && (uint64_t)n_chunks * cap <= kept_records(elements);
+    const bool keep = !st.ids_only && !lean() && (st.count || !used) && (uint64_t)n_chunks * cap <= kept_records(elements);
     HSAW_TRY(st.chunk_kept.ensure(keep ? 2 * (size_t)n_chunks * cap : 0, s));
     uint32_t* const ctl = st.chunk_hits.p;
     HSAW_CK(cudaMemsetAsync(ctl, 0, ((size_t)SC_WORDS + n_chunks) * 4, s));
