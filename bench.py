@@ -39,13 +39,13 @@ BYTES_PER_STEP = 96  # three random 32-byte sectors per live-edge draw: node rec
 # DRAM bytes (read + write) per live-edge draw of the sampler kernel from an ncu capture,
 # keyed by (hash of the kernel's source, workload).  A workload without a capture of the
 # current kernel reports traffic = null.
-NCU_TRAFFIC = {("3ac37996ed07", "rmat23-wc-eSI"): 124.5,   # profiles/k_sample_rmat23_dram.md
-               ("3ac37996ed07", "rmat26-wc-eSI"): 124.5}   # the scale-23 figure, scaled by draws
+NCU_TRAFFIC = {("c1ffc424e282", "rmat23-wc-eSI"): 124.5,   # profiles/k_sample_rmat23_dram.md
+               ("c1ffc424e282", "rmat26-wc-eSI"): 124.5}   # the scale-23 figure, scaled by draws
 
 
 def sampler_hash():
-    """Hash of k_sample's own source text and the device helpers it calls (Philox, draws,
-    edge pick, checkpoints in common.cuh)."""
+    """Hash of k_sample's own source text and the device helpers it calls (in common.cuh: Philox, draws,
+    edge pick, checkpoints; record loads, quotient, guide lookup and steps through the walk tables)."""
     csrc = os.path.join(ROOT, "paper_1702_05854_gb300", "csrc")
     src = open(os.path.join(csrc, "sample.cu")).read()
     i = src.index("constexpr int SAMPLE_WARPS")
@@ -53,9 +53,11 @@ def sampler_hash():
     common = open(os.path.join(csrc, "common.cuh")).read()
     a = common.index("// ------------------------------------------------------------------ Philox4x32-10")
     b = common.index("// ------------------------------------------------------------------ primitives")
+    c = common.index("// ------------------------------------------------------------------ walk-record steps")
+    d = common.index("// Opaque handle types of the ABI.")
     h = hashlib.sha1()
-    h.update(src[i:j].encode())
-    h.update(common[a:b].encode())
+    for part in (src[i:j], common[a:b], common[c:d]):
+        h.update(part.encode())
     return h.hexdigest()[:12]
 
 
