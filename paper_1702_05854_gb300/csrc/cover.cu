@@ -224,8 +224,8 @@ hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t
   const int64_t M = st.elem_range[em ? 1 : 0];
   cv.about = (int64_t)((double)in_stream / (double)st.count * (double)count);
   cv.crowded = lean() || (k > 0 && all && M > 0 && crowded(M, cv.about, count, k));
-  if (k > 0 && !cv.crowded && !one_by_one() && !getenv("HSAW_HIST") && peak_cluster() && in_stream < 0xFFFFFFFFll &&
-      count < 0xFFFFFFFFll && counts_by_id(M, cv.about)) {
+  if (k > 0 && !cv.crowded && !one_by_one() && !getenv("HSAW_HIST") && peak_cluster() && in_stream <= MOST_ENTRIES &&
+      count <= MOST_ENTRIES && counts_by_id(M, cv.about)) {
     cv.short_walks = in_stream < 16 * st.count;
     cv.stream = &st;
     cv.mode = mode;
@@ -238,7 +238,7 @@ hsaw_status cover_build(const Stream& st, hsaw_mode mode, int64_t first, int64_t
   HSAW_CK(cudaMemcpyAsync(&nb[1], st.node_off.p + first + count, 8, cudaMemcpyDeviceToHost, s));
   HSAW_CK(cudaStreamSynchronize(s));
   const int64_t E64 = em ? (nb[1] - (first + count)) - (nb[0] - first) : nb[1] - nb[0];
-  if (E64 >= 0xFFFFFFFFll || count >= 0xFFFFFFFFll) return fail(HSAW_E_INVALID, "cover: too many walk elements");
+  if (E64 > MOST_ENTRIES || count > MOST_ENTRIES) return fail(HSAW_E_INVALID, "cover: too many walk elements");
   const uint32_t E = (uint32_t)E64;
   cv.entries = E;
   HSAW_TRY(cv.walk_eoff.ensure((size_t)count + 1, s));

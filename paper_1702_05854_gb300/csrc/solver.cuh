@@ -80,6 +80,10 @@ hsaw_status stream_take_hits(const Graph& g, const QueryDev& qd, Stream& st, uin
 hsaw_status classify_attempts(const Graph& g, const QueryDev& qd, uint64_t first, int64_t count, int8_t* outcome,
                               int32_t* length, cudaStream_t s);
 
+// Walks and walk elements that a Cover may have.  Its kernels count them in 32 bits and step by up to 2^21
+// at a time: a step past the end must not wrap, or a loop would never end.
+constexpr int64_t MOST_ENTRIES = (1ll << 32) - (1ll << 22);
+
 // Occurrence counts and inverted index over walks [first, first + count) (a5, a6).
 struct Cover {
   int64_t walks = 0, entries = 0, unique = 0;
