@@ -390,3 +390,96 @@ def test_greedy_leaves_long_lists(capfd, monkeypatch, name, count, k, route):
         assert rounds <= 1 if route == "left at once" else rounds > 2
     oids, ogains = ost.greedy(mode, 0, count, M, k, kept_gains=True)
     assert np.array_equal(gains, ogains) and np.array_equal(ids, oids)
+
+
+def greedy_of_one_list(capfd, monkeypatch, walks, ost, g, mode, M, count, k, mask):
+    """The greedy's launch record; its picks are the oracle's."""
+    monkeypatch.setenv("HSAW_LOG_LAUNCHES", "1")
+    capfd.readouterr()
+    ids, gains = hs.hsaw_greedy(walks, g, mode, 0, count, k, candidate_mask=mask)
+    run, = greedy_records(capfd.readouterr().err)
+    oids, ogains = ost.greedy(mode, 0, count, M, k, cand_mask=mask, kept_gains=True)
+    assert np.array_equal(gains, ogains) and np.array_equal(ids, oids)
+    return run
+
+
+# 512 threads a block up to 2^14 walks, 1,024 beyond; 16 pairs a thread
+@pytest.mark.parametrize("node,pairs,whole", [(0, 8191, True), (0, 8192, True), (0, 8193, False), (0, 16_383, False),
+                                              (1, 16_383, True), (1, 16_384, True), (1, 16_385, False)])
+def test_greedy_element_of_a_block(capfd, monkeypatch, node, pairs, whole):
+    """One element in as many walks as a thread block keeps, or one more or less: the suspect, on every walk of a path,
+    or the node before it."""
+    n = 10
+    src, dst = np.arange(n - 1, dtype=np.int32), np.arange(1, n, dtype=np.int32)
+    w = np.full(n - 1, ONE, np.uint32)
+    sources = np.array([0], np.int32)
+    g, og = hs.hsaw_graph_from_edges(n, src, dst, w), oracle.Graph(n, src, dst, w)
+    ost = oracle.Stream(oracle.Query(og, sources, seed=3)).extend(20_000)
+    length = np.diff(ost.export().node_off)
+    count = int(np.nonzero(np.cumsum(length > node) == pairs)[0][0]) + 1  # a walk of l nodes starts at node l - 1
+    assert node == 0 or count > 1 << 14
+    walks = hs.hsaw_sample(g, hs.Query(sources=sources, seed=3), 0, count)
+    mask = np.zeros(n, np.uint8)
+    mask[node] = 1
+    run = greedy_of_one_list(capfd, monkeypatch, walks, ost, g, hs.HSAW_NODE, n, count, 1, mask)
+    assert run["pairs"] == pairs and run["phases"] == 1 and run["owned"] == int(whole)
+
+
+@pytest.mark.parametrize("elements,whole", [(16 * 3072 - 1, True), (16 * 3072, True), (16 * 3072 + 1, False)])
+def test_greedy_elements_of_a_block(capfd, monkeypatch, elements, whole):
+    """As many elements of one walk each as the thread blocks keep, 3,072 a block, or one more or less."""
+    n, count = 200_000, 70_000
+    src, dst, w = np.array([0], np.int32), np.array([1], np.int32), np.array([1], np.uint32)
+    sources = np.arange(n, dtype=np.int32)
+    g, og = hs.hsaw_graph_from_edges(n, src, dst, w), oracle.Graph(n, src, dst, w)
+    ost = oracle.Stream(oracle.Query(og, sources, seed=3)).extend(count)
+    walks = hs.hsaw_sample(g, hs.Query(sources=sources, seed=3), 0, count)
+    once = np.nonzero(np.bincount(ost.export().nodes[:count], minlength=n) == 1)[0]
+    mask = np.zeros(n, np.uint8)
+    mask[once[:elements]] = 1
+    assert once.size >= elements
+    run = greedy_of_one_list(capfd, monkeypatch, walks, ost, g, hs.HSAW_NODE, n, count, 3200, mask)
+    assert run["pairs"] == elements and run["phases"] == 1 and run["owned"] == int(whole)
+
+
+def small_table_graph(kind):
+    """Graphs beyond the sizes that are walked through records (128 MB of L2): tails (152 MB of records), or edges and
+    guide (45 MB, random weights)."""
+    n, m = (400_003, 9_500_001) if kind == "tails" else (60_003, 700_001)
+    src, dst = synth.chung_lu_graph(n, m, 2.1, 6)
+    return n, src, dst, synth.wc_weights(n, dst) if kind == "tails" else synth.random_lt_weights(n, dst, 7)
+
+
+@pytest.fixture(scope="module", params=["tails", "edges"])
+def small_tables(request):
+    n, src, dst, w = small_table_graph(request.param)
+    return n, src.size, hs.hsaw_graph_from_edges(n, src, dst, w), oracle.Graph(n, src, dst, w)
+
+
+@pytest.mark.parametrize("kind", ["edge", "node", "both"])
+def test_small_tables_removal(small_tables, kind):
+    """Removed edges and nodes with the small walk tables, coins on or off."""
+    n, m, g, og = small_tables
+    rng = np.random.default_rng(4)
+    er = (rng.random(m) < 0.2).astype(np.uint8) if kind != "node" else None
+    nr = (rng.random(n) < 0.1).astype(np.uint8) if kind != "edge" else None
+    sources, p = synth.sources(n, n // 50, 8), synth.probabilities(n // 50, 9)
+    for coins in (None, p):
+        ost = oracle.Stream(oracle.Query(og, sources, p_fixed=coins, edge_removed=er, node_removed=nr, seed=2)).extend(3000)
+        walks = hs.hsaw_sample(g, hs.Query(sources=sources, p_fixed=coins, seed=2), 0, 3000, edge_removed=er, node_removed=nr)
+        assert_same_stream(walks, ost, 3000)
+
+
+@pytest.mark.parametrize("coins", [False, True])
+def test_small_tables_pool(small_tables, coins):
+    """Walk pools with the small walk tables: hits, lengths and walks, and the stream past the pool's end."""
+    n, m, g, og = small_tables
+    sources = synth.sources(n, n // 200, 8)
+    p = synth.probabilities(n // 200, 9) if coins else None
+    ost = oracle.Stream(oracle.Query(og, sources, p_fixed=p, seed=2)).extend_threads(6000, threads=8)
+    inside = int(ost.export().aid[3000])  # half of the hits lie in the pool
+    try:
+        g.build_walk_pool(2, inside)
+        assert_same_stream(hs.hsaw_sample(g, hs.Query(sources=sources, p_fixed=p, seed=2), 0, 6000), ost, 6000)
+    finally:
+        g.drop_walk_pool()
