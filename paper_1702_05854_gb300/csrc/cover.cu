@@ -1,12 +1,19 @@
 // Occurrence counting, inverted index, greedy max-coverage and out-of-sample coverage
 // over the ordered HSAW stream (Alg. 4 / 7 "Greedy", Alg. 5 line 2 "Cov_{R'_t}").
 //
-// The walk elements of a range of walks are sorted by element id with their entry
-// positions (stable radix sort): the runs give the touched elements in increasing id
-// with their occurrence counts, and the run contents are the inverted index element ->
-// walks.  Greedy runs k rounds in ONE cooperative launch: a grid-wide argmax of
-// (count, -index) packed in 64 bits (ties to the smallest id), then the picked
-// element's uncovered walks are marked and every element of those walks is decremented.
+// For the greedy the walk elements are counted by element id where that is the cheaper
+// (counts_by_id, peaks.cu).  Otherwise, and for hsaw_histogram, they are sorted by element id
+// with their entry positions (stable radix sort): the runs give the touched elements in
+// increasing id with their occurrence counts, and the run contents are the inverted index
+// element -> walks.
+//
+// cover_greedy takes its picks by peaks (peaks.cu), many at a time.  The greedies here take one
+// pick at a time: an argmax of (count, -index) packed in 64 bits (ties to the smallest id), then
+// the picked element's uncovered walks are marked and every element of those walks is
+// decremented.  They have the streams whose lists are too long for the greedy by peaks
+// (peak_pairs), calls that must do with little memory, and what the environment asks for:
+// k_greedy_onchip and k_greedy_cluster in one cluster, first on the elements that occur twice
+// or more, k_greedy on the whole grid where no cluster can be had.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 

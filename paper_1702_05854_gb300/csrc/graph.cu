@@ -576,6 +576,14 @@ struct Temps {
 // small ones do, or nearly.  Sampler, G draws/s, records against small tables, R-MAT edge
 // factor 16 (L2 129 MB): equal weights, scale 18 to 23: 171/135, 111/122, 70/98, 51/63, 44/46,
 // 40/36; random weights, scale 16 to 22: 78/84, 73/85, 65/82, 54/73, 46/58, 40/40, 36/30.
+// M attempts/s at other edge factors, records against small tables: equal weights, edge factor 4, scale
+// 21 to 24: 7168/7674, 5521/6712, 4588/5045, 3939/3648; 8, scale 20 to 24: 4586/4807, 3065/4024,
+// 2305/2747, 1998/2003, 1912/1631; 32, scale 18 to 22: 2615/3046, 1393/2117, 957/1396, 779/903, 620/607;
+// 64, scale 17 to 21: 2422/2753, 1297/2252, 874/1350, 666/813, 520/526.  Random weights, edge factor 4,
+// scale 18 to 23: 52808/55342, 48652/49642, 44449/51295, 37367/44164, 31268/32594, 27746/24153; 64, scale
+// 15 to 21: 23974/28090, 21248/27152, 18875/26483, 16529/22904, 15543/17713, 14644/13173, 14191/10589.
+// The rule takes the faster of the two or one within 4% of it at 73 of 76 sizes; right at 16 M = L2 it
+// leaves up to 17% (edge factor 32, scale 18).
 static Layout choose_layout(int64_t n, int64_t m, bool eq) {
   static const double l2 = [] {
     int dev = 0, bytes = 0;

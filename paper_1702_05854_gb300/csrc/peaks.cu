@@ -142,8 +142,8 @@ __device__ __forceinline__ bool own_part(const PeakParams& P, uint32_t n, OwnPar
 // One cluster, a thread per (element, walk) pair of the list; stamps and keys in global memory
 // (L2).  Bound by latency: the barriers of a round and the dependent L2 reads before each.
 //
-// Where whole elements of the list fit the CTAs (OwnPart: 2^18 pairs on 16 CTAs, less what the
-// division at elements costs), an element's walks are looked at by one CTA alone: its count is
+// Where whole elements of the list fit the CTAs (OwnPart: 16 pairs a thread, 2^18 on 16 CTAs of 1,024
+// threads and 2^17 of 512, less what the division at elements costs; 3,072 elements a CTA), an element's walks are looked at by one CTA alone: its count is
 // that of its pairs whose walk has no stamp, so no pick takes counts down walk entry by walk
 // entry (k_take_down does that for all of a phase's walks if another phase follows), and whether
 // it is a peak is settled within the CTA, which leaves two cluster barriers a round of three.
@@ -650,7 +650,9 @@ int peak_cluster() {
 // Threads of a CTA.  Fewer warps meet at a barrier sooner, and have half the loads in flight and half
 // the room for whole elements: 512 threads against 1,024 on 5.3 K walks 266 against 298 us (stopping
 // rule query 677 against 730 us), 7-28 K walks of a pool 91-102 against 94-106, 55-222 K walks
-// 107-143 against 103-137; 32 instances of 20 K walks at once 7.47 against 7.08 ms.
+// 107-143 against 103-137; 32 instances of 20 K walks at once 7.47 against 7.08 ms.  The line lies
+// below those instances: side by side they share the SMs, and there the fewer warps cost more than the
+// barriers gain, while 20-28 K walks alone gain at most a few us.
 static unsigned peak_threads(int64_t walks) { return walks <= (1 << 14) ? 512 : 1024; }
 uint64_t peak_room(int64_t walks) { return (uint64_t)peak_cluster() * peak_threads(walks) * OWN_PAIRS; }
 
