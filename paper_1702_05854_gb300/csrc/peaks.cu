@@ -163,13 +163,14 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
   const uint32_t gtid = rank * blockDim.x + threadIdx.x, threads = C * blockDim.x;
   const uint32_t gwarp = gtid >> 5, warps = threads >> 5;
   const uint32_t n = __ldcg(&P.ctl[PC_LIST]);
-  const uint32_t keep = __ldcg(&P.ctl[PC_KEEP]);
   // the host makes room and comes back, or leaves it
-  if (n > min(P.pair_cap, max(keep, P.room)) || __ldcg(&P.ctl[PC_LIST + 1]) > P.list_cap) return;
+  if (n > min(P.pair_cap, max(__ldcg(&P.ctl[PC_KEEP]), P.room)) || __ldcg(&P.ctl[PC_LIST + 1]) > P.list_cap) return;
   const uint32_t* __restrict__ entry = P.entry + (P.from ? *P.from - P.from_sub : 0);
   const uint32_t stripe = (n + 31) / 32;
   const uint32_t floor_gain = __ldcg(&P.ctl[PC_FLOOR]);
   __shared__ OwnPart O;
+  __shared__ uint32_t s_picks;  // of earlier phases
+  if (threadIdx.x == 0) s_picks = __ldcg(&P.ctl[PC_PICKS]);
   if (threadIdx.x < 32) s_red[threadIdx.x] = 0u;  // a block may have fewer than 32 warps
   const bool owned = own_part(P, n, O, cluster);
   uint32_t walk[OWN_PAIRS], el2[OWN_PAIRS / 2] = {}, alive = 0;  // this thread's pairs; elements in 16 bits
@@ -204,14 +205,13 @@ __global__ void __launch_bounds__(1024, 1) k_greedy_peaks(const __grid_constant_
   }
   uint32_t picks = 0, g = 0, r = P.round0;
   bool stuck = false, left = false;
-  const uint32_t picks0 = __ldcg(&P.ctl[PC_PICKS]);
   for (;;) {
     ++r;
     picks = __ldcg(&P.ctl[PC_PICKS]);
-    if (!owned &&
-        (n > keep || (uint64_t)n * (r - P.round0) > 16ull * keep + (picks - picks0) * PEAK_PICK)) {
-      left = true;  // the same decision in every CTA
-      break;
+    if (!owned) {
+      const uint64_t keep = __ldcg(&P.ctl[PC_KEEP]);
+      left = n > keep || (uint64_t)n * (r - P.round0) > 16 * keep + (picks - s_picks) * PEAK_PICK;
+      if (left) break;  // the same decision in every CTA
     }
     // 1. elements at or above the floor sign their keys on their uncovered walks; the largest
     // count
